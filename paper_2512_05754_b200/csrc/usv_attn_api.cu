@@ -87,9 +87,16 @@ static int sparse_attn_impl(int B, int H, int N, int d, const void* q, const usv
     const float sc = scale == 0.f ? 1.0f / sqrtf((float)d) : scale;
     a.scale_log2 = sc * 1.4426950408889634f;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // the status word (word 0) is sticky; everything behind it starts at zero (the pairing-plan
-    // kernel does that itself: a memset between two kernels costs them their overlapped launch)
-    if (impl == 0 && attn_pair_supported(a, d)) {
+    // The status word (word 0) is sticky; everything behind it starts at zero (the first kernel of
+    // either path does that itself: a memset between two kernels costs them their overlapped launch).
+    //
+    // Small calls at d = 64 go to the mma.sync kernel alone: one launch instead of three and no
+    // pairing plan, and with all its CTAs resident at once it takes ~4 us + 1.5 us per kept key block,
+    // where plan + tcgen05 kernel + exact-list kernel take 15-25 us before the lists matter.
+    // Measured (us, mma.sync / tcgen05 path), keep 4 to 8: 32 query blocks 10 / 17, 128: 16 / 22,
+    // 384: 21 / 25, 512: 35 / 28; keep 16, 32 query blocks: 27 / 16.
+    const bool small = d == 64 && kmx <= 8 && (int64_t)B * H * NB <= 384;
+    if (impl == 0 && !small && attn_pair_supported(a, d)) {
         int rc2 = launch_pair_plan(a, plan_mem, st);
         if (rc2 != USV_OK) return rc2;
         rc2 = launch_attn_pair(a, d, st);
@@ -102,8 +109,6 @@ static int sparse_attn_impl(int B, int H, int N, int d, const void* q, const usv
         return launch_scatter_fallbacks(a, d, st);
     }
     if (y != nullptr) return fail(USV_ERR_UNSUPPORTED, "sparse_attn_unmerge: sequence too long for the tcgen05 kernel");
-    cudaError_t e = cudaMemsetAsync(static_cast<char*>(ws) + 4, 0, WS_HEADER - 4, st);
-    if (e != cudaSuccess) return fail(USV_ERR_CUDA, "sparse_attn: memset: %s", cudaGetErrorString(e));
     return launch_attn_mma(a, d, st);
 }
 

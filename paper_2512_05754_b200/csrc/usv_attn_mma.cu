@@ -1,7 +1,8 @@
 // Block-sparse attention forward, legacy tensor-core path (mma.sync m16n8k16, bf16).
 //
-// Kept as an on-device cross-check of the tcgen05 kernel and as the fallback for shapes the
-// tcgen05 kernel does not cover.  One CTA (4 warps) per (b, h, query block); each warp owns 16
+// The faster path for small calls (usv_attn_api.cu says where the line lies), the exact recomputation
+// of the query blocks the tcgen05 kernel reports, the path beyond its longest sequence, and an
+// on-device cross-check of it.  One CTA (4 warps) per (b, h, query block); each warp owns 16
 // query rows.  Selected K/V blocks stream through a double-buffered cp.async pipeline; S = QK^T
 // and O += PV run on mma.sync with the softmax kept in registers (fp32, base-2 exponentials).
 #include "usv_mma_sync.cuh"
@@ -227,6 +228,8 @@ __global__ void __launch_bounds__(128) attn_mma_kernel(const AttnArgs a) {
     dep_sync();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if (a.work_list == nullptr) {
+        // the words behind the sticky status word (fallback count, work counter, ...) start at zero
+        if (blockIdx.x == 0 && threadIdx.x < (WS_HEADER - 4) / 4) a.status[1 + threadIdx.x] = 0u;
         attn_mma_block<D>(a, blockIdx.x, smem_raw);
         return;
     }

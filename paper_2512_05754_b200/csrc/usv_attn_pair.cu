@@ -1,4 +1,5 @@
-// Block-sparse attention forward on the 5th-generation tensor cores (tcgen05 + TMEM + TMA).
+// Block-sparse attention forward on the 5th-generation tensor cores (tcgen05 + TMEM + TMA), head
+// width D = 64 or 128.
 //
 // Formulation.  The selection is per 64-row query block, but the tensor-core datapath is 128 rows
 // high and a K/V tile costs as much shared-memory bandwidth to stage as to multiply.  One work
@@ -7,7 +8,7 @@
 // per tile:
 //
 //     S[128 q x 128 keys]  = Q . K_tile^T      tcgen05.mma, A = Q in smem,        B = K in smem
-//     O[128 q x 128 d]    += P . V_tile        tcgen05.mma, A = P (bf16) in TMEM, B = V in smem
+//     O[128 q x D]        += P . V_tile        tcgen05.mma, A = P (bf16) in TMEM, B = V in smem
 //
 // A key block that only one of the two lists holds is masked for the other half of the rows
 // (its softmax weights are written as zero), so the result is exactly the per-block selection.
@@ -55,35 +56,51 @@ namespace pr {
 
 using namespace t5;
 
-constexpr int D = 128;
 constexpr int KT = 2 * USV_BLOCK;               // keys per tile = two key blocks
 constexpr int NWG = 4;                          // softmax warpgroups
-constexpr int KSTAGES = 2;                      // K tile stages
 constexpr int VSTAGES = 3;                      // V tile stages
 constexpr int SBUF = 3;                         // S/P buffers in TMEM
 constexpr int NSLOT = 4;                        // item ring
 constexpr int LCAP = 512;                       // list entries a ring slot holds (longer lists are read from global memory)
 constexpr int MAX_NB = 4096;                    // key blocks per sequence this kernel covers
-constexpr uint32_t TILE_BYTES = KT * D * 2;     // 32 KB: [d-half][128 keys][128 B]
-constexpr uint32_t SM_Q = 0;                    // the item's 128 query rows, same layout as a K tile
-constexpr uint32_t SM_K = SM_Q + TILE_BYTES;
-constexpr uint32_t SM_V = SM_K + KSTAGES * TILE_BYTES;
-constexpr uint32_t SM_BAR = SM_V + VSTAGES * TILE_BYTES;
-// barrier slots (8 bytes each)
-enum { B_QFULL = 0, B_QFREE, B_KFULL, B_KEMPTY = B_KFULL + KSTAGES, B_VFULL = B_KEMPTY + KSTAGES,
-       B_VEMPTY = B_VFULL + VSTAGES, B_SFULL = B_VEMPTY + VSTAGES, B_PFULL = B_SFULL + 2 * SBUF,
-       B_OFULL = B_PFULL + 2 * SBUF, B_OFREE, B_SUMS, B_REF = B_SUMS + NSLOT, B_IFULL = B_REF + 2 * NSLOT,
-       B_IFREE = B_IFULL + NSLOT, B_COUNT = B_IFREE + NSLOT };
-static_assert(B_COUNT <= 48, "barrier area");
-constexpr uint32_t SM_MISC = SM_BAR + 8 * 48;            // tmem base, abort flag
-constexpr uint32_t SM_FLAG = SM_MISC + 16;               // int[NSLOT][2]: a row of this side left the safe range
-constexpr uint32_t SM_REFV = SM_MISC + 64;               // float[NSLOT][128]: minus the softmax reference per row
-constexpr uint32_t SM_SUM = SM_REFV + NSLOT * 128 * 4;   // float[NSLOT][NWG][128]: partial row sums
-constexpr uint32_t SM_ITEM = SM_SUM + NSLOT * NWG * 128 * 4;   // NSLOT x { int hdr[16]; int list[LCAP]; }
 constexpr uint32_t ITEM_BYTES = 64 + LCAP * 4;
-constexpr uint32_t SM_TOTAL = SM_ITEM + NSLOT * ITEM_BYTES;
-constexpr size_t SMEM_BYTES = SM_TOTAL + 1024;           // + slack for 1024-byte alignment
-static_assert(SMEM_BYTES <= 232448, "shared memory budget");
+
+// What depends on the head width.  At D = 128 a tile's MMAs (1024 cycles) and its traffic through
+// shared memory (1280 cycles) bound it; at D = 64 both halve and the 128 x 128 exponentials (1024
+// cycles at 16 a clock) are the bound.  24 heads of 32 760 tokens at D = 64, keep 52 of 512: 1.05 ms
+// a call (640 TFLOP/s), 3.00 ms on the mma.sync kernel that served D = 64 before.  A 128-key tile of one operand is D / 64 column halves of
+// [128 keys][128 B]: 32 KB at D = 128, 16 KB at D = 64, where the shared memory left over holds
+// two more K stages (a stage takes ~1700 cycles to arrive, longer than the two tiles that
+// two stages cover at the shorter tiles of D = 64).
+template <int D>
+struct Cfg {
+    static constexpr int NH = D / 64;               // column halves of a tile
+    static constexpr int KSTAGES = D == 64 ? 4 : 2; // K tile stages
+    static constexpr uint32_t TILE_BYTES = KT * D * 2;
+    // A NaN or infinity in V of a key block that only one side selected reaches the other side's rows
+    // as 0 * inf.  At D = 64 such rows are handed to the exact kernel; at D = 128, where the interface
+    // says that they may occur, the check would cost items of one tile 1.7 % (32 more operations
+    // per row and quarter before the accumulator goes back).
+    static constexpr bool CHECK_FINITE = D == 64;
+    static constexpr uint32_t SM_Q = 0;             // the item's 128 query rows, same layout as a K tile
+    static constexpr uint32_t SM_K = SM_Q + TILE_BYTES;
+    static constexpr uint32_t SM_V = SM_K + KSTAGES * TILE_BYTES;
+    static constexpr uint32_t SM_BAR = SM_V + VSTAGES * TILE_BYTES;
+    // barrier slots (8 bytes each)
+    enum { B_QFULL = 0, B_QFREE, B_KFULL, B_KEMPTY = B_KFULL + KSTAGES, B_VFULL = B_KEMPTY + KSTAGES,
+           B_VEMPTY = B_VFULL + VSTAGES, B_SFULL = B_VEMPTY + VSTAGES, B_PFULL = B_SFULL + 2 * SBUF,
+           B_OFULL = B_PFULL + 2 * SBUF, B_OFREE, B_SUMS, B_REF = B_SUMS + NSLOT, B_IFULL = B_REF + 2 * NSLOT,
+           B_IFREE = B_IFULL + NSLOT, B_COUNT = B_IFREE + NSLOT };
+    static_assert(B_COUNT <= 56, "barrier area");
+    static constexpr uint32_t SM_MISC = SM_BAR + 8 * 56;            // tmem base, abort flag
+    static constexpr uint32_t SM_FLAG = SM_MISC + 16;               // int[NSLOT][2]: this side goes to the exact kernel
+    static constexpr uint32_t SM_REFV = SM_MISC + 64;               // float[NSLOT][128]: minus the softmax reference per row
+    static constexpr uint32_t SM_SUM = SM_REFV + NSLOT * 128 * 4;   // float[NSLOT][NWG][128]: partial row sums
+    static constexpr uint32_t SM_ITEM = SM_SUM + NSLOT * NWG * 128 * 4;   // NSLOT x { int hdr[16]; int list[LCAP]; }
+    static constexpr uint32_t SM_TOTAL = SM_ITEM + NSLOT * ITEM_BYTES;
+    static constexpr size_t SMEM_BYTES = SM_TOTAL + 1024;           // + slack for 1024-byte alignment
+    static_assert(SMEM_BYTES <= 232448, "shared memory budget");
+};
 // item header words
 enum { I_T = 0, I_NU, I_B, I_H, I_BH, I_IA, I_IB, I_SREFA, I_SREFB, I_LIST_LO, I_LIST_HI };
 
@@ -133,20 +150,24 @@ __device__ __forceinline__ const int* item_list(const int* hdr) {
                                                             (unsigned)hdr[I_LIST_LO]);
 }
 
+template <int D>
 __global__ void __launch_bounds__(NTHREADS, 1)
 attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
+    using F = Cfg<D>;
+    constexpr int KSTAGES = F::KSTAGES;
+    constexpr uint32_t TILE_BYTES = F::TILE_BYTES;
     dep_launch();   // the set-up below touches shared and tensor memory only; dep_wait() follows it
     extern __shared__ unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     unsigned char* sm = smem_raw + (base - raw);
-    auto bar = [&](int i) { return base + SM_BAR + 8u * i; };
-    volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(sm + SM_MISC);
-    volatile int* s_abort = reinterpret_cast<volatile int*>(sm + SM_MISC + 4);
-    int* s_flag = reinterpret_cast<int*>(sm + SM_FLAG);
-    float* s_refv = reinterpret_cast<float*>(sm + SM_REFV);
-    float* s_sum = reinterpret_cast<float*>(sm + SM_SUM);
-    auto hdr_of = [&](int n) { return reinterpret_cast<int*>(sm + SM_ITEM + (n % NSLOT) * ITEM_BYTES); };
+    auto bar = [&](int i) { return base + F::SM_BAR + 8u * i; };
+    volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(sm + F::SM_MISC);
+    volatile int* s_abort = reinterpret_cast<volatile int*>(sm + F::SM_MISC + 4);
+    int* s_flag = reinterpret_cast<int*>(sm + F::SM_FLAG);
+    float* s_refv = reinterpret_cast<float*>(sm + F::SM_REFV);
+    float* s_sum = reinterpret_cast<float*>(sm + F::SM_SUM);
+    auto hdr_of = [&](int n) { return reinterpret_cast<int*>(sm + F::SM_ITEM + (n % NSLOT) * ITEM_BYTES); };
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int NB = a.NB, N = a.N;
@@ -154,14 +175,14 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
     const int64_t nitems = (int64_t)a.B * a.H * NP;
 
     // ---- set-up: barriers (one per thread of the first two warps), TMEM
-    if (threadIdx.x < B_COUNT) {
+    if (threadIdx.x < F::B_COUNT) {
         const int i = threadIdx.x;
         uint32_t count = 1;                                      // Q, K/V stages, SFULL, OFULL, IFULL
-        if (i >= B_PFULL && i < B_PFULL + 2 * SBUF) count = 8;   // one per warp of a tile's two groups
-        if (i == B_OFREE) count = 4;                             // one per output warp
-        if (i >= B_SUMS && i < B_SUMS + NSLOT) count = NSOFT / 32;
-        if (i >= B_REF && i < B_REF + 2 * NSLOT) count = 2;      // the two warps of the owning group on a side
-        if (i >= B_IFREE && i < B_IFREE + NSLOT) count = 4;      // the output warps read a slot last
+        if (i >= F::B_PFULL && i < F::B_PFULL + 2 * SBUF) count = 8;   // one per warp of a tile's two groups
+        if (i == F::B_OFREE) count = 4;                             // one per output warp
+        if (i >= F::B_SUMS && i < F::B_SUMS + NSLOT) count = NSOFT / 32;
+        if (i >= F::B_REF && i < F::B_REF + 2 * NSLOT) count = 2;      // the two warps of the owning group on a side
+        if (i >= F::B_IFREE && i < F::B_IFREE + NSLOT) count = 4;      // the output warps read a slot last
         mbar_init(bar(i), count);
         if (i == 0) *s_abort = 0;
         if (i < 2 * NSLOT) s_flag[i] = 0;
@@ -169,7 +190,7 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
     }
     if (warp == W_MMA) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"(base + SM_MISC), "r"(TMEM_COLS) : "memory");
+                     ::"r"(base + F::SM_MISC), "r"(TMEM_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     fence_before();
@@ -189,7 +210,7 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
         // publishing the end marker, -2 when a bounded wait gave up.
         auto publish = [&](int n) -> int {
             int* hdr = hdr_of(n);
-            if (n >= NSLOT && !mbar_wait(bar(B_IFREE + n % NSLOT), ((n / NSLOT) - 1) & 1, s_abort, a.status, 0x8000))
+            if (n >= NSLOT && !mbar_wait(bar(F::B_IFREE + n % NSLOT), ((n / NSLOT) - 1) & 1, s_abort, a.status, 0x8000))
                 return -2;
             for (;;) {
                 int wi = 0;
@@ -198,7 +219,7 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
                 if (w >= nitems) {
                     if (lane == 0) hdr[I_T] = -1;
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(bar(B_IFULL + n % NSLOT));
+                    if (lane == 0) mbar_arrive(bar(F::B_IFULL + n % NSLOT));
                     return -1;
                 }
                 const int pair = (int)(w % NP);
@@ -256,7 +277,7 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
                     s_flag[(n % NSLOT) * 2 + 1] = 0;
                 }
                 __syncwarp();
-                if (lane == 0) mbar_arrive(bar(B_IFULL + n % NSLOT));
+                if (lane == 0) mbar_arrive(bar(F::B_IFULL + n % NSLOT));
                 return (nU + 1) >> 1;
             }
         };
@@ -264,15 +285,16 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
         auto load_q = [&](int m) -> bool {
             const int* hdr = hdr_of(m);
             const int b = hdr[I_B], h = hdr[I_H], IA = hdr[I_IA], IB = hdr[I_IB];
-            if (m >= 1 && !mbar_wait(bar(B_QFREE), (m - 1) & 1, s_abort, a.status, 0x4000)) return false;
+            if (m >= 1 && !mbar_wait(bar(F::B_QFREE), (m - 1) & 1, s_abort, a.status, 0x4000)) return false;
             if (elect_one()) {
                 // a block without a partner reads rows past the end (zero fill)
                 const int ra = IA * USV_BLOCK, rb = (IB >= 0 ? IB : NB) * USV_BLOCK;
-                mbar_expect_tx(bar(B_QFULL), TILE_BYTES);
-                tma_load_4d(base + SM_Q, &maps.q, bar(B_QFULL), 0, ra, h, b);
-                tma_load_4d(base + SM_Q + 8192, &maps.q, bar(B_QFULL), 0, rb, h, b);
-                tma_load_4d(base + SM_Q + 16384, &maps.q, bar(B_QFULL), 64, ra, h, b);
-                tma_load_4d(base + SM_Q + 24576, &maps.q, bar(B_QFULL), 64, rb, h, b);
+                mbar_expect_tx(bar(F::B_QFULL), TILE_BYTES);
+#pragma unroll
+                for (int hf = 0; hf < F::NH; ++hf) {
+                    tma_load_4d(base + F::SM_Q + hf * 16384, &maps.q, bar(F::B_QFULL), hf * 64, ra, h, b);
+                    tma_load_4d(base + F::SM_Q + hf * 16384 + 8192, &maps.q, bar(F::B_QFULL), hf * 64, rb, h, b);
+                }
             }
             __syncwarp();
             return true;
@@ -300,14 +322,15 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
                 const uint32_t ph = (g / KSTAGES) & 1;
                 const int J0 = list[2 * t] >> 2;
                 const int J1 = (2 * t + 1 < nU) ? (list[2 * t + 1] >> 2) : J0;  // odd tail: finite filler, masked
-                if (!mbar_wait(bar(B_KEMPTY + s), ph ^ 1, s_abort, a.status, 0x1)) { ok = false; break; }
-                const uint32_t dst = base + SM_K + s * TILE_BYTES;
+                if (!mbar_wait(bar(F::B_KEMPTY + s), ph ^ 1, s_abort, a.status, 0x1)) { ok = false; break; }
+                const uint32_t dst = base + F::SM_K + s * TILE_BYTES;
                 if (elect_one()) {
-                    mbar_expect_tx(bar(B_KFULL + s), TILE_BYTES);
-                    tma_load_4d(dst, &maps.k, bar(B_KFULL + s), 0, J0 * USV_BLOCK, h, b);
-                    tma_load_4d(dst + 8192, &maps.k, bar(B_KFULL + s), 0, J1 * USV_BLOCK, h, b);
-                    tma_load_4d(dst + 16384, &maps.k, bar(B_KFULL + s), 64, J0 * USV_BLOCK, h, b);
-                    tma_load_4d(dst + 24576, &maps.k, bar(B_KFULL + s), 64, J1 * USV_BLOCK, h, b);
+                    mbar_expect_tx(bar(F::B_KFULL + s), TILE_BYTES);
+#pragma unroll
+                    for (int hf = 0; hf < F::NH; ++hf) {
+                        tma_load_4d(dst + hf * 16384, &maps.k, bar(F::B_KFULL + s), hf * 64, J0 * USV_BLOCK, h, b);
+                        tma_load_4d(dst + hf * 16384 + 8192, &maps.k, bar(F::B_KFULL + s), hf * 64, J1 * USV_BLOCK, h, b);
+                    }
                 }
                 __syncwarp();
                 // This item's Q rows follow its first K tile: the Q buffer comes free one S tile
@@ -327,7 +350,7 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REG_SERVICE));
         int g = 0;
         for (int n = 0;; ++n) {
-            if (!mbar_wait(bar(B_IFULL + n % NSLOT), (n / NSLOT) & 1, s_abort, a.status, 0x10000)) break;
+            if (!mbar_wait(bar(F::B_IFULL + n % NSLOT), (n / NSLOT) & 1, s_abort, a.status, 0x10000)) break;
             const int* hdr = hdr_of(n);
             const int T = hdr[I_T];
             if (T < 0) break;
@@ -340,14 +363,15 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
                 const uint32_t phv = (g / VSTAGES) & 1;
                 const int J0 = list[2 * t] >> 2;
                 const int J1 = (2 * t + 1 < nU) ? (list[2 * t + 1] >> 2) : J0;
-                if (!mbar_wait(bar(B_VEMPTY + sv), phv ^ 1, s_abort, a.status, 0x2)) { ok = false; break; }
-                const uint32_t dst = base + SM_V + sv * TILE_BYTES;
+                if (!mbar_wait(bar(F::B_VEMPTY + sv), phv ^ 1, s_abort, a.status, 0x2)) { ok = false; break; }
+                const uint32_t dst = base + F::SM_V + sv * TILE_BYTES;
                 if (elect_one()) {
-                    mbar_expect_tx(bar(B_VFULL + sv), TILE_BYTES);
-                    tma_load_4d(dst, &maps.v, bar(B_VFULL + sv), 0, J0 * USV_BLOCK, h, b);
-                    tma_load_4d(dst + 8192, &maps.v, bar(B_VFULL + sv), 0, J1 * USV_BLOCK, h, b);
-                    tma_load_4d(dst + 16384, &maps.v, bar(B_VFULL + sv), 64, J0 * USV_BLOCK, h, b);
-                    tma_load_4d(dst + 24576, &maps.v, bar(B_VFULL + sv), 64, J1 * USV_BLOCK, h, b);
+                    mbar_expect_tx(bar(F::B_VFULL + sv), TILE_BYTES);
+#pragma unroll
+                    for (int hf = 0; hf < F::NH; ++hf) {
+                        tma_load_4d(dst + hf * 16384, &maps.v, bar(F::B_VFULL + sv), hf * 64, J0 * USV_BLOCK, h, b);
+                        tma_load_4d(dst + hf * 16384 + 8192, &maps.v, bar(F::B_VFULL + sv), hf * 64, J1 * USV_BLOCK, h, b);
+                    }
                 }
                 __syncwarp();
             }
@@ -362,20 +386,20 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
         // of that tile says so to the V producer and to the S issuer alike).
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REG_SERVICE));
         constexpr uint32_t IDESC_O = instr_desc(128, D, 0, 1);     // P (TMEM) x V (MN-major)
-        const uint64_t vdesc0 = smem_desc(base + SM_V, 16384, 1024);
+        const uint64_t vdesc0 = smem_desc(base + F::SM_V, 16384, 1024);
         int g = 0;                               // running tile
         int p_v = 0, p_buf = 0, p_b6 = 0;        // g % VSTAGES, g % SBUF, g % (2 SBUF)
         uint32_t p_vph = 0, p_ph6 = 0;           // (g / VSTAGES) & 1, (g / (2 SBUF)) & 1
         bool ok = true;
         for (int n = 0; ok; ++n) {
-            if (!mbar_wait(bar(B_IFULL + n % NSLOT), (n / NSLOT) & 1, s_abort, a.status, 0x10000)) break;
+            if (!mbar_wait(bar(F::B_IFULL + n % NSLOT), (n / NSLOT) & 1, s_abort, a.status, 0x10000)) break;
             const int T = hdr_of(n)[I_T];
             if (T < 0) break;
             for (int t = 0; t < T; ++t, ++g) {
-                if (!mbar_wait(bar(B_VFULL + p_v), p_vph, s_abort, a.status, 0x20)) { ok = false; break; }
-                if (!mbar_wait(bar(B_PFULL + p_b6), p_ph6, s_abort, a.status, 0x40)) { ok = false; break; }
+                if (!mbar_wait(bar(F::B_VFULL + p_v), p_vph, s_abort, a.status, 0x20)) { ok = false; break; }
+                if (!mbar_wait(bar(F::B_PFULL + p_b6), p_ph6, s_abort, a.status, 0x40)) { ok = false; break; }
                 // the first P.V of an item overwrites O: the item before must have been read out
-                if (t == 0 && n > 0 && !mbar_wait(bar(B_OFREE), (n - 1) & 1, s_abort, a.status, 0x2000)) { ok = false; break; }
+                if (t == 0 && n > 0 && !mbar_wait(bar(F::B_OFREE), (n - 1) & 1, s_abort, a.status, 0x2000)) { ok = false; break; }
                 fence_after();
                 const uint64_t vdesc = vdesc0 + ((p_v * TILE_BYTES) >> 4);
                 const uint32_t pb = tmem + TS + p_buf * 128;   // P: 32 columns at the head of each 64-column half
@@ -384,8 +408,8 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
                     for (int ks = 0; ks < KT / 16; ++ks)
                         umma_ts(tmem + TO, pb + (ks >> 2) * 64 + (ks & 3) * 8, vdesc + ((ks * 2048) >> 4), IDESC_O,
                                 (t > 0 || ks > 0));
-                    umma_commit(bar(B_VEMPTY + p_v));      // V stage free; S buffer p_buf free for S(g + 3)
-                    if (t == T - 1) umma_commit(bar(B_OFULL));
+                    umma_commit(bar(F::B_VEMPTY + p_v));      // V stage free; S buffer p_buf free for S(g + 3)
+                    if (t == T - 1) umma_commit(bar(F::B_OFULL));
                 }
                 __syncwarp();
                 if (++p_v == VSTAGES) { p_v = 0; p_vph ^= 1; }
@@ -398,21 +422,21 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REG_SERVICE));
         static_assert(VSTAGES == SBUF, "the V stage barrier of tile g doubles as the hand-back of S buffer g % SBUF");
         constexpr uint32_t IDESC_S = instr_desc(128, KT, 0, 0);    // Q (K-major) x K (K-major)
-        const uint64_t qdesc = smem_desc(base + SM_Q, 16, 1024);        // + byte offset >> 4
-        const uint64_t kdesc0 = smem_desc(base + SM_K, 16, 1024);
+        const uint64_t qdesc = smem_desc(base + F::SM_Q, 16, 1024);        // + byte offset >> 4
+        const uint64_t kdesc0 = smem_desc(base + F::SM_K, 16, 1024);
         int g = 0;
         int s_k = 0, s_buf = 0, s_b6 = 0;      // g % KSTAGES, g % SBUF, g % (2 SBUF)
         uint32_t s_kph = 0, s_bph = 1;         // (g / KSTAGES) & 1; parity of the hand-back of buffer s_buf: ((g / SBUF) & 1) ^ 1
         bool ok = true;
         for (int n = 0; ok; ++n) {
-            if (!mbar_wait(bar(B_IFULL + n % NSLOT), (n / NSLOT) & 1, s_abort, a.status, 0x10000)) break;
+            if (!mbar_wait(bar(F::B_IFULL + n % NSLOT), (n / NSLOT) & 1, s_abort, a.status, 0x10000)) break;
             const int T = hdr_of(n)[I_T];
             if (T < 0) break;
-            if (!mbar_wait(bar(B_QFULL), n & 1, s_abort, a.status, 0x4)) break;
+            if (!mbar_wait(bar(F::B_QFULL), n & 1, s_abort, a.status, 0x4)) break;
             for (int t = 0; t < T; ++t, ++g) {
-                if (!mbar_wait(bar(B_KFULL + s_k), s_kph, s_abort, a.status, 0x8)) { ok = false; break; }
+                if (!mbar_wait(bar(F::B_KFULL + s_k), s_kph, s_abort, a.status, 0x8)) { ok = false; break; }
                 // buffer s_buf held P(g - 3): P.V(g - 3) must be complete
-                if (g >= SBUF && !mbar_wait(bar(B_VEMPTY + s_buf), s_bph, s_abort, a.status, 0x100)) { ok = false; break; }
+                if (g >= SBUF && !mbar_wait(bar(F::B_VEMPTY + s_buf), s_bph, s_abort, a.status, 0x100)) { ok = false; break; }
                 fence_after();
                 const uint64_t kdesc = kdesc0 + ((s_k * TILE_BYTES) >> 4);
                 const uint32_t d_s = tmem + TS + s_buf * 128;
@@ -422,9 +446,9 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
                         const uint32_t off = ((ks >> 2) * 16384 + (ks & 3) * 32) >> 4;
                         umma_ss(d_s, qdesc + off, kdesc + off, IDESC_S, ks > 0);
                     }
-                    umma_commit(bar(B_SFULL + s_b6));
-                    umma_commit(bar(B_KEMPTY + s_k));             // its K stage may be refilled
-                    if (t == T - 1) umma_commit(bar(B_QFREE));    // and, after an item's last tile, the Q buffer
+                    umma_commit(bar(F::B_SFULL + s_b6));
+                    umma_commit(bar(F::B_KEMPTY + s_k));             // its K stage may be refilled
+                    if (t == T - 1) umma_commit(bar(F::B_QFREE));    // and, after an item's last tile, the Q buffer
                 }
                 __syncwarp();
                 if (++s_k == KSTAGES) { s_k = 0; s_kph ^= 1; }
@@ -440,29 +464,25 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
         const uint32_t lane_base = tmem + ((uint32_t)((warp - W_EPI) * 32) << 16);
         for (int m = 0;; ++m) {
             const int slot = m % NSLOT;
-            if (!mbar_wait(bar(B_IFULL + slot), (m / NSLOT) & 1, s_abort, a.status, 0x10000)) break;
+            if (!mbar_wait(bar(F::B_IFULL + slot), (m / NSLOT) & 1, s_abort, a.status, 0x10000)) break;
             const int* hdr = hdr_of(m);
             if (hdr[I_T] < 0) break;
             const int ib = hdr[I_B], ih = hdr[I_H], ibh = hdr[I_BH], iq = hdr[side ? I_IB : I_IA];
             const bool has_ref = hdr[side ? I_SREFB : I_SREFA] < hdr[I_NU];
             const int row = iq * USV_BLOCK + (e & 63);
             const bool live = iq >= 0 && row < N;
-            if (!mbar_wait(bar(B_SUMS + slot), (m / NSLOT) & 1, s_abort, a.status, 0x800)) break;
+            if (!mbar_wait(bar(F::B_SUMS + slot), (m / NSLOT) & 1, s_abort, a.status, 0x800)) break;
             const float* sums = s_sum + slot * (NWG * 128);
             float l = 0.f;
 #pragma unroll
             for (int q = 0; q < NWG; ++q) l += sums[q * 128 + e];
             const float nref = has_ref ? s_refv[slot * 128 + e] : 0.f;
             const bool in_range = l > 7.9e-31f && l < 1.2e30f;   // ~[2^-100, 2^100]
-            if (live && !in_range && a.fallback_list != nullptr && atomicExch(&s_flag[slot * 2 + side], 1) == 0) {
-                // first row of this query block to notice: hand the block to the exact kernel
-                const int fslot = atomicAdd(a.fallback_count, 1);
-                a.fallback_list[fslot] = ibh * NB + iq;
-            }
+            uint64_t z0 = 0, z1 = 0;   // four fp32 sums that stay 0 unless a value of the row is not finite
             const float inv = l > 0.f ? 1.0f / l : 0.f;
             if (a.lse != nullptr && live)
                 a.lse[((int64_t)ib * a.H + ih) * N + row] = (log2f(l) - nref) * 0.69314718055994531f;
-            if (!mbar_wait(bar(B_OFULL), m & 1, s_abort, a.status, 0x200)) break;
+            if (!mbar_wait(bar(F::B_OFULL), m & 1, s_abort, a.status, 0x200)) break;
             fence_after();
             // The row leaves TMEM a quarter (32 columns) at a time and is stored from registers; the
             // accumulator and the ring slot go back as soon as the last quarter has been read.
@@ -475,16 +495,33 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
                 u1 = a.unmerge_off[(int64_t)ib * (N + 1) + row + 1];
             }
 #pragma unroll 1
-            for (int qd = 0; qd < 4; ++qd) {
+            for (int qd = 0; qd < D / 32; ++qd) {
                 uint32_t r0[32];
                 tmem_ld32(lane_base + TO + qd * 32, r0);
                 tmem_wait_ld();
-                if (qd == 3) {
+#pragma unroll
+                for (int j = 0; F::CHECK_FINITE && j < 8; ++j) {
+                    z0 = fma_f32x2(pack_f32x2(__uint_as_float(r0[4 * j]), __uint_as_float(r0[4 * j + 1])), 0ull, z0);
+                    z1 = fma_f32x2(pack_f32x2(__uint_as_float(r0[4 * j + 2]), __uint_as_float(r0[4 * j + 3])), 0ull, z1);
+                }
+                if (qd == D / 32 - 1) {
+                    // A row whose sum left the safe range, or that is not finite (see CHECK_FINITE): the
+                    // first row of a query block to notice hands the block to the exact kernel, which
+                    // keeps query blocks apart.
+                    bool finite = true;
+                    if (F::CHECK_FINITE) {
+                        float za, zb;
+                        unpack_f32x2(add_f32x2(z0, z1), za, zb);
+                        finite = za + zb == 0.f;
+                    }
+                    if (live && !(in_range && finite) && a.fallback_list != nullptr &&
+                        atomicExch(&s_flag[slot * 2 + side], 1) == 0)
+                        a.fallback_list[atomicAdd(a.fallback_count, 1)] = ibh * NB + iq;
                     fence_before();
                     __syncwarp();
                     if (lane == 0) {
-                        mbar_arrive(bar(B_OFREE));
-                        mbar_arrive(bar(B_IFREE + slot));
+                        mbar_arrive(bar(F::B_OFREE));
+                        mbar_arrive(bar(F::B_IFREE + slot));
                     }
                 }
                 if (o32 != nullptr) {
@@ -531,7 +568,7 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
         unsigned refph = 0;     // bit s: phase of this side's reference barrier of ring slot s
         bool ok = true;
         for (int n = 0; ok; ++n) {
-            if (!mbar_wait(bar(B_IFULL + n % NSLOT), (n / NSLOT) & 1, s_abort, a.status, 0x10000)) { ok = false; break; }
+            if (!mbar_wait(bar(F::B_IFULL + n % NSLOT), (n / NSLOT) & 1, s_abort, a.status, 0x10000)) { ok = false; break; }
             const int* hdr = hdr_of(n);
             const int T = hdr[I_T];
             if (T < 0) break;
@@ -542,7 +579,7 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
             // block): the group that owns that slot fixes the row's softmax reference there and
             // publishes it; the other groups pick it up before their first later slot.
             const int sref = hdr[side ? I_SREFB : I_SREFA];
-            const uint32_t ref_bar = bar(B_REF + side * NSLOT + slot_n);
+            const uint32_t ref_bar = bar(F::B_REF + side * NSLOT + slot_n);
             const uint32_t ref_phase = (refph >> slot_n) & 1;
             float* refv = s_refv + slot_n * 128;
             float nref = 0.f;         // minus the softmax reference (base-2, scaled)
@@ -558,7 +595,7 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
                 const int b6 = gt % (2 * SBUF);
                 const uint32_t ph6 = (gt / (2 * SBUF)) & 1;
                 const uint32_t sbase = lane_base + TS + (gt % SBUF) * 128 + hb * 64;
-                if (!mbar_wait(bar(B_SFULL + b6), ph6, s_abort, a.status, 0x80)) { ok = false; break; }
+                if (!mbar_wait(bar(F::B_SFULL + b6), ph6, s_abort, a.status, 0x80)) { ok = false; break; }
                 fence_after();
                 if (!have_ref && sref < nU && slot >= sref) {   // (a side without any key block has sref = nU)
                     if (slot == sref) {
@@ -608,7 +645,7 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
                 tmem_wait_st();
                 fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(bar(B_PFULL + b6));
+                if (lane == 0) mbar_arrive(bar(F::B_PFULL + b6));
             }
             if (!ok) break;
             if (sref < nU) refph ^= 1u << slot_n;
@@ -616,7 +653,7 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
             unpack_f32x2(lr2, lr_lo, lr_hi);
             s_sum[slot_n * (NWG * 128) + grp * 128 + r] = lr_lo + lr_hi;
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar(B_SUMS + slot_n));
+            if (lane == 0) mbar_arrive(bar(F::B_SUMS + slot_n));
             g += T;
         }
     }
@@ -638,6 +675,8 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
 }
 
 // Fused unmerge: query blocks the exact kernel recomputed sit in o; copy them to their tokens in y.
+constexpr int DU = 128;   // head width the fused unmerge covers
+
 __global__ void __launch_bounds__(128) scatter_fallback_kernel(const AttnArgs a) {
     dep_sync();
     const int count = *a.fallback_count;
@@ -646,15 +685,15 @@ __global__ void __launch_bounds__(128) scatter_fallback_kernel(const AttnArgs a)
         const int id = a.fallback_list[w];
         const int I = id % NB, bh_ord = id / NB;
         const int b = bh_ord / a.H, h = a.head_order[bh_ord % a.H];
-        for (int idx = threadIdx.x; idx < USV_BLOCK * (D / 8); idx += 128) {
-            const int rr = idx / (D / 8), cc = idx % (D / 8);
+        for (int idx = threadIdx.x; idx < USV_BLOCK * (DU / 8); idx += 128) {
+            const int rr = idx / (DU / 8), cc = idx % (DU / 8);
             const int row = I * USV_BLOCK + rr;
             if (row >= N) continue;
             const uint4 val = *reinterpret_cast<const uint4*>(a.o + b * a.so.sb + h * a.so.sh + (int64_t)row * a.so.sn + cc * 8);
             const int u0 = a.unmerge_off[(int64_t)b * (N + 1) + row], u1 = a.unmerge_off[(int64_t)b * (N + 1) + row + 1];
             for (int u = u0; u < u1; ++u) {
                 const int tok = a.unmerge_idx[(int64_t)b * a.N_full + u];
-                *reinterpret_cast<uint4*>(a.y + ((int64_t)b * a.N_full + tok) * ((int64_t)a.H * D) + h * D + cc * 8) = val;
+                *reinterpret_cast<uint4*>(a.y + ((int64_t)b * a.N_full + tok) * ((int64_t)a.H * DU) + h * DU + cc * 8) = val;
             }
         }
     }
@@ -670,7 +709,26 @@ int launch_scatter_fallbacks(const AttnArgs& a, int d, cudaStream_t st) {
 }
 
 bool attn_pair_supported(const AttnArgs& a, int d) {
-    return d == pr::D && a.NB <= pr::MAX_NB && a.work_counter != nullptr;
+    return (d == 64 || d == 128) && a.NB <= pr::MAX_NB && a.work_counter != nullptr;
+}
+
+template <int D>
+static int launch_pair(const AttnArgs& a, int grid, const pr::Maps& maps, cudaStream_t st) {
+    cudaError_t e = cudaFuncSetAttribute(pr::attn_pair_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)pr::Cfg<D>::SMEM_BYTES);
+    if (e != cudaSuccess) return fail(USV_ERR_CUDA, "sparse_attn: smem attribute: %s", cudaGetErrorString(e));
+    // The roles redistribute the registers the CTA is launched with; a build whose launch count
+    // fell below what they ask for in total would leave the softmax warps waiting for registers
+    // that never come.  Refuse to launch such a build.
+    cudaFuncAttributes fa;
+    e = cudaFuncGetAttributes(&fa, pr::attn_pair_kernel<D>);
+    if (e != cudaSuccess) return fail(USV_ERR_CUDA, "sparse_attn: kernel attributes: %s", cudaGetErrorString(e));
+    if (fa.numRegs * (pr::NTHREADS / 32) < 16 * pr::REG_SOFT + 4 * pr::REG_EPI + 4 * pr::REG_SERVICE)
+        return fail(USV_ERR_UNSUPPORTED, "sparse_attn: kernel built with %d registers per thread, the roles need %d per lane",
+                    fa.numRegs, 16 * pr::REG_SOFT + 4 * pr::REG_EPI + 4 * pr::REG_SERVICE);
+    launch_dep(pr::attn_pair_kernel<D>, dim3(grid), dim3(pr::NTHREADS), pr::Cfg<D>::SMEM_BYTES, st, a, maps);
+    USV_CHECK_LAUNCH("attn_pair_kernel");
+    return USV_OK;
 }
 
 int launch_attn_pair(const AttnArgs& a, int d, cudaStream_t st) {
@@ -686,21 +744,7 @@ int launch_attn_pair(const AttnArgs& a, int d, cudaStream_t st) {
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
         return fail(USV_ERR_CUDA, "sparse_attn: cannot query the SM count");
     const int grid = (int)(items < sms ? items : sms);   // one persistent CTA per SM
-    cudaError_t e = cudaFuncSetAttribute(pr::attn_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)pr::SMEM_BYTES);
-    if (e != cudaSuccess) return fail(USV_ERR_CUDA, "sparse_attn: smem attribute: %s", cudaGetErrorString(e));
-    // The roles redistribute the registers the CTA is launched with; a build whose launch count
-    // fell below what they ask for in total would leave the softmax warps waiting for registers
-    // that never come.  Refuse to launch such a build.
-    cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, pr::attn_pair_kernel);
-    if (e != cudaSuccess) return fail(USV_ERR_CUDA, "sparse_attn: kernel attributes: %s", cudaGetErrorString(e));
-    if (fa.numRegs * (pr::NTHREADS / 32) < 16 * pr::REG_SOFT + 4 * pr::REG_EPI + 4 * pr::REG_SERVICE)
-        return fail(USV_ERR_UNSUPPORTED, "sparse_attn: kernel built with %d registers per thread, the roles need %d per lane",
-                    fa.numRegs, 16 * pr::REG_SOFT + 4 * pr::REG_EPI + 4 * pr::REG_SERVICE);
-    launch_dep(pr::attn_pair_kernel, dim3(grid), dim3(pr::NTHREADS), pr::SMEM_BYTES, st, a, maps);
-    USV_CHECK_LAUNCH("attn_pair_kernel");
-    return USV_OK;
+    return d == 64 ? launch_pair<64>(a, grid, maps, st) : launch_pair<128>(a, grid, maps, st);
 }
 
 }  // namespace usv

@@ -1,0 +1,62 @@
+"""The tcgen05 attention kernel where its head-width-64 form, and the hand-over of non-finite rows
+to the exact kernel, can go wrong; against the fp64 oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import usv_inputs as ui
+from parity_utils import attn_errors
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+MAX_ABS, REL_L2, REL_L2_BF16 = 2e-2, 1e-3, 2.5e-3
+
+
+@pytest.fixture(scope="module")
+def usv():
+    import paper_2512_05754_b200 as m
+    return m
+
+
+# an odd number of query blocks and a partial last block, k just above the small-call line; more
+# query blocks than that line with short lists; union lists beyond a ring slot (512 entries)
+@pytest.mark.parametrize("B,H,grid,kph", [(1, 1, (3, 9, 25), [9]), (2, 3, (5, 31, 33), [3, 1, 8]),
+                                          (1, 1, (9, 62, 66), [515])])
+def test_head_width_64(usv, B, H, grid, kph):
+    wl = ui.Workload("d64_edges", 170 + len(kph), B, H, 64, grid, (100,))
+    N, NB = wl.N, wl.NB
+    q, k, v = ui.make_qkv(wl, layout="bnhd")
+    rng = np.random.default_rng(NB)
+    sel = np.full((B, H, NB, max(kph)), -1, dtype=np.int32)
+    for b in range(B):
+        for h in range(H):
+            for i in range(NB):
+                sel[b, h, i, :kph[h]] = np.sort(rng.choice(NB, size=kph[h], replace=False))
+    o, o32, lse = usv.sparse_attn_fwd(q.to(DEV), k.to(DEV), v.to(DEV), torch.from_numpy(sel).to(DEV), kph, N=N,
+                                      return_f32=True, return_lse=True)
+    torch.cuda.synchronize()
+    assert usv.workspace_status() == 0 and usv.sparse_attn_fallbacks() == 0
+    o_ref, lse_ref = oracle.sparse_attn(q, k, v, N, sel, kph)
+    o_ref = o_ref.reshape(B, H, NB * 64, 64)[:, :, :N]
+    mx, rl2 = attn_errors(o32.cpu().numpy(), o_ref)
+    _, rl2b = attn_errors(o.float().cpu().numpy(), o_ref)
+    assert mx <= MAX_ABS and rl2 <= REL_L2 and rl2b <= REL_L2_BF16, (mx, rl2, rl2b)
+    assert np.abs(lse.cpu().numpy() - lse_ref.reshape(B, H, NB * 64)[:, :, :N]).max() <= 2e-3
+
+
+def test_an_infinity_reaches_only_the_query_blocks_that_selected_it(usv):
+    """Two query blocks share an item; the second one alone selects a block with an infinity in V.
+    Its own rows are not finite, its partner's equal the result without that block."""
+    N, NB, K, d = 64 * 12, 12, 9, 64
+    g = torch.Generator().manual_seed(d)
+    q, k, v = (torch.randn(1, 1, N, d, generator=g).to(torch.bfloat16) for _ in range(3))
+    v[:, :, 64 * 11 + 5, 3] = float("inf")
+    sel = torch.arange(K, dtype=torch.int32).expand(1, 1, NB, K).clone()
+    sel[0, 0, 1::2, K - 1] = 11
+    args = (q.to(DEV), k.to(DEV), v.to(DEV), sel.to(DEV), [K])
+    o = usv.sparse_attn_fwd(*args).float().cpu()[0, 0].reshape(NB, 64, d)
+    exact = usv.sparse_attn_fwd(*args, impl=1).float().cpu()[0, 0].reshape(NB, 64, d)
+    assert torch.isfinite(o[0::2]).all()
+    assert not torch.isfinite(o[1::2, :, 3]).any()
+    assert (o[0::2] - exact[0::2]).abs().max() <= MAX_ABS
