@@ -26,8 +26,8 @@ struct MatchTcArgs {
     Part p;
     int B, N, nA, nA_pad, nB_pad;
     const int32_t* src_idx;          // [nA] source tokens, ascending
-    uint16_t* a_h;                   // fp16 bits [B][nA_pad][128]
-    uint16_t* b_h;                   // fp16 bits [B][nB_pad][128]
+    uint16_t* a_h;                   // fp16 bits [B][nA_pad][dm]
+    uint16_t* b_h;                   // fp16 bits [B][nB_pad][dm]
     float* cand_v;                   // [B][nA][2][4] largest approximate cosines per source and tile parity, descending
     int* cand_i;                     // [B][nA][2][4] their destination ordinals
     int* exact_list;                 // sources (b * nA + rank) that need the fp32 scan of all destinations
@@ -41,9 +41,9 @@ struct MatchTcArgs {
 };
 
 // bytes of the matcher's scratch for a sequence of N tokens (any partition: sources + destinations = N)
-size_t match_tc_bytes(int B, int N);
-// mhat: fp32 unit descriptors [B,N,128]; mem: match_tc_bytes(B, N) bytes, 256-byte aligned.
-int launch_match_tc(const float* mhat, const Part& p, int B, int N, int nA, const int32_t* src_idx,
+size_t match_tc_bytes(int B, int N, int dm);
+// mhat: fp32 unit descriptors [B,N,dm], dm = 64 or 128; mem: match_tc_bytes(B, N, dm) bytes, 256-byte aligned.
+int launch_match_tc(const float* mhat, const Part& p, int B, int N, int nA, int dm, const int32_t* src_idx,
                     int32_t* jstar_s, float* u_s, void* mem, unsigned int* status, cudaStream_t st);
 
 }  // namespace usv

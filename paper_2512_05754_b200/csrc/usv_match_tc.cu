@@ -2,9 +2,9 @@
 // token the destination with the largest cosine, ties to the lowest destination.
 //
 // The cosines decide an integer (the arg-max) that is compared with an fp64 evaluation.  All
-// N_src x N_dst cosines are computed ONCE, from fp16 roundings of the fp32 unit descriptors
-// (8 tcgen05.mma, M = 128 sources, N = 128 destinations, K = 16, per 128 x 128 tile, fp32
-// accumulation), which are not exact but carry a rigorous bound: every component is off by at most
+// N_src x N_dst cosines are computed ONCE, from fp16 roundings of the fp32 unit descriptors of DM = 64
+// or 128 features (DM / 16 tcgen05.mma, M = 128 sources, N = 128 destinations, K = 16, per 128 x 128
+// tile, fp32 accumulation), which are not exact but carry a rigorous bound: every component is off by at most
 // 2^-11 relative, so a cosine of two unit vectors is off by at most sum|a_i b_i| (2^-10 + 2^-22)
 // <= 2^-10, plus ~1e-6 of accumulation: EPS = 1e-3.  The true best destination of a source
 // therefore has an approximate cosine within 2 EPS of the approximate row maximum.  Each source keeps
@@ -13,6 +13,9 @@
 // row would have chosen among them: ties to the lowest destination).  A source with a full list of
 // destinations inside the window (duplicates, near-duplicates) is handed to a plain fp32 scan of
 // all its destinations.  The result is the fp32 arg-max for every source, whatever the data.
+//
+// 21 076 sources against 7550 destinations at DM = 64: 852 us on fp32 CUDA cores, 72 us here (all four
+// kernels).
 //
 //   half_kernel         fp32 descriptors -> fp16 rows, sources (by rank) and destinations (by
 //                       ordinal) apart, zero-padded to multiples of 128 rows
@@ -36,33 +39,47 @@ namespace mt {
 
 using namespace t5;
 
-constexpr int DM = 128;
 constexpr int STAGES = 4;
 constexpr int NBUF = 3;                                 // accumulator tiles in TMEM: the hand-over of a tile between
                                                         // MMA issuer and epilogue takes longer than its MMAs
-constexpr uint32_t STAGE_BYTES = 128 * DM * 2;          // 32 KB: fp16 rows of a tile, [d-half][128 rows][128 B]
 constexpr int W_PROD = 8, W_MMA0 = 9;                   // warps 0-7: two epilogue warpgroups
 constexpr int NCAND = 8;                                // best approximate cosines kept per source and tile parity
 constexpr float EPS = 1.0e-3f;                          // bound on |approximate - exact cosine| (see above)
-constexpr uint32_t SM_B = 0;
-constexpr uint32_t SM_SCR = SM_B + STAGES * STAGE_BYTES;   // float[32][256]: a chunk of one row per epilogue thread
+constexpr uint32_t SM_SCR = 0;                          // float[32][256]: a chunk of one row per epilogue thread
 constexpr uint32_t SM_BAR = SM_SCR + 32 * 256 * 4;
 enum { B_AFULL = 0, B_BFULL = 1, B_BEMPTY = B_BFULL + STAGES, B_DFULL = B_BEMPTY + STAGES, B_DFREE = B_DFULL + 2 * NBUF,
        B_COUNT = B_DFREE + 2 * NBUF };
 static_assert(B_COUNT <= 32, "barrier area");
 constexpr uint32_t SM_MISC = SM_BAR + 8 * 32;
-constexpr uint32_t SM_TOTAL = SM_MISC + 64;
-constexpr size_t SMEM_BYTES = SM_TOTAL + 1024;
+constexpr uint32_t SM_B = (SM_MISC + 64 + 1023) / 1024 * 1024;   // STAGES tiles of fp16 rows, [d-half][128 rows][128 B]
+template <int DM>
+constexpr uint32_t STAGE_BYTES = 128 * DM * 2;          // 32 or 16 KB
+template <int DM>
+constexpr size_t SMEM_BYTES = SM_B + STAGES * STAGE_BYTES<DM> + 1024;
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t TA = 0, TD = 128;                    // A rows (fp16) at 0; D buffers at 128, 256 and 384
 static_assert(TD + NBUF * 128 <= TMEM_COLS, "TMEM budget");
 
+// DM / 32 consecutive floats per lane of a warp that holds one descriptor row
+template <int V>
+struct alignas(V * 4) Floats { float v[V]; };
+
+template <int V>
+__device__ __forceinline__ float dot(const Floats<V>& x, const Floats<V>& y) {
+    float acc = x.v[V - 1] * y.v[V - 1];
+#pragma unroll
+    for (int e = V - 2; e >= 0; --e) acc = fmaf(x.v[e], y.v[e], acc);
+    return acc;
+}
+
+template <int DM>
 __global__ void __launch_bounds__(256)
 half_kernel(const float* __restrict__ mhat, MatchTcArgs m) {
     dep_sync();
+    constexpr int V = DM / 32;
     for (int64_t w = (int64_t)blockIdx.x * 256 + threadIdx.x; w < m.zero_words; w += (int64_t)gridDim.x * 256)
         reinterpret_cast<unsigned int*>(m.exact_count)[w] = 0u;
-    // one warp per output row (4 floats per lane)
+    // one warp per output row (V floats per lane)
     const int64_t gw = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     const int64_t rows_a = (int64_t)m.B * m.nA_pad, rows_b = (int64_t)m.B * m.nB_pad;
@@ -71,16 +88,15 @@ half_kernel(const float* __restrict__ mhat, MatchTcArgs m) {
     const int64_t rr = is_b ? gw - rows_a : gw;
     const int pad = is_b ? m.nB_pad : m.nA_pad, cnt = is_b ? m.p.nB : m.nA;
     const int b = (int)(rr / pad), i = (int)(rr % pad);
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    Floats<V> v = {};
     if (i < cnt) {
         const int tok = is_b ? m.p.dst_token(i) : m.src_idx[i];
-        v = *reinterpret_cast<const float4*>(mhat + ((int64_t)b * m.N + tok) * DM + lane * 4);
+        v = *reinterpret_cast<const Floats<V>*>(mhat + ((int64_t)b * m.N + tok) * DM + lane * V);
     }
-    __half2 h01 = __floats2half2_rn(v.x, v.y), h23 = __floats2half2_rn(v.z, v.w);
-    uint2 out;
-    out.x = *reinterpret_cast<uint32_t*>(&h01);
-    out.y = *reinterpret_cast<uint32_t*>(&h23);
-    *reinterpret_cast<uint2*>((is_b ? m.b_h : m.a_h) + rr * DM + lane * 4) = out;
+    struct alignas(V * 2) { __half2 h[V / 2]; } out;
+#pragma unroll
+    for (int e = 0; e < V; e += 2) out.h[e / 2] = __floats2half2_rn(v.v[e], v.v[e + 1]);
+    *reinterpret_cast<decltype(out)*>((is_b ? m.b_h : m.a_h) + rr * DM + lane * V) = out;
     if (!is_b) {
         // A lower bound on the source's row maximum, known before the big product starts: its exact
         // cosine with the destination of its own partition block, less the error bound.  Video
@@ -90,8 +106,7 @@ half_kernel(const float* __restrict__ mhat, MatchTcArgs m) {
         float floor_v = -INFINITY;
         if (i < cnt) {
             const int own = m.p.dst_token(m.p.ord(m.src_idx[i]));
-            const float4 y = *reinterpret_cast<const float4*>(mhat + ((int64_t)b * m.N + own) * DM + lane * 4);
-            float acc = fmaf(v.x, y.x, fmaf(v.y, y.y, fmaf(v.z, y.z, v.w * y.w)));
+            float acc = dot<V>(v, *reinterpret_cast<const Floats<V>*>(mhat + ((int64_t)b * m.N + own) * DM + lane * V));
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
             floor_v = acc - 2.0f * EPS;   // exact - EPS bounds its approximate value from below; another EPS of slack
@@ -118,6 +133,7 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
         : "memory");
 }
 
+template <int DM>
 __global__ void __launch_bounds__(352, 1)
 match_tc_kernel(const MatchTcArgs m, const __grid_constant__ Maps maps) {
     dep_launch();   // the set-up below touches shared and tensor memory only; dep_wait() follows it
@@ -168,11 +184,12 @@ match_tc_kernel(const MatchTcArgs m, const __grid_constant__ Maps maps) {
             const int s = t % STAGES;
             const uint32_t ph = (t / STAGES) & 1;
             if (!mbar_wait(bar(B_BEMPTY + s), ph ^ 1, s_abort, m.status, 0x10000)) break;
-            const uint32_t dst = base + SM_B + s * STAGE_BYTES;
+            const uint32_t dst = base + SM_B + s * STAGE_BYTES<DM>;
             if (elect_one()) {
-                mbar_expect_tx(bar(B_BFULL + s), STAGE_BYTES);
-                tma_load_2d(dst, &maps.b_h, bar(B_BFULL + s), 0, row0 + t * 128);
-                tma_load_2d(dst + 16384, &maps.b_h, bar(B_BFULL + s), 64, row0 + t * 128);
+                mbar_expect_tx(bar(B_BFULL + s), STAGE_BYTES<DM>);
+#pragma unroll
+                for (int hf = 0; hf < DM / 64; ++hf)
+                    tma_load_2d(dst + hf * 16384, &maps.b_h, bar(B_BFULL + s), hf * 64, row0 + t * 128);
             }
             __syncwarp();
         }
@@ -189,7 +206,7 @@ match_tc_kernel(const MatchTcArgs m, const __grid_constant__ Maps maps) {
             if (!mbar_wait_spin(bar(B_BFULL + s), ph, s_abort, m.status, 0x40000)) break;
             if (t >= NBUF && !mbar_wait_spin(bar(B_DFREE + (t - NBUF) % (2 * NBUF)), ((t - NBUF) / (2 * NBUF)) & 1, s_abort, m.status, 0x80000)) break;
             fence_after();
-            const uint64_t bd = bdesc0 + ((s * STAGE_BYTES) >> 4);
+            const uint64_t bd = bdesc0 + ((s * STAGE_BYTES<DM>) >> 4);
             const uint32_t d = tmem + TD + buf * 128;
             if (elect_one()) {
 #pragma unroll
@@ -211,7 +228,7 @@ match_tc_kernel(const MatchTcArgs m, const __grid_constant__ Maps maps) {
             const int64_t row = (int64_t)b * m.nA_pad + a;    // padded: always in range
             const uint4* ph = reinterpret_cast<const uint4*>(m.a_h + row * DM);
 #pragma unroll
-            for (int c4 = 0; c4 < 4; ++c4) {
+            for (int c4 = 0; c4 < DM / 32; ++c4) {
                 uint32_t q[16];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
@@ -343,57 +360,87 @@ match_tc_kernel(const MatchTcArgs m, const __grid_constant__ Maps maps) {
     }
 }
 
+// fp32 cosines that decide.  DM = 128: a warp holds both rows, four products a lane, then a
+// butterfly.  DM = 64: every lane works through a whole destination row of its own, in ascending
+// feature order.  (Each width keeps one order of summation wherever a cosine is decided, so that the
+// same pair always gives the same value.)
+__device__ __forceinline__ float warp_cosine(const Floats<4>& x, const Floats<4>& y) {
+    float acc = dot<4>(x, y);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    return acc;
+}
+__device__ __forceinline__ float lane_cosine64(const float* __restrict__ x, const float* __restrict__ y) {
+    float acc = 0.f;
+#pragma unroll 4
+    for (int e = 0; e < 64; e += 4) {
+        const float4 xv = __ldg(reinterpret_cast<const float4*>(x + e)), yv = __ldg(reinterpret_cast<const float4*>(y + e));
+        acc = fmaf(xv.w, yv.w, fmaf(xv.z, yv.z, fmaf(xv.y, yv.y, fmaf(xv.x, yv.x, acc))));
+    }
+    return acc;
+}
+
 // One warp per source: the candidates inside the window (approximate cosine >= max - 2 EPS) are
 // re-evaluated in fp32; the largest wins, equal values go to the lowest destination.  A source whose
 // last kept candidate is still inside the window may have more destinations in it than were kept: it is
-// appended to the list of the exact scan.
+// appended to the list of the exact scan.  Lane c holds candidate c of the two lists (even and odd
+// destination tiles), each complete for its tiles unless its last entry is still inside the window.
+template <int DM>
 __global__ void __launch_bounds__(256)
 recheck_kernel(const float* __restrict__ mhat, MatchTcArgs m) {
     dep_sync();
+    static_assert(2 * NCAND <= 32, "one lane per candidate");
     const int64_t gw = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (gw >= (int64_t)m.B * m.nA) return;
     const int b = (int)(gw / m.nA), a = (int)(gw % m.nA);
-    // two lists per source (even and odd destination tiles), each complete for its tiles unless its
-    // last entry is still inside the window
-    float v[2 * NCAND];
-    int id[2 * NCAND];
-#pragma unroll
-    for (int c = 0; c < 2 * NCAND; ++c) {
-        v[c] = m.cand_v[gw * 2 * NCAND + c];
-        id[c] = m.cand_i[gw * 2 * NCAND + c];
-    }
-    const float window = fmaxf(v[0], v[NCAND]) - 2.0f * EPS;
-    if (v[NCAND - 1] >= window || v[2 * NCAND - 1] >= window) {   // (never true for -inf entries)
+    const int src = m.src_idx[a];
+    const float v = lane < 2 * NCAND ? m.cand_v[gw * 2 * NCAND + lane] : -INFINITY;
+    const int id = lane < 2 * NCAND ? m.cand_i[gw * 2 * NCAND + lane] : 0x7fffffff;
+    const float window = fmaxf(__shfl_sync(0xffffffffu, v, 0), __shfl_sync(0xffffffffu, v, NCAND)) - 2.0f * EPS;
+    unsigned in = __ballot_sync(0xffffffffu, v >= window);   // (never true for -inf entries)
+    if (in & ((1u << (NCAND - 1)) | (1u << (2 * NCAND - 1)))) {
         if (lane == 0) m.exact_list[atomicAdd(m.exact_count, 1)] = (int)gw;
         return;
     }
     const float* M = mhat + (int64_t)b * m.N * DM;
-    const float4 x = *reinterpret_cast<const float4*>(M + (int64_t)m.src_idx[a] * DM + lane * 4);
+    const float* X = M + (int64_t)src * DM;
     float best = -INFINITY;
     int bj = 0x7fffffff;
+    if (DM == 128) {
+        const Floats<4> x = *reinterpret_cast<const Floats<4>*>(X + lane * 4);
+        while (in) {
+            const int j = __shfl_sync(0xffffffffu, id, __ffs(in) - 1);
+            in &= in - 1;
+            const float c = warp_cosine(x, *reinterpret_cast<const Floats<4>*>(M + (int64_t)m.p.dst_token(j) * DM + lane * 4));
+            if (c > best || (c == best && j < bj)) { best = c; bj = j; }
+        }
+    } else {
+        if ((in >> lane) & 1u) {
+            best = lane_cosine64(X, M + (int64_t)m.p.dst_token(id) * DM);
+            bj = id;
+        }
 #pragma unroll
-    for (int c = 0; c < 2 * NCAND; ++c) {
-        if ((c % NCAND) == NCAND - 1 || v[c] < window) continue;   // (uniform over the warp)
-        const float4 y = *reinterpret_cast<const float4*>(M + (int64_t)m.p.dst_token(id[c]) * DM + lane * 4);
-        float acc = fmaf(x.x, y.x, fmaf(x.y, y.y, fmaf(x.z, y.z, x.w * y.w)));
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (acc > best || (acc == best && id[c] < bj)) { best = acc; bj = id[c]; }
+        for (int o = NCAND; o > 0; o >>= 1) {
+            const float ob = __shfl_xor_sync(0xffffffffu, best, o);
+            const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
+            if (ob > best || (ob == best && oj < bj)) { best = ob; bj = oj; }
+        }
     }
     if (lane == 0) {
-        m.jstar_s[gw] = m.p.dst_token(bj);
+        m.jstar_s[gw] = m.p.dst_token(bj == 0x7fffffff ? 0 : bj);   // (no comparable cosine, NaN in the metric: any destination)
         m.u_s[gw] = best;
     }
 }
 
 // fp32 scan of every destination for the listed sources (normally few or none): the same
 // summation order per cosine as recheck_kernel.  Work unit = (listed source, chunk of 256
-// destinations); a warp takes four destinations at a time so that their loads overlap; the best
-// (cosine, lowest destination) of a unit goes into the source's slot with one 64-bit atomic maximum
+// destinations); a warp takes four destinations at a time so that their loads overlap (DM = 64: one
+// a lane); the best (cosine, lowest destination) of a unit goes into the source's slot with one 64-bit atomic maximum
 // (order-preserving key of the cosine above, complement of the destination below).
 constexpr int EX_CHUNK = 256;
 
+template <int DM>
 __global__ void __launch_bounds__(256)
 match_exact_kernel(const float* __restrict__ mhat, MatchTcArgs m) {
     dep_sync();
@@ -406,27 +453,39 @@ match_exact_kernel(const float* __restrict__ mhat, MatchTcArgs m) {
         const int gw = m.exact_list[w];
         const int b = gw / m.nA, a = gw % m.nA;
         const float* M = mhat + (int64_t)b * m.N * DM;
-        const float4 x = *reinterpret_cast<const float4*>(M + (int64_t)m.src_idx[a] * DM + lane * 4);
+        const float* X = M + (int64_t)m.src_idx[a] * DM;
         unsigned long long best = 0ull;
         const int j0 = c * EX_CHUNK + warp * 32;
-#pragma unroll 1
-        for (int q = 0; q < 32; q += 4) {
-            float4 y[4];
+        auto key_of = [](float cosine, int j) {
+            return ((unsigned long long)float_key(cosine) << 32) | (0xffffffffu - (unsigned)j);
+        };
+        if (DM == 64) {
+            const int j = j0 + lane;
+            if (j < m.p.nB) best = key_of(lane_cosine64(X, M + (int64_t)m.p.dst_token(j) * DM), j);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int j = j0 + q + e;
-                y[e] = j < m.p.nB ? *reinterpret_cast<const float4*>(M + (int64_t)m.p.dst_token(j) * DM + lane * 4)
-                                  : make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int o = 16; o > 0; o >>= 1) {
+                const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
+                best = other > best ? other : best;
             }
+        } else {
+            const Floats<4> x = *reinterpret_cast<const Floats<4>*>(X + lane * 4);
+#pragma unroll 1
+            for (int q = 0; q < 32; q += 4) {
+                Floats<4> y[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int j = j0 + q + e;
-                float acc = fmaf(x.x, y[e].x, fmaf(x.y, y[e].y, fmaf(x.z, y[e].z, x.w * y[e].w)));
+                for (int e = 0; e < 4; ++e) {
+                    const int j = j0 + q + e;
+                    y[e] = j < m.p.nB ? *reinterpret_cast<const Floats<4>*>(M + (int64_t)m.p.dst_token(j) * DM + lane * 4)
+                                      : Floats<4>{};
+                }
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-                if (j < m.p.nB) {
-                    const unsigned long long key = ((unsigned long long)float_key(acc) << 32) | (0xffffffffu - (unsigned)j);
-                    best = key > best ? key : best;
+                for (int e = 0; e < 4; ++e) {
+                    const int j = j0 + q + e;
+                    const float acc = warp_cosine(x, y[e]);
+                    if (j < m.p.nB) {
+                        const unsigned long long key = key_of(acc, j);
+                        best = key > best ? key : best;
+                    }
                 }
             }
         }
@@ -456,7 +515,7 @@ match_exact_finish_kernel(MatchTcArgs m) {
     }
 }
 
-static int make_rows_map(CUtensorMap* map, const void* ptr, int64_t rows, const char* name) {
+static int make_rows_map(CUtensorMap* map, const void* ptr, int64_t rows, int DM, const char* name) {
     EncodeTiledFn fn = encode_fn();
     if (fn == nullptr) return fail(USV_ERR_CUDA, "token_merge: cuTensorMapEncodeTiled not available");
     cuuint64_t dims[2] = {(cuuint64_t)DM, (cuuint64_t)rows};
@@ -476,30 +535,31 @@ static inline int pad128(int n) { return (n + 127) / 128 * 128; }
 
 // Layout of the scratch: fp16 rows of sources and destinations (each side padded to 128 rows),
 // the candidates (value, destination) per source and tile parity, the list of the exact scan, its counter and results, the floors.
-static size_t rows_bytes(int B, int N) { return align_up((size_t)B * ((size_t)N + 256) * mt::DM * sizeof(uint16_t), 256); }
+static size_t rows_bytes(int B, int N, int dm) { return align_up((size_t)B * ((size_t)N + 256) * dm * sizeof(uint16_t), 256); }
 static size_t cand_bytes(int B, int N) { return align_up((size_t)B * N * 2 * mt::NCAND * sizeof(float), 256); }
 
 static size_t list_bytes(int B, int N) { return align_up((size_t)B * N * sizeof(int), 256); }
 
-size_t match_tc_bytes(int B, int N) {
+size_t match_tc_bytes(int B, int N, int dm) {
     // rows | candidate values | candidate destinations | exact-scan list | its counter | its results | floors
-    return rows_bytes(B, N) + 2 * cand_bytes(B, N) + list_bytes(B, N) + 256 + 2 * list_bytes(B, N) +
+    return rows_bytes(B, N, dm) + 2 * cand_bytes(B, N) + list_bytes(B, N) + 256 + 2 * list_bytes(B, N) +
            align_up((size_t)B * ((size_t)N + 128) * sizeof(float), 256);
 }
 
-int launch_match_tc(const float* mhat, const Part& p, int B, int N, int nA, const int32_t* src_idx,
-                    int32_t* jstar_s, float* u_s, void* mem, unsigned int* status, cudaStream_t st) {
+template <int dm>
+static int launch_match(const float* mhat, const Part& p, int B, int N, int nA, const int32_t* src_idx,
+                        int32_t* jstar_s, float* u_s, void* mem, unsigned int* status, cudaStream_t st) {
     MatchTcArgs m;
     m.p = p; m.B = B; m.N = N; m.nA = nA;
     m.nA_pad = pad128(nA); m.nB_pad = pad128(p.nB);
     m.src_idx = src_idx; m.jstar_s = jstar_s; m.u_s = u_s; m.status = status;
     char* base = static_cast<char*>(mem);
     m.a_h = reinterpret_cast<uint16_t*>(base);
-    m.b_h = m.a_h + (size_t)B * m.nA_pad * mt::DM;
-    m.cand_v = reinterpret_cast<float*>(base + rows_bytes(B, N));
-    m.cand_i = reinterpret_cast<int*>(base + rows_bytes(B, N) + cand_bytes(B, N));
-    m.exact_list = reinterpret_cast<int*>(base + rows_bytes(B, N) + 2 * cand_bytes(B, N));
-    char* after_list = base + rows_bytes(B, N) + 2 * cand_bytes(B, N) + list_bytes(B, N);
+    m.b_h = m.a_h + (size_t)B * m.nA_pad * dm;
+    m.cand_v = reinterpret_cast<float*>(base + rows_bytes(B, N, dm));
+    m.cand_i = reinterpret_cast<int*>(base + rows_bytes(B, N, dm) + cand_bytes(B, N));
+    m.exact_list = reinterpret_cast<int*>(base + rows_bytes(B, N, dm) + 2 * cand_bytes(B, N));
+    char* after_list = base + rows_bytes(B, N, dm) + 2 * cand_bytes(B, N) + list_bytes(B, N);
     m.exact_count = reinterpret_cast<int*>(after_list);
     m.exact_best = reinterpret_cast<unsigned long long*>(after_list + 256);
     m.floor_v = reinterpret_cast<float*>(after_list + 256 + 2 * list_bytes(B, N));
@@ -508,24 +568,30 @@ int launch_match_tc(const float* mhat, const Part& p, int B, int N, int nA, cons
     m.zero_words = (int)((256 + 2 * list_bytes(B, N)) / 4);
     cudaError_t e;
     const int64_t rows = (int64_t)B * (m.nA_pad + m.nB_pad);
-    launch_dep(mt::half_kernel, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, mhat, m);
+    launch_dep(mt::half_kernel<dm>, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, mhat, m);
     USV_CHECK_LAUNCH("half_kernel");
     mt::Maps maps;
     int rc;
-    if ((rc = mt::make_rows_map(&maps.b_h, m.b_h, (int64_t)B * m.nB_pad, "b_h")) != USV_OK) return rc;
-    e = cudaFuncSetAttribute(mt::match_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mt::SMEM_BYTES);
+    if ((rc = mt::make_rows_map(&maps.b_h, m.b_h, (int64_t)B * m.nB_pad, dm, "b_h")) != USV_OK) return rc;
+    e = cudaFuncSetAttribute(mt::match_tc_kernel<dm>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mt::SMEM_BYTES<dm>);
     if (e != cudaSuccess) return fail(USV_ERR_CUDA, "token_merge: smem attribute: %s", cudaGetErrorString(e));
     dim3 grid(m.nA_pad / 128, B);
-    launch_dep(mt::match_tc_kernel, dim3(grid), dim3(352), mt::SMEM_BYTES, st, m, maps);
+    launch_dep(mt::match_tc_kernel<dm>, dim3(grid), dim3(352), mt::SMEM_BYTES<dm>, st, m, maps);
     USV_CHECK_LAUNCH("match_tc_kernel");
     const int64_t srcs = (int64_t)B * nA;
-    launch_dep(mt::recheck_kernel, dim3((unsigned)((srcs + 7) / 8)), dim3(256), 0, st, mhat, m);
+    launch_dep(mt::recheck_kernel<dm>, dim3((unsigned)((srcs + 7) / 8)), dim3(256), 0, st, mhat, m);
     USV_CHECK_LAUNCH("recheck_kernel");
-    launch_dep(mt::match_exact_kernel, dim3(1184), dim3(256), 0, st, mhat, m);
+    launch_dep(mt::match_exact_kernel<dm>, dim3(1184), dim3(256), 0, st, mhat, m);
     USV_CHECK_LAUNCH("match_exact_kernel");
     launch_dep(mt::match_exact_finish_kernel, dim3(8), dim3(256), 0, st, m);
     USV_CHECK_LAUNCH("match_exact_finish_kernel");
     return USV_OK;
+}
+
+int launch_match_tc(const float* mhat, const Part& p, int B, int N, int nA, int dm, const int32_t* src_idx,
+                    int32_t* jstar_s, float* u_s, void* mem, unsigned int* status, cudaStream_t st) {
+    return dm == 64 ? launch_match<64>(mhat, p, B, N, nA, src_idx, jstar_s, u_s, mem, status, st)
+                    : launch_match<128>(mhat, p, B, N, nA, src_idx, jstar_s, u_s, mem, status, st);
 }
 
 }  // namespace usv

@@ -2,9 +2,9 @@
 //
 //   desc_kernel        Eq. 7-8   head-averaged, unit-normalised key descriptors (HBM stream)
 //   src_list_kernel    Eq. 6     ascending list of source tokens of the bipartite partition
-//   match_kernel       Eq. 8-9   cosine of every source against every destination of its batch
-//                                element with a fused row arg-max (fp32 CUDA cores; the result
-//                                decides an integer that is compared with an fp64 evaluation)
+//   (usv_match_tc.cu)  Eq. 8-9   cosine of every source against every destination of its batch
+//                                element with a fused row arg-max, on the tensor cores
+//   match_local_kernel           the same inside a window of partition blocks (fp32 CUDA cores)
 //   plan_select_kernel Eq. 10         radix-select of the r-th most confident source
 //   plan_assign_kernel Eq. 11, 14     ordered compaction, dst_of / pos
 //   csr_* kernels      Eq. 12    sources grouped by destination
@@ -92,97 +92,6 @@ __global__ void __launch_bounds__(256) src_list_kernel(Part p, int N, int32_t* _
         if (y % p.sh == 0) before += (x + p.sw - 1) / p.sw;     // destinations before x in this row
     }
     src_idx[n - before] = n;
-}
-
-// ---------------------------------------------------------------------------- matching
-// CTA: 256 threads, 64 sources x (all destinations in tiles of 64).  The 64 source descriptors
-// stay in shared memory for the whole sweep; destination tiles stream through in chunks of 32
-// features.  Each thread keeps the running best of its 4 rows over its 4 columns per tile;
-// columns are visited in ascending destination order and replaced only on strict improvement, so
-// equal cosines resolve to the lowest destination.
-template <int DM>
-__global__ void __launch_bounds__(256) match_kernel(const float* __restrict__ mhat, Part p, int N,
-                                                    int nA, const int32_t* __restrict__ src_idx,
-                                                    int32_t* __restrict__ jstar_s,
-                                                    float* __restrict__ u_s) {
-    dep_sync();
-    constexpr int TK = 32;
-    __shared__ __align__(16) float As[DM][64 + 4];
-    __shared__ __align__(16) float Bs[TK][64 + 4];
-    const int b = blockIdx.y;
-    const int a0 = blockIdx.x * 64;
-    const float* M = mhat + (int64_t)b * N * DM;
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-
-    for (int idx = threadIdx.x; idx < 64 * (DM / 4); idx += 256) {
-        const int r = idx / (DM / 4), c4 = idx % (DM / 4);
-        float4 v = make_float4(0, 0, 0, 0);
-        if (a0 + r < nA) v = *reinterpret_cast<const float4*>(M + (int64_t)src_idx[a0 + r] * DM + c4 * 4);
-        As[c4 * 4 + 0][r] = v.x; As[c4 * 4 + 1][r] = v.y;
-        As[c4 * 4 + 2][r] = v.z; As[c4 * 4 + 3][r] = v.w;
-    }
-    float best[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-    int besti[4] = {0x7fffffff, 0x7fffffff, 0x7fffffff, 0x7fffffff};
-    __syncthreads();
-
-    for (int j0 = 0; j0 < p.nB; j0 += 64) {
-        float acc[4][4] = {};
-        for (int k0 = 0; k0 < DM; k0 += TK) {
-#pragma unroll
-            for (int t = 0; t < 2; ++t) {
-                const int idx = threadIdx.x + t * 256;
-                const int r = idx / 8, c4 = idx % 8;
-                float4 v = make_float4(0, 0, 0, 0);
-                if (j0 + r < p.nB)
-                    v = *reinterpret_cast<const float4*>(M + (int64_t)p.dst_token(j0 + r) * DM + k0 + c4 * 4);
-                Bs[c4 * 4 + 0][r] = v.x; Bs[c4 * 4 + 1][r] = v.y;
-                Bs[c4 * 4 + 2][r] = v.z; Bs[c4 * 4 + 3][r] = v.w;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int e = 0; e < TK; ++e) {
-                const float4 av = *reinterpret_cast<const float4*>(&As[k0 + e][ty * 4]);
-                const float4 bv = *reinterpret_cast<const float4*>(&Bs[e][tx * 4]);
-                const float ar[4] = {av.x, av.y, av.z, av.w};
-                const float br[4] = {bv.x, bv.y, bv.z, bv.w};
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(ar[i], br[j], acc[i][j]);
-            }
-            __syncthreads();
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int o = j0 + tx * 4 + j;
-            if (o < p.nB) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (acc[i][j] > best[i]) {
-                        best[i] = acc[i][j];
-                        besti[i] = o;
-                    }
-            }
-        }
-    }
-    // combine the 16 threads (consecutive lanes) that share a row
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-#pragma unroll
-        for (int o = 1; o < 16; o <<= 1) {
-            const float ov = __shfl_xor_sync(0xffffffffu, best[i], o);
-            const int oi = __shfl_xor_sync(0xffffffffu, besti[i], o);
-            if (ov > best[i] || (ov == best[i] && oi < besti[i])) {
-                best[i] = ov;
-                besti[i] = oi;
-            }
-        }
-        const int a = a0 + ty * 4 + i;
-        if (tx == 0 && a < nA) {
-            jstar_s[(int64_t)b * nA + a] = p.dst_token(besti[i]);
-            u_s[(int64_t)b * nA + a] = best[i];
-        }
-    }
 }
 
 // ---------------------------------------------------------------------------- plan
@@ -632,7 +541,7 @@ static MergeWs merge_layout(int B, int N, int dm, int nA, int nB) {
     w.cursor = take((size_t)B * nB * 4);
     w.csr = take((size_t)B * nA * 4);
     w.tsel = take((size_t)B * sizeof(int2));                    // selection threshold per batch element
-    w.split = take(dm == 128 ? match_tc_bytes(B, N) : 0);       // bf16 hi/lo planes of the tensor-core matcher
+    w.split = take(dm == 128 || dm == 64 ? match_tc_bytes(B, N, dm) : 0);   // scratch of the tensor-core matcher
     w.total = o;
     return w;
 }
@@ -707,15 +616,11 @@ static int token_merge_impl(int B, int N, int C, const void* x, int Hm, int dm,
                 if (dm == 128) launch_dep(match_local_kernel<128>, dim3(lg), dim3(256), 0, s, mhat, p, N, nA, win[0], win[1], win[2], src_idx, jstar_s, u_s);
                 else launch_dep(match_local_kernel<64>, dim3(lg), dim3(256), 0, s, mhat, p, N, nA, win[0], win[1], win[2], src_idx, jstar_s, u_s);
                 USV_CHECK_LAUNCH("match_local_kernel");
-            } else if (dm == 128) {
-                // tensor cores: split-bf16 cosines (usv_match_tc.cu)
-                unsigned int* status = reinterpret_cast<unsigned int*>(base + L.status);
-                int rc = launch_match_tc(mhat, p, B, N, nA, src_idx, jstar_s, u_s, base + L.split, status, s);
-                if (rc != USV_OK) return rc;
             } else {
-                dim3 mg(ceil_div(nA, 64), B);
-                launch_dep(match_kernel<64>, dim3(mg), dim3(256), 0, s, mhat, p, N, nA, src_idx, jstar_s, u_s);
-                USV_CHECK_LAUNCH("match_kernel");
+                // tensor cores: fp16 cosines propose, fp32 decides (usv_match_tc.cu)
+                unsigned int* status = reinterpret_cast<unsigned int*>(base + L.status);
+                int rc = launch_match_tc(mhat, p, B, N, nA, dm, src_idx, jstar_s, u_s, base + L.split, status, s);
+                if (rc != USV_OK) return rc;
             }
         }
         const int2* tsel = nullptr;
