@@ -254,8 +254,7 @@ int usv_token_merge_local(int B, int N, int C, const void* x, int Hm, int dm, co
  *   usv_merge_plan_cache: from dst_of / pos of a plan (as written by usv_token_merge) into `cache`
  *     (device, 16-byte aligned, usv_merge_plan_cache_bytes(B, N) bytes, owned by the caller).
  *   usv_token_merge_apply: x_merged = merge(x) with the cached plan; same result as
- *     usv_token_merge(metric = NULL).  `cache` is not const: a destination with more than 32 merged
- *     sources has its list sorted in place on first use.
+ *     usv_token_merge(metric = NULL).
  * Grid, partition and r must be those the plan was made with.
  */
 size_t usv_merge_plan_cache_bytes(int B, int N);

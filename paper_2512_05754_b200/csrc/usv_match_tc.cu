@@ -14,8 +14,8 @@
 // destinations inside the window (duplicates, near-duplicates) is handed to a plain fp32 scan of
 // all its destinations.  The result is the fp32 arg-max for every source, whatever the data.
 //
-// 21 076 sources against 7550 destinations at DM = 64: 852 us on fp32 CUDA cores, 72 us here (all four
-// kernels).
+// 20 691 sources against 7410 destinations at DM = 64: 852 us on fp32 CUDA cores, 101 us here (all
+// kernels of this file).
 //
 //   half_kernel         fp32 descriptors -> fp16 rows, sources (by rank) and destinations (by
 //                       ordinal) apart, zero-padded to multiples of 128 rows

@@ -7,7 +7,7 @@
 //   match_local_kernel           the same inside a window of partition blocks (fp32 CUDA cores)
 //   plan_select_kernel Eq. 10         radix-select of the r-th most confident source
 //   plan_assign_kernel Eq. 11, 14     ordered compaction, dst_of / pos
-//   csr_* kernels      Eq. 12    sources grouped by destination
+//                                and the lists of merged sources per destination (Eq. 12)
 //   merge_kernel       Eq. 13-14 warp-per-row gather + mean, 16-byte accesses
 //   unmerge_kernel     Eq. 15    warp-per-row gather copy, 16-byte accesses
 #include <math.h>
@@ -81,9 +81,12 @@ __device__ __forceinline__ int block_scan_1024(int v, int* scratch, int* total) 
 // Ascending list of the source tokens (same for every batch element): the rank of a source is
 // its token index minus the number of destinations before it, which the partition gives in
 // closed form, so every token is handled independently.
-__global__ void __launch_bounds__(256) src_list_kernel(Part p, int N, int32_t* __restrict__ src_idx) {
+// It also clears the list counters that plan_assign_kernel adds to (zero_words words).
+__global__ void __launch_bounds__(256) src_list_kernel(Part p, int N, int32_t* __restrict__ src_idx,
+                                                       int32_t* __restrict__ zero, int64_t zero_words) {
     dep_sync();
     const int n = blockIdx.x * 256 + threadIdx.x;
+    for (int64_t w = n; w < zero_words; w += (int64_t)gridDim.x * 256) zero[w] = 0;
     if (n >= N || p.is_dst(n)) return;
     const int x = n % p.W, y = (n / p.W) % p.Hh, t = n / (p.W * p.Hh);
     int before = ((t + p.st - 1) / p.st) * p.nHy * p.nWx;      // whole destination frames before t
@@ -93,6 +96,27 @@ __global__ void __launch_bounds__(256) src_list_kernel(Part p, int N, int32_t* _
     }
     src_idx[n - before] = n;
 }
+
+// ---------------------------------------------------------------------------- merged-source lists
+// The sources merged into every destination, built by one atomic per source while the plan is
+// written: the first SLOTS of a destination (in order of arrival, merge_kernel sorts them) sit in a
+// 16-byte row of their own, further ones hang on a chain.  Counting, scanning and filling a CSR
+// took three more kernels (13 us at 32 760 tokens, launches included) and left merge_kernel one
+// more dependent load per row.
+struct MergeLists {
+    static constexpr int SLOTS = 4;
+    int32_t* cnt;        // [B,nB] sources of the destination, starts at zero
+    int32_t* head;       // [B,nB] 1 + the last source chained (0: none), starts at zero
+    int32_t* slots;      // [B,nB,SLOTS]
+    int32_t* next;       // [B,N]  1 + the source chained before this one (0: none)
+    int32_t* row_src;    // [B,nU] source token of every unmerged row
+    int32_t* dst_copy;   // [B,N]  copy of dst_of inside a plan cache (NULL: not wanted)
+    __device__ void push(int64_t dst, int64_t token0, int n) const {
+        const int at = atomicAdd(cnt + dst, 1);
+        if (at < SLOTS) slots[dst * SLOTS + at] = n;
+        else next[token0 + n] = atomicExch(head + dst, n + 1);
+    }
+};
 
 // ---------------------------------------------------------------------------- plan
 // One CTA (1024 threads) per batch element.  Radix-select of the r-th largest u, then an ordered
@@ -174,7 +198,7 @@ __global__ void __launch_bounds__(1024) plan_assign_kernel(Part p, int N, int nA
                                                            int32_t* __restrict__ pos,
                                                            float* __restrict__ u_out,
                                                            int32_t* __restrict__ jstar_out,
-                                                           int32_t* __restrict__ cnt) {
+                                                           const MergeLists lists) {
     dep_sync();
     __shared__ int scratch[33];
     const int b = blockIdx.y;
@@ -215,11 +239,14 @@ __global__ void __launch_bounds__(1024) plan_assign_kernel(Part p, int N, int nA
             const int n = src_idx[a];
             const int j = js[a];
             if (merged) {
+                const int o = p.ord(j);
                 d_of[n] = j;
-                ps[n] = nU + p.ord(j);
+                ps[n] = nU + o;
+                lists.push((int64_t)b * p.nB + o, (int64_t)b * N, n);
             } else {
                 d_of[n] = -1;
                 ps[n] = un_rank;
+                lists.row_src[(int64_t)b * nU + un_rank] = n;
             }
             if (u_out) u_out[(int64_t)b * N + n] = ua;
             if (jstar_out) jstar_out[(int64_t)b * N + n] = j;
@@ -230,30 +257,29 @@ __global__ void __launch_bounds__(1024) plan_assign_kernel(Part p, int N, int nA
         const int n = p.dst_token(o);
         d_of[n] = -1;
         ps[n] = nU + o;
-        cnt[(int64_t)b * p.nB + o] = 0;   // the per-destination counts of the CSR pass that follows start at zero
         if (u_out) u_out[(int64_t)b * N + n] = __int_as_float(0x7fc00000);
         if (jstar_out) jstar_out[(int64_t)b * N + n] = -1;
     }
 }
 
-// ---------------------------------------------------------------------------- CSR of M(j)
-__global__ void __launch_bounds__(256) csr_count_kernel(Part p, int N, int nU,
-                                                        const int32_t* __restrict__ dst_of,
-                                                        const int32_t* __restrict__ pos,
-                                                        int32_t* __restrict__ cnt,
-                                                        int32_t* __restrict__ row_src) {
+// The same lists from a stored plan.  cnt and head start at zero.
+__global__ void __launch_bounds__(256) plan_lists_kernel(Part p, int N, int nU,
+                                                         const int32_t* __restrict__ dst_of,
+                                                         const int32_t* __restrict__ pos,
+                                                         const MergeLists lists) {
     dep_sync();
     const int b = blockIdx.y;
     const int n = blockIdx.x * 256 + threadIdx.x;
     if (n >= N) return;
     const int j = dst_of[(int64_t)b * N + n];
-    if (j >= 0) atomicAdd(&cnt[(int64_t)b * p.nB + p.ord(j)], 1);
-    else if (!p.is_dst(n)) row_src[(int64_t)b * nU + pos[(int64_t)b * N + n]] = n;
+    if (lists.dst_copy != nullptr) lists.dst_copy[(int64_t)b * N + n] = j;
+    if (j >= 0) lists.push((int64_t)b * p.nB + p.ord(j), (int64_t)b * N, n);
+    else if (!p.is_dst(n)) lists.row_src[(int64_t)b * nU + pos[(int64_t)b * N + n]] = n;
 }
 
-// exclusive scan of cnt[b,:] -> off[b,0..nB], cursor[b,:] = off[b,:nB].  CTA (c, b) owns the
-// destinations [1024 c, 1024 c + 1024) and sums the counts before its own itself.
-__global__ void __launch_bounds__(1024) csr_scan_kernel(int nB, const int32_t* __restrict__ cnt,
+// Exclusive scan of cnt[b,:] -> off[b,0..nB], cursor[b,:] = off[b,:nB] (unmerge map).  CTA (c, b) owns the
+// rows [1024 c, 1024 c + 1024) and sums the counts before its own itself.
+__global__ void __launch_bounds__(1024) row_scan_kernel(int nB, const int32_t* __restrict__ cnt,
                                                         int32_t* __restrict__ off,
                                                         int32_t* __restrict__ cursor) {
     dep_sync();
@@ -273,21 +299,6 @@ __global__ void __launch_bounds__(1024) csr_scan_kernel(int nB, const int32_t* _
         cursor[(int64_t)b * nB + o] = e;
     }
     if (o0 + 1024 >= nB && threadIdx.x == 0) off[(int64_t)b * (nB + 1) + nB] = base + tot;
-}
-
-__global__ void __launch_bounds__(256) csr_fill_kernel(Part p, int N, int r,
-                                                       const int32_t* __restrict__ dst_of,
-                                                       int32_t* __restrict__ cursor,
-                                                       int32_t* __restrict__ csr) {
-    dep_sync();
-    const int b = blockIdx.y;
-    const int n = blockIdx.x * 256 + threadIdx.x;
-    if (n >= N) return;
-    const int j = dst_of[(int64_t)b * N + n];
-    if (j >= 0) {
-        const int slot = atomicAdd(&cursor[(int64_t)b * p.nB + p.ord(j)], 1);
-        csr[(int64_t)b * r + slot] = n;
-    }
 }
 
 // ---------------------------------------------------------------------------- local matching
@@ -334,151 +345,155 @@ __global__ void __launch_bounds__(256) match_local_kernel(const float* __restric
 }
 
 // ---------------------------------------------------------------------------- merge
-// One warp per output row.  Rows [0,nU) copy an unmerged source; rows [nU, nU+nB) hold a
-// destination averaged with its merged sources, summed in ascending source index.
-__global__ void __launch_bounds__(256) merge_kernel(Part p, int N, int C, int nU, int Nm, int r,
-                                                    const __nv_bfloat16* __restrict__ x,
-                                                    const int32_t* __restrict__ row_src,
-                                                    const int32_t* __restrict__ off,
-                                                    int32_t* __restrict__ csr,
-                                                    __nv_bfloat16* __restrict__ out, int64_t rows) {
+// HBM stream, one warp per output row.  Rows [0,nU) copy an unmerged source; rows [nU, nU+nB) hold a
+// destination averaged with its merged sources, summed in ascending source index (fp32).  Most
+// destinations have no more than two sources: their rows and the destination's are requested
+// together, G 16-byte chunks a lane each, before any is used, and only one chunk's sums are live at a
+// time, so that four CTAs share an SM.  2 x 118 800 rows of 6 KB, a quarter merged: 388 us, 6.6 TB/s, the
+// copy bandwidth of the device (392 us before); 2 x 32 760 rows of 3 KB, 40 % merged: 60 us (65 us).
+// Warps that stay and walk 1 KB segments, looking the next one's lists up ahead, were slower (96 us).
+__global__ void __launch_bounds__(256, 4) merge_kernel(Part p, int N, int C, int nU, int Nm,
+                                                       const __nv_bfloat16* __restrict__ x,
+                                                       const MergeLists lists,
+                                                       const int32_t* __restrict__ dst_of,
+                                                       __nv_bfloat16* __restrict__ out, int64_t rows) {
     dep_sync();
     const int64_t gw = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (gw >= rows) return;
     const int lane = threadIdx.x & 31;
     const int b = (int)(gw / Nm), row = (int)(gw % Nm);
     const __nv_bfloat16* xb = x + (int64_t)b * N * C;
-    uint4* dst = reinterpret_cast<uint4*>(out + ((int64_t)b * Nm + row) * C);
+    auto row_of = [&](int tok) { return reinterpret_cast<const uint4*>(xb + (int64_t)tok * C); };
+    uint4* dst = reinterpret_cast<uint4*>(out + gw * C);
     const int nvec = C / 8;
+    int len = 0, j, id = 0;
+    const int64_t od = (int64_t)b * p.nB + row - nU;
     if (row < nU) {
-        const uint4* src = reinterpret_cast<const uint4*>(xb + (int64_t)row_src[(int64_t)b * nU + row] * C);
-        for (int c = lane; c < nvec; c += 32) dst[c] = __ldg(src + c);
-        return;
+        j = lists.row_src[(int64_t)b * nU + row];
+    } else {
+        j = p.dst_token(row - nU);
+        len = lists.cnt[od];
+        if (lane < MergeLists::SLOTS) id = lists.slots[od * MergeLists::SLOTS + lane];   // (asked for beside the count)
     }
-    const int o = row - nU;
-    const int j = p.dst_token(o);
-    const int beg = off[(int64_t)b * (p.nB + 1) + o], end = off[(int64_t)b * (p.nB + 1) + o + 1];
-    const int len = end - beg;
-    int32_t* list = csr + (int64_t)b * r + beg;
-    const uint4* srcj = reinterpret_cast<const uint4*>(xb + (int64_t)j * C);
+    const uint4* srcj = row_of(j);
     if (len == 0) {
         for (int c = lane; c < nvec; c += 32) dst[c] = __ldg(srcj + c);
         return;
     }
-    int myid = 0x7fffffff;
-    if (len == 1) {
-        myid = list[0];
-    } else if (len <= 32) {
-        // rank sort in registers: lane s ends up holding the s-th smallest source index
-        const int id = lane < len ? list[lane] : 0x7fffffff;
-        int rank = 0;
+    const float inv = 1.0f / (float)(len + 1);
+    constexpr int G = 3;
+    if (len <= 2) {
+        int i0 = __shfl_sync(0xffffffffu, id, 0), i1 = len == 2 ? __shfl_sync(0xffffffffu, id, 1) : i0;
+        const uint4 *src0 = row_of(min(i0, i1)), *src1 = row_of(max(i0, i1));
+        for (int c0 = lane; c0 < nvec; c0 += 32 * G) {
+            uint4 v[G], va[G], vb[G];
 #pragma unroll
-        for (int s = 0; s < 32; ++s) {
-            const int other = __shfl_sync(0xffffffffu, id, s);
-            rank += (other < id) ? 1 : 0;
+            for (int g = 0; g < G; ++g)
+                if (c0 + g * 32 < nvec) v[g] = __ldg(srcj + c0 + g * 32);
+#pragma unroll
+            for (int g = 0; g < G; ++g)
+                if (c0 + g * 32 < nvec) va[g] = __ldg(src0 + c0 + g * 32);
+            if (len == 2) {
+#pragma unroll
+                for (int g = 0; g < G; ++g)
+                    if (c0 + g * 32 < nvec) vb[g] = __ldg(src1 + c0 + g * 32);
+            }
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+                float acc[8], f[8];
+                bf16x8_to_float(v[g], acc);
+                bf16x8_to_float(va[g], f);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) acc[e] += f[e];
+                if (len == 2) {
+                    bf16x8_to_float(vb[g], f);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) acc[e] += f[e];
+                }
+#pragma unroll
+                for (int e = 0; e < 8; ++e) acc[e] *= inv;
+                if (c0 + g * 32 < nvec) dst[c0 + g * 32] = float8_to_bf16x8(acc);
+            }
         }
-        // ids are distinct, so ranks of the valid lanes are a permutation of 0..len-1
-#pragma unroll
-        for (int s = 0; s < 32; ++s) {
+        return;
+    }
+    // Lane s < len <= 32 ends up with the s-th smallest source index.  Longer lists (rare) are found by
+    // a pass over dst_of where they are needed: it meets them in ascending order.
+    int myid = 0x7fffffff;
+    const int32_t* dob = dst_of + (int64_t)b * N;
+    if (len <= 32) {
+        if (len > MergeLists::SLOTS) {
+            int n = lists.head[od];
+            for (int s = MergeLists::SLOTS; s < len; ++s) {
+                if (lane == s) id = n - 1;
+                n = lists.next[(int64_t)b * N + n - 1];
+            }
+        }
+        if (lane >= len) id = 0x7fffffff;
+        int rank = 0;
+        for (int s = 0; s < len; ++s) rank += __shfl_sync(0xffffffffu, id, s) < id ? 1 : 0;
+        // ids are distinct, so the ranks of the valid lanes are a permutation of 0..len-1
+        for (int s = 0; s < len; ++s) {
             const int oid = __shfl_sync(0xffffffffu, id, s);
             const int orank = __shfl_sync(0xffffffffu, rank, s);
-            if (orank == lane && s < len) myid = oid;
-        }
-    } else {
-        // rare long list: in-place selection sort of the segment by this warp
-        for (int s = 0; s < len - 1; ++s) {
-            int bestv = 0x7fffffff, bestp = -1;
-            for (int t = s + lane; t < len; t += 32) {
-                const int v = list[t];
-                if (v < bestv) { bestv = v; bestp = t; }
-            }
-#pragma unroll
-            for (int w = 16; w > 0; w >>= 1) {
-                const int ov = __shfl_xor_sync(0xffffffffu, bestv, w);
-                const int op = __shfl_xor_sync(0xffffffffu, bestp, w);
-                if (ov < bestv) { bestv = ov; bestp = op; }
-            }
-            if (lane == 0 && bestp != s) {
-                const int tmp = list[s];
-                list[s] = bestv;
-                list[bestp] = tmp;
-            }
-            __syncwarp();
+            if (orank == lane) myid = oid;
         }
     }
-    const float inv = 1.0f / (float)(len + 1);
-    // G 16-byte chunks per lane at a time: the loads of one row are all in flight together, and
-    // rows are added in ascending source index (fp32)
-    constexpr int G = 3;
-    // The destination row and the first two source rows (most destinations have no more) are
-    // requested together, before any of them is used.
-    const int i0 = len <= 32 ? __shfl_sync(0xffffffffu, myid, 0) : list[0];
-    const int i1 = len < 2 ? 0 : (len <= 32 ? __shfl_sync(0xffffffffu, myid, 1) : list[1]);
-    const uint4* src0 = reinterpret_cast<const uint4*>(xb + (int64_t)i0 * C);
-    const uint4* src1 = reinterpret_cast<const uint4*>(xb + (int64_t)i1 * C);
-    for (int c0 = 0; c0 < nvec; c0 += 32 * G) {
-        float acc[G][8];
-        uint4 v[G], va[G], vb[G];
+    for (int cb = 0; cb < nvec; cb += 64) {   // (whole warps: the lanes hand the sources round)
+        const int c0 = cb + lane;
+        float acc[2][8];
+        uint4 v[2];
 #pragma unroll
-        for (int g = 0; g < G; ++g) {
-            const int c = c0 + g * 32 + lane;
-            v[g] = c < nvec ? __ldg(srcj + c) : make_uint4(0, 0, 0, 0);
-        }
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-            const int c = c0 + g * 32 + lane;
-            va[g] = c < nvec ? __ldg(src0 + c) : make_uint4(0, 0, 0, 0);
-        }
-        if (len >= 2) {
-#pragma unroll
-            for (int g = 0; g < G; ++g) {
-                const int c = c0 + g * 32 + lane;
-                vb[g] = c < nvec ? __ldg(src1 + c) : make_uint4(0, 0, 0, 0);
-            }
-        }
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
+        for (int g = 0; g < 2; ++g) {
+            v[g] = c0 + g * 32 < nvec ? __ldg(srcj + c0 + g * 32) : make_uint4(0, 0, 0, 0);
             bf16x8_to_float(v[g], acc[g]);
-            float f[8];
-            bf16x8_to_float(va[g], f);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) acc[g][e] += f[e];
         }
-        if (len >= 2) {
+        auto add = [&](const uint4* w) {
 #pragma unroll
-            for (int g = 0; g < G; ++g) {
+            for (int g = 0; g < 2; ++g) {
                 float f[8];
-                bf16x8_to_float(vb[g], f);
+                bf16x8_to_float(w[g], f);
 #pragma unroll
                 for (int e = 0; e < 8; ++e) acc[g][e] += f[e];
             }
+        };
+        auto load = [&](int tok, uint4* w) {
+            const uint4* src = row_of(tok);
+#pragma unroll
+            for (int g = 0; g < 2; ++g) w[g] = c0 + g * 32 < nvec ? __ldg(src + c0 + g * 32) : make_uint4(0, 0, 0, 0);
+        };
+        if (len <= 32) {
+            for (int s = 0; s < len; s += 2) {   // two rows in flight
+                uint4 w[2];
+                load(__shfl_sync(0xffffffffu, myid, s), v);
+                if (s + 1 < len) load(__shfl_sync(0xffffffffu, myid, s + 1), w);
+                add(v);
+                if (s + 1 < len) add(w);
+            }
+        } else {
+            for (int n0 = 0; n0 < N; n0 += 32)
+                for (unsigned found = __ballot_sync(0xffffffffu, n0 + lane < N && dob[n0 + lane] == j); found; found &= found - 1) {
+                    load(n0 + __ffs(found) - 1, v);
+                    add(v);
+                }
         }
-        for (int s = 2; s < len; ++s) {
-            const int i = len <= 32 ? __shfl_sync(0xffffffffu, myid, s) : list[s];
-            const uint4* srci = reinterpret_cast<const uint4*>(xb + (int64_t)i * C);
 #pragma unroll
-            for (int g = 0; g < G; ++g) {
-                const int c = c0 + g * 32 + lane;
-                v[g] = c < nvec ? __ldg(srci + c) : make_uint4(0, 0, 0, 0);
-            }
+        for (int g = 0; g < 2; ++g) {
+            if (c0 + g * 32 >= nvec) continue;
 #pragma unroll
-            for (int g = 0; g < G; ++g) {
-                float f[8];
-                bf16x8_to_float(v[g], f);
-#pragma unroll
-                for (int e = 0; e < 8; ++e) acc[g][e] += f[e];
-            }
-        }
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-            const int c = c0 + g * 32 + lane;
-            if (c < nvec) {
-#pragma unroll
-                for (int e = 0; e < 8; ++e) acc[g][e] *= inv;
-                dst[c] = float8_to_bf16x8(acc[g]);
-            }
+            for (int e = 0; e < 8; ++e) acc[g][e] *= inv;
+            dst[c0 + g * 32] = float8_to_bf16x8(acc[g]);
         }
     }
+}
+
+// rows: B * Nm output rows
+static int launch_merge(const Part& p, int N, int C, int nU, int Nm, int64_t rows, const void* x, const MergeLists& lists,
+                        const int32_t* dst_of, void* out, cudaStream_t st) {
+    launch_dep(merge_kernel, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, p, N, C, nU, Nm,
+               static_cast<const __nv_bfloat16*>(x), lists, dst_of, static_cast<__nv_bfloat16*>(out), rows);
+    USV_CHECK_LAUNCH("merge_kernel");
+    return USV_OK;
 }
 
 // ---------------------------------------------------------------------------- unmerge
@@ -523,7 +538,7 @@ __global__ void __launch_bounds__(256) inv_fill_kernel(int N, int Nm, const int3
 
 // ---------------------------------------------------------------------------- host side
 struct MergeWs {
-    size_t mhat, src_idx, jstar_s, u_s, row_src, cnt, off, cursor, csr, status, tsel, split, total;
+    size_t mhat, src_idx, jstar_s, u_s, row_src, cnt, head, slots, next, status, tsel, split, total;
 };
 
 static MergeWs merge_layout(int B, int N, int dm, int nA, int nB) {
@@ -536,10 +551,10 @@ static MergeWs merge_layout(int B, int N, int dm, int nA, int nB) {
     w.jstar_s = take((size_t)B * nA * 4);
     w.u_s = take((size_t)B * nA * 4);
     w.row_src = take((size_t)B * nA * 4);
-    w.cnt = take((size_t)B * nB * 4);
-    w.off = take((size_t)B * (nB + 1) * 4);
-    w.cursor = take((size_t)B * nB * 4);
-    w.csr = take((size_t)B * nA * 4);
+    w.cnt = take((size_t)B * nB * 4);                           // cnt and head are adjacent: cleared together
+    w.head = take((size_t)B * nB * 4);
+    w.slots = take((size_t)B * nB * MergeLists::SLOTS * 4);
+    w.next = take((size_t)B * N * 4);
     w.tsel = take((size_t)B * sizeof(int2));                    // selection threshold per batch element
     w.split = take(dm == 128 || dm == 64 ? match_tc_bytes(B, N, dm) : 0);   // scratch of the tensor-core matcher
     w.total = o;
@@ -594,11 +609,10 @@ static int token_merge_impl(int B, int N, int C, const void* x, int Hm, int dm,
     int32_t* src_idx = reinterpret_cast<int32_t*>(base + L.src_idx);
     int32_t* jstar_s = reinterpret_cast<int32_t*>(base + L.jstar_s);
     float* u_s = reinterpret_cast<float*>(base + L.u_s);
-    int32_t* row_src = reinterpret_cast<int32_t*>(base + L.row_src);
-    int32_t* cnt = reinterpret_cast<int32_t*>(base + L.cnt);
-    int32_t* off = reinterpret_cast<int32_t*>(base + L.off);
-    int32_t* cursor = reinterpret_cast<int32_t*>(base + L.cursor);
-    int32_t* csr = reinterpret_cast<int32_t*>(base + L.csr);
+    const MergeLists lists = {reinterpret_cast<int32_t*>(base + L.cnt), reinterpret_cast<int32_t*>(base + L.head),
+                              reinterpret_cast<int32_t*>(base + L.slots), reinterpret_cast<int32_t*>(base + L.next),
+                              reinterpret_cast<int32_t*>(base + L.row_src), nullptr};
+    const size_t zero_bytes = L.slots - L.cnt;   // cnt and head
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int nU = nA - r, Nm = N - r;
 
@@ -608,9 +622,9 @@ static int token_merge_impl(int B, int N, int C, const void* x, int Hm, int dm,
         if (dm == 128) launch_dep(desc_kernel<128>, dim3(dg), dim3(256), 0, s, static_cast<const __nv_bfloat16*>(metric), mhat, tokens, Hm);
         else launch_dep(desc_kernel<64>, dim3(dg), dim3(256), 0, s, static_cast<const __nv_bfloat16*>(metric), mhat, tokens, Hm);
         USV_CHECK_LAUNCH("desc_kernel");
+        launch_dep(src_list_kernel, dim3(ceil_div(N, 256)), dim3(256), 0, s, p, N, src_idx, lists.cnt, (int64_t)(zero_bytes / 4));
+        USV_CHECK_LAUNCH("src_list_kernel");
         if (nA > 0) {
-            launch_dep(src_list_kernel, dim3(ceil_div(N, 256)), dim3(256), 0, s, p, N, src_idx);
-            USV_CHECK_LAUNCH("src_list_kernel");
             if (win != nullptr) {
                 dim3 lg(ceil_div(nA, 8), B);
                 if (dm == 128) launch_dep(match_local_kernel<128>, dim3(lg), dim3(256), 0, s, mhat, p, N, nA, win[0], win[1], win[2], src_idx, jstar_s, u_s);
@@ -633,27 +647,15 @@ static int token_merge_impl(int B, int N, int C, const void* x, int Hm, int dm,
         // r = nA: every key is above 0; r = 0: no key is above or equal to the largest one
         dim3 pg(ceil_div(nA > p.nB ? nA : p.nB, 1024), B);
         launch_dep(plan_assign_kernel, dim3(pg), dim3(1024), 0, s, p, N, nA, r, r == nA ? 0u : 0xffffffffu, 0, tsel, src_idx, jstar_s, u_s,
-                                               dst_of, pos, u_out, jstar_out, cnt);
+                                               dst_of, pos, u_out, jstar_out, lists);
         USV_CHECK_LAUNCH("plan_assign_kernel");
     } else {
-        cudaError_t e = cudaMemsetAsync(cnt, 0, (size_t)B * p.nB * 4, s);
+        cudaError_t e = cudaMemsetAsync(lists.cnt, 0, zero_bytes, s);
         if (e != cudaSuccess) return fail(USV_ERR_CUDA, "token_merge: memset: %s", cudaGetErrorString(e));
+        launch_dep(plan_lists_kernel, dim3(ceil_div(N, 256), B), dim3(256), 0, s, p, N, nU, dst_of, pos, lists);
+        USV_CHECK_LAUNCH("plan_lists_kernel");
     }
-    dim3 tg(ceil_div(N, 256), B);
-    launch_dep(csr_count_kernel, dim3(tg), dim3(256), 0, s, p, N, nU, dst_of, pos, cnt, row_src);
-    USV_CHECK_LAUNCH("csr_count_kernel");
-    launch_dep(csr_scan_kernel, dim3(dim3(ceil_div(p.nB, 1024), B)), dim3(1024), 0, s, p.nB, cnt, off, cursor);
-    USV_CHECK_LAUNCH("csr_scan_kernel");
-    if (r > 0) {
-        launch_dep(csr_fill_kernel, dim3(tg), dim3(256), 0, s, p, N, r, dst_of, cursor, csr);
-        USV_CHECK_LAUNCH("csr_fill_kernel");
-    }
-    const int64_t rows = (int64_t)B * Nm;
-    launch_dep(merge_kernel, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, s, 
-        p, N, C, nU, Nm, r, static_cast<const __nv_bfloat16*>(x), row_src, off, csr,
-        static_cast<__nv_bfloat16*>(x_merged), rows);
-    USV_CHECK_LAUNCH("merge_kernel");
-    return USV_OK;
+    return launch_merge(p, N, C, nU, Nm, (int64_t)B * Nm, x, lists, dst_of, x_merged, s);
 }
 
 extern "C" int usv_token_unmerge(int B, int N, int Nm, int C, const void* y_merged,
@@ -676,10 +678,16 @@ extern "C" int usv_token_unmerge(int B, int N, int Nm, int C, const void* y_merg
 
 // ---------------------------------------------------------------------------- stored plan
 // What merge_kernel needs of a plan, kept by the caller beside dst_of / pos so that applying the
-// plan to further tensors is the streaming kernel alone: row_src | off | csr | (cnt, cursor scratch),
-// each B * (N + 1) ints.
+// plan to further tensors is the streaming kernel alone: cnt | head | row_src | next | dst_copy |
+// slots (SLOTS times the size), each B * (N + 1) ints.
 namespace usv {
 static size_t cache_stride(int B, int N) { return align_up((size_t)B * ((size_t)N + 1) * sizeof(int32_t), 256); }
+static MergeLists cache_lists(void* cache, int B, int N) {
+    char* base = static_cast<char*>(cache);
+    const size_t cs = cache_stride(B, N);
+    auto at = [&](int i) { return reinterpret_cast<int32_t*>(base + i * cs); };
+    return {at(0), at(1), at(5), at(3), at(2), at(4)};
+}
 
 static int fill_part(Part& p, int N, int T, int Hh, int W, int st, int sh, int sw, const char* who) {
     if (T <= 0 || Hh <= 0 || W <= 0 || (int64_t)T * Hh * W != N)
@@ -694,7 +702,7 @@ static int fill_part(Part& p, int N, int T, int Hh, int W, int st, int sh, int s
 
 extern "C" size_t usv_merge_plan_cache_bytes(int B, int N) {
     if (B <= 0 || N <= 0) return 0;
-    return 5 * usv::cache_stride(B, N);
+    return (5 + usv::MergeLists::SLOTS) * usv::cache_stride(B, N);
 }
 
 extern "C" int usv_merge_plan_cache(int B, int N, int T, int Hh, int W, int st, int sh, int sw, int r,
@@ -712,25 +720,12 @@ extern "C" int usv_merge_plan_cache(int B, int N, int T, int Hh, int W, int st, 
     if (!aligned16(cache)) return fail(USV_ERR_UNSUPPORTED, "merge_plan_cache: cache not 16-byte aligned");
     if (cache_bytes < usv_merge_plan_cache_bytes(B, N))
         return fail(USV_ERR_WORKSPACE, "merge_plan_cache: cache %zu < %zu", cache_bytes, usv_merge_plan_cache_bytes(B, N));
-    char* base = static_cast<char*>(cache);
-    const size_t cs = cache_stride(B, N);
-    int32_t* row_src = reinterpret_cast<int32_t*>(base);
-    int32_t* off = reinterpret_cast<int32_t*>(base + cs);
-    int32_t* csr = reinterpret_cast<int32_t*>(base + 2 * cs);
-    int32_t* cnt = reinterpret_cast<int32_t*>(base + 3 * cs);
-    int32_t* cursor = reinterpret_cast<int32_t*>(base + 4 * cs);
+    const MergeLists lists = cache_lists(cache, B, N);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaError_t e = cudaMemsetAsync(cnt, 0, (size_t)B * p.nB * 4, s);
+    cudaError_t e = cudaMemsetAsync(lists.cnt, 0, 2 * cache_stride(B, N), s);   // cnt and head
     if (e != cudaSuccess) return fail(USV_ERR_CUDA, "merge_plan_cache: memset: %s", cudaGetErrorString(e));
-    dim3 tg(ceil_div(N, 256), B);
-    launch_dep(csr_count_kernel, dim3(tg), dim3(256), 0, s, p, N, nA - r, dst_of, pos, cnt, row_src);
-    USV_CHECK_LAUNCH("csr_count_kernel");
-    launch_dep(csr_scan_kernel, dim3(dim3(ceil_div(p.nB, 1024), B)), dim3(1024), 0, s, p.nB, cnt, off, cursor);
-    USV_CHECK_LAUNCH("csr_scan_kernel");
-    if (r > 0) {
-        launch_dep(csr_fill_kernel, dim3(tg), dim3(256), 0, s, p, N, r, dst_of, cursor, csr);
-        USV_CHECK_LAUNCH("csr_fill_kernel");
-    }
+    launch_dep(plan_lists_kernel, dim3(ceil_div(N, 256), B), dim3(256), 0, s, p, N, nA - r, dst_of, pos, lists);
+    USV_CHECK_LAUNCH("plan_lists_kernel");
     return USV_OK;
 }
 
@@ -747,16 +742,10 @@ extern "C" int usv_token_merge_apply(int B, int N, int C, const void* x, int T, 
     if (x == nullptr || cache == nullptr || x_merged == nullptr) return fail(USV_ERR_INVALID_ARG, "token_merge_apply: null pointer");
     if (!aligned16(x) || !aligned16(x_merged) || !aligned16(cache))
         return fail(USV_ERR_UNSUPPORTED, "token_merge_apply: x/x_merged/cache not 16-byte aligned");
-    char* base = static_cast<char*>(cache);
-    const size_t cs = cache_stride(B, N);
+    const MergeLists lists = cache_lists(cache, B, N);
     const int Nm = N - r;
-    const int64_t rows = (int64_t)B * Nm;
-    launch_dep(merge_kernel, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, static_cast<cudaStream_t>(stream), 
-        p, N, C, nA - r, Nm, r, static_cast<const __nv_bfloat16*>(x), reinterpret_cast<const int32_t*>(base),
-        reinterpret_cast<const int32_t*>(base + cs), reinterpret_cast<int32_t*>(base + 2 * cs),
-        static_cast<__nv_bfloat16*>(x_merged), rows);
-    USV_CHECK_LAUNCH("merge_kernel");
-    return USV_OK;
+    return launch_merge(p, N, C, nA - r, Nm, (int64_t)B * Nm, x, lists, lists.dst_copy, x_merged,
+                        static_cast<cudaStream_t>(stream));
 }
 
 extern "C" size_t usv_unmerge_map_workspace(int B, int Nm) {
@@ -781,8 +770,8 @@ extern "C" int usv_unmerge_map(int B, int N, int Nm, const int32_t* pos, int32_t
     dim3 tg(ceil_div(N, 256), B);
     launch_dep(inv_count_kernel, dim3(tg), dim3(256), 0, s, N, Nm, pos, cnt);
     USV_CHECK_LAUNCH("inv_count_kernel");
-    launch_dep(csr_scan_kernel, dim3(dim3(ceil_div(Nm, 1024), B)), dim3(1024), 0, s, Nm, cnt, inv_off, cursor);
-    USV_CHECK_LAUNCH("csr_scan_kernel");
+    launch_dep(row_scan_kernel, dim3(dim3(ceil_div(Nm, 1024), B)), dim3(1024), 0, s, Nm, cnt, inv_off, cursor);
+    USV_CHECK_LAUNCH("row_scan_kernel");
     launch_dep(inv_fill_kernel, dim3(tg), dim3(256), 0, s, N, Nm, pos, cursor, inv_idx);
     USV_CHECK_LAUNCH("inv_fill_kernel");
     return USV_OK;
