@@ -12,7 +12,7 @@
 //                          that it never does: the long-range branch of the two-branch form).
 //   combine_kernel         the two-branch form: local-cube output and long-range output, computed
 //                          apart over disjoint key sets, fused with the softmax mass of each branch
-//                          (one warp per query row, HBM stream).
+//                          (HBM stream).
 #include "usv_common.cuh"
 
 namespace usv {
@@ -55,69 +55,84 @@ struct CombineArgs {
     float* o_f32;      // optional [B,H,N,D]
     float* lse;        // optional [B,H,N]
     int H, N;
-    int64_t rows;
 };
 
-// o = (e^lse1 o1 + e^lse2 o2) / (e^lse1 + e^lse2), one warp per (b, h, n) row, D / 32 elements per lane.
+// o = (e^lse1 o1 + e^lse2 o2) / (e^lse1 + e^lse2).  HBM stream: a thread takes 8 elements (16 bytes of
+// bf16) of CB_ROWS rows and asks for all of them before it uses any; D / 8 neighbouring threads share a
+// row.  A CTA stays inside one (b, h), so its rows need no division.  2 x 12 heads of 20 280 rows of
+// 128, bf16: 61 us = 6.2 TB/s (151 us with one warp and 8 bytes a lane per row).
+constexpr int CB_ROWS = 4;
+
 template <int D, bool F32IN>
-__global__ void __launch_bounds__(256) combine_kernel(const CombineArgs a) {
+__global__ void __launch_bounds__(256) combine_kernel(const CombineArgs a, int tiles) {
     dep_sync();
-    constexpr int EPL = D / 32;   // 4 or 2
-    const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (row >= a.rows) return;
-    const int lane = threadIdx.x & 31;
-    const int n = (int)(row % a.N);
-    const int h = (int)((row / a.N) % a.H);
-    const int64_t b = row / ((int64_t)a.N * a.H);
-    const float l1 = a.lse1[row], l2 = a.lse2[row];
-    const float m = fmaxf(l1, l2);
-    const float ms = m == -INFINITY ? 0.f : m;
-    const float w1 = expf(l1 - ms), w2 = expf(l2 - ms);
-    const float tot = w1 + w2;
-    const float inv = tot > 0.f ? 1.0f / tot : 0.f;
-    float x1[EPL], x2[EPL];
-    const int64_t off1 = b * a.s1.sb + h * a.s1.sh + (int64_t)n * a.s1.sn + lane * EPL;
-    const int64_t off2 = b * a.s2.sb + h * a.s2.sh + (int64_t)n * a.s2.sn + lane * EPL;
-    if (F32IN) {
-        const float* p1 = static_cast<const float*>(a.o1) + off1;
-        const float* p2 = static_cast<const float*>(a.o2) + off2;
-        if (EPL == 4) {
-            const float4 v1 = *reinterpret_cast<const float4*>(p1), v2 = *reinterpret_cast<const float4*>(p2);
-            x1[0] = v1.x; x1[1] = v1.y; x1[EPL - 2] = v1.z; x1[EPL - 1] = v1.w;
-            x2[0] = v2.x; x2[1] = v2.y; x2[EPL - 2] = v2.z; x2[EPL - 1] = v2.w;
+    constexpr int TPR = D / 8, RPP = 256 / TPR;   // threads per row, rows of the CTA per pass
+    constexpr int W = F32IN ? 2 : 1;              // 16-byte words of a thread's 8 elements
+    const int bh = blockIdx.x / tiles;
+    const int64_t b = bh / a.H;
+    const int h = bh % a.H;
+    const int n0 = (blockIdx.x - bh * tiles) * (RPP * CB_ROWS) + threadIdx.x / TPR;
+    const int col = threadIdx.x % TPR * 8;
+    constexpr int ES = F32IN ? 4 : 2;
+    const char* p1 = static_cast<const char*>(a.o1) + (b * a.s1.sb + h * a.s1.sh + col) * ES;
+    const char* p2 = static_cast<const char*>(a.o2) + (b * a.s2.sb + h * a.s2.sh + col) * ES;
+    const float* q1 = a.lse1 + (int64_t)bh * a.N;
+    const float* q2 = a.lse2 + (int64_t)bh * a.N;
+    uint4 v1[CB_ROWS][W], v2[CB_ROWS][W];
+    float l1[CB_ROWS], l2[CB_ROWS];
+#pragma unroll
+    for (int i = 0; i < CB_ROWS; ++i) {
+        const int n = n0 + i * RPP;
+        if (n >= a.N) break;
+        l1[i] = __ldg(q1 + n);
+        l2[i] = __ldg(q2 + n);
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            v1[i][w] = __ldg(reinterpret_cast<const uint4*>(p1 + n * a.s1.sn * ES) + w);
+            v2[i][w] = __ldg(reinterpret_cast<const uint4*>(p2 + n * a.s2.sn * ES) + w);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < CB_ROWS; ++i) {
+        const int n = n0 + i * RPP;
+        if (n >= a.N) break;
+        const float m = fmaxf(l1[i], l2[i]);
+        const float ms = m == -INFINITY ? 0.f : m;
+        const float w1 = expf(l1[i] - ms), w2 = expf(l2[i] - ms);
+        const float tot = w1 + w2;
+        const float inv = tot > 0.f ? 1.0f / tot : 0.f;
+        float x1[8], x2[8], y[8];
+        if (F32IN) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                x1[e] = __uint_as_float(reinterpret_cast<const uint32_t*>(v1[i])[e]);
+                x2[e] = __uint_as_float(reinterpret_cast<const uint32_t*>(v2[i])[e]);
+            }
         } else {
-            const float2 v1 = *reinterpret_cast<const float2*>(p1), v2 = *reinterpret_cast<const float2*>(p2);
-            x1[0] = v1.x; x1[1] = v1.y;
-            x2[0] = v2.x; x2[1] = v2.y;
+            bf16x8_to_float(v1[i][0], x1);
+            bf16x8_to_float(v2[i][0], x2);
         }
-    } else {
-        const __nv_bfloat16* p1 = static_cast<const __nv_bfloat16*>(a.o1) + off1;
-        const __nv_bfloat16* p2 = static_cast<const __nv_bfloat16*>(a.o2) + off2;
 #pragma unroll
-        for (int e = 0; e < EPL; e += 2) {
-            const uint32_t u1 = *reinterpret_cast<const uint32_t*>(p1 + e);
-            const uint32_t u2 = *reinterpret_cast<const uint32_t*>(p2 + e);
-            x1[e] = __uint_as_float(u1 << 16); x1[e + 1] = __uint_as_float(u1 & 0xffff0000u);
-            x2[e] = __uint_as_float(u2 << 16); x2[e + 1] = __uint_as_float(u2 & 0xffff0000u);
+        for (int e = 0; e < 8; ++e) {
+            // a branch without keys (weight 0) must not leak a NaN or an infinity of its (undefined) output
+            const float t1 = w1 > 0.f ? w1 * x1[e] : 0.f;
+            const float t2 = w2 > 0.f ? w2 * x2[e] : 0.f;
+            y[e] = (t1 + t2) * inv;
         }
-    }
-    float y[EPL];
+        *reinterpret_cast<uint4*>(a.o + b * a.so.sb + h * a.so.sh + n * a.so.sn + col) = float8_to_bf16x8(y);
+        const int64_t row = (int64_t)bh * a.N + n;
+        if (a.o_f32 != nullptr) {
+            float* pf = a.o_f32 + row * D + col;
+            if ((reinterpret_cast<uintptr_t>(a.o_f32) & 15u) == 0) {
+                reinterpret_cast<float4*>(pf)[0] = make_float4(y[0], y[1], y[2], y[3]);
+                reinterpret_cast<float4*>(pf)[1] = make_float4(y[4], y[5], y[6], y[7]);
+            } else {
 #pragma unroll
-    for (int e = 0; e < EPL; ++e) {
-        // a branch without keys (weight 0) must not leak a NaN or an infinity of its (undefined) output
-        const float t1 = w1 > 0.f ? w1 * x1[e] : 0.f;
-        const float t2 = w2 > 0.f ? w2 * x2[e] : 0.f;
-        y[e] = (t1 + t2) * inv;
+                for (int e = 0; e < 8; ++e) pf[e] = y[e];
+            }
+        }
+        if (a.lse != nullptr && col == 0) a.lse[row] = tot > 0.f ? ms + logf(tot) : -INFINITY;
     }
-    __nv_bfloat16* po = a.o + b * a.so.sb + h * a.so.sh + (int64_t)n * a.so.sn + lane * EPL;
-#pragma unroll
-    for (int e = 0; e < EPL; e += 2) *reinterpret_cast<uint32_t*>(po + e) = pack_bf16x2(y[e], y[e + 1]);
-    if (a.o_f32 != nullptr) {
-        float* pf = a.o_f32 + row * D + lane * EPL;
-#pragma unroll
-        for (int e = 0; e < EPL; ++e) pf[e] = y[e];
-    }
-    if (a.lse != nullptr && lane == 0) a.lse[row] = tot > 0.f ? ms + logf(tot) : -INFINITY;
 }
 
 }  // namespace usv
@@ -175,16 +190,17 @@ extern "C" int usv_attn_combine(int B, int H, int N, int d, const void* o1, cons
     a.o = static_cast<__nv_bfloat16*>(o);
     a.o_f32 = o_f32; a.lse = lse;
     a.H = H; a.N = N;
-    a.rows = (int64_t)B * H * N;
-    const int64_t blocks = (a.rows + 7) / 8;
+    const int tiles = ceil_div(N, 256 / (d / 8) * CB_ROWS);
+    const int64_t blocks = (int64_t)B * H * tiles;
     if (blocks > 2147483647LL) return fail(USV_ERR_UNSUPPORTED, "attn_combine: too many rows");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const dim3 grid((unsigned)blocks), cta(256);
     if (d == 128) {
-        if (inputs_f32) launch_dep((combine_kernel<128, true>), dim3((unsigned)blocks), dim3(256), 0, st, a);
-        else launch_dep((combine_kernel<128, false>), dim3((unsigned)blocks), dim3(256), 0, st, a);
+        if (inputs_f32) launch_dep((combine_kernel<128, true>), grid, cta, 0, st, a, tiles);
+        else launch_dep((combine_kernel<128, false>), grid, cta, 0, st, a, tiles);
     } else {
-        if (inputs_f32) launch_dep((combine_kernel<64, true>), dim3((unsigned)blocks), dim3(256), 0, st, a);
-        else launch_dep((combine_kernel<64, false>), dim3((unsigned)blocks), dim3(256), 0, st, a);
+        if (inputs_f32) launch_dep((combine_kernel<64, true>), grid, cta, 0, st, a, tiles);
+        else launch_dep((combine_kernel<64, false>), grid, cta, 0, st, a, tiles);
     }
     USV_CHECK_LAUNCH("combine_kernel");
     return USV_OK;
