@@ -144,6 +144,17 @@ __device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64
         : "memory");
 }
 
+// The same with 8-bit floating-point operands (K = 32 per instruction).
+__device__ __forceinline__ void umma_ss_f8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                           uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
 // Shared-memory matrix descriptor, 128-byte swizzle.  lbo/sbo in bytes.
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
     uint64_t d = 0;
@@ -165,6 +176,11 @@ __host__ __device__ constexpr uint32_t instr_desc(int m, int n, int a_major, int
 __host__ __device__ constexpr uint32_t instr_desc_f16(int m, int n, int a_major, int b_major) {
     return (1u << 4) | ((uint32_t)a_major << 15) | ((uint32_t)b_major << 16) | (((uint32_t)n >> 3) << 17) |
            (((uint32_t)m >> 4) << 24);
+}
+
+// e4m3 x e4m3 -> fp32, both K-major
+__host__ __device__ constexpr uint32_t instr_desc_e4m3(int m, int n) {
+    return (1u << 4) | (((uint32_t)n >> 3) << 17) | (((uint32_t)m >> 4) << 24);
 }
 
 #define USV_R16(r, o) "=r"(r[o + 0]), "=r"(r[o + 1]), "=r"(r[o + 2]), "=r"(r[o + 3]), "=r"(r[o + 4]), "=r"(r[o + 5]), \
