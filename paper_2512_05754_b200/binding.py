@@ -1,5 +1,6 @@
 """ctypes binding of libusv.so.  Same names as the C entry points, torch tensors in and out."""
 import ctypes
+import functools
 import os
 from dataclasses import dataclass
 from typing import Optional
@@ -46,9 +47,34 @@ def lib():
     L.usv_last_error.restype = ctypes.c_char_p
     L.usv_build_info.restype = ctypes.c_char_p
     L.usv_kernel_launches.restype = ctypes.c_ulonglong
-    for name in ("usv_block_scores_workspace", "usv_sparse_attn_workspace",
-                 "usv_token_merge_workspace", "usv_unmerge_map_workspace", "usv_merge_plan_cache_bytes"):
-        getattr(L, name).restype = ctypes.c_size_t
+    # Argument types, declared once: a pointer goes in as the integer that data_ptr() gives, which is
+    # several times cheaper per call than wrapping each of a call's 10 to 25 arguments in an object.
+    i, p, z, f = ctypes.c_int, ctypes.c_void_p, ctypes.c_size_t, ctypes.c_float
+    for name, args in (("usv_block_scores_workspace", (i,) * 5), ("usv_sparse_attn_workspace", (i,) * 5),
+                       ("usv_token_merge_workspace", (i,) * 5), ("usv_unmerge_map_workspace", (i,) * 2),
+                       ("usv_merge_plan_cache_bytes", (i,) * 2)):
+        getattr(L, name).restype = z
+        getattr(L, name).argtypes = args
+    for name, args in (
+            ("usv_block_scores", (i,) * 5 + (p,) * 6 + (z, p)),
+            ("usv_block_scores_noalloc", (i,) * 5 + (p,) * 6),
+            ("usv_select_blocks", (i,) * 4 + (p, p, i, p, p)),
+            ("usv_sparse_attn_fwd", (i,) * 4 + (p,) * 8 + (i,) + (p,) * 4 + (f, i, p, z, p)),
+            ("usv_sparse_attn_fwd_unmerge", (i,) * 4 + (p,) * 8 + (i,) + (p,) * 4 + (f, p, z, i) + (p,) * 4),
+            ("usv_unmerge_map", (i,) * 3 + (p,) * 4 + (z, p)),
+            ("usv_token_merge", (i,) * 3 + (p, i, i, p) + (i,) * 7 + (p,) * 6 + (z, p)),
+            ("usv_token_merge_local", (i,) * 3 + (p, i, i, p) + (i,) * 10 + (p,) * 6 + (z, p)),
+            ("usv_merge_plan_cache", (i,) * 9 + (p,) * 3 + (z, p)),
+            ("usv_token_merge_apply", (i,) * 3 + (p,) + (i,) * 7 + (p,) * 3),
+            ("usv_token_unmerge", (i,) * 4 + (p,) * 4),
+            ("usv_attn_entropy", (i,) * 4 + (p,) * 6 + (i, p, f) + (p,) * 4),
+            ("usv_force_own_block", (i,) * 4 + (p,) * 2),
+            ("usv_exclude_own_block", (i,) * 4 + (p,) * 2),
+            ("usv_cube_order", (i,) * 6 + (p,) * 3),
+            ("usv_workspace_init", (p, p)), ("usv_workspace_status", (p, p)),
+            ("usv_selftest_wait_timeout", (p, ctypes.c_uint, p)), ("usv_sparse_attn_fallbacks", (p, p, p)),
+            ("usv_attn_combine", (i,) * 4 + (p,) * 6 + (i,) + (p,) * 5)):
+        getattr(L, name).argtypes = args
     _lib = L
     return L
 
@@ -63,11 +89,13 @@ def kernel_launches():
 
 
 def _ptr(t):
-    return ctypes.c_void_p(0 if t is None else t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(device):
-    return ctypes.c_void_p(torch.cuda.current_stream(device).cuda_stream)
+    """The current stream's handle as an integer (without building a torch.cuda.Stream object)."""
+    index = device.index
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if index is None else index)
 
 
 def _check(status, where):
@@ -75,10 +103,16 @@ def _check(status, where):
         raise USVError(status, where)
 
 
+@functools.lru_cache(maxsize=512)
+def _strides(sb, sh, sn):
+    """Pointer to a usv_strides with these values (read-only, so that it can be shared)."""
+    return ctypes.pointer(_Strides(sb, sh, sn))
+
+
 def _view(t, name):
     if t.dim() != 4 or t.dtype != torch.bfloat16 or not t.is_cuda or t.stride(3) != 1:
         raise ValueError("%s must be a CUDA bf16 [B,H,N,d] view with a contiguous last axis" % name)
-    return _Strides(t.stride(0), t.stride(1), t.stride(2))
+    return _strides(*t.stride()[:3])
 
 
 _ws_cache = {}
@@ -90,7 +124,7 @@ WS_HEADER = 256
 def _workspace(device, nbytes):
     """Grow-only scratch buffer per (device, stream).  Its header (status word) starts at zero
     and is carried over when the buffer grows, so that workspace_status() sees every call."""
-    key = (device.index, torch.cuda.current_stream(device).cuda_stream)
+    key = (device.index, _stream(device))
     buf = _ws_cache.get(key)
     if buf is None or buf.numel() < nbytes:
         new = torch.empty(max(int(nbytes), WS_HEADER), dtype=torch.uint8, device=device)
@@ -102,11 +136,21 @@ def _workspace(device, nbytes):
     return buf
 
 
+@functools.lru_cache(maxsize=512)
+def _k_values(ks):
+    """(int32 array, largest entry) of a tuple of Python ints; the library only reads the array."""
+    return (ctypes.c_int32 * len(ks))(*ks), max(ks)
+
+
 def _k_array(k_per_head, H):
-    ks = [int(x) for x in k_per_head]
+    ks = tuple(k_per_head)
     if len(ks) != H:
         raise ValueError("k_per_head needs one entry per head")
-    return (ctypes.c_int32 * H)(*ks), max(ks)
+    for x in ks:
+        if type(x) is not int:
+            ks = tuple(int(y) for y in ks)
+            break
+    return _k_values(ks)
 
 
 def block_scores(q, k, Nq=None, Nk=None, out=None):
@@ -121,8 +165,8 @@ def block_scores(q, k, Nq=None, Nk=None, out=None):
     L = lib()
     need = L.usv_block_scores_workspace(B, H, Nq, Nk, d)
     ws = _workspace(q.device, need)
-    _check(L.usv_block_scores(B, H, Nq, Nk, d, _ptr(q), ctypes.byref(sq), _ptr(k),
-                              ctypes.byref(sk), _ptr(out), _ptr(ws), ctypes.c_size_t(ws.numel()),
+    _check(L.usv_block_scores(B, H, Nq, Nk, d, _ptr(q), sq, _ptr(k),
+                              sk, _ptr(out), _ptr(ws), ws.numel(),
                               _stream(q.device)), "usv_block_scores")
     return out
 
@@ -141,8 +185,8 @@ def block_scores_noalloc(q, k, Nq=None, Nk=None, out=None):
     NBq, NBk = (Nq + BLOCK - 1) // BLOCK, (Nk + BLOCK - 1) // BLOCK
     if out is None:
         out = torch.empty((B, H, NBq, NBk), dtype=torch.float32, device=q.device)
-    _check(lib().usv_block_scores_noalloc(B, H, Nq, Nk, d, _ptr(q), ctypes.byref(sq), _ptr(k),
-                                          ctypes.byref(sk), _ptr(out), _stream(q.device)),
+    _check(lib().usv_block_scores_noalloc(B, H, Nq, Nk, d, _ptr(q), sq, _ptr(k),
+                                          sk, _ptr(out), _stream(q.device)),
            "usv_block_scores_noalloc")
     return out
 
@@ -191,10 +235,10 @@ def sparse_attn_fwd(q, k, v, sel, k_per_head, N=None, scale=0.0, out=None, retur
     L = lib()
     need = L.usv_sparse_attn_workspace(B, H, N, d, kmax)
     ws = _workspace(q.device, need)
-    _check(L.usv_sparse_attn_fwd(B, H, N, d, _ptr(q), ctypes.byref(sq), _ptr(k), ctypes.byref(sk),
-                                 _ptr(v), ctypes.byref(sv), _ptr(sel), karr, kmax, _ptr(out),
-                                 ctypes.byref(so), _ptr(o32), _ptr(lse), ctypes.c_float(scale),
-                                 int(impl), _ptr(ws), ctypes.c_size_t(ws.numel()),
+    _check(L.usv_sparse_attn_fwd(B, H, N, d, _ptr(q), sq, _ptr(k), sk,
+                                 _ptr(v), sv, _ptr(sel), karr, kmax, _ptr(out),
+                                 so, _ptr(o32), _ptr(lse), scale,
+                                 int(impl), _ptr(ws), ws.numel(),
                                  _stream(q.device)), "usv_sparse_attn_fwd")
     res = (out,)
     if return_f32:
@@ -218,7 +262,7 @@ def selftest_wait_timeout(limit_us=1000, device=None):
     reports USV_ERR_TIMEOUT afterwards (once)."""
     device = torch.device("cuda", torch.cuda.current_device()) if device is None else device
     ws = _workspace(device, WS_HEADER)
-    _check(lib().usv_selftest_wait_timeout(_ptr(ws), ctypes.c_uint(int(limit_us)), _stream(device)),
+    _check(lib().usv_selftest_wait_timeout(_ptr(ws), int(limit_us), _stream(device)),
            "usv_selftest_wait_timeout")
 
 
@@ -281,13 +325,13 @@ def token_merge(x, metric, grid, part, r, plan=None, debug=False, window=None, o
     if window is None:
         _check(L.usv_token_merge(B, N, C, _ptr(x), Hm, dm, _ptr(metric), T, Hh, W, st, sh, sw, int(r),
                                  _ptr(out), _ptr(plan.dst_of), _ptr(plan.pos), _ptr(u), _ptr(js),
-                                 _ptr(ws), ctypes.c_size_t(ws.numel()), _stream(dev)),
+                                 _ptr(ws), ws.numel(), _stream(dev)),
                "usv_token_merge")
     else:
         wt, wh, ww = (int(v) for v in window)
         _check(L.usv_token_merge_local(B, N, C, _ptr(x), Hm, dm, _ptr(metric), T, Hh, W, st, sh, sw, wt, wh, ww,
                                        int(r), _ptr(out), _ptr(plan.dst_of), _ptr(plan.pos), _ptr(u), _ptr(js),
-                                       _ptr(ws), ctypes.c_size_t(ws.numel()), _stream(dev)),
+                                       _ptr(ws), ws.numel(), _stream(dev)),
                "usv_token_merge_local")
     return out, plan
 
@@ -321,8 +365,8 @@ def attn_entropy(q, k, sel, k_per_head, lse, N=None, scale=0.0):
     marg = torch.empty((B, N), dtype=torch.float32, device=q.device)
     ent = torch.empty((B,), dtype=torch.float32, device=q.device)
     ws = _workspace(q.device, WS_HEADER)
-    _check(lib().usv_attn_entropy(B, H, N, d, _ptr(q), ctypes.byref(sq), _ptr(k), ctypes.byref(sk), _ptr(sel),
-                                  karr, sel.shape[3], _ptr(lse), ctypes.c_float(scale), _ptr(marg), _ptr(ent),
+    _check(lib().usv_attn_entropy(B, H, N, d, _ptr(q), sq, _ptr(k), sk, _ptr(sel),
+                                  karr, sel.shape[3], _ptr(lse), scale, _ptr(marg), _ptr(ent),
                                   _ptr(ws), _stream(q.device)), "usv_attn_entropy")
     return marg, ent
 
@@ -349,7 +393,7 @@ def cube_order(grid, cube=(4, 4, 4), device=None, want_inverse=True):
     n = max(T * Hh * W, 1)
     perm = torch.empty((n,), dtype=torch.int32, device=device)
     inv = torch.empty((n,), dtype=torch.int32, device=device) if want_inverse else None
-    _check(lib().usv_cube_order(T, Hh, W, ct, ch, cw, _ptr(perm), _ptr(inv) if want_inverse else None,
+    _check(lib().usv_cube_order(T, Hh, W, ct, ch, cw, _ptr(perm), _ptr(inv),
                                 _stream(device)), "usv_cube_order")
     return perm, inv
 
@@ -393,15 +437,14 @@ def attn_combine(o1, lse1, o2, lse2, out=None, return_f32=False, return_lse=Fals
     for l in (lse1, lse2):
         if l.dtype != torch.float32 or not l.is_contiguous() or tuple(l.shape) != (B, H, N):
             raise ValueError("lse must be a contiguous fp32 [B,H,N] tensor")
-    s1 = _Strides(o1.stride(0), o1.stride(1), o1.stride(2))
-    s2 = _Strides(o2.stride(0), o2.stride(1), o2.stride(2))
+    s1, s2 = _strides(*o1.stride()[:3]), _strides(*o2.stride()[:3])
     if out is None:
         out = torch.empty((B, H, N, d), dtype=torch.bfloat16, device=o1.device)
     so = _view(out, "o")
     o32 = torch.empty((B, H, N, d), dtype=torch.float32, device=o1.device) if return_f32 else None
     lse = torch.empty((B, H, N), dtype=torch.float32, device=o1.device) if return_lse else None
-    _check(lib().usv_attn_combine(B, H, N, d, _ptr(o1), ctypes.byref(s1), _ptr(lse1), _ptr(o2), ctypes.byref(s2),
-                                  _ptr(lse2), 1 if o1.dtype == torch.float32 else 0, _ptr(out), ctypes.byref(so),
+    _check(lib().usv_attn_combine(B, H, N, d, _ptr(o1), s1, _ptr(lse1), _ptr(o2), s2,
+                                  _ptr(lse2), 1 if o1.dtype == torch.float32 else 0, _ptr(out), so,
                                   _ptr(o32), _ptr(lse), _stream(o1.device)), "usv_attn_combine")
     res = (out,)
     if return_f32:
@@ -421,7 +464,7 @@ def unmerge_map(pos, Nm):
     idx = torch.empty((B, N), dtype=torch.int32, device=pos.device)
     L = lib()
     ws = _workspace(pos.device, L.usv_unmerge_map_workspace(B, int(Nm)))
-    _check(L.usv_unmerge_map(B, N, int(Nm), _ptr(pos), _ptr(off), _ptr(idx), _ptr(ws), ctypes.c_size_t(ws.numel()),
+    _check(L.usv_unmerge_map(B, N, int(Nm), _ptr(pos), _ptr(off), _ptr(idx), _ptr(ws), ws.numel(),
                              _stream(pos.device)), "usv_unmerge_map")
     return off, idx
 
@@ -447,10 +490,10 @@ def sparse_attn_fwd_unmerge(q, k, v, sel, k_per_head, umap, N_full, N=None, scal
     lse = torch.empty((B, H, N), dtype=torch.float32, device=q.device) if return_lse else None
     L = lib()
     ws = _workspace(q.device, L.usv_sparse_attn_workspace(B, H, N, d, kmax))
-    _check(L.usv_sparse_attn_fwd_unmerge(B, H, N, d, _ptr(q), ctypes.byref(sq), _ptr(k), ctypes.byref(sk),
-                                         _ptr(v), ctypes.byref(sv), _ptr(sel), karr, kmax, _ptr(scratch),
-                                         ctypes.byref(so), _ptr(o32), _ptr(lse), ctypes.c_float(scale), _ptr(ws),
-                                         ctypes.c_size_t(ws.numel()), int(N_full), _ptr(off), _ptr(idx), _ptr(out),
+    _check(L.usv_sparse_attn_fwd_unmerge(B, H, N, d, _ptr(q), sq, _ptr(k), sk,
+                                         _ptr(v), sv, _ptr(sel), karr, kmax, _ptr(scratch),
+                                         so, _ptr(o32), _ptr(lse), scale, _ptr(ws),
+                                         ws.numel(), int(N_full), _ptr(off), _ptr(idx), _ptr(out),
                                          _stream(q.device)), "usv_sparse_attn_fwd_unmerge")
     res = (out,)
     if return_f32:
@@ -471,7 +514,7 @@ def merge_plan_cache(plan):
         nbytes = L.usv_merge_plan_cache_bytes(B, N)
         cache = torch.empty(int(nbytes), dtype=torch.uint8, device=plan.pos.device)
         _check(L.usv_merge_plan_cache(B, N, T, Hh, W, st, sh, sw, int(plan.r), _ptr(plan.dst_of), _ptr(plan.pos),
-                                      _ptr(cache), ctypes.c_size_t(nbytes), _stream(plan.pos.device)),
+                                      _ptr(cache), nbytes, _stream(plan.pos.device)),
                "usv_merge_plan_cache")
         plan.cache = cache
     return plan.cache
