@@ -1,228 +1,268 @@
-// Top-k key-block selection.
+// Top-k key-block selection: a row of scores in the registers of one warp (up to 1536 scores) or of a few.
 //
-// Rows of up to 2048 scores: one WARP per row, select_warp_kernel (with more of a row per lane
-// the register file holds too few warps: measured slower than the CTA kernel below).  The
-// row sits in registers as order-preserving keys, striped over the lanes; the key T of the k-th
-// largest element is found bit by bit (at most 32 warp-wide counts, fewer when a candidate cuts
-// the row at exactly k), then every element above T and the first (k - above) elements equal to
-// T are emitted in ascending index (two ballots per 32 elements give the positions).
-//
-// Longer rows: one CTA per row, select_kernel.
-//
-// The row is mapped to order-preserving 32-bit keys in shared memory.  Four 8-bit radix passes
-// (most significant digit first) find the key T of the k-th largest element and the number of
-// elements strictly above it.  The output pass gives every thread a contiguous stretch of the
-// row: it counts what it keeps (every key above T, and the first (k - above) keys equal to T,
-// which is exactly "k largest, ties to the lowest index"), one block-wide scan places it, and it
-// writes its indices in ascending order.  Rows that keep everything skip the search.
+// The k-th largest score is bracketed by probes: two counts of the scores at or above a value per
+// step.  The first two values come from the mean and spread of the row as if it were normal, the next
+// from interpolation, until at most 32 scores lie between the probes on either side of k (two to four
+// steps on video-like rows).  Those are ranked directly, and everything above the last one kept, with
+// its equals up to its index, is written in ascending order: "k largest, ties to the lowest index".
+// Rows where that does not work out (NaN, no spread, many equal scores at the cut) take a search bit
+// by bit over order-preserving keys.
+#include <math.h>
+
 #include "usv_common.cuh"
 
 namespace usv {
 
-constexpr int SEL_THREADS = 256;
 constexpr int SEL_MAX_NB = 8192;
 
 struct SelHeads {
     int k[USV_MAX_HEADS];
+    float z[2][USV_MAX_HEADS];   // where the first two probes lie, in standard deviations from the mean
 };
 
-// Block-wide exclusive scan of one int per thread (SEL_THREADS threads); returns the exclusive
-// prefix and writes the block total to *total.  `scratch` holds >= 9 ints.
-__device__ __forceinline__ int block_excl_scan(int v, int* scratch, int* total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int incl = warp_incl_scan(v);
-    if (lane == 31) scratch[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        int w = lane < SEL_THREADS / 32 ? scratch[lane] : 0;
-        int wi = warp_incl_scan(w);
-        if (lane < SEL_THREADS / 32) scratch[lane] = wi - w;
-        if (lane == SEL_THREADS / 32 - 1) scratch[8] = wi;
-    }
-    __syncthreads();
-    const int res = scratch[warp] + incl - v;
-    *total = scratch[8];
-    __syncthreads();
-    return res;
-}
+constexpr int CANDS = 32;       // scores between the probes that are ranked directly (one per lane)
+constexpr int MAX_STEPS = 10;
 
-__global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __restrict__ scores,
-                                                             int32_t* __restrict__ sel, int H,
-                                                             int NBq, int NBk, int kmax,
-                                                             const SelHeads heads) {
+// W warps per row (W = 1: eight rows a CTA, no barrier).  The row passes through shared memory: warp w
+// gets the scores [w 32 KPL, ...) with coalesced asynchronous copies, and lane l of it takes KPL consecutive
+// ones (KPL is odd: no bank conflicts), so that a lane's kept indices are consecutive in the output.
+// Issue slots bound it.  40 heads x 1182 x 1182, keep 60: 113 us (316 us with the row striped over the
+// lanes, a search bit by bit, and two ballots per 32 scores on the way out); 12 x 3023 x 3023, keep 152: 186 us
+// (442 us with one CTA a row and radix passes in shared memory).
+template <int W, int KPL>
+__global__ void __launch_bounds__(W == 1 ? 256 : W * 32) select_kernel(const float* __restrict__ scores,
+                                                                      int32_t* __restrict__ sel, int H, int NBq,
+                                                                      int NBk, int kmax, const SelHeads heads,
+                                                                      int64_t rows) {
     dep_sync();
-    extern __shared__ uint32_t keys[];   // NBk order-preserving keys
-    __shared__ int hist[256];
-    __shared__ int scratch[9];
-    __shared__ uint32_t s_prefix;
-    __shared__ int s_remaining, s_eq_total;
-
-    const int row = blockIdx.x;  // (b*H + h)*NBq + I
-    const int h = (row / NBq) % H;
-    const int k = heads.k[h];
-    const float* src = scores + (int64_t)row * NBk;
-    int32_t* out = sel + (int64_t)row * kmax;
-
-    if (k >= NBk) {   // keep everything: no search
-        for (int j = threadIdx.x; j < NBk; j += SEL_THREADS) out[j] = j;
-        for (int t = NBk + threadIdx.x; t < kmax; t += SEL_THREADS) out[t] = -1;
-        return;
-    }
-    for (int j = threadIdx.x; j < NBk; j += SEL_THREADS) keys[j] = float_key(src[j]);
-    if (threadIdx.x == 0) {
-        s_prefix = 0;
-        s_remaining = k;
-    }
-    __syncthreads();
-
-    // Radix select: after the pass for digit `shift`, s_prefix holds the top bits of T and
-    // s_remaining the rank of T among the elements that share those bits.
-    for (int shift = 24; shift >= 0; shift -= 8) {
-        hist[threadIdx.x] = 0;
-        __syncthreads();
-        const uint32_t prefix = s_prefix;
-        const uint32_t mask = shift == 24 ? 0u : (0xffffffffu << (shift + 8));
-        for (int j = threadIdx.x; j < NBk; j += SEL_THREADS) {
-            const uint32_t key = keys[j];
-            if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255], 1);
-        }
-        __syncthreads();
-        if (threadIdx.x < 32) {
-            // 256 bins, scanned from the top; each lane owns 8 consecutive bins.
-            const int lane = threadIdx.x;
-            const int remaining = s_remaining;  // read by every lane before the scan's shuffles
-            int local[8], sum = 0;
-#pragma unroll
-            for (int t = 0; t < 8; ++t) {
-                local[t] = hist[255 - (lane * 8 + t)];
-                sum += local[t];
-            }
-            const int incl = warp_incl_scan(sum);
-            int before = incl - sum;  // elements in bins above this lane's bins
-#pragma unroll
-            for (int t = 0; t < 8; ++t) {
-                if (before < remaining && remaining <= before + local[t]) {
-                    s_prefix = prefix | ((uint32_t)(255 - (lane * 8 + t)) << shift);
-                    s_remaining = remaining - before;
-                    s_eq_total = local[t];   // after the last pass: how many keys equal T
-                }
-                before += local[t];
-            }
-        }
-        __syncthreads();
-    }
-    const uint32_t T = s_prefix;
-    const int need_eq = s_remaining;  // how many elements equal to T are kept (lowest indices)
-    const bool all_eq = need_eq == s_eq_total;   // no tie straddles the cut (the usual case)
-
-    // Ordered output.  Thread t owns the contiguous indices [t L, t L + L): it counts what it keeps,
-    // one block-wide scan gives its first output slot, and it writes its indices in order.
-    const int L = (NBk + SEL_THREADS - 1) / SEL_THREADS;
-    const int j0 = threadIdx.x * L, j1 = min(j0 + L, NBk);
-    int eq_base = 0;
-    if (!all_eq) {   // ties across the cut: the lowest indices among the equal keys win
-        int ne = 0;
-        for (int j = j0; j < j1; ++j) ne += keys[j] == T ? 1 : 0;
-        int tot;
-        eq_base = block_excl_scan(ne, scratch, &tot);
-    }
-    int cnt = 0;
-    {
-        int eq_seen = eq_base;
-        for (int j = j0; j < j1; ++j) {
-            const uint32_t key = keys[j];
-            if (key > T) ++cnt;
-            else if (key == T) { if (all_eq || eq_seen < need_eq) ++cnt; ++eq_seen; }
-        }
-    }
-    int tot_out;
-    int p = block_excl_scan(cnt, scratch, &tot_out);
-    {
-        int eq_seen = eq_base;
-        for (int j = j0; j < j1; ++j) {
-            const uint32_t key = keys[j];
-            bool take = key > T;
-            if (key == T) { take = all_eq || eq_seen < need_eq; ++eq_seen; }
-            if (take) out[p++] = j;
-        }
-    }
-    for (int t = k + threadIdx.x; t < kmax; t += SEL_THREADS) out[t] = -1;
-}
-
-// One warp per row; lane l holds the scores of indices i * 32 + l, i < KPL (every load of the
-// row is one contiguous 128-byte line per warp).
-template <int KPL>
-__global__ void __launch_bounds__(256, 2) select_warp_kernel(const float* __restrict__ scores,
-                                                          int32_t* __restrict__ sel, int H, int NBq,
-                                                          int NBk, int kmax, const SelHeads heads,
-                                                          int64_t rows) {
-    dep_sync();
-    const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (row >= rows) return;
-    const int lane = threadIdx.x & 31;
-    const uint32_t lt = (1u << lane) - 1u;
+    static_assert(KPL % 2 == 1 && KPL <= 64, "");
+    constexpr int G = W == 1 ? 8 : 1;               // rows per CTA
+    constexpr int SEG = 32 * KPL;                   // scores per warp
+    extern __shared__ float s_rows[];               // [G or W warps][SEG]
+    __shared__ float s_val[G][CANDS];
+    __shared__ int s_n[G];
+    __shared__ int s_cnt[2][W];
+    __shared__ float s_sum[3][W];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int g = W == 1 ? warp : 0, w = W == 1 ? 0 : warp;
+    const int64_t row = (int64_t)blockIdx.x * G + g;
+    if (row >= rows) return;                         // (W = 1: a whole warp; W > 1: never)
     const int h = (int)((row / NBq) % H);
     const int k = heads.k[h];
-    const float* src = scores + row * NBk;
+    const int tid = w * 32 + lane;                   // thread of the row
     int32_t* out = sel + row * kmax;
-    if (k >= NBk) {   // keep everything: no search (uniform over the warp)
-        for (int j = lane; j < NBk; j += 32) out[j] = j;
-        for (int t = NBk + lane; t < kmax; t += 32) out[t] = -1;
+    if (k >= NBk) {   // keep everything: no search (uniform over the row)
+        for (int j = tid; j < NBk; j += W * 32) out[j] = j;
+        for (int t = NBk + tid; t < kmax; t += W * 32) out[t] = -1;
         return;
     }
-    uint32_t key[KPL];
+    auto sync = [] { if (W == 1) __syncwarp(); else __syncthreads(); };
+    const int j0 = w * SEG;
+    float* buf = s_rows + warp * SEG;
+    {
+        const float* src = scores + row * NBk + j0 + lane;
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(buf) + lane * 4;
+        const int mine = NBk - j0 - lane;            // this lane copies the scores i * 32 < mine
 #pragma unroll
-    for (int i = 0; i < KPL; ++i) key[i] = (i * 32 + lane < NBk) ? float_key(__ldg(src + i * 32 + lane)) : 0u;   // 0 < any real key
-    // Largest T with count(key >= T) >= k, one bit at a time.  As soon as a candidate leaves
-    // exactly k keys at or above it, those k are the answer and no tie can straddle the cut.
-    // The bits above the highest one in which two real keys differ are common to all of them and
-    // to T: the search starts below them.
-    uint32_t kor = 0u, kand = 0xffffffffu;
-#pragma unroll
-    for (int i = 0; i < KPL; ++i)
-        if (i * 32 + lane < NBk) { kor |= key[i]; kand &= key[i]; }
-    kor = __reduce_or_sync(0xffffffffu, kor);
-    kand = __reduce_and_sync(0xffffffffu, kand);
-    const uint32_t diff = kor ^ kand;
-    const int top = diff ? 31 - __clz(diff) : -1;               // highest differing bit (-1: all keys equal)
-    uint32_t T = top >= 31 ? 0u : (kand & ~((2u << (top < 0 ? 0 : top)) - 1u));
-    if (top < 0) T = kand;
-    bool exact = false;
-#pragma unroll 1
-    for (int bit = top; bit >= 0; --bit) {
-        const uint32_t cand = T | (1u << bit);
-        int c = 0;
-#pragma unroll
-        for (int i = 0; i < KPL; ++i) c += key[i] >= cand ? 1 : 0;
-        const int tot = __reduce_add_sync(0xffffffffu, c);
-        if (tot >= k) T = cand;
-        if (tot == k) { exact = true; break; }
+        for (int i = 0; i < KPL; ++i) {
+            if (i * 32 < mine) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + i * 128), "l"(src + i * 32) : "memory");
+            else buf[i * 32 + lane] = -INFINITY;     // past the end: no probe counts it
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
     }
-    // keys above the cut are kept; of the keys equal to T (the k-th largest key, when the search
-    // ran to the last bit) the lowest indices fill what is left
-    const uint32_t cut = exact ? T - 1u : T;   // kept outright: key > cut
-    int need_eq = 0;
-    if (!exact) {
-        int ngt = 0;
+    for (int t = k + tid; t < kmax; t += W * 32) out[t] = -1;
+    if (tid == 0) s_n[g] = 0;
+    sync();
+    float x[KPL];
 #pragma unroll
-        for (int i = 0; i < KPL; ++i) ngt += key[i] > T ? 1 : 0;
-        need_eq = k - __reduce_add_sync(0xffffffffu, ngt);
-    }
-    int base = 0, eq_seen = 0;
+    for (int i = 0; i < KPL; ++i) x[i] = buf[lane * KPL + i];
+    const int first = j0 + lane * KPL;               // index of x[0]
+
+    // sum of one int over the row; `turn` alternates between the calls (one barrier each)
+    int turn = 0;
+    auto total = [&](int c) {
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (W == 1) return c;
+        if (lane == 0) s_cnt[turn][w] = c;
+        __syncthreads();
+        c = 0;
+#pragma unroll
+        for (int q = 0; q < W; ++q) c += s_cnt[turn][q];
+        turn ^= 1;
+        return c;
+    };
+    // exclusive sum over the lanes of the row, in index order
+    auto before = [&](int c) {
+        const int incl = warp_incl_scan(c);
+        int b = incl - c;
+        if (W > 1) {
+            if (lane == 31) s_cnt[turn][w] = incl;
+            __syncthreads();
+            for (int q = 0; q < w; ++q) b += s_cnt[turn][q];
+            turn ^= 1;
+        }
+        return b;
+    };
+
+    // 1. mean and spread of the finite scores
+    bool nan = false;
+    float sum = 0.f, sq = 0.f, cnt = 0.f;
 #pragma unroll
     for (int i = 0; i < KPL; ++i) {
-        if (i * 32 < NBk) {   // uniform over the warp
-            const bool gt = key[i] > cut;
-            const bool eq = !exact && key[i] == T && i * 32 + lane < NBk;
-            const uint32_t eqb = __ballot_sync(0xffffffffu, eq);
-            const bool take = gt || (eq && eq_seen + __popc(eqb & lt) < need_eq);
-            const uint32_t tkb = __ballot_sync(0xffffffffu, take);
-            if (take) out[base + __popc(tkb & lt)] = i * 32 + lane;
-            base += __popc(tkb);
-            eq_seen += __popc(eqb);
+        if (fabsf(x[i]) <= 3.402823466e38f) { sum += x[i]; sq = fmaf(x[i], x[i], sq); cnt += 1.f; }
+        nan |= x[i] != x[i];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        sq += __shfl_xor_sync(0xffffffffu, sq, o);
+        cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+    }
+    if (__any_sync(0xffffffffu, nan)) sum = __int_as_float(0x7fc00000);   // (reaches every warp of the row through the sum)
+    if (W > 1) {
+        if (lane == 0) { s_sum[0][w] = sum; s_sum[1][w] = sq; s_sum[2][w] = cnt; }
+        __syncthreads();
+        sum = sq = cnt = 0.f;
+#pragma unroll
+        for (int q = 0; q < W; ++q) { sum += s_sum[0][q]; sq += s_sum[1][q]; cnt += s_sum[2][q]; }
+    }
+    const float mean = sum / cnt;
+    const float sd = sqrtf(fmaxf(sq / cnt - mean * mean, 0.f));
+    float last_v = 0.f;     // the last score kept
+    bool found = false;
+    if (sd > 0.f && sd < 1e30f && fabsf(mean) < 1e30f) {   // (uniform over the row)
+        // 2. two probes a step, aimed at a few ranks on either side of k: first from the normal
+        // distribution of that mean and spread, then by interpolation between the bracketing probes
+        float lo = -INFINITY, hi = INFINITY;   // count(x >= lo) = c_lo >= k > c_hi = count(x >= hi)
+        int c_lo = NBk, c_hi = 0;
+        float t1 = fmaf(sd, heads.z[0][h], mean), t2 = fmaf(sd, heads.z[1][h], mean), reach = 0.5f * sd;
+#pragma unroll 1
+        for (int step = 0; step < MAX_STEPS; ++step) {
+            int c = 0;
+#pragma unroll
+            for (int i = 0; i < KPL; ++i) {
+                if (x[i] >= t1) c += 1;
+                if (x[i] >= t2) c += 0x10000;
+            }
+            c = total(c);
+            const int c1 = c & 0xffff, c2 = c >> 16;
+            if (c1 >= k) { lo = t1; c_lo = c1; } else { hi = t1; c_hi = c1; }
+            if (c2 >= k) { lo = t2; c_lo = c2; } else if (c1 >= k) { hi = t2; c_hi = c2; }
+            if (c_lo - c_hi <= CANDS && hi < INFINITY && lo > -INFINITY) { found = true; break; }
+            if (hi == INFINITY) {
+                t1 = lo + reach;
+                t2 = t1 + reach;
+                reach *= 4.f;
+            } else if (lo == -INFINITY) {
+                t2 = hi - reach;
+                t1 = t2 - reach;
+                reach *= 4.f;
+            } else {
+                const float span = hi - lo, per = span / (float)(c_lo - c_hi);
+                const float at = lo + per * (float)(c_lo - k);
+                const float side = fmaxf(12.f * per, 0.02f * span);
+                t1 = fmaxf(at - side, lo + 0.02f * span);
+                t2 = fminf(at + side, hi - 0.02f * span);
+                if (!(t1 > lo && t2 > t1 && t2 < hi)) break;   // the bracket has no room left
+            }
+        }
+        if (found) {
+            // 3. rank the few scores between the probes: the (k - c_hi)-th is the last one kept, unless
+            // equal scores lie on both sides of the cut
+            const int n = c_lo - c_hi, need = k - c_hi;
+            uint32_t in[2] = {0, 0};
+#pragma unroll
+            for (int i = 0; i < KPL; ++i)
+                if (x[i] >= lo && x[i] < hi) in[i / 32] |= 1u << (i % 32);
+            if (in[0] | in[1]) {
+                int at = atomicAdd(&s_n[g], __popc(in[0]) + __popc(in[1]));
+#pragma unroll
+                for (int q = 0; q < 2; ++q)
+                    for (uint32_t m = in[q]; m; m &= m - 1) s_val[g][at++] = buf[lane * KPL + q * 32 + __ffs(m) - 1];
+            }
+            sync();
+            const float v = lane < n ? s_val[g][lane] : 0.f;
+            int above = 0, equal = 0;
+            for (int q = 0; q < n; ++q) {
+                const float vq = __shfl_sync(0xffffffffu, v, q);
+                above += vq > v ? 1 : 0;
+                equal += vq == v ? 1 : 0;
+            }
+            // (among equal scores exactly the last of the kept ones has above + equal == need, if they all are kept)
+            const uint32_t at = __ballot_sync(0xffffffffu, lane < n && above + equal == need);
+            found = at != 0;
+            last_v = __shfl_sync(0xffffffffu, v, at ? __ffs(at) - 1 : 0);
         }
     }
-    for (int t = k + lane; t < kmax; t += 32) out[t] = -1;
+    uint32_t take[2] = {0, 0};                        // bit i: x[i] is kept
+    if (found) {
+#pragma unroll
+        for (int i = 0; i < KPL; ++i)
+            if (x[i] >= last_v) take[i / 32] |= 1u << (i % 32);
+    } else {
+        // Rare (NaN, no spread, no room between the probes, equal scores at the cut): the key of the k-th
+        // largest score bit by bit, then the first of the equal keys.
+        auto is = [&](int i) { return first + i < NBk; };
+        uint32_t T = 0;
+#pragma unroll 1
+        for (int bit = 31; bit >= 0; --bit) {
+            const uint32_t cand = T | (1u << bit);
+            int c = 0;
+#pragma unroll
+            for (int i = 0; i < KPL; ++i) c += is(i) && float_key(x[i]) >= cand ? 1 : 0;
+            if (total(c) >= k) T = cand;
+        }
+        int above = 0, equal = 0;
+#pragma unroll
+        for (int i = 0; i < KPL; ++i) {
+            above += is(i) && float_key(x[i]) > T ? 1 : 0;
+            equal += is(i) && float_key(x[i]) == T ? 1 : 0;
+        }
+        const int need = k - total(above);
+        int seen = before(equal);
+#pragma unroll
+        for (int i = 0; i < KPL; ++i) {
+            const bool tie = is(i) && float_key(x[i]) == T;
+            if ((tie && seen < need) || (is(i) && float_key(x[i]) > T)) take[i / 32] |= 1u << (i % 32);
+            seen += tie ? 1 : 0;
+        }
+    }
+    // 4. the kept indices in ascending order
+    int at = before(__popc(take[0]) + __popc(take[1]));
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+        for (uint32_t m = take[q]; m; m &= m - 1) out[at++] = first + q * 32 + __ffs(m) - 1;
+}
+
+template <int W, int KPL>
+static cudaError_t launch_select(const float* scores, int32_t* sel, int H, int NBq, int NBk, int kmax, const SelHeads& heads,
+                                 int64_t rows, cudaStream_t st) {
+    constexpr int WARPS = W == 1 ? 8 : W;
+    constexpr size_t smem = (size_t)WARPS * 32 * KPL * sizeof(float);
+    if (smem > 40 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(select_kernel<W, KPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    return launch_dep(select_kernel<W, KPL>, dim3((unsigned)(W == 1 ? (rows + 7) / 8 : rows)), dim3(WARPS * 32), smem, st,
+                      scores, sel, H, NBq, NBk, kmax, heads, rows);
+}
+
+// Standard deviations above the mean at which a normal distribution has a share p (0 < p < 1) of its
+// mass above: rational approximation 26.2.23 of Abramowitz and Stegun (error below 4.5e-4).
+static float upper_quantile(float p) {
+    const float q = p < 0.5f ? p : 1.f - p;
+    const float t = sqrtf(-2.f * logf(q));
+    const float z = t - (2.515517f + t * (0.802853f + t * 0.010328f)) /
+                            (1.f + t * (1.432788f + t * (0.189269f + t * 0.001308f)));
+    return p < 0.5f ? z : -z;
+}
+
+// Probes at a sixth of the smaller side (but at least 8 ranks) below and above rank k.
+static void first_probes(SelHeads& heads, int h, int NBk) {
+    const float n = (float)NBk, k = (float)heads.k[h];
+    const float side = fmaxf(8.f, fminf(k, n - k) / 6.f);
+    heads.z[0][h] = upper_quantile(fminf(k + side, n - 0.5f) / n);
+    heads.z[1][h] = upper_quantile(fmaxf(k - side, 0.5f) / n);
 }
 
 }  // namespace usv
@@ -249,15 +289,24 @@ extern "C" int usv_select_blocks(int B, int H, int NBq, int NBk, const float* sc
     const int64_t rows = (int64_t)B * H * NBq;
     if (rows > 2147483647LL) return fail(USV_ERR_UNSUPPORTED, "select_blocks: too many rows");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const unsigned wg = (unsigned)((rows + 7) / 8);
-#define USV_SEL_WARP(KPL) launch_dep(select_warp_kernel<KPL>, dim3(wg), dim3(256), 0, st, scores, sel, H, NBq, NBk, kmax, heads, rows)
-    if (NBk <= 256) USV_SEL_WARP(8);
-    else if (NBk <= 512) USV_SEL_WARP(16);
-    else if (NBk <= 1024) USV_SEL_WARP(32);
-    else if (NBk <= 1536) USV_SEL_WARP(48);
-    else if (NBk <= 2048) USV_SEL_WARP(64);
-    else launch_dep(select_kernel, dim3((unsigned)rows), dim3(SEL_THREADS), (size_t)NBk * sizeof(uint32_t), st, scores, sel, H, NBq, NBk, kmax, heads);
-#undef USV_SEL_WARP
+    for (int h = 0; h < H; ++h) first_probes(heads, h, NBk);
+#define USV_SEL(W, KPL) launch_select<W, KPL>(scores, sel, H, NBq, NBk, kmax, heads, rows, st)
+    // The smallest form that holds the row.  One warp a row up to 544 scores (512 scores, 12 288 rows: 16.7 us,
+    // 22.4 with two warps), then two: at 1182 scores and 47 280 rows two warps of 19 scores a lane take
+    // 113 us and one warp of 37 119 us; at 3023 and 36 276 rows two warps take 186 us, four 239 us.
+    if (NBk <= 288) USV_SEL(1, 9);
+    else if (NBk <= 352) USV_SEL(1, 11);
+    else if (NBk <= 544) USV_SEL(1, 17);
+    else if (NBk <= 832) USV_SEL(2, 13);
+    else if (NBk <= 1088) USV_SEL(2, 17);
+    else if (NBk <= 1216) USV_SEL(2, 19);
+    else if (NBk <= 1472) USV_SEL(2, 23);
+    else if (NBk <= 2112) USV_SEL(2, 33);
+    else if (NBk <= 3136) USV_SEL(2, 49);
+    else if (NBk <= 4224) USV_SEL(4, 33);
+    else if (NBk <= 6272) USV_SEL(4, 49);
+    else USV_SEL(8, 33);
+#undef USV_SEL
     USV_CHECK_LAUNCH("select_kernel");
     return USV_OK;
 }

@@ -1,0 +1,56 @@
+"""Top-k selection where the probe search can go wrong: row lengths at the edges of every form of the
+kernel, rows without spread, heavy tails, infinities, NaN, ties across the cut, the smallest and largest
+k.  Exact against an ordering of the same fp32 values by (key, index)."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.fixture(scope="module")
+def usv():
+    import paper_2512_05754_b200 as m
+    return m
+
+
+def _reference(scores, ks):
+    """Order-preserving integer keys (-0 as +0, NaN between the negative and the other values), k largest, ties to the lower index."""
+    u = (scores + np.float32(0)).view(np.uint32).astype(np.int64)
+    key = np.where(u & 0x80000000, 0xffffffff - u, u | 0x80000000)
+    key = np.where(np.isnan(scores), 0x7fffffff, key)
+    order = np.argsort(-key, axis=-1, kind="stable")
+    out = np.full(scores.shape[:-1] + (max(ks),), -1, dtype=np.int32)
+    for h, k in enumerate(ks):
+        out[:, h, :, :k] = np.sort(order[:, h, :, :k], axis=-1)
+    return out
+
+
+EDGES = [1, 2, 31, 33, 288, 289, 352, 353, 544, 545, 832, 833, 1088, 1089, 1216, 1217, 1472, 1473, 2112, 2113, 3136, 3137,
+         4224, 4225, 6272, 6273, 8192]
+
+
+@pytest.mark.parametrize("NB", EDGES)
+def test_rows_of_every_kind(usv, NB):
+    rng = np.random.default_rng(NB)
+    rows = []
+    x = rng.standard_normal(NB)
+    rows.append(x)                                            # what the first probes assume
+    rows.append(np.sin(np.arange(NB) * 0.1) * 3 + 0.1 * x)    # two-sided, light tails
+    rows.append(rng.standard_cauchy(NB))                      # outliers far beyond the spread
+    rows.append(np.exp(8 * x))                                # one-sided over many octaves
+    rows.append(np.round(2 * x))                              # a handful of values: ties across the cut
+    rows.append(np.full(NB, -0.25))                           # one value
+    rows.append(np.where(rng.random(NB) < 0.5, 0.0, -0.0))    # both zeros are equal
+    rows.append(1e30 * x)                                     # squares overflow
+    y = x.copy(); y[NB // 2] = np.inf; rows.append(y)         # an own block forced in
+    y = x.copy(); y[NB // 3] = -np.inf; rows.append(y)        # and one kept out
+    y = x.copy(); y[rng.random(NB) < 0.7] = -np.inf; rows.append(y)
+    y = x.copy(); y[0] = np.nan; rows.append(y)
+    scores = np.stack(rows).astype(np.float32)[None, None].repeat(4, axis=1)
+    ks = [1, max(1, NB // 10), max(1, (2 * NB) // 3), max(1, NB - 1)]
+    sel = usv.select_blocks(torch.from_numpy(scores).to(DEV), ks, kmax=max(ks) + 3).cpu().numpy()
+    ref = _reference(scores, ks)
+    assert np.array_equal(sel[..., :max(ks)], ref)
+    assert (sel[..., max(ks):] == -1).all()
