@@ -75,7 +75,7 @@ unsigned long long usv_kernel_launches(void);
  * q: bf16 view [B,H,Nq,d], k: bf16 view [B,H,Nk,d]; d in {64,128}.
  * scores: fp32 [B,H,NBq,NBk] contiguous (written).  ws: pooled means (and, at d = 128, the bf16
  * operand planes of the tensor-core product, which is accumulated in fp32 from a three-way split
- * of every fp32 mean and is fp32-accurate), see *_workspace().
+ * of every fp32 mean and is fp32-accurate; small calls use fp32 CUDA cores), see *_workspace().
  */
 size_t usv_block_scores_workspace(int B, int H, int Nq, int Nk, int d);
 int usv_block_scores(int B, int H, int Nq, int Nk, int d, const void* q, const usv_strides* sq,

@@ -247,11 +247,11 @@ int launch_attn_mma(const AttnArgs& a, int d, cudaStream_t st) {
     if (d == 128) {
         cudaFuncSetAttribute(attn_mma_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)MmaSmem<128>::BYTES);
-        launch_dep(attn_mma_kernel<128>, dim3((unsigned)grid), dim3(128), MmaSmem<128>::BYTES, st, a);
+        launch_dep_smem(attn_mma_kernel<128>, dim3((unsigned)grid), dim3(128), MmaSmem<128>::BYTES, st, a);
     } else {
         cudaFuncSetAttribute(attn_mma_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)MmaSmem<64>::BYTES);
-        launch_dep(attn_mma_kernel<64>, dim3((unsigned)grid), dim3(128), MmaSmem<64>::BYTES, st, a);
+        launch_dep_smem(attn_mma_kernel<64>, dim3((unsigned)grid), dim3(128), MmaSmem<64>::BYTES, st, a);
     }
     USV_CHECK_LAUNCH("attn_mma_kernel");
     return USV_OK;

@@ -507,15 +507,15 @@ int launch_pair_plan(AttnArgs& a, void* mem, cudaStream_t st) {
         uint16_t* by_rank = reinterpret_cast<uint16_t*>(base + L.by_rank);
         ord = {by_rank, reinterpret_cast<uint8_t*>(base + L.taken), reinterpret_cast<int*>(base + L.count), 1};
         const int64_t rows = (int64_t)BH * a.NB;
-        launch_dep(plan::plan_keys_kernel, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, a, keys, ord.count);
+        launch_dep_smem(plan::plan_keys_kernel, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, a, keys, ord.count);
         USV_CHECK_LAUNCH("plan_keys_kernel");
-        launch_dep(plan::plan_sort_kernel, dim3(2 * BH), dim3(1024), 0, st, a.NB, keys, by_rank);
+        launch_dep_smem(plan::plan_sort_kernel, dim3(2 * BH), dim3(1024), 0, st, a.NB, keys, by_rank);
         USV_CHECK_LAUNCH("plan_sort_kernel");
-        launch_dep(plan::pair_plan_kernel, grid, dim3(plan::THREADS), smem, st, a, pairs, lists, ord, nbuf);
+        launch_dep_smem(plan::pair_plan_kernel, grid, dim3(plan::THREADS), smem, st, a, pairs, lists, ord, nbuf);
         USV_CHECK_LAUNCH("pair_plan_kernel (first pass)");
         ord.pass = 2;
     }
-    launch_dep(plan::pair_plan_kernel, grid, dim3(plan::THREADS), smem, st, a, pairs, lists, ord, nbuf);
+    launch_dep_smem(plan::pair_plan_kernel, grid, dim3(plan::THREADS), smem, st, a, pairs, lists, ord, nbuf);
     USV_CHECK_LAUNCH("pair_plan_kernel");
     return USV_OK;
 }

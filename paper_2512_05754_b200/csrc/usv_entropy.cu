@@ -188,7 +188,7 @@ extern "C" int usv_attn_entropy(int B, int H, int N, int d, const void* q, const
         launch_dep(key_marginal_kernel<64>, dim3((unsigned)grid), dim3(128), smem, st, a);
     }
     if (d != 128) USV_CHECK_LAUNCH("key_marginal_kernel");
-    launch_dep(entropy_kernel, dim3(B), dim3(1024), 0, st, key_marginal, N, entropy);
+    launch_dep_smem(entropy_kernel, dim3(B), dim3(1024), 0, st, key_marginal, N, entropy);
     USV_CHECK_LAUNCH("entropy_kernel");
     return USV_OK;
 }

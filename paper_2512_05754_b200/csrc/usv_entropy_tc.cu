@@ -201,7 +201,7 @@ int launch_marginal_tc(const MargArgs& a, cudaStream_t st) {
     cudaError_t e = cudaFuncSetAttribute(et::marginal_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)et::SMEM_BYTES);
     if (e != cudaSuccess) return fail(USV_ERR_CUDA, "attn_entropy: smem attribute: %s", cudaGetErrorString(e));
-    launch_dep(et::marginal_tc_kernel, dim3((unsigned)grid), dim3(et::NTHREADS), et::SMEM_BYTES, st, a, maps);
+    launch_dep_smem(et::marginal_tc_kernel, dim3((unsigned)grid), dim3(et::NTHREADS), et::SMEM_BYTES, st, a, maps);
     USV_CHECK_LAUNCH("marginal_tc_kernel");
     return USV_OK;
 }

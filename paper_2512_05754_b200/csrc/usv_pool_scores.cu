@@ -5,6 +5,7 @@
 //                   rows of a block.  At d = 128 it also writes the three bf16 planes
 //                   (mean = hi + mid + lo) that the tensor-core score kernel multiplies, so the
 //                   fp32 means are not read back for a separate split pass.
+//   scores_small_kernel : the scores of small calls, fp32 CUDA cores (both head widths).
 //   scores_kernel : fp32 CUDA-core NT GEMM per (b,h), 64x64 output tile, 4x4 per thread.
 //                   Kept in fp32 (not bf16 tensor cores) because the result decides an integer
 //                   (the top-k set) that is compared with an fp64 evaluation.
@@ -22,12 +23,18 @@ struct PoolArgs {
     // (NULL: not wanted); rows NB .. NB_pad - 1 are written as zero
     __nv_bfloat16* planes[2];
     int NB_pad[2];
+    int span;           // consecutive blocks per CTA
 };
 
 // D = head dim (64 or 128).  Threads: 128.  A row of D bf16 is D/8 uint4; TPR threads per row.
-// A CTA pools POOL_SPAN consecutive blocks of one (tensor, b, h); the loads of the next block are
-// issued before the current one is reduced, so that the CTA always has a block in flight.
+// A CTA pools `span` consecutive blocks of one (tensor, b, h); the loads of the next block are issued
+// before the current one is reduced, so that the CTA always has a block in flight.  Up to four blocks
+// where there are enough of them to fill the GPU, fewer (and more CTAs) for small calls.
 constexpr int POOL_SPAN = 4;
+static int pool_span(int64_t blocks) {
+    const int64_t s = blocks / 1480;   // ten CTAs per SM
+    return s < 1 ? 1 : (s < POOL_SPAN ? (int)s : POOL_SPAN);
+}
 
 template <int D>
 __global__ void __launch_bounds__(128) pool_kernel(const PoolArgs a) {
@@ -37,9 +44,9 @@ __global__ void __launch_bounds__(128) pool_kernel(const PoolArgs a) {
     constexpr int ITERS = USV_BLOCK / RPI;
     const int which = blockIdx.z;
     const int NB = a.NB[which];
-    const int I0 = blockIdx.x * POOL_SPAN;
+    const int I0 = blockIdx.x * a.span;
     if (I0 >= NB) return;
-    const int I1 = min(I0 + POOL_SPAN, NB);
+    const int I1 = min(I0 + a.span, NB);
     const int bh = blockIdx.y;
     const int b = bh / a.H, h = bh % a.H;
     const int N = a.N[which];
@@ -168,6 +175,74 @@ __global__ void __launch_bounds__(256) scores_kernel(const float* __restrict__ q
     }
 }
 
+// The same product for small calls: 32 x 32 output tiles, 64 features of both operands in shared memory
+// after one round of loads, 2 x 2 outputs a thread, features in ascending order as above.  (All 128
+// features at once need 34 KB, and with that another split of the SM's memory than pool_kernel has.)
+constexpr int SCT = 32;
+
+template <int D>
+__global__ void __launch_bounds__(256) scores_small_kernel(const float* __restrict__ qbar, const float* __restrict__ kbar,
+                                                           float* __restrict__ scores, int NBq, int NBk, float scale) {
+    dep_sync();
+    constexpr int TK = 64;
+    __shared__ __align__(16) float As[SCT][TK + 4];
+    __shared__ __align__(16) float Bs[SCT][TK + 4];
+    const int bh = blockIdx.z;
+    const int i0 = blockIdx.y * SCT, j0 = blockIdx.x * SCT;
+    const float4* A = reinterpret_cast<const float4*>(qbar + (int64_t)bh * NBq * D);
+    const float4* Bm = reinterpret_cast<const float4*>(kbar + (int64_t)bh * NBk * D);
+    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+    constexpr int L = SCT * TK / 4 / 256;   // 16-byte loads per thread, operand and round
+    float4 va[D / TK][L], vb[D / TK][L];
+#pragma unroll
+    for (int k = 0; k < D / TK; ++k)
+#pragma unroll
+        for (int l = 0; l < L; ++l) {
+            const int r = ty + 16 * l, c = k * (TK / 4) + tx;
+            va[k][l] = i0 + r < NBq ? A[(int64_t)(i0 + r) * (D / 4) + c] : make_float4(0, 0, 0, 0);
+            vb[k][l] = j0 + r < NBk ? Bm[(int64_t)(j0 + r) * (D / 4) + c] : make_float4(0, 0, 0, 0);
+        }
+    float acc[2][2] = {};
+#pragma unroll
+    for (int k = 0; k < D / TK; ++k) {
+        if (k > 0) __syncthreads();
+#pragma unroll
+        for (int l = 0; l < L; ++l) {
+            *reinterpret_cast<float4*>(&As[ty + 16 * l][tx * 4]) = va[k][l];
+            *reinterpret_cast<float4*>(&Bs[ty + 16 * l][tx * 4]) = vb[k][l];
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int e = 0; e < TK; e += 4) {
+            float4 av[2], bv[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                av[i] = *reinterpret_cast<const float4*>(&As[ty + 16 * i][e]);
+                bv[i] = *reinterpret_cast<const float4*>(&Bs[tx + 16 * i][e]);
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 2; ++j)
+                    acc[i][j] = fmaf(av[i].w, bv[j].w, fmaf(av[i].z, bv[j].z, fmaf(av[i].y, bv[j].y, fmaf(av[i].x, bv[j].x, acc[i][j]))));
+        }
+    }
+    float* out = scores + (int64_t)bh * NBq * NBk;
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int I = i0 + ty + 16 * i, J = j0 + tx + 16 * j;
+            if (I < NBq && J < NBk) out[(int64_t)I * NBk + J] = acc[i][j] * scale;
+        }
+}
+
+// The small form takes calls of at most this many 32 x 32 tiles.  Whole calls, us, with the kernels for large
+// calls / with this one: d = 64, 12 tiles 5.9 / 4.0, 256: 10.8 / 8.1, 768: 13.8 / 13.6, 1024: 11.9 / 12.9;
+// d = 128 (tensor-core kernel), 12 tiles 13.5 / 6.1, 256: 15.0 / 10.0, 768: 27.9 / 27.9, 1024: 18.5 / 22.4.
+constexpr int64_t SMALL_TILES = 700;
+static int64_t small_tiles(int BH, int NBq, int NBk) { return (int64_t)BH * ceil_div(NBq, SCT) * ceil_div(NBk, SCT); }
+
 }  // namespace usv
 
 extern "C" size_t usv_block_scores_workspace(int B, int H, int Nq, int Nk, int d) {
@@ -213,17 +288,27 @@ extern "C" int usv_block_scores(int B, int H, int Nq, int Nk, int d, const void*
     a.planes[0] = a.planes[1] = nullptr;
     a.NB_pad[0] = a.NB_pad[1] = 0;
     void* tc_mem = reinterpret_cast<char*>(kbar) + align_up((size_t)B * H * NBk * d * sizeof(float), 256);
-    if (d == 128) scores_tc_planes(tc_mem, B * H, NBq, NBk, &a.planes[0], &a.planes[1], &a.NB_pad[0], &a.NB_pad[1]);
-    dim3 pg(ceil_div(NBq > NBk ? NBq : NBk, POOL_SPAN), B * H, 2);
+    const int64_t tiles = small_tiles(B * H, NBq, NBk);
+    const bool small = tiles <= SMALL_TILES;
+    if (d == 128 && !small) scores_tc_planes(tc_mem, B * H, NBq, NBk, &a.planes[0], &a.planes[1], &a.NB_pad[0], &a.NB_pad[1]);
+    a.span = pool_span((int64_t)B * H * (NBq + NBk));
+    dim3 pg(ceil_div(NBq > NBk ? NBq : NBk, a.span), B * H, 2);
     if (d == 128) launch_dep(pool_kernel<128>, dim3(pg), dim3(128), 0, st, a);
     else launch_dep(pool_kernel<64>, dim3(pg), dim3(128), 0, st, a);
     USV_CHECK_LAUNCH("pool_kernel");
 
+    const float sc = 1.0f / sqrtf((float)d);
+    if (small) {
+        dim3 tg(ceil_div(NBk, SCT), ceil_div(NBq, SCT), B * H);
+        if (d == 128) launch_dep(scores_small_kernel<128>, tg, dim3(256), 0, st, qbar, kbar, scores, NBq, NBk, sc);
+        else launch_dep(scores_small_kernel<64>, tg, dim3(256), 0, st, qbar, kbar, scores, NBq, NBk, sc);
+        USV_CHECK_LAUNCH("scores_small_kernel");
+        return USV_OK;
+    }
     if (d == 128)
-        return launch_scores_tc(scores, B * H, NBq, NBk, 1.0f / sqrtf((float)d), tc_mem,
-                                static_cast<unsigned int*>(ws), st);
+        return launch_scores_tc(scores, B * H, NBq, NBk, sc, tc_mem, static_cast<unsigned int*>(ws), st);
     dim3 sg(ceil_div(NBk, 64), ceil_div(NBq, 64), B * H);
-    launch_dep(scores_kernel, dim3(sg), dim3(256), 0, st, qbar, kbar, scores, NBq, NBk, d, 1.0f / sqrtf((float)d));
+    launch_dep(scores_kernel, dim3(sg), dim3(256), 0, st, qbar, kbar, scores, NBq, NBk, d, sc);
     USV_CHECK_LAUNCH("scores_kernel");
     return USV_OK;
 }
@@ -298,7 +383,8 @@ extern "C" int usv_block_scores_noalloc(int B, int H, int Nq, int Nk, int d, con
     a.H = H;
     a.planes[0] = a.planes[1] = nullptr;
     a.NB_pad[0] = a.NB_pad[1] = 0;
-    dim3 pg(ceil_div(NBq > NBk ? NBq : NBk, POOL_SPAN), B * H, 2);
+    a.span = pool_span((int64_t)B * H * (NBq + NBk));
+    dim3 pg(ceil_div(NBq > NBk ? NBq : NBk, a.span), B * H, 2);
     if (d == 128) pool_kernel<128><<<pg, 128, 0, st>>>(a);
     else pool_kernel<64><<<pg, 128, 0, st>>>(a);
     USV_CHECK_LAUNCH("pool_kernel (noalloc)");

@@ -243,7 +243,7 @@ static cudaError_t launch_select(const float* scores, int32_t* sel, int H, int N
         cudaError_t e = cudaFuncSetAttribute(select_kernel<W, KPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    return launch_dep(select_kernel<W, KPL>, dim3((unsigned)(W == 1 ? (rows + 7) / 8 : rows)), dim3(WARPS * 32), smem, st,
+    return launch_dep_smem(select_kernel<W, KPL>, dim3((unsigned)(W == 1 ? (rows + 7) / 8 : rows)), dim3(WARPS * 32), smem, st,
                       scores, sel, H, NBq, NBk, kmax, heads, rows);
 }
 
