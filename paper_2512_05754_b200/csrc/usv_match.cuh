@@ -4,20 +4,80 @@
 
 namespace usv {
 
+// Division of 0 <= n < 2^31 by a divisor that the host knows: multiply, add, shift (Granlund and
+// Montgomery, "Division by invariant integers using multiplication", 1994).
+struct Div {
+    uint32_t m = 0, s = 0;
+    int d = 1;
+    Div() = default;
+    explicit Div(int divisor) : d(divisor) {
+        while ((1ll << s) < d) ++s;
+        m = (uint32_t)((((1ull << s) - d) << 32) / d + 1);
+    }
+    __host__ __device__ int quot(int n) const {
+#ifdef __CUDA_ARCH__
+        return (int)((__umulhi(m, (uint32_t)n) + (uint32_t)n) >> s);
+#else
+        return n / d;
+#endif
+    }
+    // quotient; n becomes the remainder
+    __host__ __device__ int split(int& n) const {
+        const int q = quot(n);
+        n -= q * d;
+        return q;
+    }
+};
+
+// Every kernel of the merge looks tokens up in the partition, most of them once per warp: with
+// hardware division that was a dozen divisions of ~25 instructions a token.
 struct Part {
     int T, Hh, W, st, sh, sw;
     int nHy, nWx, nB;  // destinations per axis (y, x) and in total
-    __host__ __device__ bool is_dst(int n) const {
-        const int x = n % W, y = (n / W) % Hh, t = n / (W * Hh);
-        return (t % st == 0) && (y % sh == 0) && (x % sw == 0);
+    Div dW, dH, dst, dsh, dsw, dWx, dHy;
+    Part() = default;
+    Part(int T_, int Hh_, int W_, int st_, int sh_, int sw_)
+        : T(T_), Hh(Hh_), W(W_), st(st_), sh(sh_), sw(sw_), nHy(ceil_div(Hh_, sh_)), nWx(ceil_div(W_, sw_)),
+          nB(ceil_div(T_, st_) * nHy * nWx), dW(W_), dH(Hh_), dst(st_), dsh(sh_), dsw(sw_), dWx(nWx), dHy(nHy) {}
+    // n = (t, y, x) in raster order
+    __host__ __device__ void coords(int n, int& t, int& y, int& x) const {
+        x = n;
+        y = dW.split(x);
+        t = dH.split(y);
     }
-    // ordinal (ascending token order) of a destination token
+    // Whether token n is a destination, and its place: ordinal among the destinations (ascending token
+    // order) or rank among the sources (its index minus the destinations before it).
+    __host__ __device__ bool place(int n, int& at) const {
+        int t, y, x;
+        coords(n, t, y, x);
+        int rt = t, ry = y, rx = x;
+        const int bt = dst.split(rt), by = dsh.split(ry), bx = dsw.split(rx);
+        if ((rt | ry | rx) == 0) {
+            at = (bt * nHy + by) * nWx + bx;
+            return true;
+        }
+        int before = (bt + (rt != 0)) * nHy * nWx;                 // whole destination frames before t
+        if (rt == 0) {
+            before += (by + (ry != 0)) * nWx;                      // whole destination rows before y
+            if (ry == 0) before += bx + (rx != 0);                 // destinations before x in this row
+        }
+        at = n - before;
+        return false;
+    }
+    __host__ __device__ bool is_dst(int n) const {
+        int at;
+        return place(n, at);
+    }
+    // ordinal of the destination of n's partition block
     __host__ __device__ int ord(int n) const {
-        const int x = n % W, y = (n / W) % Hh, t = n / (W * Hh);
-        return ((t / st) * nHy + y / sh) * nWx + x / sw;
+        int t, y, x;
+        coords(n, t, y, x);
+        return (dst.quot(t) * nHy + dsh.quot(y)) * nWx + dsw.quot(x);
     }
     __host__ __device__ int dst_token(int o) const {
-        const int dx = o % nWx, dy = (o / nWx) % nHy, dt = o / (nWx * nHy);
+        int dx = o;
+        int dy = dWx.split(dx);
+        const int dt = dHy.split(dy);
         return ((dt * st) * Hh + dy * sh) * W + dx * sw;
     }
 };
@@ -26,15 +86,14 @@ struct MatchTcArgs {
     Part p;
     int B, N, nA, nA_pad, nB_pad;
     const int32_t* src_idx;          // [nA] source tokens, ascending
-    uint16_t* a_h;                   // fp16 bits [B][nA_pad][dm]
-    uint16_t* b_h;                   // fp16 bits [B][nB_pad][dm]
-    float* cand_v;                   // [B][nA][2][4] largest approximate cosines per source and tile parity, descending
-    int* cand_i;                     // [B][nA][2][4] their destination ordinals
+    uint16_t* a_h;                   // fp16 bits [B][nA_pad][dm]: sources by rank, zero-padded
+    uint16_t* b_h;                   // fp16 bits [B][nB_pad][dm]: destinations by ordinal, zero-padded
+    float* cand_v;                   // [B][nA][2][8] largest approximate cosines per source and tile parity, descending
+    int* cand_i;                     // [B][nA][2][8] their destination ordinals
     int* exact_list;                 // sources (b * nA + rank) that need the fp32 scan of all destinations
     int* exact_count;
-    int zero_words;              // 32-bit words from exact_count on that half_kernel sets to zero
+    int* exact_done;                 // one slot per list entry: chunks of the scan that are finished
     unsigned long long* exact_best;  // one slot per list entry: (key of the best cosine << 32) | ~destination
-    float* floor_v;                  // [B][nA_pad] lower bound on each source's approximate row maximum
     int32_t* jstar_s;                // [B][nA] best destination TOKEN per source rank
     float* u_s;                      // [B][nA] its cosine
     unsigned int* status;            // device status word for bounded waits (may be NULL)
@@ -42,8 +101,11 @@ struct MatchTcArgs {
 
 // bytes of the matcher's scratch for a sequence of N tokens (any partition: sources + destinations = N)
 size_t match_tc_bytes(int B, int N, int dm);
-// mhat: fp32 unit descriptors [B,N,dm], dm = 64 or 128; mem: match_tc_bytes(B, N, dm) bytes, 256-byte aligned.
-int launch_match_tc(const float* mhat, const Part& p, int B, int N, int nA, int dm, const int32_t* src_idx,
-                    int32_t* jstar_s, float* u_s, void* mem, unsigned int* status, cudaStream_t st);
+// Fills in what m.p, m.B, m.N and m.nA leave open; mem: match_tc_bytes(B, N, dm) bytes, 256-byte aligned.
+void match_tc_args(MatchTcArgs& m, int dm, const int32_t* src_idx, int32_t* jstar_s, float* u_s, void* mem,
+                   unsigned int* status);
+// mhat: fp32 unit descriptors [B,N,dm], dm = 64 or 128.  a_h, b_h and a zero exact_count have been
+// written by kernels before it in the stream.
+int launch_match_tc(const float* mhat, const MatchTcArgs& m, int dm, cudaStream_t st);
 
 }  // namespace usv

@@ -17,7 +17,7 @@
 // 20 691 sources against 7410 destinations at DM = 64: 852 us on fp32 CUDA cores, 101 us here (all
 // kernels of this file).
 //
-//   half_kernel         fp32 descriptors -> fp16 rows, sources (by rank) and destinations (by
+//   (usv_merge.cu)      desc_kernel writes the fp16 rows, sources (by rank) and destinations (by
 //                       ordinal) apart, zero-padded to multiples of 128 rows
 //   match_tc_kernel     one CTA per 128 sources: their rows sit in TMEM as the A operand, the
 //                       destination rows stream through shared memory (TMA, 4 stages); warp 8 =
@@ -46,7 +46,8 @@ constexpr int W_PROD = 8, W_MMA0 = 9;                   // warps 0-7: two epilog
 constexpr int NCAND = 8;                                // best approximate cosines kept per source and tile parity
 constexpr float EPS = 1.0e-3f;                          // bound on |approximate - exact cosine| (see above)
 constexpr uint32_t SM_SCR = 0;                          // float[32][256]: a chunk of one row per epilogue thread
-constexpr uint32_t SM_BAR = SM_SCR + 32 * 256 * 4;
+constexpr uint32_t SM_FLOOR = SM_SCR + 32 * 256 * 4;     // float[128]: floor per source row
+constexpr uint32_t SM_BAR = SM_FLOOR + 128 * 4;
 enum { B_AFULL = 0, B_BFULL = 1, B_BEMPTY = B_BFULL + STAGES, B_DFULL = B_BEMPTY + STAGES, B_DFREE = B_DFULL + 2 * NBUF,
        B_COUNT = B_DFREE + 2 * NBUF };
 static_assert(B_COUNT <= 32, "barrier area");
@@ -70,49 +71,6 @@ __device__ __forceinline__ float dot(const Floats<V>& x, const Floats<V>& y) {
 #pragma unroll
     for (int e = V - 2; e >= 0; --e) acc = fmaf(x.v[e], y.v[e], acc);
     return acc;
-}
-
-template <int DM>
-__global__ void __launch_bounds__(256)
-half_kernel(const float* __restrict__ mhat, MatchTcArgs m) {
-    dep_sync();
-    constexpr int V = DM / 32;
-    for (int64_t w = (int64_t)blockIdx.x * 256 + threadIdx.x; w < m.zero_words; w += (int64_t)gridDim.x * 256)
-        reinterpret_cast<unsigned int*>(m.exact_count)[w] = 0u;
-    // one warp per output row (V floats per lane)
-    const int64_t gw = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    const int64_t rows_a = (int64_t)m.B * m.nA_pad, rows_b = (int64_t)m.B * m.nB_pad;
-    if (gw >= rows_a + rows_b) return;
-    const bool is_b = gw >= rows_a;
-    const int64_t rr = is_b ? gw - rows_a : gw;
-    const int pad = is_b ? m.nB_pad : m.nA_pad, cnt = is_b ? m.p.nB : m.nA;
-    const int b = (int)(rr / pad), i = (int)(rr % pad);
-    Floats<V> v = {};
-    if (i < cnt) {
-        const int tok = is_b ? m.p.dst_token(i) : m.src_idx[i];
-        v = *reinterpret_cast<const Floats<V>*>(mhat + ((int64_t)b * m.N + tok) * DM + lane * V);
-    }
-    struct alignas(V * 2) { __half2 h[V / 2]; } out;
-#pragma unroll
-    for (int e = 0; e < V; e += 2) out.h[e / 2] = __floats2half2_rn(v.v[e], v.v[e + 1]);
-    *reinterpret_cast<decltype(out)*>((is_b ? m.b_h : m.a_h) + rr * DM + lane * V) = out;
-    if (!is_b) {
-        // A lower bound on the source's row maximum, known before the big product starts: its exact
-        // cosine with the destination of its own partition block, less the error bound.  Video
-        // tokens mostly match a neighbour, so the bound is usually close to the maximum and the
-        // matcher's window is narrow from the first tile on.  (Any value that cannot exceed the
-        // approximate row maximum is a valid floor; a poor one only costs time.)
-        float floor_v = -INFINITY;
-        if (i < cnt) {
-            const int own = m.p.dst_token(m.p.ord(m.src_idx[i]));
-            float acc = dot<V>(v, *reinterpret_cast<const Floats<V>*>(mhat + ((int64_t)b * m.N + own) * DM + lane * V));
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            floor_v = acc - 2.0f * EPS;   // exact - EPS bounds its approximate value from below; another EPS of slack
-        }
-        if (lane == 0) m.floor_v[rr] = floor_v;
-    }
 }
 
 struct Maps {
@@ -250,7 +208,36 @@ match_tc_kernel(const MatchTcArgs m, const __grid_constant__ Maps maps) {
 #pragma unroll
         for (int c = 0; c < NCAND; ++c) { cval[c] = -INFINITY; cidx[c] = 0; }
         float vmax = -INFINITY, vlast = -INFINITY;
-        const float floor_v = m.floor_v[(int64_t)b * m.nA_pad + a];   // never above the row's approximate maximum
+        // A lower bound on the row's approximate maximum, known before the first tile: the cosine of
+        // the fp16 rows of the source and of the destination of its own partition block, less
+        // the accumulation error.  Video tokens mostly match a neighbour, so the bound is usually
+        // close to the maximum and the window is narrow from the first tile on.  (Any value that cannot
+        // exceed the approximate maximum is a valid floor; a poor one only costs time.)  Group 1
+        // works it out while group 0 fills the A operand.
+        float* s_floor = reinterpret_cast<float*>(sm + SM_FLOOR);
+        if (eg == 1) {
+            float c0 = 0.f, c1 = 0.f;
+            if (a < m.nA) {
+                const int own = m.p.ord(m.src_idx[a]);
+                const uint4* px = reinterpret_cast<const uint4*>(m.a_h + ((int64_t)b * m.nA_pad + a) * DM);
+                const uint4* py = reinterpret_cast<const uint4*>(m.b_h + ((int64_t)b * m.nB_pad + own) * DM);
+#pragma unroll 4
+                for (int i = 0; i < DM / 8; ++i) {
+                    const uint4 xv = __ldg(px + i), yv = __ldg(py + i);
+                    const uint32_t xw[4] = {xv.x, xv.y, xv.z, xv.w}, yw[4] = {yv.x, yv.y, yv.z, yv.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float2 fx = __half22float2(*reinterpret_cast<const __half2*>(xw + e));
+                        const float2 fy = __half22float2(*reinterpret_cast<const __half2*>(yw + e));
+                        c0 = fmaf(fx.x, fy.x, c0);
+                        c1 = fmaf(fx.y, fy.y, c1);
+                    }
+                }
+            }
+            s_floor[r] = c0 + c1 - 1e-5f;   // (sums of 128 products of unit vectors, two orders: 2e-6 apart at most)
+        }
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        const float floor_v = s_floor[r];
         bool ok = true;
         for (int t = eg; t < T; t += 2) {
             const int buf = t % NBUF;
@@ -400,7 +387,12 @@ recheck_kernel(const float* __restrict__ mhat, MatchTcArgs m) {
     const float window = fmaxf(__shfl_sync(0xffffffffu, v, 0), __shfl_sync(0xffffffffu, v, NCAND)) - 2.0f * EPS;
     unsigned in = __ballot_sync(0xffffffffu, v >= window);   // (never true for -inf entries)
     if (in & ((1u << (NCAND - 1)) | (1u << (2 * NCAND - 1)))) {
-        if (lane == 0) m.exact_list[atomicAdd(m.exact_count, 1)] = (int)gw;
+        if (lane == 0) {
+            const int w = atomicAdd(m.exact_count, 1);
+            m.exact_list[w] = (int)gw;
+            m.exact_done[w] = 0;
+            m.exact_best[w] = 0ull;
+        }
         return;
     }
     const float* M = mhat + (int64_t)b * m.N * DM;
@@ -495,23 +487,17 @@ match_exact_kernel(const float* __restrict__ mhat, MatchTcArgs m) {
             unsigned long long bb = s_key[0];
             for (int q = 1; q < 8; ++q) bb = s_key[q] > bb ? s_key[q] : bb;
             atomicMax(m.exact_best + w, bb);
+            __threadfence();
+            if (atomicAdd(m.exact_done + w, 1) == nchunks - 1) {   // the last chunk of this source: every best is in
+                __threadfence();
+                const unsigned long long key = atomicMax(m.exact_best + w, 0ull);
+                const uint32_t fk = (uint32_t)(key >> 32);
+                const uint32_t bits = (fk & 0x80000000u) ? (fk & 0x7fffffffu) : ~fk;    // inverse of float_key
+                m.jstar_s[gw] = m.p.dst_token((int)(0xffffffffu - (uint32_t)key));
+                m.u_s[gw] = __uint_as_float(bits);
+            }
         }
         __syncthreads();
-    }
-}
-
-__global__ void __launch_bounds__(256)
-match_exact_finish_kernel(MatchTcArgs m) {
-    dep_sync();
-    const int count = *m.exact_count;
-    for (int w = blockIdx.x * 256 + threadIdx.x; w < count; w += gridDim.x * 256) {
-        const unsigned long long key = m.exact_best[w];
-        const uint32_t fk = (uint32_t)(key >> 32);
-        const uint32_t bits = (fk & 0x80000000u) ? (fk & 0x7fffffffu) : ~fk;    // inverse of float_key
-        const int j = (int)(0xffffffffu - (uint32_t)key);
-        const int gw = m.exact_list[w];
-        m.jstar_s[gw] = m.p.dst_token(j);
-        m.u_s[gw] = __uint_as_float(bits);
     }
 }
 
@@ -533,65 +519,52 @@ static int make_rows_map(CUtensorMap* map, const void* ptr, int64_t rows, int DM
 
 static inline int pad128(int n) { return (n + 127) / 128 * 128; }
 
-// Layout of the scratch: fp16 rows of sources and destinations (each side padded to 128 rows),
-// the candidates (value, destination) per source and tile parity, the list of the exact scan, its counter and results, the floors.
 static size_t rows_bytes(int B, int N, int dm) { return align_up((size_t)B * ((size_t)N + 256) * dm * sizeof(uint16_t), 256); }
 static size_t cand_bytes(int B, int N) { return align_up((size_t)B * N * 2 * mt::NCAND * sizeof(float), 256); }
-
 static size_t list_bytes(int B, int N) { return align_up((size_t)B * N * sizeof(int), 256); }
 
 size_t match_tc_bytes(int B, int N, int dm) {
-    // rows | candidate values | candidate destinations | exact-scan list | its counter | its results | floors
-    return rows_bytes(B, N, dm) + 2 * cand_bytes(B, N) + list_bytes(B, N) + 256 + 2 * list_bytes(B, N) +
-           align_up((size_t)B * ((size_t)N + 128) * sizeof(float), 256);
+    // fp16 rows | candidate values | candidate destinations | exact scan: list, chunk counters, results, counter
+    return rows_bytes(B, N, dm) + 2 * cand_bytes(B, N) + 4 * list_bytes(B, N) + 256;
+}
+
+void match_tc_args(MatchTcArgs& m, int dm, const int32_t* src_idx, int32_t* jstar_s, float* u_s, void* mem,
+                   unsigned int* status) {
+    const int B = m.B, N = m.N;
+    m.nA_pad = pad128(m.nA); m.nB_pad = pad128(m.p.nB);
+    m.src_idx = src_idx; m.jstar_s = jstar_s; m.u_s = u_s; m.status = status;
+    char* at = static_cast<char*>(mem);
+    auto take = [&](size_t bytes) { char* p = at; at += bytes; return p; };
+    m.a_h = reinterpret_cast<uint16_t*>(take(rows_bytes(B, N, dm)));
+    m.b_h = m.a_h + (size_t)B * m.nA_pad * dm;
+    m.cand_v = reinterpret_cast<float*>(take(cand_bytes(B, N)));
+    m.cand_i = reinterpret_cast<int*>(take(cand_bytes(B, N)));
+    m.exact_list = reinterpret_cast<int*>(take(list_bytes(B, N)));
+    m.exact_done = reinterpret_cast<int*>(take(list_bytes(B, N)));
+    m.exact_best = reinterpret_cast<unsigned long long*>(take(2 * list_bytes(B, N)));
+    m.exact_count = reinterpret_cast<int*>(take(256));
 }
 
 template <int dm>
-static int launch_match(const float* mhat, const Part& p, int B, int N, int nA, const int32_t* src_idx,
-                        int32_t* jstar_s, float* u_s, void* mem, unsigned int* status, cudaStream_t st) {
-    MatchTcArgs m;
-    m.p = p; m.B = B; m.N = N; m.nA = nA;
-    m.nA_pad = pad128(nA); m.nB_pad = pad128(p.nB);
-    m.src_idx = src_idx; m.jstar_s = jstar_s; m.u_s = u_s; m.status = status;
-    char* base = static_cast<char*>(mem);
-    m.a_h = reinterpret_cast<uint16_t*>(base);
-    m.b_h = m.a_h + (size_t)B * m.nA_pad * dm;
-    m.cand_v = reinterpret_cast<float*>(base + rows_bytes(B, N, dm));
-    m.cand_i = reinterpret_cast<int*>(base + rows_bytes(B, N, dm) + cand_bytes(B, N));
-    m.exact_list = reinterpret_cast<int*>(base + rows_bytes(B, N, dm) + 2 * cand_bytes(B, N));
-    char* after_list = base + rows_bytes(B, N, dm) + 2 * cand_bytes(B, N) + list_bytes(B, N);
-    m.exact_count = reinterpret_cast<int*>(after_list);
-    m.exact_best = reinterpret_cast<unsigned long long*>(after_list + 256);
-    m.floor_v = reinterpret_cast<float*>(after_list + 256 + 2 * list_bytes(B, N));
-    // counter and result slots of the exact scan start at zero: they are adjacent, and half_kernel
-    // clears them (a memset between two kernels costs them their overlapped launch)
-    m.zero_words = (int)((256 + 2 * list_bytes(B, N)) / 4);
-    cudaError_t e;
-    const int64_t rows = (int64_t)B * (m.nA_pad + m.nB_pad);
-    launch_dep(mt::half_kernel<dm>, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, mhat, m);
-    USV_CHECK_LAUNCH("half_kernel");
+static int launch_match(const float* mhat, const MatchTcArgs& m, cudaStream_t st) {
     mt::Maps maps;
     int rc;
-    if ((rc = mt::make_rows_map(&maps.b_h, m.b_h, (int64_t)B * m.nB_pad, dm, "b_h")) != USV_OK) return rc;
-    e = cudaFuncSetAttribute(mt::match_tc_kernel<dm>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mt::SMEM_BYTES<dm>);
+    if ((rc = mt::make_rows_map(&maps.b_h, m.b_h, (int64_t)m.B * m.nB_pad, dm, "b_h")) != USV_OK) return rc;
+    cudaError_t e = cudaFuncSetAttribute(mt::match_tc_kernel<dm>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mt::SMEM_BYTES<dm>);
     if (e != cudaSuccess) return fail(USV_ERR_CUDA, "token_merge: smem attribute: %s", cudaGetErrorString(e));
-    dim3 grid(m.nA_pad / 128, B);
+    dim3 grid(m.nA_pad / 128, m.B);
     launch_dep(mt::match_tc_kernel<dm>, dim3(grid), dim3(352), mt::SMEM_BYTES<dm>, st, m, maps);
     USV_CHECK_LAUNCH("match_tc_kernel");
-    const int64_t srcs = (int64_t)B * nA;
+    const int64_t srcs = (int64_t)m.B * m.nA;
     launch_dep(mt::recheck_kernel<dm>, dim3((unsigned)((srcs + 7) / 8)), dim3(256), 0, st, mhat, m);
     USV_CHECK_LAUNCH("recheck_kernel");
-    launch_dep(mt::match_exact_kernel<dm>, dim3(1184), dim3(256), 0, st, mhat, m);
+    launch_dep(mt::match_exact_kernel<dm>, dim3(592), dim3(256), 0, st, mhat, m);
     USV_CHECK_LAUNCH("match_exact_kernel");
-    launch_dep(mt::match_exact_finish_kernel, dim3(8), dim3(256), 0, st, m);
-    USV_CHECK_LAUNCH("match_exact_finish_kernel");
     return USV_OK;
 }
 
-int launch_match_tc(const float* mhat, const Part& p, int B, int N, int nA, int dm, const int32_t* src_idx,
-                    int32_t* jstar_s, float* u_s, void* mem, unsigned int* status, cudaStream_t st) {
-    return dm == 64 ? launch_match<64>(mhat, p, B, N, nA, src_idx, jstar_s, u_s, mem, status, st)
-                    : launch_match<128>(mhat, p, B, N, nA, src_idx, jstar_s, u_s, mem, status, st);
+int launch_match_tc(const float* mhat, const MatchTcArgs& m, int dm, cudaStream_t st) {
+    return dm == 64 ? launch_match<64>(mhat, m, st) : launch_match<128>(mhat, m, st);
 }
 
 }  // namespace usv

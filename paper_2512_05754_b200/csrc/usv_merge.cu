@@ -1,7 +1,7 @@
 // Token merge / unmerge (Sec. 3.3 of the USV paper).
 //
 //   desc_kernel        Eq. 7-8   head-averaged, unit-normalised key descriptors (HBM stream)
-//   src_list_kernel    Eq. 6     ascending list of source tokens of the bipartite partition
+//                                and the ascending list of source tokens of the partition (Eq. 6)
 //   (usv_match_tc.cu)  Eq. 8-9   cosine of every source against every destination of its batch
 //                                element with a fused row arg-max, on the tensor cores
 //   match_local_kernel           the same inside a window of partition blocks (fp32 CUDA cores)
@@ -10,6 +10,7 @@
 //                                and the lists of merged sources per destination (Eq. 12)
 //   merge_kernel       Eq. 13-14 warp-per-row gather + mean, 16-byte accesses
 //   unmerge_kernel     Eq. 15    warp-per-row gather copy, 16-byte accesses
+#include <cuda_fp16.h>
 #include <math.h>
 
 #include "usv_match.cuh"
@@ -17,19 +18,38 @@
 namespace usv {
 
 // ---------------------------------------------------------------------------- descriptors
-// One warp per token.  DM/8 lanes cover one head's row with 16-byte loads; 32/(DM/8) heads are
-// read in parallel and combined with shuffles.
+// HBM stream, one warp per token.  DM/8 lanes cover one head's row with 16-byte loads; 32/(DM/8) heads
+// are read in parallel and combined with shuffles.  Besides the fp32 descriptors the warp writes what
+// it has at hand without another pass: the tokens of the sources by rank, and for the tensor-core
+// matcher (m.a_h != NULL) the fp16 rows of sources and destinations.  (Kernels of their own for those
+// took 17 us at 32 760 tokens, 86 us at 2 x 118 800.  One warp per partition block, which could also
+// compare sources with their destination, left too few loads in flight: 432 us at 2 x 118 800, 270 us
+// this way.)  It also clears what later kernels count in: `zero` (zero_words words), exact_count.
 template <int DM>
 __global__ void __launch_bounds__(256) desc_kernel(const __nv_bfloat16* __restrict__ metric,
-                                                   float* __restrict__ mhat, int64_t tokens,
-                                                   int Hm) {
+                                                   float* __restrict__ mhat, int Hm,
+                                                   int32_t* __restrict__ src_idx, int32_t* __restrict__ zero,
+                                                   int64_t zero_words, const MatchTcArgs m) {
     dep_sync();
     constexpr int LPH = DM / 8;    // lanes per head row
     constexpr int HPW = 32 / LPH;  // heads handled at once
-    const int64_t tok = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (tok >= tokens) return;
+    if (blockIdx.y == 0) {
+        for (int64_t w = (int64_t)blockIdx.x * 256 + threadIdx.x; w < zero_words; w += (int64_t)gridDim.x * 256) zero[w] = 0;
+        if (blockIdx.x == 0 && threadIdx.x == 0 && m.a_h != nullptr) *m.exact_count = 0;
+    }
+    const int b = blockIdx.y, n = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     const int chunk = lane % LPH, hsub = lane / LPH;
+    if (n >= m.N) {
+        // the rows that pad sources and destinations to multiples of 128
+        const int i = n - m.N, pa = m.nA_pad - m.nA;
+        if (m.a_h == nullptr || i >= pa + m.nB_pad - m.p.nB || hsub != 0) return;
+        uint16_t* row = i < pa ? m.a_h + ((int64_t)b * m.nA_pad + m.nA + i) * DM
+                               : m.b_h + ((int64_t)b * m.nB_pad + m.p.nB + i - pa) * DM;
+        *reinterpret_cast<uint4*>(row + chunk * 8) = make_uint4(0, 0, 0, 0);
+        return;
+    }
+    const int64_t tok = (int64_t)b * m.N + n;
     const __nv_bfloat16* src = metric + tok * Hm * DM + chunk * 8;
     float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     for (int h = hsub; h < Hm; h += HPW) {
@@ -52,11 +72,21 @@ __global__ void __launch_bounds__(256) desc_kernel(const __nv_bfloat16* __restri
 #pragma unroll
     for (int o = 1; o < LPH; o <<= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
     const float inv = 1.0f / fmaxf(sqrtf(n2), 1e-12f);
-    if (hsub == 0) {
-        float* dst = mhat + tok * DM + chunk * 8;
-        *reinterpret_cast<float4*>(dst) = make_float4(acc[0] * inv, acc[1] * inv, acc[2] * inv, acc[3] * inv);
-        *reinterpret_cast<float4*>(dst + 4) = make_float4(acc[4] * inv, acc[5] * inv, acc[6] * inv, acc[7] * inv);
-    }
+    if (hsub != 0) return;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[e] *= inv;
+    float* dst = mhat + tok * DM + chunk * 8;
+    *reinterpret_cast<float4*>(dst) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+    *reinterpret_cast<float4*>(dst + 4) = make_float4(acc[4], acc[5], acc[6], acc[7]);
+    int at;
+    const bool is_dst = m.p.place(n, at);
+    if (!is_dst && b == 0 && lane == 0) src_idx[at] = n;
+    if (m.a_h == nullptr) return;
+    uint16_t* row = is_dst ? m.b_h + ((int64_t)b * m.nB_pad + at) * DM : m.a_h + ((int64_t)b * m.nA_pad + at) * DM;
+    struct alignas(16) { __half2 h[4]; } out;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) out.h[e] = __floats2half2_rn(acc[2 * e], acc[2 * e + 1]);
+    *reinterpret_cast<decltype(out)*>(row + chunk * 8) = out;
 }
 
 // ---------------------------------------------------------------------------- block scan (1024)
@@ -76,25 +106,6 @@ __device__ __forceinline__ int block_scan_1024(int v, int* scratch, int* total) 
     *total = scratch[32];
     __syncthreads();
     return res;
-}
-
-// Ascending list of the source tokens (same for every batch element): the rank of a source is
-// its token index minus the number of destinations before it, which the partition gives in
-// closed form, so every token is handled independently.
-// It also clears the list counters that plan_assign_kernel adds to (zero_words words).
-__global__ void __launch_bounds__(256) src_list_kernel(Part p, int N, int32_t* __restrict__ src_idx,
-                                                       int32_t* __restrict__ zero, int64_t zero_words) {
-    dep_sync();
-    const int n = blockIdx.x * 256 + threadIdx.x;
-    for (int64_t w = n; w < zero_words; w += (int64_t)gridDim.x * 256) zero[w] = 0;
-    if (n >= N || p.is_dst(n)) return;
-    const int x = n % p.W, y = (n / p.W) % p.Hh, t = n / (p.W * p.Hh);
-    int before = ((t + p.st - 1) / p.st) * p.nHy * p.nWx;      // whole destination frames before t
-    if (t % p.st == 0) {
-        before += ((y + p.sh - 1) / p.sh) * p.nWx;              // whole destination rows before y
-        if (y % p.sh == 0) before += (x + p.sw - 1) / p.sw;     // destinations before x in this row
-    }
-    src_idx[n - before] = n;
 }
 
 // ---------------------------------------------------------------------------- merged-source lists
@@ -319,8 +330,9 @@ __global__ void __launch_bounds__(256) match_local_kernel(const float* __restric
     const int lane = threadIdx.x & 31;
     const float* mb = mhat + (int64_t)b * N * DM;
     const int i = src_idx[a];
-    const int x = i % p.W, y = (i / p.W) % p.Hh, t = i / (p.W * p.Hh);
-    const int bt = t / p.st, by = y / p.sh, bx = x / p.sw;
+    int t, y, x;
+    p.coords(i, t, y, x);
+    const int bt = p.dst.quot(t), by = p.dsh.quot(y), bx = p.dsw.quot(x);
     const int nBt = p.nB / (p.nHy * p.nWx);
     float mi[V];
 #pragma unroll
@@ -588,10 +600,7 @@ static int token_merge_impl(int B, int N, int C, const void* x, int Hm, int dm,
         return fail(USV_ERR_INVALID_ARG, "token_merge: null pointer");
     if (!aligned16(x) || !aligned16(x_merged) || !aligned16(ws))
         return fail(USV_ERR_UNSUPPORTED, "token_merge: x/x_merged/ws not 16-byte aligned");
-    Part p;
-    p.T = T; p.Hh = Hh; p.W = W; p.st = st; p.sh = sh; p.sw = sw;
-    p.nHy = ceil_div(Hh, sh); p.nWx = ceil_div(W, sw);
-    p.nB = ceil_div(T, st) * p.nHy * p.nWx;
+    const Part p(T, Hh, W, st, sh, sw);
     const int nA = N - p.nB;
     if (r < 0 || r > nA) return fail(USV_ERR_INVALID_ARG, "token_merge: r=%d outside [0,%d] (number of sources)", r, nA);
     if (metric != nullptr) {
@@ -617,13 +626,15 @@ static int token_merge_impl(int B, int N, int C, const void* x, int Hm, int dm,
     const int nU = nA - r, Nm = N - r;
 
     if (metric != nullptr) {
-        const int64_t tokens = (int64_t)B * N;
-        const unsigned dg = (unsigned)((tokens + 7) / 8);
-        if (dm == 128) launch_dep(desc_kernel<128>, dim3(dg), dim3(256), 0, s, static_cast<const __nv_bfloat16*>(metric), mhat, tokens, Hm);
-        else launch_dep(desc_kernel<64>, dim3(dg), dim3(256), 0, s, static_cast<const __nv_bfloat16*>(metric), mhat, tokens, Hm);
+        MatchTcArgs m = {};
+        m.p = p; m.B = B; m.N = N; m.nA = nA;
+        if (nA > 0 && win == nullptr)
+            match_tc_args(m, dm, src_idx, jstar_s, u_s, base + L.split, reinterpret_cast<unsigned int*>(base + L.status));
+        // one warp per token, and one per padding row
+        const dim3 dg(ceil_div(m.a_h != nullptr ? m.nA_pad + m.nB_pad : N, 8), B);
+        if (dm == 128) launch_dep(desc_kernel<128>, dg, dim3(256), 0, s, static_cast<const __nv_bfloat16*>(metric), mhat, Hm, src_idx, lists.cnt, (int64_t)(zero_bytes / 4), m);
+        else launch_dep(desc_kernel<64>, dg, dim3(256), 0, s, static_cast<const __nv_bfloat16*>(metric), mhat, Hm, src_idx, lists.cnt, (int64_t)(zero_bytes / 4), m);
         USV_CHECK_LAUNCH("desc_kernel");
-        launch_dep(src_list_kernel, dim3(ceil_div(N, 256)), dim3(256), 0, s, p, N, src_idx, lists.cnt, (int64_t)(zero_bytes / 4));
-        USV_CHECK_LAUNCH("src_list_kernel");
         if (nA > 0) {
             if (win != nullptr) {
                 dim3 lg(ceil_div(nA, 8), B);
@@ -632,8 +643,7 @@ static int token_merge_impl(int B, int N, int C, const void* x, int Hm, int dm,
                 USV_CHECK_LAUNCH("match_local_kernel");
             } else {
                 // tensor cores: fp16 cosines propose, fp32 decides (usv_match_tc.cu)
-                unsigned int* status = reinterpret_cast<unsigned int*>(base + L.status);
-                int rc = launch_match_tc(mhat, p, B, N, nA, dm, src_idx, jstar_s, u_s, base + L.split, status, s);
+                int rc = launch_match_tc(mhat, m, dm, s);
                 if (rc != USV_OK) return rc;
             }
         }
@@ -693,9 +703,7 @@ static int fill_part(Part& p, int N, int T, int Hh, int W, int st, int sh, int s
     if (T <= 0 || Hh <= 0 || W <= 0 || (int64_t)T * Hh * W != N)
         return fail(USV_ERR_INVALID_ARG, "%s: T*Hh*W = %lld != N = %d", who, (long long)T * Hh * W, N);
     if (st <= 0 || sh <= 0 || sw <= 0) return fail(USV_ERR_INVALID_ARG, "%s: partition sizes must be positive", who);
-    p.T = T; p.Hh = Hh; p.W = W; p.st = st; p.sh = sh; p.sw = sw;
-    p.nHy = ceil_div(Hh, sh); p.nWx = ceil_div(W, sw);
-    p.nB = ceil_div(T, st) * p.nHy * p.nWx;
+    p = Part(T, Hh, W, st, sh, sw);
     return USV_OK;
 }
 }  // namespace usv
