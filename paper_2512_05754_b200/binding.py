@@ -1,6 +1,8 @@
-"""ctypes binding of libusv.so.  Same names as the C entry points, torch tensors in and out."""
+"""Binding of libusv.so.  Same names as the C entry points, torch tensors in and out.  The calls of the
+hot path go through the CPython module _usv (csrc/usv_py.cpp), the others through ctypes."""
 import ctypes
 import functools
+import importlib.util
 import os
 from dataclasses import dataclass
 from typing import Optional
@@ -47,8 +49,6 @@ def lib():
     L.usv_last_error.restype = ctypes.c_char_p
     L.usv_build_info.restype = ctypes.c_char_p
     L.usv_kernel_launches.restype = ctypes.c_ulonglong
-    # Argument types, declared once: a pointer goes in as the integer that data_ptr() gives, which is
-    # several times cheaper per call than wrapping each of a call's 10 to 25 arguments in an object.
     i, p, z, f = ctypes.c_int, ctypes.c_void_p, ctypes.c_size_t, ctypes.c_float
     for name, args in (("usv_block_scores_workspace", (i,) * 5), ("usv_sparse_attn_workspace", (i,) * 5),
                        ("usv_token_merge_workspace", (i,) * 5), ("usv_unmerge_map_workspace", (i,) * 2),
@@ -56,27 +56,41 @@ def lib():
         getattr(L, name).restype = z
         getattr(L, name).argtypes = args
     for name, args in (
-            ("usv_block_scores", (i,) * 5 + (p,) * 6 + (z, p)),
             ("usv_block_scores_noalloc", (i,) * 5 + (p,) * 6),
-            ("usv_select_blocks", (i,) * 4 + (p, p, i, p, p)),
-            ("usv_sparse_attn_fwd", (i,) * 4 + (p,) * 8 + (i,) + (p,) * 4 + (f, i, p, z, p)),
             ("usv_sparse_attn_fwd_unmerge", (i,) * 4 + (p,) * 8 + (i,) + (p,) * 4 + (f, p, z, i) + (p,) * 4),
             ("usv_unmerge_map", (i,) * 3 + (p,) * 4 + (z, p)),
-            ("usv_token_merge", (i,) * 3 + (p, i, i, p) + (i,) * 7 + (p,) * 6 + (z, p)),
-            ("usv_token_merge_local", (i,) * 3 + (p, i, i, p) + (i,) * 10 + (p,) * 6 + (z, p)),
-            ("usv_merge_plan_cache", (i,) * 9 + (p,) * 3 + (z, p)),
-            ("usv_token_merge_apply", (i,) * 3 + (p,) + (i,) * 7 + (p,) * 3),
-            ("usv_token_unmerge", (i,) * 4 + (p,) * 4),
-            ("usv_attn_entropy", (i,) * 4 + (p,) * 6 + (i, p, f) + (p,) * 4),
-            ("usv_force_own_block", (i,) * 4 + (p,) * 2),
-            ("usv_exclude_own_block", (i,) * 4 + (p,) * 2),
             ("usv_cube_order", (i,) * 6 + (p,) * 3),
-            ("usv_workspace_init", (p, p)), ("usv_workspace_status", (p, p)),
-            ("usv_selftest_wait_timeout", (p, ctypes.c_uint, p)), ("usv_sparse_attn_fallbacks", (p, p, p)),
-            ("usv_attn_combine", (i,) * 4 + (p,) * 6 + (i,) + (p,) * 5)):
+            ("usv_workspace_status", (p, p)), ("usv_selftest_wait_timeout", (p, ctypes.c_uint, p)),
+            ("usv_sparse_attn_fallbacks", (p, p, p))):
         getattr(L, name).argtypes = args
     _lib = L
     return L
+
+
+def _load_native():
+    lib()                       # builds what is missing
+    if not os.path.exists(_build.MODULE):
+        try:
+            _build.build()
+        except Exception as e:  # no silent fallback
+            raise ImportError("_usv.so is not built and could not be built: %s" % e)
+    spec = importlib.util.spec_from_file_location("_usv", _build.MODULE)
+    module = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(module)
+    module.on_error(_check)
+    return module
+
+
+class _Native:
+    """Stands for the module until its first use."""
+
+    def __getattr__(self, name):
+        global _native
+        _native = _load_native()
+        return getattr(_native, name)
+
+
+_native = _Native()
 
 
 def build_info():
@@ -115,25 +129,15 @@ def _view(t, name):
     return _strides(*t.stride()[:3])
 
 
-_ws_cache = {}
-
-
 WS_HEADER = 256
 
 
 def _workspace(device, nbytes):
-    """Grow-only scratch buffer per (device, stream).  Its header (status word) starts at zero
-    and is carried over when the buffer grows, so that workspace_status() sees every call."""
-    key = (device.index, _stream(device))
-    buf = _ws_cache.get(key)
-    if buf is None or buf.numel() < nbytes:
-        new = torch.empty(max(int(nbytes), WS_HEADER), dtype=torch.uint8, device=device)
-        if buf is None:
-            _check(lib().usv_workspace_init(_ptr(new), _stream(device)), "usv_workspace_init")
-        else:
-            new[:WS_HEADER].copy_(buf[:WS_HEADER])
-        _ws_cache[key] = buf = new
-    return buf
+    """Grow-only scratch buffer per (device, stream), kept by the native module and shared with its calls.
+    Its header (status word) starts at zero and is carried over when the buffer grows, so that
+    workspace_status() sees every call."""
+    index = device.index
+    return _native.workspace(torch.cuda.current_device() if index is None else index, int(nbytes))
 
 
 @functools.lru_cache(maxsize=512)
@@ -155,20 +159,7 @@ def _k_array(k_per_head, H):
 
 def block_scores(q, k, Nq=None, Nk=None, out=None):
     """scores[b,h,I,J] of the pooled 64-token blocks; fp32 [B,H,NBq,NBk]."""
-    sq, sk = _view(q, "q"), _view(k, "k")
-    B, H, nq, d = q.shape
-    Nq = nq if Nq is None else int(Nq)
-    Nk = k.shape[2] if Nk is None else int(Nk)
-    NBq, NBk = (Nq + BLOCK - 1) // BLOCK, (Nk + BLOCK - 1) // BLOCK
-    if out is None:
-        out = torch.empty((B, H, NBq, NBk), dtype=torch.float32, device=q.device)
-    L = lib()
-    need = L.usv_block_scores_workspace(B, H, Nq, Nk, d)
-    ws = _workspace(q.device, need)
-    _check(L.usv_block_scores(B, H, Nq, Nk, d, _ptr(q), sq, _ptr(k),
-                              sk, _ptr(out), _ptr(ws), ws.numel(),
-                              _stream(q.device)), "usv_block_scores")
-    return out
+    return _native.block_scores(q, k, Nq, Nk, out)
 
 
 def block_scores_noalloc(q, k, Nq=None, Nk=None, out=None):
@@ -193,16 +184,7 @@ def block_scores_noalloc(q, k, Nq=None, Nk=None, out=None):
 
 def select_blocks(scores, k_per_head, kmax=None, out=None):
     """Top-k key blocks per (b,h,I), ascending, ties to the lowest index; int32 [B,H,NBq,kmax]."""
-    if scores.dtype != torch.float32 or not scores.is_cuda or not scores.is_contiguous():
-        raise ValueError("scores must be a contiguous CUDA fp32 tensor")
-    B, H, NBq, NBk = scores.shape
-    karr, kmx = _k_array(k_per_head, H)
-    kmax = kmx if kmax is None else int(kmax)
-    if out is None:
-        out = torch.empty((B, H, NBq, kmax), dtype=torch.int32, device=scores.device)
-    _check(lib().usv_select_blocks(B, H, NBq, NBk, _ptr(scores), karr, kmax, _ptr(out),
-                                   _stream(scores.device)), "usv_select_blocks")
-    return out
+    return _native.select_blocks(scores, k_per_head, kmax, out)
 
 
 def sparse_attn_fwd(q, k, v, sel, k_per_head, N=None, scale=0.0, out=None, return_f32=False,
@@ -210,42 +192,7 @@ def sparse_attn_fwd(q, k, v, sel, k_per_head, N=None, scale=0.0, out=None, retur
     """Block-sparse attention forward.  Returns o (bf16, layout of q) and, if asked for, the
     un-rounded fp32 output [B,H,N,d] and the log-sum-exp [B,H,N] (written into out_f32 / out_lse
     when those contiguous fp32 tensors are given)."""
-    sq, sk, sv = _view(q, "q"), _view(k, "k"), _view(v, "v")
-    B, H, n, d = q.shape
-    N = n if N is None else int(N)
-    if sel.dtype != torch.int32 or not sel.is_contiguous() or not sel.is_cuda:
-        raise ValueError("sel must be a contiguous CUDA int32 tensor")
-    kmax = sel.shape[3]
-    karr, _ = _k_array(k_per_head, H)
-    if out is None:
-        if q.is_contiguous():
-            out = torch.empty_like(q)
-        else:   # token-major memory [B,N,H,d], returned as a [B,H,N,d] view
-            out = torch.empty((B, n, H, d), dtype=q.dtype, device=q.device).permute(0, 2, 1, 3)
-    so = _view(out, "o")
-    o32 = lse = None
-    if return_f32:
-        o32 = torch.empty((B, H, N, d), dtype=torch.float32, device=q.device) if out_f32 is None else out_f32
-        if o32.dtype != torch.float32 or not o32.is_contiguous() or tuple(o32.shape) != (B, H, N, d):
-            raise ValueError("out_f32 must be a contiguous fp32 [B,H,N,d] tensor")
-    if return_lse:
-        lse = torch.empty((B, H, N), dtype=torch.float32, device=q.device) if out_lse is None else out_lse
-        if lse.dtype != torch.float32 or not lse.is_contiguous() or tuple(lse.shape) != (B, H, N):
-            raise ValueError("out_lse must be a contiguous fp32 [B,H,N] tensor")
-    L = lib()
-    need = L.usv_sparse_attn_workspace(B, H, N, d, kmax)
-    ws = _workspace(q.device, need)
-    _check(L.usv_sparse_attn_fwd(B, H, N, d, _ptr(q), sq, _ptr(k), sk,
-                                 _ptr(v), sv, _ptr(sel), karr, kmax, _ptr(out),
-                                 so, _ptr(o32), _ptr(lse), scale,
-                                 int(impl), _ptr(ws), ws.numel(),
-                                 _stream(q.device)), "usv_sparse_attn_fwd")
-    res = (out,)
-    if return_f32:
-        res += (o32,)
-    if return_lse:
-        res += (lse,)
-    return res if len(res) > 1 else out
+    return _native.sparse_attn_fwd(q, k, v, sel, k_per_head, N, scale, out, return_f32, return_lse, impl, out_f32, out_lse)
 
 
 def workspace_status(device=None):
@@ -293,82 +240,23 @@ def token_merge(x, metric, grid, part, r, plan=None, debug=False, window=None, o
     metric=None the given `plan` is applied.  `window` = (wt, wh, ww) keeps the matching inside
     the partition blocks that near the source's own block (None: all destinations).
     Returns (x_merged [B,N-r,C], plan)."""
-    if x.dim() != 3 or x.dtype != torch.bfloat16 or not x.is_cuda or not x.is_contiguous():
-        raise ValueError("x must be a contiguous CUDA bf16 [B,N,C] tensor")
-    B, N, C = x.shape
-    T, Hh, W = grid
-    st, sh, sw = part
-    dev = x.device
-    if metric is None:
-        if plan is None:
-            raise ValueError("either metric or plan is needed")
-        Hm = dm = 0
-        u = js = None
-    else:
-        if metric.dim() != 4 or metric.dtype != torch.bfloat16 or not metric.is_contiguous():
-            raise ValueError("metric must be a contiguous CUDA bf16 [B,N,Hm,dm] tensor")
-        Hm, dm = metric.shape[2], metric.shape[3]
-        plan = MergePlan(torch.empty((B, N), dtype=torch.int32, device=dev),
-                         torch.empty((B, N), dtype=torch.int32, device=dev), tuple(grid),
-                         tuple(part), int(r))
-        if debug:
-            plan.u = torch.empty((B, N), dtype=torch.float32, device=dev)
-            plan.jstar = torch.empty((B, N), dtype=torch.int32, device=dev)
-        u, js = plan.u, plan.jstar
-    if out is None:
-        out = torch.empty((B, max(N - r, 0), C), dtype=torch.bfloat16, device=dev)
-    elif out.dtype != torch.bfloat16 or not out.is_contiguous() or tuple(out.shape) != (B, N - r, C):
-        raise ValueError("out must be a contiguous bf16 [B,N-r,C] tensor")
-    L = lib()
-    need = L.usv_token_merge_workspace(B, N, C, Hm, dm if dm else 128)
-    ws = _workspace(dev, need)
-    if window is None:
-        _check(L.usv_token_merge(B, N, C, _ptr(x), Hm, dm, _ptr(metric), T, Hh, W, st, sh, sw, int(r),
-                                 _ptr(out), _ptr(plan.dst_of), _ptr(plan.pos), _ptr(u), _ptr(js),
-                                 _ptr(ws), ws.numel(), _stream(dev)),
-               "usv_token_merge")
-    else:
-        wt, wh, ww = (int(v) for v in window)
-        _check(L.usv_token_merge_local(B, N, C, _ptr(x), Hm, dm, _ptr(metric), T, Hh, W, st, sh, sw, wt, wh, ww,
-                                       int(r), _ptr(out), _ptr(plan.dst_of), _ptr(plan.pos), _ptr(u), _ptr(js),
-                                       _ptr(ws), ws.numel(), _stream(dev)),
-               "usv_token_merge_local")
-    return out, plan
+    if metric is None and plan is not None:
+        out, _, _, _, _ = _native.token_merge(x, None, grid, part, r, plan.dst_of, plan.pos, False, window, out)
+        return out, plan
+    out, dst_of, pos, u, jstar = _native.token_merge(x, metric, grid, part, r, None, None, debug, window, out)
+    return out, MergePlan(dst_of, pos, tuple(grid), tuple(part), int(r), u, jstar)
 
 
 def token_unmerge(y_merged, pos, out=None):
     """y[b,n,:] = y_merged[b,pos[b,n],:]."""
-    if (y_merged.dim() != 3 or y_merged.dtype != torch.bfloat16 or not y_merged.is_cuda
-            or not y_merged.is_contiguous()):
-        raise ValueError("y_merged must be a contiguous CUDA bf16 [B,Nm,C] tensor")
-    B, Nm, C = y_merged.shape
-    N = pos.shape[1]
-    if out is None:
-        out = torch.empty((B, N, C), dtype=torch.bfloat16, device=y_merged.device)
-    _check(lib().usv_token_unmerge(B, N, Nm, C, _ptr(y_merged), _ptr(pos), _ptr(out),
-                                   _stream(y_merged.device)), "usv_token_unmerge")
-    return out
+    return _native.token_unmerge(y_merged, pos, out)
 
 
 def attn_entropy(q, k, sel, k_per_head, lse, N=None, scale=0.0):
     """Key marginal [B,N] of the block-masked attention weights averaged over heads and queries,
     and its entropy normalised by log N [B].  `lse` is the log-sum-exp of sparse_attn_fwd for the
     same q, k, sel."""
-    sq, sk = _view(q, "q"), _view(k, "k")
-    B, H, n, d = q.shape
-    N = n if N is None else int(N)
-    if sel.dtype != torch.int32 or not sel.is_contiguous() or not sel.is_cuda:
-        raise ValueError("sel must be a contiguous CUDA int32 tensor")
-    if lse.dtype != torch.float32 or not lse.is_contiguous() or tuple(lse.shape) != (B, H, N):
-        raise ValueError("lse must be a contiguous CUDA fp32 [B,H,N] tensor")
-    karr, _ = _k_array(k_per_head, H)
-    marg = torch.empty((B, N), dtype=torch.float32, device=q.device)
-    ent = torch.empty((B,), dtype=torch.float32, device=q.device)
-    ws = _workspace(q.device, WS_HEADER)
-    _check(lib().usv_attn_entropy(B, H, N, d, _ptr(q), sq, _ptr(k), sk, _ptr(sel),
-                                  karr, sel.shape[3], _ptr(lse), scale, _ptr(marg), _ptr(ent),
-                                  _ptr(ws), _stream(q.device)), "usv_attn_entropy")
-    return marg, ent
+    return _native.attn_entropy(q, k, sel, k_per_head, lse, N, scale)
 
 
 def allocate_sparsity(entropy, gamma, rho_bar, rho_min, rho_max):
@@ -408,50 +296,19 @@ def permute_tokens(x, index):
 
 def force_own_block(scores):
     """In place: scores[b,h,I,I] = +inf, so that select_blocks keeps every query block's own block."""
-    if scores.dtype != torch.float32 or not scores.is_contiguous() or not scores.is_cuda or scores.dim() != 4:
-        raise ValueError("scores must be a contiguous CUDA fp32 [B,H,NBq,NBk] tensor")
-    B, H, NBq, NBk = scores.shape
-    _check(lib().usv_force_own_block(B, H, NBq, NBk, _ptr(scores), _stream(scores.device)), "usv_force_own_block")
-    return scores
+    return _native.set_own_block(scores, False)
 
 
 def exclude_own_block(scores):
     """In place: scores[b,h,I,I] = -inf, so that select_blocks never keeps a query block's own block
     (the long-range branch of the two-branch form)."""
-    if scores.dtype != torch.float32 or not scores.is_contiguous() or not scores.is_cuda or scores.dim() != 4:
-        raise ValueError("scores must be a contiguous CUDA fp32 [B,H,NBq,NBk] tensor")
-    B, H, NBq, NBk = scores.shape
-    _check(lib().usv_exclude_own_block(B, H, NBq, NBk, _ptr(scores), _stream(scores.device)), "usv_exclude_own_block")
-    return scores
+    return _native.set_own_block(scores, True)
 
 
 def attn_combine(o1, lse1, o2, lse2, out=None, return_f32=False, return_lse=False):
     """Fuses two attention branches over disjoint key sets by their softmax mass.  o1, o2: [B,H,N,d]
     views, both bf16 or both fp32; lse1, lse2: fp32 [B,H,N].  Returns o (bf16) [, o_f32] [, lse]."""
-    if o1.dtype != o2.dtype or o1.dtype not in (torch.bfloat16, torch.float32):
-        raise ValueError("o1 and o2 must both be bf16 or both be fp32")
-    for t in (o1, o2):
-        if t.dim() != 4 or not t.is_cuda or t.stride(3) != 1:
-            raise ValueError("branch outputs must be CUDA [B,H,N,d] views with a contiguous last axis")
-    B, H, N, d = o1.shape
-    for l in (lse1, lse2):
-        if l.dtype != torch.float32 or not l.is_contiguous() or tuple(l.shape) != (B, H, N):
-            raise ValueError("lse must be a contiguous fp32 [B,H,N] tensor")
-    s1, s2 = _strides(*o1.stride()[:3]), _strides(*o2.stride()[:3])
-    if out is None:
-        out = torch.empty((B, H, N, d), dtype=torch.bfloat16, device=o1.device)
-    so = _view(out, "o")
-    o32 = torch.empty((B, H, N, d), dtype=torch.float32, device=o1.device) if return_f32 else None
-    lse = torch.empty((B, H, N), dtype=torch.float32, device=o1.device) if return_lse else None
-    _check(lib().usv_attn_combine(B, H, N, d, _ptr(o1), s1, _ptr(lse1), _ptr(o2), s2,
-                                  _ptr(lse2), 1 if o1.dtype == torch.float32 else 0, _ptr(out), so,
-                                  _ptr(o32), _ptr(lse), _stream(o1.device)), "usv_attn_combine")
-    res = (out,)
-    if return_f32:
-        res += (o32,)
-    if return_lse:
-        res += (lse,)
-    return res if len(res) > 1 else out
+    return _native.attn_combine(o1, lse1, o2, lse2, out, return_f32, return_lse)
 
 
 def unmerge_map(pos, Nm):
@@ -507,30 +364,11 @@ def merge_plan_cache(plan):
     """Builds (once) and returns the merged-source lists of a plan, kept on the plan object, so that
     token_merge_apply is the streaming merge kernel alone."""
     if plan.cache is None:
-        B, N = plan.pos.shape
-        T, Hh, W = plan.grid
-        st, sh, sw = plan.part
-        L = lib()
-        nbytes = L.usv_merge_plan_cache_bytes(B, N)
-        cache = torch.empty(int(nbytes), dtype=torch.uint8, device=plan.pos.device)
-        _check(L.usv_merge_plan_cache(B, N, T, Hh, W, st, sh, sw, int(plan.r), _ptr(plan.dst_of), _ptr(plan.pos),
-                                      _ptr(cache), nbytes, _stream(plan.pos.device)),
-               "usv_merge_plan_cache")
-        plan.cache = cache
+        plan.cache = _native.merge_plan_cache(plan.dst_of, plan.pos, plan.grid, plan.part, plan.r)
     return plan.cache
 
 
 def token_merge_apply(x, plan, out=None):
     """Merges x [B,N,C] (bf16) with a stored plan through its cached lists; same result as
     token_merge(x, None, ..., plan=plan)."""
-    if x.dim() != 3 or x.dtype != torch.bfloat16 or not x.is_cuda or not x.is_contiguous():
-        raise ValueError("x must be a contiguous CUDA bf16 [B,N,C] tensor")
-    B, N, C = x.shape
-    T, Hh, W = plan.grid
-    st, sh, sw = plan.part
-    cache = merge_plan_cache(plan)
-    if out is None:
-        out = torch.empty((B, N - plan.r, C), dtype=torch.bfloat16, device=x.device)
-    _check(lib().usv_token_merge_apply(B, N, C, _ptr(x), T, Hh, W, st, sh, sw, int(plan.r), _ptr(cache), _ptr(out),
-                                       _stream(x.device)), "usv_token_merge_apply")
-    return out
+    return _native.token_merge_apply(x, plan.grid, plan.part, plan.r, merge_plan_cache(plan), out)

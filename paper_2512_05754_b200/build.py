@@ -1,13 +1,16 @@
-"""Builds libusv.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds libusv.so (the C-ABI CUDA library, nvcc for sm_100a) and _usv.so (the CPython module that
+calls it from torch tensors, g++) in-tree."""
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libusv.so")
+MODULE = os.path.join(HERE, "_usv.so")
 
 
 def sources():
@@ -23,7 +26,48 @@ def _stale():
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def start_module(force=False):
+    """Starts compiling csrc/usv_py.cpp against the installed torch, unless _usv.so is newer than its
+    sources; returns (process, object file) or None."""
+    src = os.path.join(CSRC, "usv_py.cpp")
+    deps = [src] + glob.glob(os.path.join(ROOT, "include", "*.h"))
+    if not force and os.path.exists(MODULE) and all(os.path.getmtime(MODULE) > os.path.getmtime(d) for d in deps):
+        return None
+    import torch
+    t = os.path.join(os.path.dirname(torch.__file__), "include")
+    obj = os.path.join(HERE, "_build", "usv_py.o")
+    os.makedirs(os.path.dirname(obj), exist_ok=True)
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-w", "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+           "-I", os.path.join(ROOT, "include"), "-isystem", t, "-isystem", os.path.join(t, "torch", "csrc", "api", "include"),
+           "-isystem", sysconfig.get_paths()["include"], "-isystem", "/usr/local/cuda/include", "-c", src, "-o", obj]
+    return subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT), obj
+
+
+def finish_module(started):
+    """Waits for the compiler and links _usv.so beside libusv.so."""
+    if started is None:
+        return
+    import torch
+    proc, obj = started
+    out, _ = proc.communicate()
+    if proc.returncode != 0:
+        sys.stderr.write(out.decode())
+        raise RuntimeError("g++ failed on usv_py.cpp")
+    tl = os.path.join(os.path.dirname(torch.__file__), "lib")
+    subprocess.run(["g++", "-shared", "-o", MODULE, obj, "-L", HERE, "-l:libusv.so", "-L", tl, "-lc10", "-lc10_cuda",
+                    "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python", "-ltorch", "-Wl,-rpath,$ORIGIN", "-Wl,-rpath," + tl],
+                   check=True)
+
+
 def build(force=False, verbose=False):
+    """Compile every .cu under csrc/ into libusv.so, and the CPython module; returns the library path."""
+    module = start_module(force)
+    build_lib(force, verbose)
+    finish_module(module)
+    return LIB
+
+
+def build_lib(force=False, verbose=False):
     """Compile every .cu under csrc/ into libusv.so; returns the library path."""
     if not force and not _stale():
         return LIB
