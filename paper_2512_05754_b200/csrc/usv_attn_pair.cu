@@ -67,8 +67,8 @@ constexpr uint32_t ITEM_BYTES = 64 + LCAP * 4;
 
 // What depends on the head width.  At D = 128 a tile's MMAs (1024 cycles) and its traffic through
 // shared memory (1280 cycles) bound it; at D = 64 both halve and the 128 x 128 exponentials (1024
-// cycles at 16 a clock) are the bound.  24 heads of 32 760 tokens at D = 64, keep 52 of 512: 1.05 ms
-// a call (640 TFLOP/s), 3.00 ms on the mma.sync kernel that served D = 64 before.  A 128-key tile of one operand is D / 64 column halves of
+// cycles at 16 a clock) are the bound.  24 heads of 32 760 tokens at D = 64, keep 52 of 512: 0.86 ms
+// a call (780 TFLOP/s), 3.00 ms on the mma.sync kernel.  A 128-key tile of one operand is D / 64 column halves of
 // [128 keys][128 B]: 32 KB at D = 128, 16 KB at D = 64, where the shared memory left over holds
 // two more K stages (a stage takes ~1700 cycles to arrive, longer than the two tiles that
 // two stages cover at the shorter tiles of D = 64).
@@ -85,7 +85,18 @@ struct Cfg {
     static constexpr uint32_t SM_Q = 0;             // the item's 128 query rows, same layout as a K tile
     static constexpr uint32_t SM_K = SM_Q + TILE_BYTES;
     static constexpr uint32_t SM_V = SM_K + KSTAGES * TILE_BYTES;
-    static constexpr uint32_t SM_BAR = SM_V + VSTAGES * TILE_BYTES;
+    // At D = 64 the row sums come out of the P.V product: its B operand has 16 more columns, all ones, read
+    // from a block of their own (128 keys x 128 B) behind the V stages.  That takes the unpacking and
+    // adding of the rounded weights, a third of the softmax's instructions, off the warps that bound
+    // the kernel.  (D = 128 has no tensor memory left for the 16 columns.)
+    static constexpr bool SUM_COL = D == 64;
+    // Every POLY-th pair of exponentials goes to the FMA pipe (0: none).  24 heads x 512 blocks at D = 64, keep
+    // 52: none 880 us, one in eight 843, one in four 844, one in three 874, half 947; at D = 128, where the
+    // special-function unit is not the bound, 636, 639, 652, 665 and 750 us (12 heads).
+    static constexpr int POLY = D == 64 ? 5 : 0;
+    static constexpr int ND = SUM_COL ? D + 16 : D;   // columns of the P.V product
+    static constexpr uint32_t SM_ONES = SM_V + VSTAGES * TILE_BYTES;
+    static constexpr uint32_t SM_BAR = SM_ONES + (SUM_COL ? KT * 128 : 0);
     // barrier slots (8 bytes each)
     enum { B_QFULL = 0, B_QFREE, B_KFULL, B_KEMPTY = B_KFULL + KSTAGES, B_VFULL = B_KEMPTY + KSTAGES,
            B_VEMPTY = B_VFULL + VSTAGES, B_SFULL = B_VEMPTY + VSTAGES, B_PFULL = B_SFULL + 2 * SBUF,
@@ -107,7 +118,7 @@ enum { I_T = 0, I_NU, I_B, I_H, I_BH, I_IA, I_IB, I_SREFA, I_SREFB, I_LIST_LO, I
 // TMEM columns: O | S/P buffer 0 | S/P buffer 1 | S/P buffer 2
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t TO = 0, TS = 128;
-static_assert(TS + SBUF * 128 <= TMEM_COLS, "TMEM budget");
+static_assert(TS + SBUF * 128 <= TMEM_COLS && Cfg<64>::ND <= 128 && Cfg<128>::ND <= 128, "TMEM budget");
 
 constexpr int NSOFT = NWG * 128;   // softmax threads
 constexpr int NTHREADS = NSOFT + 128 + 128;   // + output warpgroup + service warpgroup
@@ -122,24 +133,30 @@ struct Maps {
     CUtensorMap q, k, v;
 };
 
-// exp2 of 32 scaled logits -> 16 packed bf16 pairs; adds the weights, as rounded to bf16 (what
+// exp2 of 32 scaled logits -> 16 packed bf16 pairs; with SUM adds the weights, as rounded to bf16 (what
 // the P.V product multiplies by), to the two lanes of `acc`, so that numerator and denominator of
 // a row carry the same rounding.  Two logits at a time on the packed-fp32 pipe.
-template <bool MASKED>
+template <bool MASKED, bool SUM, int POLY>
 __device__ __forceinline__ void weights32(const uint32_t* sr, uint32_t* pk, uint64_t c2, uint64_t nref2, int col0,
                                           int nvalid, uint64_t& acc) {
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
         const uint64_t x2 = fma_f32x2(pack_f32x2(__uint_as_float(sr[2 * j]), __uint_as_float(sr[2 * j + 1])), c2, nref2);
-        float x0, x1;
-        unpack_f32x2(x2, x0, x1);
-        float p0 = ex2(x0), p1 = ex2(x1);
+        float p0, p1;
+        if (POLY && j % (POLY ? POLY : 1) == POLY - 1) {
+            exp2_fma(x2, p0, p1);
+        } else {
+            float x0, x1;
+            unpack_f32x2(x2, x0, x1);
+            p0 = ex2(x0);
+            p1 = ex2(x1);
+        }
         if (MASKED) {
             if (col0 + 2 * j >= nvalid) p0 = 0.f;
             if (col0 + 2 * j + 1 >= nvalid) p1 = 0.f;
         }
         pk[j] = pack_bf16x2(p0, p1);
-        acc = add_f32x2(acc, pack_f32x2(__uint_as_float(pk[j] << 16), __uint_as_float(pk[j] & 0xffff0000u)));
+        if (SUM) acc = add_f32x2(acc, pack_f32x2(__uint_as_float(pk[j] << 16), __uint_as_float(pk[j] & 0xffff0000u)));
     }
 }
 
@@ -187,6 +204,11 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
         if (i == 0) *s_abort = 0;
         if (i < 2 * NSLOT) s_flag[i] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (F::SUM_COL) {
+        for (int i = threadIdx.x; i < KT * 128 / 16; i += NTHREADS)
+            reinterpret_cast<uint4*>(sm + F::SM_ONES)[i] = make_uint4(0x3f803f80u, 0x3f803f80u, 0x3f803f80u, 0x3f803f80u);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     if (warp == W_MMA) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
@@ -385,8 +407,11 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
         // TMEM buffer of P(g - 3) and is issued once P.V(g - 3) is COMPLETE (the V stage barrier
         // of that tile says so to the V producer and to the S issuer alike).
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REG_SERVICE));
-        constexpr uint32_t IDESC_O = instr_desc(128, D, 0, 1);     // P (TMEM) x V (MN-major)
-        const uint64_t vdesc0 = smem_desc(base + F::SM_V, 16384, 1024);
+        constexpr uint32_t IDESC_O = instr_desc(128, F::ND, 0, 1);     // P (TMEM) x V (MN-major)
+        // from one 64-column half of V to the next, or to the ones: per stage the descriptor moves on by
+        // a tile, and the distance to the ones shrinks by as much
+        const uint64_t vdesc0 = smem_desc(base + F::SM_V, F::SUM_COL ? F::SM_ONES - F::SM_V : 16384, 1024);
+        constexpr uint64_t VSTEP = (uint64_t)(TILE_BYTES >> 4) - (F::SUM_COL ? (uint64_t)(TILE_BYTES >> 4) << 16 : 0);
         int g = 0;                               // running tile
         int p_v = 0, p_buf = 0, p_b6 = 0;        // g % VSTAGES, g % SBUF, g % (2 SBUF)
         uint32_t p_vph = 0, p_ph6 = 0;           // (g / VSTAGES) & 1, (g / (2 SBUF)) & 1
@@ -401,7 +426,7 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
                 // the first P.V of an item overwrites O: the item before must have been read out
                 if (t == 0 && n > 0 && !mbar_wait(bar(F::B_OFREE), (n - 1) & 1, s_abort, a.status, 0x2000)) { ok = false; break; }
                 fence_after();
-                const uint64_t vdesc = vdesc0 + ((p_v * TILE_BYTES) >> 4);
+                const uint64_t vdesc = vdesc0 + p_v * VSTEP;
                 const uint32_t pb = tmem + TS + p_buf * 128;   // P: 32 columns at the head of each 64-column half
                 if (elect_one()) {
 #pragma unroll
@@ -472,18 +497,29 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
             const int row = iq * USV_BLOCK + (e & 63);
             const bool live = iq >= 0 && row < N;
             if (!mbar_wait(bar(F::B_SUMS + slot), (m / NSLOT) & 1, s_abort, a.status, 0x800)) break;
-            const float* sums = s_sum + slot * (NWG * 128);
             float l = 0.f;
+            if (F::SUM_COL) {
+                if (!mbar_wait(bar(F::B_OFULL), m & 1, s_abort, a.status, 0x200)) break;
+                fence_after();
+                uint32_t sum;
+                tmem_ld1(lane_base + TO + D, sum);
+                tmem_wait_ld();
+                l = __uint_as_float(sum);
+            } else {
+                const float* sums = s_sum + slot * (NWG * 128);
 #pragma unroll
-            for (int q = 0; q < NWG; ++q) l += sums[q * 128 + e];
+                for (int q = 0; q < NWG; ++q) l += sums[q * 128 + e];
+            }
             const float nref = has_ref ? s_refv[slot * 128 + e] : 0.f;
             const bool in_range = l > 7.9e-31f && l < 1.2e30f;   // ~[2^-100, 2^100]
             uint64_t z0 = 0, z1 = 0;   // four fp32 sums that stay 0 unless a value of the row is not finite
             const float inv = l > 0.f ? 1.0f / l : 0.f;
             if (a.lse != nullptr && live)
                 a.lse[((int64_t)ib * a.H + ih) * N + row] = (log2f(l) - nref) * 0.69314718055994531f;
-            if (!mbar_wait(bar(F::B_OFULL), m & 1, s_abort, a.status, 0x200)) break;
-            fence_after();
+            if (!F::SUM_COL) {
+                if (!mbar_wait(bar(F::B_OFULL), m & 1, s_abort, a.status, 0x200)) break;
+                fence_after();
+            }
             // The row leaves TMEM a quarter (32 columns) at a time and is stored from registers; the
             // accumulator and the ring slot go back as soon as the last quarter has been read.
             float* o32 = (a.o_f32 != nullptr && live) ? a.o_f32 + (((int64_t)ib * a.H + ih) * N + row) * D : nullptr;
@@ -628,13 +664,13 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
                     uint32_t sx[32];
                     tmem_ld32(sbase, sx);
                     tmem_wait_ld();
-                    if (nv >= USV_BLOCK) weights32<false>(sx, pk0, c2, nref2, 0, nv, lr2);
-                    else weights32<true>(sx, pk0, c2, nref2, 0, nv, lr2);
+                    if (nv >= USV_BLOCK) weights32<false, !F::SUM_COL, F::POLY>(sx, pk0, c2, nref2, 0, nv, lr2);
+                    else weights32<true, !F::SUM_COL, F::POLY>(sx, pk0, c2, nref2, 0, nv, lr2);
                     tmem_ld32(sbase + 32, sx);
                     tmem_wait_ld();
                     tmem_st16(sbase, pk0);
-                    if (nv >= USV_BLOCK) weights32<false>(sx, pk1, c2, nref2, 32, nv, lr2);
-                    else weights32<true>(sx, pk1, c2, nref2, 32, nv, lr2);
+                    if (nv >= USV_BLOCK) weights32<false, !F::SUM_COL, F::POLY>(sx, pk1, c2, nref2, 32, nv, lr2);
+                    else weights32<true, !F::SUM_COL, F::POLY>(sx, pk1, c2, nref2, 32, nv, lr2);
                     tmem_st16(sbase + 16, pk1);
                 } else {
 #pragma unroll
@@ -649,9 +685,11 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
             }
             if (!ok) break;
             if (sref < nU) refph ^= 1u << slot_n;
-            float lr_lo, lr_hi;
-            unpack_f32x2(lr2, lr_lo, lr_hi);
-            s_sum[slot_n * (NWG * 128) + grp * 128 + r] = lr_lo + lr_hi;
+            if (!F::SUM_COL) {
+                float lr_lo, lr_hi;
+                unpack_f32x2(lr2, lr_lo, lr_hi);
+                s_sum[slot_n * (NWG * 128) + grp * 128 + r] = lr_lo + lr_hi;
+            }
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(F::B_SUMS + slot_n));
             g += T;

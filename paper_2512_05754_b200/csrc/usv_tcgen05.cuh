@@ -201,6 +201,10 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
         : "r"(taddr)
         : "memory");
 }
+// one 32-bit column
+__device__ __forceinline__ void tmem_ld1(uint32_t taddr, uint32_t& r) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr) : "memory");
+}
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // registers -> 16 consecutive 32-bit columns of this thread's TMEM lane
@@ -244,6 +248,39 @@ __device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
     uint64_t d;
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
+}
+
+__device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t both(float v) { return pack_f32x2(v, v); }
+
+// 2^x of a packed pair on the FMA pipe, for kernels that the special-function unit (16 results a clock and
+// SM) bounds: x = n + f with |f| <= 1/2, a polynomial of degree 5 for 2^f (interpolation of 2^f at the
+// Chebyshev nodes; relative error 1.0e-7, 2.2e-7 as evaluated, ex2.approx: 2.4e-7), times 2^n.  Below
+// -126 the result stays 2^-126, at 128 and above it is infinite, NaN stays NaN.
+__device__ __forceinline__ void exp2_fma(uint64_t x2, float& p0, float& p1) {
+    float x0, x1;
+    unpack_f32x2(x2, x0, x1);
+    asm("max.NaN.f32 %0, %0, %1;" : "+f"(x0) : "f"(-126.f));
+    asm("max.NaN.f32 %0, %0, %1;" : "+f"(x1) : "f"(-126.f));
+    asm("min.NaN.f32 %0, %0, %1;" : "+f"(x0) : "f"(128.f));
+    asm("min.NaN.f32 %0, %0, %1;" : "+f"(x1) : "f"(128.f));
+    const uint64_t x = pack_f32x2(x0, x1);
+    const uint64_t t = add_f32x2(x, both(12582912.f + 127.f));       // 1.5 * 2^23: n + 127 in the low bits
+    const uint64_t n = add_f32x2(t, both(-12582912.f - 127.f));
+    const uint64_t f = fma_f32x2(n, both(-1.f), x);
+    uint64_t p = fma_f32x2(both(0.0013390863314270973f), f, both(0.009676031768321991f));
+    p = fma_f32x2(p, f, both(0.055503569543361664f));
+    p = fma_f32x2(p, f, both(0.2402210682630539f));
+    p = fma_f32x2(p, f, both(0.6931471824645996f));
+    p = fma_f32x2(p, f, both(1.0000001192092896f));
+    float t0, t1;
+    unpack_f32x2(t, t0, t1);
+    const uint64_t scale = pack_f32x2(__uint_as_float(__float_as_uint(t0) << 23), __uint_as_float(__float_as_uint(t1) << 23));
+    unpack_f32x2(mul_f32x2(p, scale), p0, p1);
 }
 
 // ---- host side: tensor maps through the driver entry point (no link-time libcuda dependency)
