@@ -747,6 +747,9 @@ int launch_scatter_fallbacks(const AttnArgs& a, int d, cudaStream_t st) {
 }
 
 bool attn_pair_supported(const AttnArgs& a, int d) {
+    // heads or batch elements that share their rows (stride 0) are left to the mma.sync kernel
+    for (const usv_strides* v : {&a.sq, &a.sk, &a.sv})
+        if ((a.H > 1 && v->sh == 0) || (a.B > 1 && v->sb == 0)) return false;
     return (d == 64 || d == 128) && a.NB <= pr::MAX_NB && a.work_counter != nullptr;
 }
 

@@ -1,4 +1,4 @@
-// Arguments of the key-marginal kernels (Sec. 3.4, Eq. 16) and the launcher of the tcgen05 one.
+// Arguments of the key-marginal kernel (Sec. 3.4, Eq. 16) and its launcher.
 #pragma once
 #include "usv_common.cuh"
 
@@ -13,11 +13,12 @@ struct MargArgs {
     unsigned int* status; // device status word the bounded waits report to (may be NULL)
     int B, H, N, NB, kmax;
     float scale_log2;     // softmax scale * log2(e)
+    float inv_scale;      // 1 / softmax scale
     float inv_hn;         // 1 / (H N)
     int k_per_head[USV_MAX_HEADS];
 };
 
-// d = 128 on the tensor cores (usv_entropy_tc.cu); marg must be zero.
-int launch_marginal_tc(const MargArgs& a, cudaStream_t st);
+// usv_entropy_tc.cu; marg must be zero.
+int launch_marginal_tc(const MargArgs& a, int d, cudaStream_t st);
 
 }  // namespace usv

@@ -1,20 +1,34 @@
 // Key marginal of the block-masked attention (Sec. 3.4, Eq. 16) on the 5th-generation tensor
-// cores, d = 128.
+// cores, head width D = 64 or 128.
 //
 //     abar[b,j] = 1/(H N) sum_h sum_i A(h,i,j),   A(h,i,j) = exp(scale <q_i,k_j> - lse_i)
 //
 // with lse_i the log-sum-exp the attention forward wrote.  Only the logits are needed, and the
-// sum runs over the queries, so the product is taken transposed: one CTA per (b, h, query block)
-// walks the block's selected key blocks two at a time and computes
+// sum runs over the queries, so the product is taken transposed: one CTA per (b, h, two
+// consecutive query blocks) walks the union of the two lists two key blocks at a time and computes
 //
-//     S^T[128 keys x 64 queries] = K_tile . Q^T      tcgen05.mma, A = K tile in smem, B = Q in smem
+//     S^T[128 keys x 128 queries] = K_tile . Q^T      tcgen05.mma, A = K tile in smem, B = Q in smem
 //
-// into one of four 64-column TMEM buffers.  Keys live on TMEM lanes: thread r of the four
-// consumer warps owns key r of the tile, exponentiates its 64 logits against the queries'
-// log-sum-exp (held in registers) and adds the sum to abar with one atomic per key and tile.
-// A CTA needs 82 KB of shared memory and 256 TMEM columns, so two share an SM and fill each
-// other's gaps.  Warp 4 is the TMA producer, warp 5 the MMA issuer and TMEM owner.  All waits
-// are bounded; a role that gives up raises the CTA's abort flag and the others follow.
+// into one of two 128-column TMEM buffers.  Keys live on TMEM lanes: thread r of a warpgroup owns
+// key r of the tile and one warpgroup serves each query block: it exponentiates the 64 logits of
+// its side and adds their sum to abar with one atomic per key and tile; it skips a key block that
+// its side did not select.  The log-sum-exp enters through the product itself: one more K = 16 step
+// multiplies a K operand of ones by -lse / scale, split into three bf16 terms (24 bits), so that no
+// thread has to hold 64 of them and twice as many warps fit.
+//
+// Bounds at D = 128: 128 x 128 exponentials a tile are 1024 cycles at 16 a clock, less what one side
+// skips; the tile's traffic through shared memory (32 KB in by TMA, 64 KB + 8 KB out to the MMAs) is
+// 830.  With one query block a CTA the traffic was 640 cycles for half as many exponentials.
+// Measured with the entropy (us; one query block a CTA at D = 128, mma.sync at D = 64, before): 12 heads x 512
+// blocks, D = 128, keep 52: 492 -> 439, all blocks: 4490 -> 3600; 24 heads, D = 64, keep 52: 2548 -> 775;
+// 8 heads x 2325 blocks, D = 128, keep 117, where neighbours share less: 3310 -> 3320.
+//
+// The union is built as a list in shared memory: two bitmaps over the key blocks, compacted by one warp.
+// CTAs that run at the same time start at different entries of it, those near their own query blocks:
+// their atomic adds would otherwise meet on the same keys.  A launch covers a window of 16 384 key blocks.
+// Two CTAs share an SM and fill each other's gaps.  Warp 8 is the TMA producer, warp 9 the MMA
+// issuer and TMEM owner.  All waits are bounded; a role that gives up raises the CTA's abort flag and
+// the others follow.
 #include "usv_entropy.cuh"
 #include "usv_tcgen05.cuh"
 
@@ -24,25 +38,36 @@ namespace et {
 
 using namespace t5;
 
-constexpr int D = 128;
 constexpr int KT = 2 * USV_BLOCK;               // keys per tile = two key blocks
-constexpr int KSTAGES = 2;                      // two CTAs share an SM and cover each other's waits
-constexpr int NBUF = 4;                         // S^T buffers of 64 columns
-constexpr uint32_t TILE_BYTES = KT * D * 2;     // 32 KB: [d-half][128 keys][128 B]
-constexpr uint32_t Q_BYTES = USV_BLOCK * D * 2; // 16 KB: [d-half][64 queries][128 B]
-constexpr uint32_t SM_Q = 0;
-constexpr uint32_t SM_K = SM_Q + Q_BYTES;
-constexpr uint32_t SM_BAR = SM_K + KSTAGES * TILE_BYTES;
-enum { B_QFULL = 0, B_KFULL, B_KEMPTY = B_KFULL + KSTAGES, B_SFULL = B_KEMPTY + KSTAGES,
-       B_SFREE = B_SFULL + NBUF, B_COUNT = B_SFREE + NBUF };
-constexpr uint32_t SM_MISC = SM_BAR + 8 * 16;   // tmem base, abort flag
-constexpr uint32_t SM_TOTAL = SM_MISC + 64;
-constexpr size_t SMEM_BYTES = SM_TOTAL + 1024;  // + slack for 1024-byte alignment
-static_assert(B_COUNT <= 16, "barrier area");
-static_assert(2 * SMEM_BYTES <= 232448, "two CTAs per SM");
+constexpr int QT = 2 * USV_BLOCK;               // queries per CTA = two query blocks
+constexpr int NBUF = 2;                         // S^T buffers of 128 columns
+constexpr int WINDOW = 1 << 14;                 // key blocks a launch covers (16-bit list entries)
+constexpr uint32_t AUG_BYTES = 128 * 32;        // [128 rows][16 bf16]
 
-constexpr uint32_t TMEM_COLS = 256;
-constexpr int NCONS = 128;                      // consumer threads
+template <int D>
+struct Cfg {
+    static constexpr int NH = D / 64;                   // column halves of a tile
+    static constexpr int KSTAGES = D == 64 ? 4 : 2;
+    // every POLY-th pair of exponentials goes to the FMA pipe (at 12 / 24 heads as above: none 448 / 822 us, one
+    // in eight 439 / 820, in five 439 / 775, in four 439 / 813)
+    static constexpr int POLY = D == 64 ? 5 : 4;
+    static constexpr uint32_t TILE_BYTES = KT * D * 2;  // [d-half][128 rows][128 B], for K and Q alike
+    static constexpr uint32_t SM_Q = 0;
+    static constexpr uint32_t SM_K = SM_Q + TILE_BYTES;
+    static constexpr uint32_t SM_AUGK = SM_K + KSTAGES * TILE_BYTES;   // ones
+    static constexpr uint32_t SM_AUGQ = SM_AUGK + AUG_BYTES;           // -lse / scale, three terms a row
+    static constexpr uint32_t SM_BAR = SM_AUGQ + AUG_BYTES;
+    static constexpr uint32_t SM_MISC = SM_BAR + 8 * 16;               // tmem base, abort flag, union size
+    static constexpr uint32_t SM_LIST = SM_MISC + 64;                  // union: (key block - window) << 2 | in-A | in-B << 1
+    enum { B_QFULL = 0, B_KFULL, B_KEMPTY = B_KFULL + KSTAGES, B_SFULL = B_KEMPTY + KSTAGES,
+           B_SFREE = B_SFULL + NBUF, B_COUNT = B_SFREE + NBUF };
+    static_assert(B_COUNT <= 16, "barrier area");
+    static_assert(2 * (WINDOW / 32) * 4 <= KSTAGES * TILE_BYTES, "the bitmaps lie in the K stages");
+    static size_t smem_bytes(int entries) { return SM_LIST + 2 * (size_t)entries + 1024; }   // + slack for alignment
+};
+
+constexpr uint32_t TMEM_COLS = NBUF * QT;
+constexpr int NCONS = 256;                      // consumer threads: one warpgroup per query block
 constexpr int NTHREADS = NCONS + 64;
 constexpr int W_TMA = NCONS / 32, W_MMA = NCONS / 32 + 1;
 
@@ -50,35 +75,60 @@ struct Maps {
     CUtensorMap q, k;
 };
 
+// exp2 of two scaled logits; pair i of a row, every POLY-th one on the FMA pipe
+template <int POLY>
+__device__ __forceinline__ uint64_t weight2(int i, uint32_t a, uint32_t b, uint64_t c2) {
+    const uint64_t x2 = mul_f32x2(pack_f32x2(__uint_as_float(a), __uint_as_float(b)), c2);
+    float p0, p1;
+    if (POLY && i % (POLY ? POLY : 1) == POLY - 1) {
+        exp2_fma(x2, p0, p1);
+    } else {
+        float x0, x1;
+        unpack_f32x2(x2, x0, x1);
+        p0 = ex2(x0);
+        p1 = ex2(x1);
+    }
+    return pack_f32x2(p0, p1);
+}
+
+template <int D>
 __global__ void __launch_bounds__(NTHREADS, 2)
-marginal_tc_kernel(const MargArgs a, const __grid_constant__ Maps maps) {
+marginal_tc_kernel(const MargArgs a, int w0, const __grid_constant__ Maps maps) {
+    using F = Cfg<D>;
+    constexpr int KSTAGES = F::KSTAGES;
+    constexpr uint32_t TILE_BYTES = F::TILE_BYTES;
     dep_launch();   // the set-up below touches shared and tensor memory only; dep_wait() follows it
     extern __shared__ unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     unsigned char* sm = smem_raw + (base - raw);
-    auto bar = [&](int i) { return base + SM_BAR + 8u * i; };
-    volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(sm + SM_MISC);
-    volatile int* s_abort = reinterpret_cast<volatile int*>(sm + SM_MISC + 4);
+    auto bar = [&](int i) { return base + F::SM_BAR + 8u * i; };
+    volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(sm + F::SM_MISC);
+    volatile int* s_abort = reinterpret_cast<volatile int*>(sm + F::SM_MISC + 4);
+    volatile int* s_union = reinterpret_cast<volatile int*>(sm + F::SM_MISC + 8);   // entries, first one taken
+    uint32_t* s_bits = reinterpret_cast<uint32_t*>(sm + F::SM_K);
+    uint16_t* s_list = reinterpret_cast<uint16_t*>(sm + F::SM_LIST);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int N = a.N;
-    const int I = blockIdx.x % a.NB;
-    const int bh = blockIdx.x / a.NB;
+    const int N = a.N, NB = a.NB;
+    const int NP = (NB + 1) >> 1, words = (min(NB - w0, WINDOW) + 31) >> 5;   // key blocks [w0, w0 + 32 words)
+    const int I = 2 * (blockIdx.x % NP);
+    const int bh = blockIdx.x / NP;
     const int b = bh / a.H, h = bh % a.H;
     const int kh = a.k_per_head[h];
-    const int T = (kh + 1) >> 1;   // tiles of two list entries
-    const int32_t* sel = a.sel + ((int64_t)bh * a.NB + I) * a.kmax;
 
-    if (threadIdx.x < B_COUNT) {
+    if (threadIdx.x < F::B_COUNT) {
         const int i = threadIdx.x;
-        mbar_init(bar(i), (i >= B_SFREE && i < B_SFREE + NBUF) ? NCONS / 32 : 1);
-        if (i == 0) *s_abort = 0;
+        mbar_init(bar(i), (i >= F::B_SFREE && i < F::B_SFREE + NBUF) ? NCONS / 32 : 1);
+        if (i == 0) { *s_abort = 0; s_union[1] = 0; }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    for (int i = threadIdx.x; i < 2 * words; i += NTHREADS) s_bits[i] = 0;
+    for (int i = threadIdx.x; i < (int)AUG_BYTES / 16; i += NTHREADS)
+        reinterpret_cast<uint4*>(sm + F::SM_AUGK)[i] = make_uint4(0x3f803f80u, 0x3f803f80u, 0x3f803f80u, 0x3f803f80u);
     if (warp == W_MMA) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"(base + SM_MISC), "r"(TMEM_COLS) : "memory");
+                     ::"r"(base + F::SM_MISC), "r"(TMEM_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     fence_before();
@@ -87,90 +137,146 @@ marginal_tc_kernel(const MargArgs a, const __grid_constant__ Maps maps) {
     dep_wait();
     const uint32_t tmem = *s_tmem;
 
-    if (warp == W_TMA) {
-        // ===== producer: the query block once, then the key tiles =================================
-        if (elect_one()) {
-            mbar_expect_tx(bar(B_QFULL), Q_BYTES);
-            tma_load_4d(base + SM_Q, &maps.q, bar(B_QFULL), 0, I * USV_BLOCK, h, b);
-            tma_load_4d(base + SM_Q + 8192, &maps.q, bar(B_QFULL), 64, I * USV_BLOCK, h, b);
+    // ---- the query rows on their way, the lists as bitmaps, the log-sum-exp as an operand
+    if (warp == W_TMA && elect_one()) {
+        const int hq = a.sq.sh ? h : 0, bq = a.sq.sb ? b : 0;
+        mbar_expect_tx(bar(F::B_QFULL), TILE_BYTES);
+#pragma unroll
+        for (int hf = 0; hf < F::NH; ++hf) {
+            tma_load_4d(base + F::SM_Q + hf * 16384, &maps.q, bar(F::B_QFULL), hf * 64, I * USV_BLOCK, hq, bq);
+            tma_load_4d(base + F::SM_Q + hf * 16384 + 8192, &maps.q, bar(F::B_QFULL), hf * 64, (I + 1) * USV_BLOCK, hq, bq);
         }
-        __syncwarp();
-        int n0 = T > 0 ? sel[0] : -1, n1 = (T > 0 && 1 < kh) ? sel[1] : -1;   // entries of the next tile, fetched ahead
+    }
+    for (int i = threadIdx.x; i < 2 * kh; i += NTHREADS) {
+        const int side = i >= kh;
+        if (I + side >= NB) continue;
+        const int e = a.sel[((int64_t)bh * NB + I + side) * a.kmax + (i - side * kh)];
+        if (e >= w0 && e < NB && e - w0 < WINDOW) atomicOr(&s_bits[side * words + ((e - w0) >> 5)], 1u << (e & 31));
+    }
+    if (threadIdx.x < QT) {
+        // a query at or beyond N counts nothing
+        const int row = I * USV_BLOCK + threadIdx.x;
+        const float x = row < N ? -a.lse[(int64_t)bh * N + row] * a.inv_scale : -1e30f;
+        const __nv_bfloat16 hi = __float2bfloat16(x);
+        float r = x - __bfloat162float(hi);
+        if (!isfinite(x)) r = 0.f;
+        const __nv_bfloat16 mid = __float2bfloat16(r);
+        const __nv_bfloat16 lo = __float2bfloat16(r - __bfloat162float(mid));
+        // rows of 32 bytes, 32-byte swizzle: the other operand is all ones, so it does not matter where
+        // in its row a term lies
+        uint4* dst = reinterpret_cast<uint4*>(sm + F::SM_AUGQ + threadIdx.x * 32);
+        dst[0] = make_uint4((uint32_t)__bfloat16_as_ushort(hi) | ((uint32_t)__bfloat16_as_ushort(mid) << 16),
+                            __bfloat16_as_ushort(lo), 0, 0);
+        dst[1] = make_uint4(0, 0, 0, 0);
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
+    if (warp == 0) {
+        int n = 0;
+        for (int i0 = 0; i0 < words; i0 += 32) {
+            const int i = i0 + lane;
+            const uint32_t ba = i < words ? s_bits[i] : 0, bb = i < words ? s_bits[words + i] : 0;
+            uint32_t m = ba | bb;
+            const int incl = warp_incl_scan(__popc(m));
+            int at = n + incl - __popc(m);
+            if (i == (I - w0) >> 5) s_union[1] = at;
+            for (; m; m &= m - 1) {
+                const int bit = __ffs(m) - 1;
+                s_list[at++] = (uint16_t)((i * 32 + bit) << 2 | ((ba >> bit) & 1u) | ((bb >> bit) & 1u) << 1);
+            }
+            n += __shfl_sync(0xffffffffu, incl, 31);
+        }
+        if (lane == 0) s_union[0] = n;
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the K stages go to the TMA
+    }
+    __syncthreads();
+    const int nU = s_union[0], T = (nU + 1) >> 1;   // tiles of two key blocks
+    const int first = s_union[1] < nU ? s_union[1] : 0;
+    // n-th entry from `first` on, around the end; 0 (no side) behind the last one
+    auto entry = [&](int n) -> int {
+        const int i = first + n;
+        return n < nU ? s_list[i < nU ? i : i - nU] : 0;
+    };
+
+    if (warp == W_TMA) {
+        // ===== producer: the key tiles =============================================================
+        const int hk = a.sk.sh ? h : 0, bk = a.sk.sb ? b : 0;
         for (int t = 0; t < T; ++t) {
             const int s = t % KSTAGES;
-            const uint32_t ph = (t / KSTAGES) & 1;
-            // an entry may be -1 (no block): any finite tile will do, its keys are not counted
-            const int e0 = n0, e1 = n1;
-            n0 = (2 * t + 2 < kh) ? sel[2 * t + 2] : -1;
-            n1 = (2 * t + 3 < kh) ? sel[2 * t + 3] : -1;
-            const int J0 = e0 >= 0 ? e0 : 0, J1 = e1 >= 0 ? e1 : J0;
-            if (!mbar_wait(bar(B_KEMPTY + s), ph ^ 1, s_abort, a.status, 0x1000000u)) break;
-            const uint32_t dst = base + SM_K + s * TILE_BYTES;
+            const int J0 = w0 + (entry(2 * t) >> 2), J1 = w0 + (entry(2 * t + 1) >> 2);   // odd tail: any tile, not counted
+            if (!mbar_wait(bar(F::B_KEMPTY + s), ((t / KSTAGES) & 1) ^ 1, s_abort, a.status, 0x1000000u)) break;
+            const uint32_t dst = base + F::SM_K + s * TILE_BYTES;
             if (elect_one()) {
-                mbar_expect_tx(bar(B_KFULL + s), TILE_BYTES);
-                tma_load_4d(dst, &maps.k, bar(B_KFULL + s), 0, J0 * USV_BLOCK, h, b);
-                tma_load_4d(dst + 8192, &maps.k, bar(B_KFULL + s), 0, J1 * USV_BLOCK, h, b);
-                tma_load_4d(dst + 16384, &maps.k, bar(B_KFULL + s), 64, J0 * USV_BLOCK, h, b);
-                tma_load_4d(dst + 24576, &maps.k, bar(B_KFULL + s), 64, J1 * USV_BLOCK, h, b);
+                mbar_expect_tx(bar(F::B_KFULL + s), TILE_BYTES);
+#pragma unroll
+                for (int hf = 0; hf < F::NH; ++hf) {
+                    tma_load_4d(dst + hf * 16384, &maps.k, bar(F::B_KFULL + s), hf * 64, J0 * USV_BLOCK, hk, bk);
+                    tma_load_4d(dst + hf * 16384 + 8192, &maps.k, bar(F::B_KFULL + s), hf * 64, J1 * USV_BLOCK, hk, bk);
+                }
             }
             __syncwarp();
         }
     } else if (warp == W_MMA) {
         // ===== MMA issuer ==========================================================================
-        constexpr uint32_t IDESC = instr_desc(128, USV_BLOCK, 0, 0);    // K tile (K-major) x Q (K-major)
-        const uint64_t kdesc0 = smem_desc(base + SM_K, 16, 1024);
-        const uint64_t qdesc0 = smem_desc(base + SM_Q, 16, 1024);
-        bool ok = mbar_wait(bar(B_QFULL), 0, s_abort, a.status, 0x2000000u);
+        constexpr uint32_t IDESC = instr_desc(128, QT, 0, 0);    // K tile (K-major) x Q (K-major)
+        const uint64_t kdesc0 = smem_desc(base + F::SM_K, 16, 1024);
+        const uint64_t qdesc0 = smem_desc(base + F::SM_Q, 16, 1024);
+        const uint64_t augk = smem_desc_32b(base + F::SM_AUGK), augq = smem_desc_32b(base + F::SM_AUGQ);
+        bool ok = mbar_wait(bar(F::B_QFULL), 0, s_abort, a.status, 0x2000000u);
         for (int t = 0; ok && t < T; ++t) {
             const int s = t % KSTAGES;
             const int bf = t % NBUF;
-            if (!mbar_wait(bar(B_KFULL + s), (t / KSTAGES) & 1, s_abort, a.status, 0x4000000u)) break;
-            if (t >= NBUF && !mbar_wait(bar(B_SFREE + bf), ((t / NBUF) - 1) & 1, s_abort, a.status, 0x8000000u)) break;
+            if (!mbar_wait(bar(F::B_KFULL + s), (t / KSTAGES) & 1, s_abort, a.status, 0x4000000u)) break;
+            if (t >= NBUF && !mbar_wait(bar(F::B_SFREE + bf), ((t / NBUF) - 1) & 1, s_abort, a.status, 0x8000000u)) break;
             fence_after();
             const uint64_t kdesc = kdesc0 + ((s * TILE_BYTES) >> 4);
             if (elect_one()) {
 #pragma unroll
-                for (int ks = 0; ks < D / 16; ++ks)
-                    umma_ss(tmem + bf * 64, kdesc + (((ks >> 2) * 16384 + (ks & 3) * 32) >> 4),
-                            qdesc0 + (((ks >> 2) * 8192 + (ks & 3) * 32) >> 4), IDESC, ks > 0);
-                umma_commit(bar(B_SFULL + bf));
-                umma_commit(bar(B_KEMPTY + s));
+                for (int ks = 0; ks < D / 16; ++ks) {
+                    const uint32_t off = ((ks >> 2) * 16384 + (ks & 3) * 32) >> 4;
+                    umma_ss(tmem + bf * QT, kdesc + off, qdesc0 + off, IDESC, ks > 0);
+                }
+                umma_ss(tmem + bf * QT, augk, augq, IDESC, 1);
+                umma_commit(bar(F::B_SFULL + bf));
+                umma_commit(bar(F::B_KEMPTY + s));
             }
             __syncwarp();
         }
     } else {
-        // ===== consumers: thread r <-> TMEM lane r <-> key r of the tile ===========================
-        const int r = threadIdx.x;
-        const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
-        const float c = a.scale_log2;
-        // minus the base-2 log-sum-exp of the block's 64 queries; a query at or beyond N counts nothing
-        float nl2[USV_BLOCK];
-#pragma unroll
-        for (int qi = 0; qi < USV_BLOCK; ++qi) {
-            const int row = I * USV_BLOCK + qi;
-            nl2[qi] = row < N ? -a.lse[(int64_t)bh * N + row] * 1.4426950408889634f : -INFINITY;
-        }
+        // ===== consumers: thread r of a group <-> TMEM lane r <-> key r of the tile =================
+        const int side = warp >> 2;                      // query block this warpgroup serves
+        const int r = threadIdx.x & 127;
+        const int second = r >> 6;                      // which key block of the tile (uniform per warp)
+        const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16) + side * USV_BLOCK;
+        const uint64_t c2 = both(a.scale_log2);
         float* marg = a.marg + (int64_t)b * N;
         for (int t = 0; t < T; ++t) {
             const int bf = t % NBUF;
-            const int e = (2 * t + (r >> 6) < kh) ? sel[2 * t + (r >> 6)] : -1;   // this key's block
-            if (!mbar_wait(bar(B_SFULL + bf), (t / NBUF) & 1, s_abort, a.status, 0x10000000u)) break;
+            const int e = entry(2 * t + second);
+            const bool mine = (e >> side) & 1;
+            if (!mbar_wait(bar(F::B_SFULL + bf), (t / NBUF) & 1, s_abort, a.status, 0x10000000u)) break;
+            if (!mine) {
+                if (lane == 0) mbar_arrive(bar(F::B_SFREE + bf));
+                continue;
+            }
             fence_after();
             uint32_t s0[32], s1[32];
-            tmem_ld32(lane_base + bf * 64, s0);
-            tmem_ld32(lane_base + bf * 64 + 32, s1);
+            tmem_ld32(lane_base + bf * QT, s0);
+            tmem_ld32(lane_base + bf * QT + 32, s1);
             tmem_wait_ld();
             fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar(B_SFREE + bf));   // the logits are in registers
-            float acc0 = 0.f, acc1 = 0.f;
+            if (lane == 0) mbar_arrive(bar(F::B_SFREE + bf));   // the logits are in registers
+            uint64_t acc = 0, acc1 = 0;
 #pragma unroll
-            for (int qi = 0; qi < 32; ++qi) {
-                acc0 += ex2(fmaf(__uint_as_float(s0[qi]), c, nl2[qi]));
-                acc1 += ex2(fmaf(__uint_as_float(s1[qi]), c, nl2[32 + qi]));
+            for (int i = 0; i < 16; ++i) {
+                acc = add_f32x2(acc, weight2<F::POLY>(i, s0[2 * i], s0[2 * i + 1], c2));
+                acc1 = add_f32x2(acc1, weight2<F::POLY>(i, s1[2 * i], s1[2 * i + 1], c2));
             }
-            const int j = e * USV_BLOCK + (r & 63);
-            if (e >= 0 && j < N) atomicAdd(marg + j, (acc0 + acc1) * a.inv_hn);
+            float x, y;
+            unpack_f32x2(add_f32x2(acc, acc1), x, y);
+            const int j = (w0 + (e >> 2)) * USV_BLOCK + (r & 63);
+            if (j < N) atomicAdd(marg + j, (x + y) * a.inv_hn);
         }
     }
 
@@ -190,20 +296,30 @@ marginal_tc_kernel(const MargArgs a, const __grid_constant__ Maps maps) {
     }
 }
 
+template <int D>
+static int launch(const MargArgs& a, cudaStream_t st) {
+    Maps maps;
+    int rc;
+    if ((rc = make_bhnd_map(&maps.q, a.q, a.sq, a.B, a.H, a.N, D, "q")) != USV_OK) return rc;
+    if ((rc = make_bhnd_map(&maps.k, a.k, a.sk, a.B, a.H, a.N, D, "k")) != USV_OK) return rc;
+    const int64_t grid = (int64_t)a.B * a.H * ((a.NB + 1) / 2);
+    int kmx = 0;
+    for (int h = 0; h < a.H; ++h) kmx = a.k_per_head[h] > kmx ? a.k_per_head[h] : kmx;
+    const int widest = a.NB < WINDOW ? a.NB : WINDOW;
+    const size_t smem = Cfg<D>::smem_bytes(widest < 2 * kmx ? widest : 2 * kmx);
+    cudaError_t e = cudaFuncSetAttribute(marginal_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return fail(USV_ERR_CUDA, "attn_entropy: smem attribute: %s", cudaGetErrorString(e));
+    for (int w0 = 0; w0 < a.NB; w0 += WINDOW) {
+        launch_dep_smem(marginal_tc_kernel<D>, dim3((unsigned)grid), dim3(NTHREADS), smem, st, a, w0, maps);
+        USV_CHECK_LAUNCH("marginal_tc_kernel");
+    }
+    return USV_OK;
+}
+
 }  // namespace et
 
-int launch_marginal_tc(const MargArgs& a, cudaStream_t st) {
-    et::Maps maps;
-    int rc;
-    if ((rc = t5::make_bhnd_map(&maps.q, a.q, a.sq, a.B, a.H, a.N, et::D, "q")) != USV_OK) return rc;
-    if ((rc = t5::make_bhnd_map(&maps.k, a.k, a.sk, a.B, a.H, a.N, et::D, "k")) != USV_OK) return rc;
-    const int64_t grid = (int64_t)a.B * a.H * a.NB;
-    cudaError_t e = cudaFuncSetAttribute(et::marginal_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)et::SMEM_BYTES);
-    if (e != cudaSuccess) return fail(USV_ERR_CUDA, "attn_entropy: smem attribute: %s", cudaGetErrorString(e));
-    launch_dep_smem(et::marginal_tc_kernel, dim3((unsigned)grid), dim3(et::NTHREADS), et::SMEM_BYTES, st, a, maps);
-    USV_CHECK_LAUNCH("marginal_tc_kernel");
-    return USV_OK;
+int launch_marginal_tc(const MargArgs& a, int d, cudaStream_t st) {
+    return d == 64 ? et::launch<64>(a, st) : et::launch<128>(a, st);
 }
 
 }  // namespace usv

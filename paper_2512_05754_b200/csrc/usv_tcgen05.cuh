@@ -166,6 +166,17 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
     return d;
 }
 
+// The same for K-major rows of 32 bytes (one K = 16 step of bf16), 32-byte swizzle.
+__device__ __forceinline__ uint64_t smem_desc_32b(uint32_t addr) {
+    uint64_t d = 0;
+    d |= (uint64_t)((addr >> 4) & 0x3fff);
+    d |= (uint64_t)1 << 16;           // leading offset: not used by swizzled K-major operands
+    d |= (uint64_t)(256 >> 4) << 32;  // 8 rows
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)6 << 61;           // SWIZZLE_32B
+    return d;
+}
+
 // Instruction descriptor: bf16 x bf16 -> fp32, M x N tile; majors: 0 = K-major, 1 = MN-major.
 __host__ __device__ constexpr uint32_t instr_desc(int m, int n, int a_major, int b_major) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a_major << 15) | ((uint32_t)b_major << 16) |
@@ -301,14 +312,16 @@ inline EncodeTiledFn encode_fn() {
 }
 
 // bf16 [B,H,N,d] view -> rank-4 map (d, N, H, B), box 64 x 64 x 1 x 1, 128-byte swizzle; rows
-// at or beyond N read as zero.
+// at or beyond N read as zero.  A dimension with stride 0 (heads or batch elements that share
+// their rows) has extent 1 in the map: the kernel gives coordinate 0 for it.
 inline int make_bhnd_map(CUtensorMap* m, const void* ptr, const usv_strides& s, int B, int H, int N, int d,
                          const char* name) {
     EncodeTiledFn fn = encode_fn();
     if (fn == nullptr) return fail(USV_ERR_CUDA, "sparse_attn: cuTensorMapEncodeTiled not available");
-    cuuint64_t dims[4] = {(cuuint64_t)d, (cuuint64_t)N, (cuuint64_t)H, (cuuint64_t)B};
-    cuuint64_t strides[3] = {(cuuint64_t)s.sn * 2, (cuuint64_t)(H > 1 ? s.sh : s.sn * N) * 2,
-                             (cuuint64_t)(B > 1 ? s.sb : (H > 1 ? s.sh * H : s.sn * N)) * 2};
+    const bool heads = H > 1 && s.sh != 0, batch = B > 1 && s.sb != 0;
+    cuuint64_t dims[4] = {(cuuint64_t)d, (cuuint64_t)N, (cuuint64_t)(heads ? H : 1), (cuuint64_t)(batch ? B : 1)};
+    cuuint64_t strides[3] = {(cuuint64_t)s.sn * 2, (cuuint64_t)(heads ? s.sh : s.sn * N) * 2,
+                             (cuuint64_t)(batch ? s.sb : (heads ? s.sh * H : s.sn * N)) * 2};
     for (int i = 0; i < 3; ++i)
         if (strides[i] == 0 || (strides[i] & 15))
             return fail(USV_ERR_UNSUPPORTED, "sparse_attn: %s stride %d not TMA-compatible", name, i);

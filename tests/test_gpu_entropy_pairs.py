@@ -1,0 +1,44 @@
+"""Key marginal where the tcgen05 kernel can go wrong: both head widths, one block and odd block counts (a
+CTA whose second query block does not exist), a partial last block, lists from one block to all, holes
+in a list, heads that share their keys.  The reference is the same sum in PyTorch fp64 from the fp32
+log-sum-exp of the call; bf16 logits are exact products summed in fp32, so a weight differs by |logit| x 2^-20
+or so plus the exponential's 2^-21, and a sum of weights by less than 1e-4 of its size."""
+import pytest
+import torch
+
+DEV = "cuda:0"
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("B,H,N,d,kph,shared,holes", [
+    (1, 1, 37, 64, [1], False, False), (1, 1, 64, 128, [1], False, False), (2, 2, 129, 64, [3, 1], False, False),
+    (1, 3, 1000, 128, [16, 2, 7], False, True), (2, 2, 1000, 64, [5, 16], True, True),
+    (1, 2, 64 * 65 + 1, 64, [66, 9], False, False), (1, 2, 64 * 65 + 1, 128, [9, 66], True, False)])
+def test_marginal_against_fp64(B, H, N, d, kph, shared, holes):
+    import paper_2512_05754_b200 as usv
+    g = torch.Generator().manual_seed(N + d)
+    NB = -(-N // 64)
+    q = (2 * torch.randn(B, H, N, d, generator=g)).to(torch.bfloat16).to(DEV)
+    k = torch.randn(B, 1 if shared else H, N, d, generator=g).to(torch.bfloat16).to(DEV).expand(B, H, N, d)
+    kmax = max(kph)
+    sel = torch.full((B, H, NB, kmax), -1, dtype=torch.int32)
+    for b in range(B):
+        for h in range(H):
+            for i in range(NB):
+                row = torch.randperm(NB, generator=g)[:kph[h]].sort().values.int()
+                if holes and i % 3 == 1 and kph[h] > 1:
+                    row[kph[h] // 2] = -1
+                sel[b, h, i, :kph[h]] = row
+    keep = torch.zeros(B, H, NB, NB + 1, dtype=torch.bool)
+    keep.scatter_(3, torch.where(sel < 0, NB, sel).long(), True)
+    mask = keep[..., :NB].repeat_interleave(64, 2).repeat_interleave(64, 3)[:, :, :N, :N].to(DEV)
+    s = (q.double() @ k.double().transpose(-1, -2)) * d ** -0.5
+    lse = torch.logsumexp(s.masked_fill(~mask, -torch.inf), -1).float()
+    ref = torch.where(mask, (s - lse.double()[..., None]).exp(), 0.0).sum((1, 2)) / (H * N)
+    marg, ent = usv.attn_entropy(q, k, sel.to(DEV), kph, lse)
+    torch.cuda.synchronize()
+    assert usv.workspace_status() == 0
+    assert (marg.double() - ref).abs().max() <= 1e-4 * ref.max()
+    assert torch.equal(marg == 0, ref == 0)
+    h = -torch.where(ref > 0, ref * ref.clamp_min(1e-300).log(), 0.0).sum(1) / torch.log(torch.tensor(float(N)))
+    assert (ent.double().cpu() - h.cpu()).abs().max() <= 1e-4
