@@ -73,7 +73,7 @@ unsigned long long usv_kernel_launches(void);
  *     scores[b,h,I,J] = < mean_q[b,h,I,:], mean_k[b,h,J,:] > / sqrt(d)          (fp32).
  *
  * q: bf16 view [B,H,Nq,d], k: bf16 view [B,H,Nk,d]; d in {64,128}.
- * scores: fp32 [B,H,NBq,NBk] contiguous (written).  ws: pooled means (and, at d = 128, the bf16
+ * scores: fp32 [B,H,NBq,NBk] contiguous (written).  ws: pooled means (and the bf16
  * operand planes of the tensor-core product, which is accumulated in fp32 from a three-way split
  * of every fp32 mean and is fp32-accurate; small calls use fp32 CUDA cores), see *_workspace().
  */

@@ -2,13 +2,12 @@
 //
 //   pool_kernel   : one CTA per (tensor, b, h, four blocks); 16-byte loads, the next block in
 //                   flight while the current one is reduced (fp32 tree), mean over the VALID
-//                   rows of a block.  At d = 128 it also writes the three bf16 planes
+//                   rows of a block.  It also writes the three bf16 planes
 //                   (mean = hi + mid + lo) that the tensor-core score kernel multiplies, so the
 //                   fp32 means are not read back for a separate split pass.
 //   scores_small_kernel : the scores of small calls, fp32 CUDA cores (both head widths).
-//   scores_kernel : fp32 CUDA-core NT GEMM per (b,h), 64x64 output tile, 4x4 per thread.
-//                   Kept in fp32 (not bf16 tensor cores) because the result decides an integer
-//                   (the top-k set) that is compared with an fp64 evaluation.
+//   scores_kernel : fp32 CUDA-core NT GEMM per (b,h), 64x64 output tile, 4x4 per thread, for the entry
+//                   point without caller scratch, which has no room for the planes.
 #include "usv_scores.cuh"
 
 namespace usv {
@@ -19,7 +18,7 @@ struct PoolArgs {
     int N[2], NB[2];
     float* out[2];  // [B,H,NB,d]
     int H;
-    // d = 128 with the tensor-core score kernel: bf16 planes [3][B*H][NB_pad][128] per tensor
+    // for the tensor-core score kernel: bf16 planes [3][B*H][NB_pad][d] per tensor
     // (NULL: not wanted); rows NB .. NB_pad - 1 are written as zero
     __nv_bfloat16* planes[2];
     int NB_pad[2];
@@ -248,10 +247,10 @@ static int64_t small_tiles(int BH, int NBq, int NBk) { return (int64_t)BH * ceil
 extern "C" size_t usv_block_scores_workspace(int B, int H, int Nq, int Nk, int d) {
     if (B <= 0 || H <= 0 || Nq <= 0 || Nk <= 0 || d <= 0) return 0;
     const size_t nbq = usv::ceil_div(Nq, USV_BLOCK), nbk = usv::ceil_div(Nk, USV_BLOCK);
-    // header, pooled means of q and k; at d = 128 also the bf16 planes of the tensor-core scores kernel
+    // header, pooled means of q and k, the bf16 planes of the tensor-core scores kernel
     return usv::WS_HEADER + usv::align_up((size_t)B * H * nbq * d * sizeof(float), 256) +
            usv::align_up((size_t)B * H * nbk * d * sizeof(float), 256) +
-           (d == 128 ? usv::scores_tc_bytes(B * H, (int)nbq, (int)nbk) : 0);
+           (d == 64 || d == 128 ? usv::scores_tc_bytes(B * H, (int)nbq, (int)nbk, d) : 0);
 }
 
 extern "C" int usv_block_scores(int B, int H, int Nq, int Nk, int d, const void* q,
@@ -290,7 +289,7 @@ extern "C" int usv_block_scores(int B, int H, int Nq, int Nk, int d, const void*
     void* tc_mem = reinterpret_cast<char*>(kbar) + align_up((size_t)B * H * NBk * d * sizeof(float), 256);
     const int64_t tiles = small_tiles(B * H, NBq, NBk);
     const bool small = tiles <= SMALL_TILES;
-    if (d == 128 && !small) scores_tc_planes(tc_mem, B * H, NBq, NBk, &a.planes[0], &a.planes[1], &a.NB_pad[0], &a.NB_pad[1]);
+    if (!small) scores_tc_planes(tc_mem, B * H, NBq, NBk, d, &a.planes[0], &a.planes[1], &a.NB_pad[0], &a.NB_pad[1]);
     a.span = pool_span((int64_t)B * H * (NBq + NBk));
     dim3 pg(ceil_div(NBq > NBk ? NBq : NBk, a.span), B * H, 2);
     if (d == 128) launch_dep(pool_kernel<128>, dim3(pg), dim3(128), 0, st, a);
@@ -305,12 +304,7 @@ extern "C" int usv_block_scores(int B, int H, int Nq, int Nk, int d, const void*
         USV_CHECK_LAUNCH("scores_small_kernel");
         return USV_OK;
     }
-    if (d == 128)
-        return launch_scores_tc(scores, B * H, NBq, NBk, sc, tc_mem, static_cast<unsigned int*>(ws), st);
-    dim3 sg(ceil_div(NBk, 64), ceil_div(NBq, 64), B * H);
-    launch_dep(scores_kernel, dim3(sg), dim3(256), 0, st, qbar, kbar, scores, NBq, NBk, d, sc);
-    USV_CHECK_LAUNCH("scores_kernel");
-    return USV_OK;
+    return launch_scores_tc(scores, B * H, NBq, NBk, d, sc, tc_mem, static_cast<unsigned int*>(ws), st);
 }
 
 // ------------------------------------------------------------------------------------------
