@@ -111,11 +111,11 @@ __device__ __forceinline__ int block_scan_1024(int v, int* scratch, int* total) 
 // ---------------------------------------------------------------------------- merged-source lists
 // The sources merged into every destination, built by one atomic per source while the plan is
 // written: the first SLOTS of a destination (in order of arrival, merge_kernel sorts them) sit in a
-// 16-byte row of their own, further ones hang on a chain.  Counting, scanning and filling a CSR
+// 32-byte row of their own, further ones hang on a chain.  Counting, scanning and filling a CSR
 // took three more kernels (13 us at 32 760 tokens, launches included) and left merge_kernel one
 // more dependent load per row.
 struct MergeLists {
-    static constexpr int SLOTS = 4;
+    static constexpr int SLOTS = 8;
     int32_t* cnt;        // [B,nB] sources of the destination, starts at zero
     int32_t* head;       // [B,nB] 1 + the last source chained (0: none), starts at zero
     int32_t* slots;      // [B,nB,SLOTS]
@@ -315,41 +315,73 @@ __global__ void __launch_bounds__(1024) row_scan_kernel(int nB, const int32_t* _
 // ---------------------------------------------------------------------------- local matching
 // The other reading of Sec. 3.3 (matching kept inside neighbouring 3D blocks): Eq. 8-9 with the
 // arg-max over the destinations of the partition blocks within (wt, wh, ww) blocks of the
-// source's own block.  One warp per source; the lanes split the descriptor, the candidates are
-// visited in ascending destination index and a later one wins only when strictly better.
+// source's own block; a later destination wins only when strictly better.  One warp per source, 32
+// candidates in ascending order at a time: the lanes split the descriptors, all candidates' rows are
+// requested before any is used, and the 32 sums over lanes are taken together (at every step a lane
+// hands half of its candidates over: 31 shuffles, where one candidate after the other takes 160), which
+// leaves candidate l in lane l.  Bound: issue slots and the reads of the candidates from L1.  2 x 16 380
+// sources, 27 candidates of 128: 73 -> 41 us (46 us without the bound on registers).
 template <int DM>
-__global__ void __launch_bounds__(256) match_local_kernel(const float* __restrict__ mhat, Part p, int N, int nA,
+__global__ void __launch_bounds__(256, 3) match_local_kernel(const float* __restrict__ mhat, Part p, int N, int nA,
                                                           int wt, int wh, int ww,
                                                           const int32_t* __restrict__ src_idx,
                                                           int32_t* __restrict__ jstar_s, float* __restrict__ u_s) {
     dep_sync();
     constexpr int V = DM / 32;   // floats per lane
+    struct alignas(4 * V) Vec { float f[V]; };
     const int a = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (a >= nA) return;
     const int b = blockIdx.y;
     const int lane = threadIdx.x & 31;
-    const float* mb = mhat + (int64_t)b * N * DM;
+    const float* mb = mhat + (int64_t)b * N * DM + lane * V;
     const int i = src_idx[a];
     int t, y, x;
     p.coords(i, t, y, x);
     const int bt = p.dst.quot(t), by = p.dsh.quot(y), bx = p.dsw.quot(x);
     const int nBt = p.nB / (p.nHy * p.nWx);
-    float mi[V];
-#pragma unroll
-    for (int e = 0; e < V; ++e) mi[e] = mb[(int64_t)i * DM + lane * V + e];
+    const int t0 = max(bt - wt, 0), y0 = max(by - wh, 0), x0 = max(bx - ww, 0);
+    const int ny = min(by + wh, p.nHy - 1) - y0 + 1, nx = min(bx + ww, p.nWx - 1) - x0 + 1;
+    const int64_t count = (int64_t)(min(bt + wt, nBt - 1) - t0 + 1) * ny * nx;   // (the block's own destination is among them)
+    const Vec mi = *reinterpret_cast<const Vec*>(mb + (int64_t)i * DM);
     float best = -INFINITY;
     int jbest = -1;
-    for (int ct = max(bt - wt, 0); ct <= min(bt + wt, nBt - 1); ++ct)
-        for (int cy = max(by - wh, 0); cy <= min(by + wh, p.nHy - 1); ++cy)
-            for (int cx = max(bx - ww, 0); cx <= min(bx + ww, p.nWx - 1); ++cx) {
-                const int j = ((ct * p.st) * p.Hh + cy * p.sh) * p.W + cx * p.sw;
-                float c = 0.f;
+    for (int64_t k0 = 0; k0 < count; k0 += 32) {
+        const int n = (int)min((int64_t)32, count - k0);
+        const int k = (int)k0 + min(lane, n - 1);
+        const int row = k / nx, ct = row / ny;
+        const int jk = (((t0 + ct) * p.st) * p.Hh + (y0 + row - ct * ny) * p.sh) * p.W + (x0 + k - row * nx) * p.sw;
+        float c[32];
 #pragma unroll
-                for (int e = 0; e < V; ++e) c = fmaf(mi[e], mb[(int64_t)j * DM + lane * V + e], c);
+        for (int q0 = 0; q0 < 32; q0 += 8) {
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-                if (c > best) { best = c; jbest = j; }
+            for (int q = q0; q < q0 + 8; ++q) c[q] = 0.f;
+            if (q0 < n) {
+                Vec mj[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    mj[q] = *reinterpret_cast<const Vec*>(mb + (int64_t)__shfl_sync(0xffffffffu, jk, q0 + q) * DM);
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+#pragma unroll
+                    for (int e = 0; e < V; ++e) c[q0 + q] = fmaf(mi.f[e], mj[q].f[e], c[q0 + q]);
             }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const bool up = lane & o;
+#pragma unroll
+            for (int q = 0; q < o; ++q) {
+                const float give = up ? c[q] : c[q + o], keep = up ? c[q + o] : c[q];
+                c[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+            }
+        }
+        const uint32_t key = lane < n && c[0] > -INFINITY ? float_key(c[0]) : 0u;   // NaN never wins
+        const uint32_t top = __reduce_max_sync(0xffffffffu, key);
+        const int w = __ffs(__ballot_sync(0xffffffffu, key == top)) - 1;
+        const float cw = __shfl_sync(0xffffffffu, c[0], w);
+        const int jw = __shfl_sync(0xffffffffu, jk, w);
+        if (top != 0 && cw > best) { best = cw; jbest = jw; }
+    }
     if (lane == 0) {
         jstar_s[(int64_t)b * nA + a] = jbest;
         u_s[(int64_t)b * nA + a] = best;
@@ -361,19 +393,30 @@ __global__ void __launch_bounds__(256) match_local_kernel(const float* __restric
 // destination averaged with its merged sources, summed in ascending source index (fp32).  Most
 // destinations have no more than two sources: their rows and the destination's are requested
 // together, G 16-byte chunks a lane each, before any is used, and only one chunk's sums are live at a
-// time, so that four CTAs share an SM.  2 x 118 800 rows of 6 KB, a quarter merged: 388 us, 6.6 TB/s, the
-// copy bandwidth of the device (392 us before); 2 x 32 760 rows of 3 KB, 40 % merged: 60 us (65 us).
-// Warps that stay and walk 1 KB segments, looking the next one's lists up ahead, were slower (96 us).
-__global__ void __launch_bounds__(256, 4) merge_kernel(Part p, int N, int C, int nU, int Nm,
+// time.  Longer lists take ROWS rows of two chunks at a time.  The destinations come first: a row with a
+// long list takes several times a copy's time, and at the end of the grid it is all that runs.  Four
+// warps a CTA, so that one long row keeps few others' registers.  Calls of a stored plan, us (256 threads,
+// copies first, two rows at a time before; x the copy bandwidth of the device): 2 x 118 800 rows of 6 KB, a
+// quarter merged: 393 -> 378 (1.03); 2 x 32 760 rows of 3 KB, 40 % merged: 62 -> 53 (0.93); 28 101 rows
+// of 3 KB, blocks of 2 x 2, a quarter merged, up to ten sources a row: 42.6 -> 27.3 (0.85); 32 760 rows,
+// blocks of 2 x 2 x 2, 40 %: 48 -> 29.  ROWS = 3 or 5, 6 or 8 CTAs an SM: within 5 % either way.
+// Warps that stay and walk 1 KB segments, looking the next one's lists up ahead, were slower (96 us
+// where 65).
+__global__ void __launch_bounds__(128, 7) merge_kernel(Part p, int N, int C, int nU, int Nm,
                                                        const __nv_bfloat16* __restrict__ x,
                                                        const MergeLists lists,
                                                        const int32_t* __restrict__ dst_of,
                                                        __nv_bfloat16* __restrict__ out, int64_t rows) {
     dep_sync();
-    const int64_t gw = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (gw >= rows) return;
+    const int64_t w = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
+    if (w >= rows) return;
     const int lane = threadIdx.x & 31;
-    const int b = (int)(gw / Nm), row = (int)(gw % Nm);
+    // the destinations of all batch elements first, the plain copies last
+    const bool is_copy = w >= (int64_t)(rows / Nm) * p.nB;
+    const int64_t wi = is_copy ? w - (int64_t)(rows / Nm) * p.nB : w;
+    const int per = is_copy ? nU : p.nB;
+    const int b = (int)(wi / per), row = (int)(wi - (int64_t)b * per) + (is_copy ? 0 : nU);
+    const int64_t gw = (int64_t)b * Nm + row;
     const __nv_bfloat16* xb = x + (int64_t)b * N * C;
     auto row_of = [&](int tok) { return reinterpret_cast<const uint4*>(xb + (int64_t)tok * C); };
     uint4* dst = reinterpret_cast<uint4*>(out + gw * C);
@@ -393,7 +436,7 @@ __global__ void __launch_bounds__(256, 4) merge_kernel(Part p, int N, int C, int
         return;
     }
     const float inv = 1.0f / (float)(len + 1);
-    constexpr int G = 3;
+    constexpr int G = 3, ROWS = 4;
     if (len <= 2) {
         int i0 = __shfl_sync(0xffffffffu, id, 0), i1 = len == 2 ? __shfl_sync(0xffffffffu, id, 1) : i0;
         const uint4 *src0 = row_of(min(i0, i1)), *src1 = row_of(max(i0, i1));
@@ -429,11 +472,11 @@ __global__ void __launch_bounds__(256, 4) merge_kernel(Part p, int N, int C, int
         }
         return;
     }
-    // Lane s < len <= 32 ends up with the s-th smallest source index.  Longer lists (rare) are found by
-    // a pass over dst_of where they are needed: it meets them in ascending order.
-    int myid = 0x7fffffff;
+    // Lane 0 holds the destination's token, lane s + 1 the s-th smallest source.  Lists beyond 31 (rare) are
+    // found by a pass over dst_of where they are needed: it meets them in ascending order.
+    int myid = j;
     const int32_t* dob = dst_of + (int64_t)b * N;
-    if (len <= 32) {
+    if (len <= 31) {
         if (len > MergeLists::SLOTS) {
             int n = lists.head[od];
             for (int s = MergeLists::SLOTS; s < len; ++s) {
@@ -448,18 +491,14 @@ __global__ void __launch_bounds__(256, 4) merge_kernel(Part p, int N, int C, int
         for (int s = 0; s < len; ++s) {
             const int oid = __shfl_sync(0xffffffffu, id, s);
             const int orank = __shfl_sync(0xffffffffu, rank, s);
-            if (orank == lane) myid = oid;
+            if (orank + 1 == lane) myid = oid;
         }
     }
-    for (int cb = 0; cb < nvec; cb += 64) {   // (whole warps: the lanes hand the sources round)
+    for (int cb = 0; cb < nvec; cb += 64) {   // (whole warps: the lanes hand the rows round)
         const int c0 = cb + lane;
         float acc[2][8];
-        uint4 v[2];
 #pragma unroll
-        for (int g = 0; g < 2; ++g) {
-            v[g] = c0 + g * 32 < nvec ? __ldg(srcj + c0 + g * 32) : make_uint4(0, 0, 0, 0);
-            bf16x8_to_float(v[g], acc[g]);
-        }
+        for (int e = 0; e < 8; ++e) acc[0][e] = acc[1][e] = -0.f;   // (-0 + x is x for every x)
         auto add = [&](const uint4* w) {
 #pragma unroll
             for (int g = 0; g < 2; ++g) {
@@ -474,15 +513,20 @@ __global__ void __launch_bounds__(256, 4) merge_kernel(Part p, int N, int C, int
 #pragma unroll
             for (int g = 0; g < 2; ++g) w[g] = c0 + g * 32 < nvec ? __ldg(src + c0 + g * 32) : make_uint4(0, 0, 0, 0);
         };
-        if (len <= 32) {
-            for (int s = 0; s < len; s += 2) {   // two rows in flight
-                uint4 w[2];
-                load(__shfl_sync(0xffffffffu, myid, s), v);
-                if (s + 1 < len) load(__shfl_sync(0xffffffffu, myid, s + 1), w);
-                add(v);
-                if (s + 1 < len) add(w);
+        if (len <= 31) {
+            for (int s = 0; s <= len; s += ROWS) {   // ROWS rows in flight
+                uint4 w[ROWS][2];
+#pragma unroll
+                for (int q = 0; q < ROWS; ++q)
+                    if (s + q <= len) load(__shfl_sync(0xffffffffu, myid, s + q), w[q]);
+#pragma unroll
+                for (int q = 0; q < ROWS; ++q)
+                    if (s + q <= len) add(w[q]);
             }
         } else {
+            uint4 v[2];
+            load(j, v);
+            add(v);
             for (int n0 = 0; n0 < N; n0 += 32)
                 for (unsigned found = __ballot_sync(0xffffffffu, n0 + lane < N && dob[n0 + lane] == j); found; found &= found - 1) {
                     load(n0 + __ffs(found) - 1, v);
@@ -502,7 +546,7 @@ __global__ void __launch_bounds__(256, 4) merge_kernel(Part p, int N, int C, int
 // rows: B * Nm output rows
 static int launch_merge(const Part& p, int N, int C, int nU, int Nm, int64_t rows, const void* x, const MergeLists& lists,
                         const int32_t* dst_of, void* out, cudaStream_t st) {
-    launch_dep(merge_kernel, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, p, N, C, nU, Nm,
+    launch_dep(merge_kernel, dim3((unsigned)((rows + 3) / 4)), dim3(128), 0, st, p, N, C, nU, Nm,
                static_cast<const __nv_bfloat16*>(x), lists, dst_of, static_cast<__nv_bfloat16*>(out), rows);
     USV_CHECK_LAUNCH("merge_kernel");
     return USV_OK;

@@ -1,0 +1,46 @@
+"""Merging at the edges of the local matcher's groups of 32 candidates and of the slots a destination has
+for its sources.  A window over the whole grid has to give the global matcher's plan, ties (equal
+destinations) included; rows with 7 to 9 sources are compared with the oracle's merge of the plan."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from parity_utils import bf16_ulp_distance, bits
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.mark.parametrize("dm", [64, 128])
+@pytest.mark.parametrize("nB", [1, 7, 8, 9, 31, 32, 33, 64, 65])
+def test_candidate_counts(nB, dm):
+    import paper_2512_05754_b200 as usv
+    grid, part, N = (1, 1, 2 * nB), (1, 1, 2), 2 * nB
+    g = torch.Generator().manual_seed(nB + dm)
+    x = torch.randn(2, N, 64, generator=g).to(torch.bfloat16).to(DEV)
+    metric = torch.randn(2, N, 2, dm, generator=g).to(torch.bfloat16)
+    metric[:, nB // 2 * 2] = metric[:, 0]                     # two destinations alike: the lower one wins
+    metric[0, 1] = metric[0, 0]
+    metric = metric.to(DEV)
+    r = max(1, nB // 2)
+    xg, pg = usv.token_merge(x, metric, grid, part, r, debug=True)
+    xl, pl = usv.token_merge(x, metric, grid, part, r, debug=True, window=(0, 0, nB))
+    assert torch.equal(pg.dst_of, pl.dst_of) and torch.equal(pg.pos, pl.pos) and torch.equal(xg, xl)
+
+
+def test_slots_of_a_destination():
+    import paper_2512_05754_b200 as usv
+    grid, part, N = (1, 4, 32), (1, 1, 2), 128                # 64 sources, 64 destinations
+    dst = np.nonzero(oracle.destination_mask(grid, part))[0]
+    src = list(np.random.default_rng(3).permutation(np.nonzero(~oracle.destination_mask(grid, part))[0]))
+    g = torch.Generator().manual_seed(7)
+    metric = torch.randn(1, N, 2, 64, generator=g)
+    for t, n in enumerate([7, 8, 9, 4, 16]):
+        for _ in range(n):
+            metric[0, src.pop()] = metric[0, dst[9 * t]]
+    x = torch.randn(1, N, 520, generator=g).to(torch.bfloat16)
+    xm, plan = usv.token_merge(x.to(DEV), metric.to(torch.bfloat16).to(DEV), grid, part, 44)
+    ref = oracle.round_to_bf16(oracle.merge_apply(x, plan.dst_of.cpu().numpy(), plan.pos.cpu().numpy(), N - 44))
+    assert bf16_ulp_distance(bits(xm), ref).max() <= 1
+    assert torch.equal(usv.token_merge_apply(x.to(DEV), plan), xm)
