@@ -32,6 +32,7 @@ struct AttnArgs {
     int N_full;
     const int* work_list;   // list mode of the exact kernel (NULL = one CTA per query block)
     const int* work_count;
+    const uint16_t* work_flags;   // flag mode: the query blocks whose flag is not 0; their number goes to fallback_count
     int B, H, N, NB, kmax;
     float scale_log2;    // softmax scale * log2(e)
     int k_per_head[USV_MAX_HEADS];
@@ -40,6 +41,8 @@ struct AttnArgs {
 
 int launch_attn_mma(const AttnArgs& a, int d, cudaStream_t st);
 bool attn_pair_supported(const AttnArgs& a, int d);
+// whether the call is too small for a pairing plan: a.pairs stays NULL, and fallback_list takes flags
+bool attn_pair_direct(const AttnArgs& a);
 int launch_attn_pair(const AttnArgs& a, int d, cudaStream_t st);
 // fused unmerge: copies the query blocks the exact kernel recomputed (into o) to their original tokens in y
 int launch_scatter_fallbacks(const AttnArgs& a, int d, cudaStream_t st);

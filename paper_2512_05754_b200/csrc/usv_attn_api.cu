@@ -79,6 +79,7 @@ static int sparse_attn_impl(int B, int H, int N, int d, const void* q, const usv
     a.list_batch = 0;
     a.work_list = nullptr;
     a.work_count = nullptr;
+    a.work_flags = nullptr;
     a.unmerge_off = unmerge_off;
     a.unmerge_idx = unmerge_idx;
     a.y = static_cast<__nv_bfloat16*>(y);
@@ -97,10 +98,14 @@ static int sparse_attn_impl(int B, int H, int N, int d, const void* q, const usv
     // 384: 21 / 25, 512: 35 / 28; keep 16, 32 query blocks: 27 / 16.
     const bool small = d == 64 && kmx <= 8 && (int64_t)B * H * NB <= 384;
     if (impl == 0 && !small && attn_pair_supported(a, d)) {
-        int rc2 = launch_pair_plan(a, plan_mem, st);
-        if (rc2 != USV_OK) return rc2;
-        rc2 = launch_attn_pair(a, d, st);
-        if (rc2 != USV_OK) return rc2;
+        int rc2;
+        if (attn_pair_direct(a)) {
+            if ((rc2 = launch_attn_pair(a, d, st)) != USV_OK) return rc2;
+            a.work_flags = reinterpret_cast<const uint16_t*>(a.fallback_list);
+            return launch_attn_mma(a, d, st);
+        }
+        if ((rc2 = launch_pair_plan(a, plan_mem, st)) != USV_OK) return rc2;
+        if ((rc2 = launch_attn_pair(a, d, st)) != USV_OK) return rc2;
         // exact recomputation of the (normally zero) query blocks the fast kernel reported
         a.work_list = a.fallback_list;
         a.work_count = a.fallback_count;

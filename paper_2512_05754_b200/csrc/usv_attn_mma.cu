@@ -222,11 +222,36 @@ __device__ __forceinline__ void attn_mma_block(const AttnArgs& a, const int work
     }
 }
 
-// One CTA per query block, or (list mode) a fixed grid whose CTAs walk a device-side work list.
-template <int D>
+// One CTA per query block, or a fixed grid whose CTAs walk a device-side work list or take every gridDim-th
+// block's flag.
+template <int D, bool FLAGS>
 __global__ void __launch_bounds__(128) attn_mma_kernel(const AttnArgs a) {
     dep_sync();
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (FLAGS) {
+        const int blocks = a.B * a.H * a.NB;
+        if (blockIdx.x == 0) {   // how many there are
+            __shared__ int s_count;
+            if (threadIdx.x == 0) s_count = 0;
+            __syncthreads();
+            int count = 0;
+            for (int i = threadIdx.x; i < blocks; i += 128) count += a.work_flags[i] != 0;
+            if (count) atomicAdd(&s_count, count);
+            __syncthreads();
+            if (threadIdx.x == 0) *a.fallback_count = s_count;
+        }
+        const int stride = gridDim.x;
+        for (int i0 = blockIdx.x; i0 < blocks; i0 += 128 * stride) {
+            const int64_t mine = i0 + (int64_t)threadIdx.x * stride;
+            if (!__syncthreads_or(mine < blocks && a.work_flags[mine] != 0)) continue;
+            for (int64_t i = i0; i < blocks && i < i0 + 128 * (int64_t)stride; i += stride)
+                if (a.work_flags[i] != 0) {
+                    attn_mma_block<D>(a, (int)i, smem_raw);
+                    __syncthreads();
+                }
+        }
+        return;
+    }
     if (a.work_list == nullptr) {
         // the words behind the sticky status word (fallback count, work counter, ...) start at zero
         if (blockIdx.x == 0 && threadIdx.x < (WS_HEADER - 4) / 4) a.status[1 + threadIdx.x] = 0u;
@@ -243,16 +268,14 @@ __global__ void __launch_bounds__(128) attn_mma_kernel(const AttnArgs a) {
 int launch_attn_mma(const AttnArgs& a, int d, cudaStream_t st) {
     int64_t grid = (int64_t)a.B * a.H * a.NB;
     if (grid > 2147483647LL) return fail(USV_ERR_UNSUPPORTED, "sparse_attn: too many query blocks");
-    if (a.work_list != nullptr && grid > 296) grid = 296;
-    if (d == 128) {
-        cudaFuncSetAttribute(attn_mma_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)MmaSmem<128>::BYTES);
-        launch_dep_smem(attn_mma_kernel<128>, dim3((unsigned)grid), dim3(128), MmaSmem<128>::BYTES, st, a);
-    } else {
-        cudaFuncSetAttribute(attn_mma_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)MmaSmem<64>::BYTES);
-        launch_dep_smem(attn_mma_kernel<64>, dim3((unsigned)grid), dim3(128), MmaSmem<64>::BYTES, st, a);
-    }
+    if ((a.work_list != nullptr || a.work_flags != nullptr) && grid > 296) grid = 296;
+    auto launch = [&](auto kernel, size_t smem) {
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        launch_dep_smem(kernel, dim3((unsigned)grid), dim3(128), smem, st, a);
+    };
+    const bool flags = a.work_flags != nullptr;
+    if (d == 128) launch(flags ? attn_mma_kernel<128, true> : attn_mma_kernel<128, false>, MmaSmem<128>::BYTES);
+    else launch(flags ? attn_mma_kernel<64, true> : attn_mma_kernel<64, false>, MmaSmem<64>::BYTES);
     USV_CHECK_LAUNCH("attn_mma_kernel");
     return USV_OK;
 }

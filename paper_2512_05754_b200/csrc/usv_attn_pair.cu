@@ -167,7 +167,10 @@ __device__ __forceinline__ const int* item_list(const int* hdr) {
                                                             (unsigned)hdr[I_LIST_LO]);
 }
 
-template <int D>
+// DIRECT: no pairing plan (see attn_pair_direct).  Neighbouring query blocks share an item, the CTAs take the
+// items in turn, the scout builds an item's list from the two selection rows, and a query block that the
+// exact kernel has to recompute is flagged (one byte per 32 of its rows) instead of listed.
+template <int D, bool DIRECT>
 __global__ void __launch_bounds__(NTHREADS, 1)
 attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
     using F = Cfg<D>;
@@ -230,14 +233,21 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
         // into ring slot n and publish it; a pair without any key block gets its defined output
         // (zeros) right here and is not published.  Returns the item's tile count, -1 after
         // publishing the end marker, -2 when a bounded wait gave up.
+        int64_t turn = blockIdx.x;
         auto publish = [&](int n) -> int {
             int* hdr = hdr_of(n);
             if (n >= NSLOT && !mbar_wait(bar(F::B_IFREE + n % NSLOT), ((n / NSLOT) - 1) & 1, s_abort, a.status, 0x8000))
                 return -2;
             for (;;) {
-                int wi = 0;
-                if (lane == 0) wi = atomicAdd(a.work_counter, 1);
-                const int64_t w = __shfl_sync(0xffffffffu, wi, 0);
+                int64_t w;
+                if (DIRECT) {
+                    w = turn;
+                    turn += gridDim.x;
+                } else {
+                    int wi = 0;
+                    if (lane == 0) wi = atomicAdd(a.work_counter, 1);
+                    w = __shfl_sync(0xffffffffu, wi, 0);
+                }
                 if (w >= nitems) {
                     if (lane == 0) hdr[I_T] = -1;
                     __syncwarp();
@@ -248,11 +258,42 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
                 const int bh_ord = (int)(w / NP);
                 const int b = bh_ord / a.H;
                 const int h = a.head_order[bh_ord % a.H];
-                const int2 pq = a.pairs[((int64_t)b * a.H + h) * NP + pair];   // similarity-driven pairing
-                const int* pl = a.lists + b * a.list_batch + a.list_off[h] +
-                                (int64_t)pair * list_stride(a.k_per_head[h], NB);
-                const int nU = __ldg(pl);
+                int2 pq;
+                const int* pl = nullptr;
+                int nU;
+                if (DIRECT) {
+                    // a word of either row's bitmap per lane, the union as a list in the ring slot
+                    pq = make_int2(2 * pair, 2 * pair + 1 < NB ? 2 * pair + 1 : -1);
+                    const int kh = a.k_per_head[h];
+                    const int32_t* row = a.sel + (((int64_t)b * a.H + h) * NB + pq.x) * a.kmax;
+                    uint32_t ba = 0, bb = 0;
+                    for (int i0 = 0; i0 < kh; i0 += 32) {
+                        const int i = i0 + lane;
+                        const int ea = i < kh ? __ldg(row + i) : -1, eb = i < kh && pq.y >= 0 ? __ldg(row + a.kmax + i) : -1;
+                        const int m = min(32, kh - i0);
+#pragma unroll 4
+                        for (int q = 0; q < m; ++q) {
+                            const int ja = __shfl_sync(0xffffffffu, ea, q), jb = __shfl_sync(0xffffffffu, eb, q);
+                            if (ja >= 0 && ja < NB && (ja >> 5) == lane) ba |= 1u << (ja & 31);
+                            if (jb >= 0 && jb < NB && (jb >> 5) == lane) bb |= 1u << (jb & 31);
+                        }
+                    }
+                    uint32_t u = ba | bb;
+                    const int incl = warp_incl_scan(__popc(u));
+                    nU = __shfl_sync(0xffffffffu, incl, 31);
+                    for (int at = 16 + incl - __popc(u); u != 0; u &= u - 1) {
+                        const int bit = __ffs(u) - 1;
+                        hdr[at++] = ((lane * 32 + bit) << 2) | ((ba >> bit) & 1u) | (((bb >> bit) & 1u) << 1);
+                    }
+                    __syncwarp();
+                } else {
+                    pq = a.pairs[((int64_t)b * a.H + h) * NP + pair];   // similarity-driven pairing
+                    pl = a.lists + b * a.list_batch + a.list_off[h] + (int64_t)pair * list_stride(a.k_per_head[h], NB);
+                    nU = __ldg(pl);
+                }
                 if (nU == 0) {
+                    if (DIRECT && lane < 2 && (lane == 0 || pq.y >= 0))
+                        reinterpret_cast<uint16_t*>(a.fallback_list)[(int64_t)bh_ord * NB + pq.x + lane] = 0;
                     // no valid key block at all: defined output (zeros, log-sum-exp 0), as the exact kernel does
                     __nv_bfloat16* O = a.o + b * a.so.sb + h * a.so.sh;
                     for (int idx = lane; idx < 128 * (D / 8); idx += 32) {
@@ -281,8 +322,8 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
                 int srefA = nU, srefB = nU;   // first union slot that block A / block B may see
                 for (int i0 = 0; i0 < nU; i0 += 32) {
                     const int idx = i0 + lane;
-                    const int e = idx < nU ? __ldg(pl + 1 + idx) : 0;
-                    if (nU <= LCAP && idx < nU) hdr[16 + idx] = e;
+                    const int e = idx >= nU ? 0 : (DIRECT ? hdr[16 + idx] : __ldg(pl + 1 + idx));
+                    if (!DIRECT && nU <= LCAP && idx < nU) hdr[16 + idx] = e;
                     const unsigned ba = __ballot_sync(0xffffffffu, e & 1), bb = __ballot_sync(0xffffffffu, e & 2);
                     if (srefA == nU && ba) srefA = i0 + __ffs(ba) - 1;
                     if (srefB == nU && bb) srefB = i0 + __ffs(bb) - 1;
@@ -550,9 +591,14 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
                         unpack_f32x2(add_f32x2(z0, z1), za, zb);
                         finite = za + zb == 0.f;
                     }
-                    if (live && !(in_range && finite) && a.fallback_list != nullptr &&
-                        atomicExch(&s_flag[slot * 2 + side], 1) == 0)
+                    if (DIRECT) {
+                        const bool any = __any_sync(0xffffffffu, live && !(in_range && finite));
+                        if (lane == 0 && iq >= 0)
+                            reinterpret_cast<uint8_t*>(a.fallback_list)[2 * ((int64_t)ibh * NB + iq) + (warp & 1)] = any;
+                    } else if (live && !(in_range && finite) && a.fallback_list != nullptr &&
+                               atomicExch(&s_flag[slot * 2 + side], 1) == 0) {
                         a.fallback_list[atomicAdd(a.fallback_count, 1)] = ibh * NB + iq;
+                    }
                     fence_before();
                     __syncwarp();
                     if (lane == 0) {
@@ -753,21 +799,38 @@ bool attn_pair_supported(const AttnArgs& a, int d) {
     return (d == 64 || d == 128) && a.NB <= pr::MAX_NB && a.work_counter != nullptr;
 }
 
-template <int D>
+// The pairing plan takes 8 to 10 us, partly hidden, before the first query block is computed, and saves a
+// tenth to a sixth of the attention kernel's work: it does not pay in small calls, here those that keep at
+// most DIRECT_WORK key blocks over all query blocks.  Whole calls, us, with the plan / without it, at key
+// blocks kept: D = 128, 2.7 k 29.1 / 26.4, 3.5 k 32.3 / 26.7, 5 k (two heads of 160 blocks) 42.2 / 35.2, 7 k
+// 40.8 / 39.5, 12 k 51.4 / 50.8, 14 k 55.5 / 61.0, 24 k 76 / 80; D = 64, 4.6 k 30.3 / 25.4, 14 k 45.8 / 47.4,
+// 38 k 81 / 93.  (Beyond 1024 blocks or lists of 256 the scout's registers and ring slots do not hold a union.)
+bool attn_pair_direct(const AttnArgs& a) {
+    constexpr int64_t DIRECT_WORK = 10000;
+    int64_t kept = 0;
+    int most = 0;
+    for (int h = 0; h < a.H; ++h) {
+        kept += a.k_per_head[h];
+        most = a.k_per_head[h] > most ? a.k_per_head[h] : most;
+    }
+    return a.y == nullptr && a.NB <= 1024 && 2 * most <= pr::LCAP && (int64_t)a.B * a.NB * kept <= DIRECT_WORK;
+}
+
+template <int D, bool DIRECT>
 static int launch_pair(const AttnArgs& a, int grid, const pr::Maps& maps, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(pr::attn_pair_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(pr::attn_pair_kernel<D, DIRECT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)pr::Cfg<D>::SMEM_BYTES);
     if (e != cudaSuccess) return fail(USV_ERR_CUDA, "sparse_attn: smem attribute: %s", cudaGetErrorString(e));
     // The roles redistribute the registers the CTA is launched with; a build whose launch count
     // fell below what they ask for in total would leave the softmax warps waiting for registers
     // that never come.  Refuse to launch such a build.
     cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, pr::attn_pair_kernel<D>);
+    e = cudaFuncGetAttributes(&fa, pr::attn_pair_kernel<D, DIRECT>);
     if (e != cudaSuccess) return fail(USV_ERR_CUDA, "sparse_attn: kernel attributes: %s", cudaGetErrorString(e));
     if (fa.numRegs * (pr::NTHREADS / 32) < 16 * pr::REG_SOFT + 4 * pr::REG_EPI + 4 * pr::REG_SERVICE)
         return fail(USV_ERR_UNSUPPORTED, "sparse_attn: kernel built with %d registers per thread, the roles need %d per lane",
                     fa.numRegs, 16 * pr::REG_SOFT + 4 * pr::REG_EPI + 4 * pr::REG_SERVICE);
-    launch_dep(pr::attn_pair_kernel<D>, dim3(grid), dim3(pr::NTHREADS), pr::Cfg<D>::SMEM_BYTES, st, a, maps);
+    launch_dep(pr::attn_pair_kernel<D, DIRECT>, dim3(grid), dim3(pr::NTHREADS), pr::Cfg<D>::SMEM_BYTES, st, a, maps);
     USV_CHECK_LAUNCH("attn_pair_kernel");
     return USV_OK;
 }
@@ -785,7 +848,8 @@ int launch_attn_pair(const AttnArgs& a, int d, cudaStream_t st) {
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
         return fail(USV_ERR_CUDA, "sparse_attn: cannot query the SM count");
     const int grid = (int)(items < sms ? items : sms);   // one persistent CTA per SM
-    return d == 64 ? launch_pair<64>(a, grid, maps, st) : launch_pair<128>(a, grid, maps, st);
+    if (a.pairs == nullptr) return d == 64 ? launch_pair<64, true>(a, grid, maps, st) : launch_pair<128, true>(a, grid, maps, st);
+    return d == 64 ? launch_pair<64, false>(a, grid, maps, st) : launch_pair<128, false>(a, grid, maps, st);
 }
 
 }  // namespace usv

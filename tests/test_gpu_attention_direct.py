@@ -1,0 +1,48 @@
+"""Small attention calls, which run without a pairing plan, on either side of their limits (kept key blocks,
+1024 blocks, lists of 256): odd and single blocks, holes, blocks without keys, rows handed to the exact
+kernel, several items a CTA.  Reference: the mma.sync kernel, which computes query blocks one by one; both
+round the weights to bf16 (white-noise V: 1.4e-3 each against fp64)."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("B,H,NB,kph,cut", [
+    (1, 1, 1, [1], 13), (1, 2, 2, [2, 1], 0), (1, 1, 5, [5], 63), (2, 3, 33, [33, 9, 1], 7), (1, 9, 111, [10] * 9, 0),
+    (1, 9, 112, [10] * 9, 1), (1, 1, 1024, [9], 0), (1, 1, 1025, [9], 0), (1, 1, 38, [33], 5)])
+def test_small_calls(d, B, H, NB, kph, cut):
+    import paper_2512_05754_b200 as usv
+    N, kmax = 64 * NB - cut, max(kph)
+    g = torch.Generator(device=DEV).manual_seed(NB + d)
+    q, k, v = (torch.randn(B, H, N, d, generator=g, device=DEV).to(torch.bfloat16) for _ in range(3))
+    rng = np.random.default_rng(NB)
+    sel = np.full((B, H, NB, kmax), -1, dtype=np.int32)
+    for b in range(B):
+        for h in range(H):
+            for i in range(NB):
+                sel[b, h, i, :kph[h]] = np.sort(rng.choice(NB, size=kph[h], replace=False))
+            if NB > 4:
+                sel[b, h, 2, kph[h] // 2] = -1        # a hole
+                sel[b, h, 3] = -1                     # no keys, its partner has some
+    empty = 0
+    if NB > 30:
+        sel[0, 0, 10:12] = -1                         # a whole item without keys
+        empty = 2
+        k[0, 0, 64 * 7:64 * 8] *= 60                  # logits far above the first block's: the exact kernel's rows
+    sel = torch.from_numpy(sel).to(DEV)
+    o, o32, lse = usv.sparse_attn_fwd(q, k, v, sel, kph, return_f32=True, return_lse=True, out_f32=torch.full((B, H, N, d), 7e9, device=DEV))
+    torch.cuda.synchronize()
+    assert usv.workspace_status() == 0
+    again = usv.sparse_attn_fallbacks()
+    _, e32, elxe = usv.sparse_attn_fwd(q, k, v, sel, kph, return_f32=True, return_lse=True, impl=1)
+    assert ((o32 - e32).double().norm() / e32.double().norm()).item() <= 3e-3
+    assert (o32 - e32).abs().max().item() <= 2e-2 and (lse - elxe).abs().max().item() <= 2e-3
+    assert (o.float() - o32).abs().max().item() <= 2.0 ** -8 * o32.abs().max().item()
+    if NB > 4 and not (d == 64 and kmax <= 8 and B * H * NB <= 384):   # (those run on the mma.sync kernel anyway)
+        assert again >= B * H                         # the blocks without keys beside a partner that has some
+    if empty:
+        assert (o[0, 0, 640:768] == 0).all() and again < B * H * NB
