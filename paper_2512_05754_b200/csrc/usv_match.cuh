@@ -88,8 +88,9 @@ struct MatchTcArgs {
     const int32_t* src_idx;          // [nA] source tokens, ascending
     uint16_t* a_h;                   // fp16 bits [B][nA_pad][dm]: sources by rank, zero-padded
     uint16_t* b_h;                   // fp16 bits [B][nB_pad][dm]: destinations by ordinal, zero-padded
-    float* cand_v;                   // [B][nA][2][8] largest approximate cosines per source and tile parity, descending
-    int* cand_i;                     // [B][nA][2][8] their destination ordinals
+    int parts;                       // 1, 2 or 4 CTAs share the destinations of 128 sources
+    float* cand_v;                   // [B][nA][parts][2][8] largest approximate cosines per source, part and tile parity, descending
+    int* cand_i;                     // [B][nA][parts][2][8] their destination ordinals
     int* exact_list;                 // sources (b * nA + rank) that need the fp32 scan of all destinations
     int* exact_count;
     int* exact_done;                 // one slot per list entry: chunks of the scan that are finished

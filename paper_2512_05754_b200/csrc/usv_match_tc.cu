@@ -105,8 +105,10 @@ match_tc_kernel(const MatchTcArgs m, const __grid_constant__ Maps maps) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b = blockIdx.y;
     const int a0 = blockIdx.x * 128;
-    const int T = m.nB_pad / 128;   // destination tiles, walked in the same order by every CTA (walking them
-                                    // in rotated orders, so that the CTAs ask for different L2 lines, was slower)
+    // destination tiles [t_lo, t_lo + T), walked in the same order by every CTA (walking them in rotated
+    // orders, so that the CTAs ask for different L2 lines, was slower)
+    const int t_all = m.nB_pad / 128, t_per = (t_all + m.parts - 1) / m.parts;
+    const int t_lo = min(t_all, (int)blockIdx.z * t_per), T = min(t_per, t_all - t_lo);
 
     if (threadIdx.x == 0) {
         mbar_init(bar(B_AFULL), 4);
@@ -137,7 +139,7 @@ match_tc_kernel(const MatchTcArgs m, const __grid_constant__ Maps maps) {
 
     if (warp == W_PROD) {
         // ===== TMA producer: destination rows =====
-        const int row0 = b * m.nB_pad;
+        const int row0 = b * m.nB_pad + t_lo * 128;
         for (int t = 0; t < T; ++t) {
             const int s = t % STAGES;
             const uint32_t ph = (t / STAGES) & 1;
@@ -243,7 +245,7 @@ match_tc_kernel(const MatchTcArgs m, const __grid_constant__ Maps maps) {
             const int buf = t % NBUF;
             if (!mbar_wait_spin(bar(B_DFULL + t % (2 * NBUF)), (t / (2 * NBUF)) & 1, s_abort, m.status, 0x100000)) { ok = false; break; }
             fence_after();
-            const int nvalid = m.p.nB - t * 128;   // destinations of this tile that exist
+            const int nvalid = m.p.nB - (t_lo + t) * 128;   // destinations of this tile that exist
             // the whole 128-column row in one go (four loads in flight, one wait), then the buffer goes back
             uint32_t sr[128];
 #pragma unroll
@@ -302,7 +304,7 @@ match_tc_kernel(const MatchTcArgs m, const __grid_constant__ Maps maps) {
                             mask &= mask - 1;
                             const float v = scr[j * 256];
                             if (v >= fmaxf(vmax, floor_v) - 2.0f * EPS && v > vlast) {
-                                const int idx = t * 128 + ch * 32 + j;
+                                const int idx = (t_lo + t) * 128 + ch * 32 + j;
                                 // descending cosine, then ascending destination: the entries the
                                 // new one beats move down one place, the last one drops out
                                 bool placed = false;
@@ -325,7 +327,7 @@ match_tc_kernel(const MatchTcArgs m, const __grid_constant__ Maps maps) {
             }
         }
         if (ok && a < m.nA) {
-            const int64_t g4 = (((int64_t)b * m.nA + a) * 2 + eg) * NCAND;
+            const int64_t g4 = ((((int64_t)b * m.nA + a) * m.parts + blockIdx.z) * 2 + eg) * NCAND;
 #pragma unroll
             for (int c = 0; c < NCAND; ++c) {
                 m.cand_v[g4 + c] = cval[c];
@@ -370,23 +372,36 @@ __device__ __forceinline__ float lane_cosine64(const float* __restrict__ x, cons
 // One warp per source: the candidates inside the window (approximate cosine >= max - 2 EPS) are
 // re-evaluated in fp32; the largest wins, equal values go to the lowest destination.  A source whose
 // last kept candidate is still inside the window may have more destinations in it than were kept: it is
-// appended to the list of the exact scan.  Lane c holds candidate c of the two lists (even and odd
-// destination tiles), each complete for its tiles unless its last entry is still inside the window.
+// appended to the list of the exact scan.  Lane c holds candidates c and c + 32 of the two lists per part
+// (even and odd destination tiles), each complete for its tiles unless its last entry is still inside the
+// window.
 template <int DM>
 __global__ void __launch_bounds__(256)
 recheck_kernel(const float* __restrict__ mhat, MatchTcArgs m) {
     dep_sync();
-    static_assert(2 * NCAND <= 32, "one lane per candidate");
+    static_assert(NCAND == 8, "four lists a warp");
     const int64_t gw = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (gw >= (int64_t)m.B * m.nA) return;
     const int b = (int)(gw / m.nA), a = (int)(gw % m.nA);
     const int src = m.src_idx[a];
-    const float v = lane < 2 * NCAND ? m.cand_v[gw * 2 * NCAND + lane] : -INFINITY;
-    const int id = lane < 2 * NCAND ? m.cand_i[gw * 2 * NCAND + lane] : 0x7fffffff;
-    const float window = fmaxf(__shfl_sync(0xffffffffu, v, 0), __shfl_sync(0xffffffffu, v, NCAND)) - 2.0f * EPS;
-    unsigned in = __ballot_sync(0xffffffffu, v >= window);   // (never true for -inf entries)
-    if (in & ((1u << (NCAND - 1)) | (1u << (2 * NCAND - 1)))) {
+    const int total = m.parts * 2 * NCAND;
+    float v[2];
+    int id[2];
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+        const int c = g * 32 + lane;
+        v[g] = c < total ? m.cand_v[gw * total + c] : -INFINITY;
+        id[g] = c < total ? m.cand_i[gw * total + c] : 0x7fffffff;
+    }
+    float top = fmaxf(v[0], v[1]);
+#pragma unroll
+    for (int o = NCAND; o < 32; o <<= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+    const float window = __shfl_sync(0xffffffffu, top, 0) - 2.0f * EPS;   // (a list's first entry is its largest)
+    unsigned in[2];
+#pragma unroll
+    for (int g = 0; g < 2; ++g) in[g] = __ballot_sync(0xffffffffu, v[g] >= window);   // (never true for -inf entries)
+    if ((in[0] | in[1]) & 0x80808080u) {
         if (lane == 0) {
             const int w = atomicAdd(m.exact_count, 1);
             m.exact_list[w] = (int)gw;
@@ -401,19 +416,23 @@ recheck_kernel(const float* __restrict__ mhat, MatchTcArgs m) {
     int bj = 0x7fffffff;
     if (DM == 128) {
         const Floats<4> x = *reinterpret_cast<const Floats<4>*>(X + lane * 4);
-        while (in) {
-            const int j = __shfl_sync(0xffffffffu, id, __ffs(in) - 1);
-            in &= in - 1;
-            const float c = warp_cosine(x, *reinterpret_cast<const Floats<4>*>(M + (int64_t)m.p.dst_token(j) * DM + lane * 4));
-            if (c > best || (c == best && j < bj)) { best = c; bj = j; }
-        }
-    } else {
-        if ((in >> lane) & 1u) {
-            best = lane_cosine64(X, M + (int64_t)m.p.dst_token(id) * DM);
-            bj = id;
-        }
 #pragma unroll
-        for (int o = NCAND; o > 0; o >>= 1) {
+        for (int g = 0; g < 2; ++g)
+            while (in[g]) {
+                const int j = __shfl_sync(0xffffffffu, id[g], __ffs(in[g]) - 1);
+                in[g] &= in[g] - 1;
+                const float c = warp_cosine(x, *reinterpret_cast<const Floats<4>*>(M + (int64_t)m.p.dst_token(j) * DM + lane * 4));
+                if (c > best || (c == best && j < bj)) { best = c; bj = j; }
+            }
+    } else {
+#pragma unroll
+        for (int g = 0; g < 2; ++g)
+            if ((in[g] >> lane) & 1u) {
+                const float c = lane_cosine64(X, M + (int64_t)m.p.dst_token(id[g]) * DM);
+                if (c > best || (c == best && id[g] < bj)) { best = c; bj = id[g]; }
+            }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
             const float ob = __shfl_xor_sync(0xffffffffu, best, o);
             const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
             if (ob > best || (ob == best && oj < bj)) { best = ob; bj = oj; }
@@ -520,7 +539,26 @@ static int make_rows_map(CUtensorMap* map, const void* ptr, int64_t rows, int DM
 static inline int pad128(int n) { return (n + 127) / 128 * 128; }
 
 static size_t rows_bytes(int B, int N, int dm) { return align_up((size_t)B * ((size_t)N + 256) * dm * sizeof(uint16_t), 256); }
-static size_t cand_bytes(int B, int N) { return align_up((size_t)B * N * 2 * mt::NCAND * sizeof(float), 256); }
+// several parts for up to PARTS_MAX_SOURCES sources only
+constexpr int64_t PARTS_MAX_SOURCES = 32768;
+static size_t cand_bytes(int B, int N) {
+    const int64_t n = (int64_t)B * N, few = n < PARTS_MAX_SOURCES ? n : PARTS_MAX_SOURCES;
+    return align_up((size_t)(n > 4 * few ? n : 4 * few) * 2 * mt::NCAND * sizeof(float), 256);
+}
+// CTAs that share the destinations of 128 sources: one CTA an SM is resident, its start takes as long as
+// eight destination tiles (sixteen gives the same times).  Whole merges, us, one part / as chosen: 4680
+// tokens 59.7 / 50.5, 9600 55.3 / 50.1, 12 000 57.7 / 53.3, 28 101 (162 CTAs) 145.5 / 137, 39 000 (153 CTAs)
+// 196 / 178.
+static int match_parts(int B, int nA, int nB) {
+    if ((int64_t)B * nA > PARTS_MAX_SOURCES) return 1;
+    const int ctas = B * ceil_div(nA, 128), tiles = ceil_div(nB, 128);
+    int best = 1, least = 0;
+    for (int parts = 1; parts <= 4 && parts <= tiles; parts *= 2) {
+        const int time = ceil_div(ctas * parts, 148) * (8 + ceil_div(tiles, parts));
+        if (parts == 1 || time < least) { best = parts; least = time; }
+    }
+    return best;
+}
 static size_t list_bytes(int B, int N) { return align_up((size_t)B * N * sizeof(int), 256); }
 
 size_t match_tc_bytes(int B, int N, int dm) {
@@ -533,6 +571,7 @@ void match_tc_args(MatchTcArgs& m, int dm, const int32_t* src_idx, int32_t* jsta
     const int B = m.B, N = m.N;
     m.nA_pad = pad128(m.nA); m.nB_pad = pad128(m.p.nB);
     m.src_idx = src_idx; m.jstar_s = jstar_s; m.u_s = u_s; m.status = status;
+    m.parts = match_parts(B, m.nA, m.p.nB);
     char* at = static_cast<char*>(mem);
     auto take = [&](size_t bytes) { char* p = at; at += bytes; return p; };
     m.a_h = reinterpret_cast<uint16_t*>(take(rows_bytes(B, N, dm)));
@@ -552,7 +591,7 @@ static int launch_match(const float* mhat, const MatchTcArgs& m, cudaStream_t st
     if ((rc = mt::make_rows_map(&maps.b_h, m.b_h, (int64_t)m.B * m.nB_pad, dm, "b_h")) != USV_OK) return rc;
     cudaError_t e = cudaFuncSetAttribute(mt::match_tc_kernel<dm>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mt::SMEM_BYTES<dm>);
     if (e != cudaSuccess) return fail(USV_ERR_CUDA, "token_merge: smem attribute: %s", cudaGetErrorString(e));
-    dim3 grid(m.nA_pad / 128, m.B);
+    dim3 grid(m.nA_pad / 128, m.B, m.parts);
     launch_dep(mt::match_tc_kernel<dm>, dim3(grid), dim3(352), mt::SMEM_BYTES<dm>, st, m, maps);
     USV_CHECK_LAUNCH("match_tc_kernel");
     const int64_t srcs = (int64_t)m.B * m.nA;
