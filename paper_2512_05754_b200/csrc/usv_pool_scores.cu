@@ -247,10 +247,12 @@ static int64_t small_tiles(int BH, int NBq, int NBk) { return (int64_t)BH * ceil
 extern "C" size_t usv_block_scores_workspace(int B, int H, int Nq, int Nk, int d) {
     if (B <= 0 || H <= 0 || Nq <= 0 || Nk <= 0 || d <= 0) return 0;
     const size_t nbq = usv::ceil_div(Nq, USV_BLOCK), nbk = usv::ceil_div(Nk, USV_BLOCK);
-    // header, pooled means of q and k, the bf16 planes of the tensor-core scores kernel
+    // header, pooled means of q and k, the bf16 planes of the tensor-core scores kernel (small calls at d = 64
+    // never had them, and do not run it)
+    const bool planes = d == 128 || (d == 64 && usv::small_tiles(B * H, (int)nbq, (int)nbk) > usv::SMALL_TILES);
     return usv::WS_HEADER + usv::align_up((size_t)B * H * nbq * d * sizeof(float), 256) +
            usv::align_up((size_t)B * H * nbk * d * sizeof(float), 256) +
-           (d == 64 || d == 128 ? usv::scores_tc_bytes(B * H, (int)nbq, (int)nbk, d) : 0);
+           (planes ? usv::scores_tc_bytes(B * H, (int)nbq, (int)nbk, d) : 0);
 }
 
 extern "C" int usv_block_scores(int B, int H, int Nq, int Nk, int d, const void* q,
