@@ -42,7 +42,7 @@ struct AttnArgs {
 int launch_attn_mma(const AttnArgs& a, int d, cudaStream_t st);
 bool attn_pair_supported(const AttnArgs& a, int d);
 // whether the call is too small for a pairing plan: a.pairs stays NULL, and fallback_list takes flags
-bool attn_pair_direct(const AttnArgs& a);
+bool attn_pair_direct(const AttnArgs& a, int d);
 int launch_attn_pair(const AttnArgs& a, int d, cudaStream_t st);
 // fused unmerge: copies the query blocks the exact kernel recomputed (into o) to their original tokens in y
 int launch_scatter_fallbacks(const AttnArgs& a, int d, cudaStream_t st);

@@ -99,7 +99,7 @@ static int sparse_attn_impl(int B, int H, int N, int d, const void* q, const usv
     const bool small = d == 64 && kmx <= 8 && (int64_t)B * H * NB <= 384;
     if (impl == 0 && !small && attn_pair_supported(a, d)) {
         int rc2;
-        if (attn_pair_direct(a)) {
+        if (attn_pair_direct(a, d)) {
             if ((rc2 = launch_attn_pair(a, d, st)) != USV_OK) return rc2;
             a.work_flags = reinterpret_cast<const uint16_t*>(a.fallback_list);
             return launch_attn_mma(a, d, st);

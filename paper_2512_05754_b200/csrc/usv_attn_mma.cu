@@ -235,7 +235,14 @@ __global__ void __launch_bounds__(128) attn_mma_kernel(const AttnArgs a) {
             if (threadIdx.x == 0) s_count = 0;
             __syncthreads();
             int count = 0;
-            for (int i = threadIdx.x; i < blocks; i += 128) count += a.work_flags[i] != 0;
+#pragma unroll 4
+            for (int i = threadIdx.x; i < blocks / 8; i += 128) {
+                const uint4 f = reinterpret_cast<const uint4*>(a.work_flags)[i];
+                const uint32_t w[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) count += ((w[e] & 0xffffu) != 0) + ((w[e] >> 16) != 0);
+            }
+            if (threadIdx.x < blocks % 8) count += a.work_flags[blocks / 8 * 8 + threadIdx.x] != 0;
             if (count) atomicAdd(&s_count, count);
             __syncthreads();
             if (threadIdx.x == 0) *a.fallback_count = s_count;

@@ -805,15 +805,20 @@ bool attn_pair_supported(const AttnArgs& a, int d) {
 // blocks kept: D = 128, 2.7 k 29.1 / 26.4, 3.5 k 32.3 / 26.7, 5 k (two heads of 160 blocks) 42.2 / 35.2, 7 k
 // 40.8 / 39.5, 12 k 51.4 / 50.8, 14 k 55.5 / 61.0, 24 k 76 / 80; D = 64, 4.6 k 30.3 / 25.4, 14 k 45.8 / 47.4,
 // 38 k 81 / 93.  (Beyond 1024 blocks or lists of 256 the scout's registers and ring slots do not hold a union.)
-bool attn_pair_direct(const AttnArgs& a) {
+// With short lists the scout's work per item counts, which bounds the number of blocks too, lower where a
+// tile takes longer: D = 128, 3 heads x 220 blocks, keep 11 45.1 / 40.7, 24 x 72, keep 4 47.2 / 48.3, 12 x 120,
+// keep 6 48.3 / 47.2, 16 x 120, keep 3 48.0 / 51.4, 24 x 317, keep 1 114 / 140; D = 64, 24 x 72, keep 4 38.8 / 35.4.
+bool attn_pair_direct(const AttnArgs& a, int d) {
     constexpr int64_t DIRECT_WORK = 10000;
+    const int64_t most_blocks = d == 64 ? 1800 : 1000;
     int64_t kept = 0;
     int most = 0;
     for (int h = 0; h < a.H; ++h) {
         kept += a.k_per_head[h];
         most = a.k_per_head[h] > most ? a.k_per_head[h] : most;
     }
-    return a.y == nullptr && a.NB <= 1024 && 2 * most <= pr::LCAP && (int64_t)a.B * a.NB * kept <= DIRECT_WORK;
+    return a.y == nullptr && a.NB <= 1024 && 2 * most <= pr::LCAP && (int64_t)a.B * a.H * a.NB <= most_blocks &&
+           (int64_t)a.B * a.NB * kept <= DIRECT_WORK;
 }
 
 template <int D, bool DIRECT>

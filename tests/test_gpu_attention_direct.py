@@ -1,6 +1,6 @@
 """Small attention calls, which run without a pairing plan, on either side of their limits (kept key blocks,
-1024 blocks, lists of 256): odd and single blocks, holes, blocks without keys, rows handed to the exact
-kernel, several items a CTA.  Reference: the mma.sync kernel, which computes query blocks one by one; both
+blocks in all and in a sequence, lists of 256): odd and single blocks, holes, blocks without keys, rows handed
+to the exact kernel, several items a CTA.  Reference: the mma.sync kernel, which computes query blocks one by one; both
 round the weights to bf16 (white-noise V: 1.4e-3 each against fp64)."""
 import numpy as np
 import pytest
@@ -13,7 +13,8 @@ DEV = "cuda:0"
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("B,H,NB,kph,cut", [
     (1, 1, 1, [1], 13), (1, 2, 2, [2, 1], 0), (1, 1, 5, [5], 63), (2, 3, 33, [33, 9, 1], 7), (1, 9, 111, [10] * 9, 0),
-    (1, 9, 112, [10] * 9, 1), (1, 1, 1024, [9], 0), (1, 1, 1025, [9], 0), (1, 1, 38, [33], 5)])
+    (1, 9, 112, [10] * 9, 1), (1, 1, 1024, [9], 0), (1, 1, 1025, [9], 0), (1, 1, 38, [33], 5), (1, 2, 500, [1] * 2, 17),
+    (1, 2, 501, [1] * 2, 0), (1, 2, 900, [2] * 2, 0), (1, 2, 901, [2] * 2, 0)])
 def test_small_calls(d, B, H, NB, kph, cut):
     import paper_2512_05754_b200 as usv
     N, kmax = 64 * NB - cut, max(kph)
@@ -26,7 +27,8 @@ def test_small_calls(d, B, H, NB, kph, cut):
             for i in range(NB):
                 sel[b, h, i, :kph[h]] = np.sort(rng.choice(NB, size=kph[h], replace=False))
             if NB > 4:
-                sel[b, h, 2, kph[h] // 2] = -1        # a hole
+                if kph[h] > 1:
+                    sel[b, h, 2, kph[h] // 2] = -1    # a hole
                 sel[b, h, 3] = -1                     # no keys, its partner has some
     empty = 0
     if NB > 30:
