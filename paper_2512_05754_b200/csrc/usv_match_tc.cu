@@ -19,13 +19,13 @@
 //
 //   (usv_merge.cu)      desc_kernel writes the fp16 rows, sources (by rank) and destinations (by
 //                       ordinal) apart, zero-padded to multiples of 128 rows
-//   match_tc_kernel     one CTA per 128 sources: their rows sit in TMEM as the A operand, the
+//   match_tc_kernel     one CTA per 128 sources and part of the destinations: the sources sit in TMEM as the A operand, the
 //                       destination rows stream through shared memory (TMA, 4 stages); warp 8 =
 //                       TMA producer, warps 9-10 = MMA issuers on alternate tiles, warps 0-3 / 4-7 =
 //                       two groups of one thread per source row, reading the 128 x 128 tiles of even /
 //                       odd index out of TMEM (three accumulator tiles in rotation) and keeping the eight best (value,
 //                       destination) inside the window of their running maximum, ascending destinations
-//   recheck_kernel      per source: the candidates inside the window in fp32 -> j*, u; sources
+//   recheck_kernel      per source: the candidates of all parts inside the window in fp32 -> j*, u; sources
 //                       with a full window are listed
 //   match_exact_kernel  fp32 scan of every destination for the listed sources (normally none)
 #include <cuda_fp16.h>
