@@ -125,6 +125,11 @@ __device__ __forceinline__ uint32_t float_key(float f) {
 // a NaN that an addition returns the compiler may assume what it likes, here one way and there another.
 __device__ __forceinline__ uint32_t float_key_any(float f) { return f == f ? float_key(f) : 0x7fffffffu; }
 
+// The warp's index, in a form that the compiler knows to be the same in all its lanes: the branch into a warp's role is
+// then uniform to it, and loop counters, addresses and descriptors behind it stay in uniform registers, which the
+// issuing warps of the tcgen05 kernels would otherwise fill for every instruction from one lane's.
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+
 __device__ __forceinline__ int warp_incl_scan(int v) {
     const int lane = threadIdx.x & 31;
 #pragma unroll

@@ -111,7 +111,7 @@ marginal_tc_kernel(const MargArgs a, int w0, const __grid_constant__ Maps maps) 
     uint32_t* s_bits = reinterpret_cast<uint32_t*>(sm + F::SM_K);
     uint16_t* s_list = reinterpret_cast<uint16_t*>(sm + F::SM_LIST);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int N = a.N, NB = a.NB;
     const int NP = (NB + PER - 1) / PER, words = (min(NB - w0, WINDOW) + 31) >> 5;   // key blocks [w0, w0 + 32 words)
     const int I = PER * (blockIdx.x % NP);

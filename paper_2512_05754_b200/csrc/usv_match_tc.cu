@@ -102,7 +102,7 @@ match_tc_kernel(const MatchTcArgs m, const __grid_constant__ Maps maps) {
     auto bar = [&](int i) { return base + SM_BAR + 8u * i; };
     volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(sm + SM_MISC);
     volatile int* s_abort = reinterpret_cast<volatile int*>(sm + SM_MISC + 4);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int b = blockIdx.y;
     const int a0 = blockIdx.x * 128;
     // destination tiles [t_lo, t_lo + T), walked in the same order by every CTA (walking them in rotated

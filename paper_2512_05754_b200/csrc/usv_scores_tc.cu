@@ -79,7 +79,7 @@ scores_tc_kernel(const Args m, const __grid_constant__ Maps maps) {
     auto bar = [&](int i) { return base + F::SM_BAR + 8u * i; };
     volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(sm + F::SM_MISC);
     volatile int* s_abort = reinterpret_cast<volatile int*>(sm + F::SM_MISC + 4);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int bh = blockIdx.y;
     const int i0 = blockIdx.x * 128;
     // key-block tiles [t_lo, t_hi) of this CTA: the column range is split over blockIdx.z so that
