@@ -292,6 +292,14 @@ int usv_attn_entropy(int B, int H, int N, int d, const void* q, const usv_stride
                      const int32_t* k_per_head, int kmax, const float* lse, float scale,
                      float* key_marginal, float* entropy, void* ws, void* stream);
 
+/* The same with scratch memory, with which large calls are faster: query blocks whose lists overlap are paired first.
+ * ws: as above, ws_bytes of it; with fewer than usv_attn_entropy_workspace() bytes (or NULL) the call is usv_attn_entropy. */
+size_t usv_attn_entropy_workspace(int B, int H, int N, int kmax);
+int usv_attn_entropy_ws(int B, int H, int N, int d, const void* q, const usv_strides* sq,
+                        const void* k, const usv_strides* sk, const int32_t* sel,
+                        const int32_t* k_per_head, int kmax, const float* lse, float scale,
+                        float* key_marginal, float* entropy, void* ws, size_t ws_bytes, void* stream);
+
 /* Entropy-aware allocation over the L layers of one step (Eq. 18-19), plain host arithmetic:
  *     w_l = (1 - h_l)^gamma ,   rho_l = clip(rho_min, rho_max, rho_bar * w_l / mean_l'(w_l')).
  * entropy, rho: HOST arrays of L floats; gamma >= 1; every h_l in [0,1].  If every w_l is zero

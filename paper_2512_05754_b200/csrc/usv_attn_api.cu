@@ -106,7 +106,7 @@ static int sparse_attn_impl(int B, int H, int N, int d, const void* q, const usv
             a.work_flags = reinterpret_cast<const uint16_t*>(a.fallback_list);
             return launch_attn_mma(a, d, st);
         }
-        if ((rc2 = launch_pair_plan(a, plan_mem, st)) != USV_OK) return rc2;
+        if ((rc2 = launch_pair_plan(a, plan_mem, false, st)) != USV_OK) return rc2;
         if ((rc2 = launch_attn_pair(a, d, st)) != USV_OK) return rc2;
         // exact recomputation of the (normally zero) query blocks the fast kernel reported
         a.work_list = a.fallback_list;

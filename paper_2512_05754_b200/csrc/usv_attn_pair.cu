@@ -62,7 +62,7 @@ constexpr int VSTAGES = 3;                      // V tile stages
 constexpr int SBUF = 3;                         // S/P buffers in TMEM
 constexpr int NSLOT = 4;                        // item ring
 constexpr int LCAP = 512;                       // list entries a ring slot holds (longer lists are read from global memory)
-constexpr int MAX_NB = 4096;                    // key blocks per sequence this kernel covers
+constexpr int MAX_NB = PLAN_MAX_NB;             // key blocks per sequence this kernel covers
 constexpr uint32_t ITEM_BYTES = 64 + LCAP * 4;
 
 // What depends on the head width.  At D = 128 a tile's MMAs (1024 cycles) and its traffic through

@@ -42,6 +42,7 @@ struct Order {
     uint8_t* taken;            // [B*H][NB] written by the first pass: 1 = paired
     int* count;                // [B*H] pairs written so far (starts at zero)
     int pass;                  // 0: one pass in index order (the rest unused); 1, 2: first and second of two
+    int as_listed;             // lists of as many entries as there are key blocks are read too (the marginal's may have holes)
 };
 
 __device__ __forceinline__ uint32_t mix12(uint32_t x, uint32_t a, uint32_t b) {   // a bijection of 0 .. 4095
@@ -179,7 +180,7 @@ pair_plan_kernel(const AttnArgs a, int2* __restrict__ pairs, int* __restrict__ l
     // its CTAs, already resident, would leave room for one CTA of this kernel an SM instead of two (D = 64, 12 heads x 256
     // blocks, keep 26: 134 us a call, 138 with the wait behind the signal).
     dep_wait();
-    const bool full = kh >= NB;   // every list is the full set: no overlaps to compute
+    const bool full = kh >= NB && !ord.as_listed;   // every list is the full set: no overlaps to compute
     if (warp == 0 && !full) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(t5::smem_u32(&s_tmem)), "r"(128u) : "memory");
@@ -199,7 +200,7 @@ pair_plan_kernel(const AttnArgs a, int2* __restrict__ pairs, int* __restrict__ l
         if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(128u) : "memory");
     };
     // the words behind the sticky status word (fallback count, work counter, ...) start at zero
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < (WS_HEADER - 4) / 4) a.status[1 + threadIdx.x] = 0u;
+    if (a.work_counter != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < (WS_HEADER - 4) / 4) a.status[1 + threadIdx.x] = 0u;
 
     if (full) {
         if (ord.pass == 2) return;   // (done by the first pass)
@@ -497,7 +498,7 @@ struct PlanLayout {
 
 size_t pair_plan_bytes(int B, int H, int NB, const int32_t* k_per_head) { return PlanLayout(B, H, NB, k_per_head).total; }
 
-int launch_pair_plan(AttnArgs& a, void* mem, cudaStream_t st) {
+int launch_pair_plan(AttnArgs& a, void* mem, bool as_listed, cudaStream_t st) {
     const int NP = (a.NB + 1) / 2, BH = a.B * a.H;
     char* base = static_cast<char*>(mem);
     const PlanLayout L(a.B, a.H, a.NB, a.k_per_head);
@@ -517,11 +518,11 @@ int launch_pair_plan(AttnArgs& a, void* mem, cudaStream_t st) {
     cudaError_t e = cudaFuncSetAttribute(plan::pair_plan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan::MOST_SMEM);
     if (e != cudaSuccess) return fail(USV_ERR_CUDA, "sparse_attn: plan smem attribute: %s", cudaGetErrorString(e));
     const dim3 grid((a.NB + plan::CH - 1) / plan::CH, BH);
-    plan::Order ord = {nullptr, nullptr, nullptr, 0};
+    plan::Order ord = {nullptr, nullptr, nullptr, 0, as_listed};
     if (plan::plan_ordered(a)) {
         uint32_t* keys = reinterpret_cast<uint32_t*>(base + L.keys);
         uint16_t* by_rank = reinterpret_cast<uint16_t*>(base + L.by_rank);
-        ord = {by_rank, reinterpret_cast<uint8_t*>(base + L.taken), reinterpret_cast<int*>(base + L.count), 1};
+        ord = {by_rank, reinterpret_cast<uint8_t*>(base + L.taken), reinterpret_cast<int*>(base + L.count), 1, as_listed};
         const int64_t rows = (int64_t)BH * a.NB;
         launch_dep_smem(plan::plan_keys_kernel, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, a, keys, ord.count);
         USV_CHECK_LAUNCH("plan_keys_kernel");

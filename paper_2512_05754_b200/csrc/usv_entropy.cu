@@ -40,10 +40,10 @@ __global__ void __launch_bounds__(1024) entropy_kernel(const float* __restrict__
 
 }  // namespace usv
 
-extern "C" int usv_attn_entropy(int B, int H, int N, int d, const void* q, const usv_strides* sq,
-                                const void* k, const usv_strides* sk, const int32_t* sel,
-                                const int32_t* k_per_head, int kmax, const float* lse, float scale,
-                                float* key_marginal, float* entropy, void* ws, void* stream) {
+static int attn_entropy_impl(int B, int H, int N, int d, const void* q, const usv_strides* sq,
+                             const void* k, const usv_strides* sk, const int32_t* sel,
+                             const int32_t* k_per_head, int kmax, const float* lse, float scale,
+                             float* key_marginal, float* entropy, void* ws, bool room, void* stream) {
     using namespace usv;
     if (B <= 0 || H <= 0 || N <= 0) return fail(USV_ERR_INVALID_ARG, "attn_entropy: B,H,N must be positive");
     if (d != 64 && d != 128) return fail(USV_ERR_UNSUPPORTED, "attn_entropy: d=%d (need 64 or 128)", d);
@@ -75,13 +75,40 @@ extern "C" int usv_attn_entropy(int B, int H, int N, int d, const void* q, const
     const float sc = scale == 0.f ? 1.0f / sqrtf((float)d) : scale;
     a.scale_log2 = sc * 1.4426950408889634f;
     a.inv_hn = 1.0f / ((float)H * (float)N);
+    a.pairs = nullptr;
+    a.lists = nullptr;
+    a.list_batch = 0;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e = cudaMemsetAsync(key_marginal, 0, (size_t)B * N * sizeof(float), st);
     if (e != cudaSuccess) return fail(USV_ERR_CUDA, "attn_entropy: memset: %s", cudaGetErrorString(e));
+    int sms;
+    if ((rc = sm_count(&sms)) != USV_OK) return rc;
+    if (room && marginal_planned(a, sms) && (rc = launch_marginal_plan(a, static_cast<char*>(ws) + WS_HEADER, st)) != USV_OK)
+        return rc;
     if ((rc = launch_marginal_tc(a, d, st)) != USV_OK) return rc;
     launch_dep_smem(entropy_kernel, dim3(B), dim3(1024), 0, st, key_marginal, N, entropy);
     USV_CHECK_LAUNCH("entropy_kernel");
     return USV_OK;
+}
+
+extern "C" int usv_attn_entropy(int B, int H, int N, int d, const void* q, const usv_strides* sq,
+                                const void* k, const usv_strides* sk, const int32_t* sel,
+                                const int32_t* k_per_head, int kmax, const float* lse, float scale,
+                                float* key_marginal, float* entropy, void* ws, void* stream) {
+    return attn_entropy_impl(B, H, N, d, q, sq, k, sk, sel, k_per_head, kmax, lse, scale, key_marginal, entropy, ws, false, stream);
+}
+
+extern "C" size_t usv_attn_entropy_workspace(int B, int H, int N, int kmax) {
+    if (B <= 0 || H <= 0 || N <= 0 || H > USV_MAX_HEADS) return usv::WS_HEADER;
+    return usv::WS_HEADER + usv::marginal_plan_bytes(B, H, usv::ceil_div(N, USV_BLOCK), kmax);
+}
+
+extern "C" int usv_attn_entropy_ws(int B, int H, int N, int d, const void* q, const usv_strides* sq,
+                                   const void* k, const usv_strides* sk, const int32_t* sel,
+                                   const int32_t* k_per_head, int kmax, const float* lse, float scale,
+                                   float* key_marginal, float* entropy, void* ws, size_t ws_bytes, void* stream) {
+    const bool room = ws != nullptr && ws_bytes >= usv_attn_entropy_workspace(B, H, N, kmax);
+    return attn_entropy_impl(B, H, N, d, q, sq, k, sk, sel, k_per_head, kmax, lse, scale, key_marginal, entropy, ws, room, stream);
 }
 
 extern "C" int usv_allocate_sparsity(int L, const float* entropy, float gamma, float rho_bar, float rho_min,

@@ -15,9 +15,18 @@ struct MargArgs {
     float scale_log2;     // softmax scale * log2(e)
     float inv_hn;         // 1 / (H N)
     int k_per_head[USV_MAX_HEADS];
+    // Pairs of query blocks and their union lists as usv_attn_plan.cu writes them; NULL: neighbours are paired.
+    const int2* pairs;
+    const int* lists;
+    int64_t list_batch, list_off[USV_MAX_HEADS];
 };
 
 // usv_entropy_tc.cu; marg must be zero.
 int launch_marginal_tc(const MargArgs& a, int d, cudaStream_t st);
+// whether a pairing plan pays for the call
+bool marginal_planned(const MargArgs& a, int sms);
+size_t marginal_plan_bytes(int B, int H, int NB, int kmax);
+// Enqueues the plan of the call in mem and points a to it.
+int launch_marginal_plan(MargArgs& a, void* mem, cudaStream_t st);
 
 }  // namespace usv

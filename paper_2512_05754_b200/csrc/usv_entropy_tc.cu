@@ -5,7 +5,8 @@
 //
 // with lse_i the log-sum-exp the attention forward wrote.  Only the logits are needed, and the
 // sum runs over the queries, so the product is taken transposed: one CTA per (b, h, two
-// consecutive query blocks; one in small calls) walks the union of the two lists two key blocks at a time and computes
+// consecutive query blocks, in large calls two with overlapping lists; one in small calls) walks the union of the two
+// lists two key blocks at a time and computes
 //
 //     S^T[128 keys x 128 queries] = K_tile . Q^T      tcgen05.mma, A = K tile in smem, B = Q in smem
 //
@@ -25,12 +26,14 @@
 // blocks of random keys, keep 52, D = 128: 607 -> 437, D = 64: 1324 -> 385; 8 x 1182, keep 60, D = 128: 924 -> 820,
 // D = 64: 2274 -> 690.
 //
-// The union is built as a list in shared memory: two bitmaps over the key blocks, compacted by one warp.
+// The union is built as a list in shared memory (two bitmaps over the key blocks, compacted by one warp), or copied from
+// the pairing plan of a large call.
 // CTAs that run at the same time start at different entries of it, those near their own query blocks:
 // their atomic adds would otherwise meet on the same keys.  A launch covers a window of 16 384 key blocks.
 // Two CTAs share an SM and fill each other's gaps.  Warp 8 is the TMA producer, warp 9 the MMA
 // issuer and TMEM owner.  All waits are bounded; a role that gives up raises the CTA's abort flag and
 // the others follow.
+#include "usv_attn.cuh"
 #include "usv_entropy.cuh"
 #include "usv_tcgen05.cuh"
 
@@ -44,6 +47,7 @@ constexpr int KT = 2 * USV_BLOCK;               // keys per tile = two key block
 constexpr int QT = 2 * USV_BLOCK;               // queries per CTA = two query blocks
 constexpr int NBUF = 2;                         // S^T buffers of 128 columns
 constexpr int WINDOW = 1 << 14;                 // key blocks a launch covers (16-bit list entries)
+constexpr int64_t PLAN_MIN_WORK = 500000;       // kept key blocks over all query blocks
 
 template <int D>
 struct Cfg {
@@ -92,8 +96,8 @@ __device__ __forceinline__ uint64_t weight2(int i, uint32_t a, uint32_t b, uint6
     return pack_f32x2(p0, p1);
 }
 
-// PER: query blocks a CTA
-template <int D, int PER>
+// PER: query blocks a CTA; PLANNED: which two, and their union, come from a pairing plan
+template <int D, int PER, bool PLANNED>
 __global__ void __launch_bounds__(NTHREADS, 2)
 marginal_tc_kernel(const MargArgs a, int w0, const __grid_constant__ Maps maps) {
     using F = Cfg<D>;
@@ -114,8 +118,6 @@ marginal_tc_kernel(const MargArgs a, int w0, const __grid_constant__ Maps maps) 
     const int warp = warp_index(), lane = threadIdx.x & 31;
     const int N = a.N, NB = a.NB;
     const int NP = (NB + PER - 1) / PER, words = (min(NB - w0, WINDOW) + 31) >> 5;   // key blocks [w0, w0 + 32 words)
-    const int I = PER * (blockIdx.x % NP);
-    const int last = min(I + PER, NB);   // query blocks [I, last)
     const int bh = blockIdx.x / NP;
     const int b = bh / a.H, h = bh % a.H;
     const int kh = a.k_per_head[h];
@@ -126,7 +128,7 @@ marginal_tc_kernel(const MargArgs a, int w0, const __grid_constant__ Maps maps) 
         if (i == 0) { *s_abort = 0; s_union[1] = 0; }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    for (int i = threadIdx.x; i < 2 * words; i += NTHREADS) s_bits[i] = 0;
+    for (int i = threadIdx.x; !PLANNED && i < 2 * words; i += NTHREADS) s_bits[i] = 0;
     if (warp == W_MMA) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(base + F::SM_MISC), "r"(TMEM_COLS) : "memory");
@@ -138,6 +140,10 @@ marginal_tc_kernel(const MargArgs a, int w0, const __grid_constant__ Maps maps) 
     dep_sync();
     const uint32_t tmem = *s_tmem;
 
+    // the CTA's query blocks, the second one -1 or NB where there is none
+    const int2 blk = PLANNED ? a.pairs[blockIdx.x] : make_int2(PER * (blockIdx.x % NP), PER * (blockIdx.x % NP) + 1);
+    const int I = blk.x, last = min(I + PER, NB);   // (without a plan the CTA has blocks [I, last))
+
     // ---- the query rows on their way, the lists as bitmaps, the log-sum-exps
     if (warp == W_TMA && elect_one()) {
         const int hq = a.sq.sh ? h : 0, bq = a.sq.sb ? b : 0;
@@ -146,9 +152,10 @@ marginal_tc_kernel(const MargArgs a, int w0, const __grid_constant__ Maps maps) 
         for (int hf = 0; hf < F::NH; ++hf)
 #pragma unroll
             for (int p = 0; p < PER; ++p)
-                tma_load_4d(base + F::SM_Q + hf * 16384 + p * 8192, &maps.q, bar(F::B_QFULL), hf * 64, (I + p) * USV_BLOCK, hq, bq);
+                tma_load_4d(base + F::SM_Q + hf * 16384 + p * 8192, &maps.q, bar(F::B_QFULL), hf * 64,
+                            (p == 0 ? I : (blk.y < 0 ? NB : blk.y)) * USV_BLOCK, hq, bq);   // (rows past the end: zeros)
     }
-    for (int i = threadIdx.x; i < PER * kh; i += NTHREADS) {
+    for (int i = threadIdx.x; !PLANNED && i < PER * kh; i += NTHREADS) {
         const int side = i >= kh;
         if (I + side >= last) continue;
         const int e = a.sel[((int64_t)bh * NB + I + side) * a.kmax + (i - side * kh)];
@@ -156,13 +163,26 @@ marginal_tc_kernel(const MargArgs a, int w0, const __grid_constant__ Maps maps) 
     }
     if (threadIdx.x < USV_BLOCK * PER) {
         // a query at or beyond N counts nothing
-        const int row = I * USV_BLOCK + threadIdx.x;
+        const int row = (threadIdx.x < USV_BLOCK ? I : blk.y) * USV_BLOCK + (threadIdx.x & (USV_BLOCK - 1));
         reinterpret_cast<float*>(sm + F::SM_LSE)[threadIdx.x] =
-            row < N ? -a.lse[(int64_t)bh * N + row] * 1.4426950408889634f : -INFINITY;
+            row >= 0 && row < N ? -a.lse[(int64_t)bh * N + row] * 1.4426950408889634f : -INFINITY;
+    }
+    if (PLANNED) {
+        const int* pl = a.lists + b * a.list_batch + a.list_off[h] + (int64_t)(blockIdx.x % NP) * list_stride(kh, NB);
+        const int n = __ldg(pl);
+        int before = 0;   // entries below the CTA's own block
+        for (int i = threadIdx.x; i < n; i += NTHREADS) {
+            const int e = __ldg(pl + 1 + i);
+            s_list[i] = (uint16_t)e;
+            before += (e >> 2) < I;
+        }
+        before = __reduce_add_sync(0xffffffffu, before);
+        if (lane == 0 && before) atomicAdd(const_cast<int*>(s_union + 1), before);
+        if (threadIdx.x == 0) s_union[0] = n;
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
-    if (warp == 0) {
+    if (!PLANNED && warp == 0) {
         int n = 0;
         for (int i0 = 0; i0 < words; i0 += 32) {
             const int i = i0 + lane;
@@ -180,7 +200,7 @@ marginal_tc_kernel(const MargArgs a, int w0, const __grid_constant__ Maps maps) 
         if (lane == 0) s_union[0] = n;
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the K stages go to the TMA
     }
-    __syncthreads();
+    if (!PLANNED) __syncthreads();
     const int nU = s_union[0], T = (nU + 1) >> 1;   // tiles of two key blocks
     const int first = s_union[1] < nU ? s_union[1] : 0;
     // n-th entry from `first` on, around the end; 0 (no side) behind the last one
@@ -289,7 +309,7 @@ marginal_tc_kernel(const MargArgs a, int w0, const __grid_constant__ Maps maps) 
     }
 }
 
-template <int D, int PER>
+template <int D, int PER, bool PLANNED>
 static int launch(const MargArgs& a, cudaStream_t st) {
     Maps maps;
     int rc;
@@ -301,11 +321,11 @@ static int launch(const MargArgs& a, cudaStream_t st) {
     const int widest = a.NB < WINDOW ? a.NB : WINDOW;
     const size_t smem = Cfg<D>::smem_bytes(widest < 2 * kmx ? widest : 2 * kmx);
     // (the limit is the function's, not the call's: always the most any call needs, for calls from several threads)
-    cudaError_t e = cudaFuncSetAttribute(marginal_tc_kernel<D, PER>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(marginal_tc_kernel<D, PER, PLANNED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)Cfg<D>::smem_bytes(WINDOW));
     if (e != cudaSuccess) return fail(USV_ERR_CUDA, "attn_entropy: smem attribute: %s", cudaGetErrorString(e));
     for (int w0 = 0; w0 < a.NB; w0 += WINDOW) {
-        launch_dep_smem(marginal_tc_kernel<D, PER>, dim3((unsigned)grid), dim3(NTHREADS), smem, st, a, w0, maps);
+        launch_dep_smem(marginal_tc_kernel<D, PER, PLANNED>, dim3((unsigned)grid), dim3(NTHREADS), smem, st, a, w0, maps);
         USV_CHECK_LAUNCH("marginal_tc_kernel");
     }
     return USV_OK;
@@ -313,9 +333,7 @@ static int launch(const MargArgs& a, cudaStream_t st) {
 
 }  // namespace et
 
-int launch_marginal_tc(const MargArgs& a, int d, cudaStream_t st) {
-    int rc, sms;
-    if ((rc = sm_count(&sms)) != USV_OK) return rc;
+static bool marginal_single(const MargArgs& a, int sms) {
     // One query block a CTA where all of them are resident together (two CTAs an SM): such a call takes as long as one walk
     // over a list, and a union is longer than a list.  So too, up to twice as many, where lists are long and hold so little
     // of the sequence that neighbours need not share much.  Marginal + entropy, us, two blocks a CTA / one, D = 128 (D = 64),
@@ -325,9 +343,54 @@ int launch_marginal_tc(const MargArgs& a, int d, cudaStream_t st) {
     int kmx = 0;
     for (int h = 0; h < a.H; ++h) kmx = a.k_per_head[h] > kmx ? a.k_per_head[h] : kmx;
     const int64_t blocks = (int64_t)a.B * a.H * a.NB;
-    const bool one = blocks <= 2 * sms || (blocks <= 4 * sms && kmx >= 16 && 4 * kmx <= a.NB);
-    if (d == 64) return one ? et::launch<64, 1>(a, st) : et::launch<64, 2>(a, st);
-    return one ? et::launch<128, 1>(a, st) : et::launch<128, 2>(a, st);
+    return blocks <= 2 * sms || (blocks <= 4 * sms && kmx >= 16 && 4 * kmx <= a.NB);
+}
+
+// The plan costs 8 to 20 us (40 where the blocks are ordered first) and takes a quarter of the tiles away: the union of two
+// paired lists is 1.28 to 1.35 times a list, that of neighbours in index 1.9 times.  Marginal + entropy of video inputs, us,
+// neighbours / paired: 12 heads x 122 blocks, keep 13 48 / 58; 12 x 317, keep 39 226 / 220; 12 x 512, keep 52 496 / 493;
+// 24 x 512 at D = 64 786 / 750; 40 x 1182, keep 60 5074 / 4405; 12 x 3023, keep 152 10 093 / 8139.  Long lists overlap
+// anyway: 12 x 512, keep 180 1573 / 1578; 16 x 317, keep 317, 80, 32 and 16 851 / 838.
+bool marginal_planned(const MargArgs& a, int sms) {
+    int64_t kept = 0;
+    int heads = 0;
+    for (int h = 0; h < a.H; ++h)
+        if (a.k_per_head[h] < a.NB) {
+            kept += a.k_per_head[h];
+            ++heads;
+        }
+    return a.NB <= PLAN_MAX_NB && !marginal_single(a, sms) && (int64_t)a.B * a.NB * kept >= et::PLAN_MIN_WORK &&
+           4 * kept <= (int64_t)heads * a.NB;
+}
+
+size_t marginal_plan_bytes(int B, int H, int NB, int kmax) {
+    int32_t kk[USV_MAX_HEADS];
+    for (int h = 0; h < H; ++h) kk[h] = kmax < 1 ? 1 : (kmax > NB ? NB : kmax);
+    return pair_plan_bytes(B, H, NB, kk);
+}
+
+int launch_marginal_plan(MargArgs& a, void* mem, cudaStream_t st) {
+    AttnArgs p = {};
+    p.sel = a.sel;
+    p.status = a.status;
+    p.B = a.B; p.H = a.H; p.N = a.N; p.NB = a.NB; p.kmax = a.kmax;
+    for (int h = 0; h < a.H; ++h) p.k_per_head[h] = a.k_per_head[h];
+    const int rc = launch_pair_plan(p, mem, true, st);
+    if (rc != USV_OK) return rc;
+    a.pairs = p.pairs;
+    a.lists = p.lists;
+    a.list_batch = p.list_batch;
+    for (int h = 0; h < a.H; ++h) a.list_off[h] = p.list_off[h];
+    return USV_OK;
+}
+
+int launch_marginal_tc(const MargArgs& a, int d, cudaStream_t st) {
+    int rc, sms;
+    if ((rc = sm_count(&sms)) != USV_OK) return rc;
+    if (a.pairs != nullptr) return d == 64 ? et::launch<64, 2, true>(a, st) : et::launch<128, 2, true>(a, st);
+    const bool one = marginal_single(a, sms);
+    if (d == 64) return one ? et::launch<64, 1, false>(a, st) : et::launch<64, 2, false>(a, st);
+    return one ? et::launch<128, 1, false>(a, st) : et::launch<128, 2, false>(a, st);
 }
 
 }  // namespace usv
