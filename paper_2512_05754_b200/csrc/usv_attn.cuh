@@ -35,6 +35,7 @@ struct AttnArgs {
     const uint16_t* work_flags;   // flag mode: the query blocks whose flag is not 0; their number goes to fallback_count
     int B, H, N, NB, kmax;
     float scale_log2;    // softmax scale * log2(e)
+    int full_heads;      // the first of head_order, which keep every key block, are left to attn_dense_kernel
     int k_per_head[USV_MAX_HEADS];
     int head_order[USV_MAX_HEADS];  // heads sorted by descending k: heavy work is issued first
 };
@@ -44,6 +45,9 @@ bool attn_pair_supported(const AttnArgs& a, int d);
 // whether the call is too small for a pairing plan: a.pairs stays NULL, and fallback_list takes flags
 bool attn_pair_direct(const AttnArgs& a, int d);
 int launch_attn_pair(const AttnArgs& a, int d, cudaStream_t st);
+// Heads that keep every key block and are better computed by the kernel of usv_attn_dense.cu (the first of a.head_order); 0: none.
+int attn_dense_heads(const AttnArgs& a, int d);
+int launch_attn_dense(const AttnArgs& a, cudaStream_t st);
 // fused unmerge: copies the query blocks the exact kernel recomputed (into o) to their original tokens in y
 int launch_scatter_fallbacks(const AttnArgs& a, int d, cudaStream_t st);
 // ints one pair's list occupies for a head that keeps k of NB key blocks (header + entries)

@@ -85,6 +85,7 @@ static int sparse_attn_impl(int B, int H, int N, int d, const void* q, const usv
     a.y = static_cast<__nv_bfloat16*>(y);
     a.N_full = N_full;
     a.B = B; a.H = H; a.N = N; a.NB = NB; a.kmax = kmax;
+    a.full_heads = 0;
     const float sc = scale == 0.f ? 1.0f / sqrtf((float)d) : scale;
     a.scale_log2 = sc * 1.4426950408889634f;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -106,8 +107,15 @@ static int sparse_attn_impl(int B, int H, int N, int d, const void* q, const usv
             a.work_flags = reinterpret_cast<const uint16_t*>(a.fallback_list);
             return launch_attn_mma(a, d, st);
         }
-        if ((rc2 = launch_pair_plan(a, plan_mem, false, st)) != USV_OK) return rc2;
-        if ((rc2 = launch_attn_pair(a, d, st)) != USV_OK) return rc2;
+        a.full_heads = attn_dense_heads(a, d);
+        if (a.full_heads < H) {
+            if ((rc2 = launch_pair_plan(a, plan_mem, false, st)) != USV_OK) return rc2;
+        } else {
+            cudaError_t e = cudaMemsetAsync(a.status + 1, 0, WS_HEADER - 4, st);   // (what the plan does otherwise)
+            if (e != cudaSuccess) return fail(USV_ERR_CUDA, "sparse_attn: memset: %s", cudaGetErrorString(e));
+        }
+        if (a.full_heads > 0 && (rc2 = launch_attn_dense(a, st)) != USV_OK) return rc2;
+        if (a.full_heads < H && (rc2 = launch_attn_pair(a, d, st)) != USV_OK) return rc2;
         // exact recomputation of the (normally zero) query blocks the fast kernel reported
         a.work_list = a.fallback_list;
         a.work_count = a.fallback_count;

@@ -48,7 +48,7 @@
 // skipped a phase could not tell it from the one two before).  All waits are bounded; a wait
 // that gives up sets the device status word and every role leaves its loop.
 #include "usv_attn.cuh"
-#include "usv_tcgen05.cuh"
+#include "usv_attn_softmax.cuh"
 
 namespace usv {
 
@@ -133,35 +133,6 @@ struct Maps {
     CUtensorMap q, k, v;
 };
 
-// exp2 of 32 scaled logits -> 16 packed bf16 pairs; adds to the two lanes of `acc` nothing, the weights as rounded to
-// bf16 (what the P.V product multiplies by, so that numerator and denominator of a row carry the same
-// rounding), or the weights before the rounding (for the log-sum-exp).  Two logits at a time on the packed-fp32 pipe.
-enum { SUM_NONE = 0, SUM_ROUNDED = 1, SUM_EXACT = 2 };
-template <bool MASKED, int SUM, int POLY>
-__device__ __forceinline__ void weights32(const uint32_t* sr, uint32_t* pk, uint64_t c2, uint64_t nref2, int col0,
-                                          int nvalid, uint64_t& acc) {
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        const uint64_t x2 = fma_f32x2(pack_f32x2(__uint_as_float(sr[2 * j]), __uint_as_float(sr[2 * j + 1])), c2, nref2);
-        float p0, p1;
-        if (POLY && j % (POLY ? POLY : 1) == POLY - 1) {
-            exp2_fma(x2, p0, p1);
-        } else {
-            float x0, x1;
-            unpack_f32x2(x2, x0, x1);
-            p0 = ex2(x0);
-            p1 = ex2(x1);
-        }
-        if (MASKED) {
-            if (col0 + 2 * j >= nvalid) p0 = 0.f;
-            if (col0 + 2 * j + 1 >= nvalid) p1 = 0.f;
-        }
-        pk[j] = pack_bf16x2(p0, p1);
-        if (SUM == SUM_ROUNDED) acc = add_f32x2(acc, pack_f32x2(__uint_as_float(pk[j] << 16), __uint_as_float(pk[j] & 0xffff0000u)));
-        if (SUM == SUM_EXACT) acc = add_f32x2(acc, pack_f32x2(p0, p1));
-    }
-}
-
 // nU entries: (key block << 2) | in-A | in-B << 1, ascending (ring slot or global memory)
 __device__ __forceinline__ const int* item_list(const int* hdr) {
     return hdr[I_NU] <= LCAP ? hdr + 16
@@ -202,7 +173,8 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
     const int warp = warp_index(), lane = threadIdx.x & 31;
     const int NB = a.NB, N = a.N;
     const int NP = (NB + 1) >> 1;                 // query-block pairs per (b, h)
-    const int64_t nitems = (int64_t)a.B * a.H * NP;
+    const int heads = a.H - a.full_heads;         // (the first ones of head_order are computed elsewhere)
+    const int64_t nitems = (int64_t)a.B * heads * NP;
 
     // ---- set-up: barriers (one per thread of the first two warps), TMEM
     if (threadIdx.x < F::B_COUNT) {
@@ -265,9 +237,9 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
                     return -1;
                 }
                 const int pair = (int)(w % NP);
-                const int bh_ord = (int)(w / NP);
-                const int b = bh_ord / a.H;
-                const int h = a.head_order[bh_ord % a.H];
+                const int b = (int)(w / NP) / heads;
+                const int bh_ord = b * a.H + a.full_heads + (int)(w / NP) % heads;
+                const int h = a.head_order[bh_ord - b * a.H];
                 int2 pq;
                 const int* pl = nullptr;
                 int nU;
@@ -862,7 +834,7 @@ int launch_attn_pair(const AttnArgs& a, int d, cudaStream_t st) {
     if ((rc = t5::make_bhnd_map(&maps.q, a.q, a.sq, a.B, a.H, a.N, d, "q")) != USV_OK) return rc;
     if ((rc = t5::make_bhnd_map(&maps.k, a.k, a.sk, a.B, a.H, a.N, d, "k")) != USV_OK) return rc;
     if ((rc = t5::make_bhnd_map(&maps.v, a.v, a.sv, a.B, a.H, a.N, d, "v")) != USV_OK) return rc;
-    const int64_t items = (int64_t)a.B * a.H * ((a.NB + 1) / 2);
+    const int64_t items = (int64_t)a.B * (a.H - a.full_heads) * ((a.NB + 1) / 2);
     if (items > 2000000000LL) return fail(USV_ERR_UNSUPPORTED, "sparse_attn: too many query blocks");
     if ((rc = sm_count(&sms)) != USV_OK) return rc;
     const int grid = (int)(items < sms ? items : sms);   // one persistent CTA per SM

@@ -203,7 +203,7 @@ pair_plan_kernel(const AttnArgs a, int2* __restrict__ pairs, int* __restrict__ l
     if (a.work_counter != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < (WS_HEADER - 4) / 4) a.status[1 + threadIdx.x] = 0u;
 
     if (full) {
-        if (ord.pass == 2) return;   // (done by the first pass)
+        if (ord.pass == 2 || a.full_heads > 0) return;   // (done by the first pass, or not wanted)
         out_pairs += blockIdx.x * (CH / 2);
         out_lists += (int64_t)blockIdx.x * (CH / 2) * lstride;
         // every list is the full set: pairing is arbitrary and every key block belongs to both sides
