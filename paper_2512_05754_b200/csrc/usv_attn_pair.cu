@@ -29,17 +29,19 @@
 //   warps 0-15   four softmax warpgroups sharing the 128 rows (thread r of every group <-> TMEM
 //                lane r <-> query row r).  Group g works on the tiles of running parity g >> 1
 //                and there on key block g & 1 of the tile (64 logit columns).
-//   warps 16-19  output: thread e <-> query row e reads the finished O row out of TMEM a quarter at
-//                a time, hands the accumulator back and stores from registers (to o, or, with the
+//   warps 16-19  output: thread e <-> query row e reads the finished O row out of TMEM, hands the
+//                accumulator back and stores from registers (to o, or, with the
 //                unmerge folded in, to every original token that reads the row back), while the
-//                softmax groups are already in the next item.
-//   warp 20      scout + K producer: draws the next item, copies its key-block list into a ring
-//                slot in shared memory and publishes it, fetches Q and the K tiles (TMA).
+//                softmax groups are already in the next item.  Warp 16 is the scout too: it draws items two
+//                ahead, copies their key-block lists into ring slots in shared memory and publishes them.  (That takes
+//                3000 to 6000 cycles of round trips to the L2 and of issue slots it has to wait for.  In the K producer, where
+//                it stood before, the third K tile of an item waited for it.)
+//   warp 20      Q and K producer (TMA).
 //   warp 21      P.V issuer and TMEM owner.
 //   warp 22      V producer (TMA).
 //   warp 23      S issuer.
 // The CTA is launched with 80 registers per thread and the roles re-divide them at their start
-// (setmaxnreg): the softmax loop needs more than the launch allows for 768 threads, the others less.
+// (setmaxnreg): softmax and output (a whole row as bf16 pairs) need more than the launch allows for 768 threads, the others less.
 //
 // TMEM holds O and THREE S buffers; running tile g uses buffer g mod 3.  The weights P are
 // written back, as bf16 pairs, into the columns their logits came from, so a buffer goes
@@ -61,6 +63,7 @@ constexpr int NWG = 4;                          // softmax warpgroups
 constexpr int VSTAGES = 3;                      // V tile stages
 constexpr int SBUF = 3;                         // S/P buffers in TMEM
 constexpr int NSLOT = 4;                        // item ring
+constexpr int LOOK = 2;                         // items published ahead of the one whose output is next (at most NSLOT - 1)
 constexpr int LCAP = 512;                       // list entries a ring slot holds (longer lists are read from global memory)
 constexpr int MAX_NB = PLAN_MAX_NB;             // key blocks per sequence this kernel covers
 constexpr uint32_t ITEM_BYTES = 64 + LCAP * 4;
@@ -125,8 +128,8 @@ constexpr int NTHREADS = NSOFT + 128 + 128;   // + output warpgroup + service wa
 constexpr int W_EPI = NSOFT / 32, W_TMA = W_EPI + 4, W_MMA = W_EPI + 5, W_TMA_V = W_EPI + 6, W_MMA_S = W_EPI + 7;
 // Registers per thread after the roles part ways (setmaxnreg, whole warpgroups).  A CTA can only
 // redistribute what it was launched with: 24 warps x 80 registers = 1920 per lane, and
-// 16 x 96 + 4 x 56 + 4 x 40 = 1920.  (A request beyond the pool would wait forever.)
-constexpr int REG_LAUNCH = 80, REG_SOFT = 96, REG_EPI = 56, REG_SERVICE = 40;
+// 16 x 88 + 4 x 88 + 4 x 40 = 1920.  (A request beyond the pool would wait forever.)
+constexpr int REG_LAUNCH = 80, REG_SOFT = 88, REG_EPI = 88, REG_SERVICE = 40;
 static_assert(16 * REG_SOFT + 4 * REG_EPI + 4 * REG_SERVICE <= 24 * REG_LAUNCH, "register pool of the CTA");
 
 struct Maps {
@@ -138,6 +141,24 @@ __device__ __forceinline__ const int* item_list(const int* hdr) {
     return hdr[I_NU] <= LCAP ? hdr + 16
                              : reinterpret_cast<const int*>(((unsigned long long)(unsigned)hdr[I_LIST_HI] << 32) |
                                                             (unsigned)hdr[I_LIST_LO]);
+}
+
+// Four lanes of a warp, four pieces of 16 bytes each: lane i of the four gets piece i of all four.
+__device__ __forceinline__ void quad_transpose(uint32_t* x, int lane) {
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (i & o) continue;
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                const uint32_t got = __shfl_xor_sync(0xffffffffu, up ? x[4 * i + w] : x[4 * (i + o) + w], o);
+                if (up) x[4 * i + w] = got;
+                else x[4 * (i + o) + w] = got;
+            }
+        }
+    }
 }
 
 // DIRECT: no pairing plan (see attn_pair_direct).  Neighbouring query blocks share an item, the CTAs take the
@@ -209,123 +230,8 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
     // (softmax warps): setmaxnreg, whole warpgroups.
 
     if (warp == W_TMA) {
+        // ===== Q and K producer (whole warp in the loop, one elected lane issues) ================
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REG_SERVICE));
-        // ===== scout + K producer (whole warp in the loop, one elected lane issues) ==============
-        // publish(n): draw work until an item with at least one key block turns up, copy its list
-        // into ring slot n and publish it; a pair without any key block gets its defined output
-        // (zeros) right here and is not published.  Returns the item's tile count, -1 after
-        // publishing the end marker, -2 when a bounded wait gave up.
-        int64_t turn = blockIdx.x;
-        auto publish = [&](int n) -> int {
-            int* hdr = hdr_of(n);
-            if (n >= NSLOT && !mbar_wait(bar(F::B_IFREE + n % NSLOT), ((n / NSLOT) - 1) & 1, s_abort, a.status, 0x8000))
-                return -2;
-            for (;;) {
-                int64_t w;
-                if (DIRECT) {
-                    w = turn;
-                    turn += gridDim.x;
-                } else {
-                    int wi = 0;
-                    if (lane == 0) wi = atomicAdd(a.work_counter, 1);
-                    w = __shfl_sync(0xffffffffu, wi, 0);
-                }
-                if (w >= nitems) {
-                    if (lane == 0) hdr[I_T] = -1;
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar(F::B_IFULL + n % NSLOT));
-                    return -1;
-                }
-                const int pair = (int)(w % NP);
-                const int b = (int)(w / NP) / heads;
-                const int bh_ord = b * a.H + a.full_heads + (int)(w / NP) % heads;
-                const int h = a.head_order[bh_ord - b * a.H];
-                int2 pq;
-                const int* pl = nullptr;
-                int nU;
-                if (DIRECT) {
-                    // a word of either row's bitmap per lane, the union as a list in the ring slot
-                    pq = make_int2(2 * pair, 2 * pair + 1 < NB ? 2 * pair + 1 : -1);
-                    const int kh = a.k_per_head[h];
-                    const int32_t* row = a.sel + (((int64_t)b * a.H + h) * NB + pq.x) * a.kmax;
-                    uint32_t ba = 0, bb = 0;
-                    for (int i0 = 0; i0 < kh; i0 += 32) {
-                        const int i = i0 + lane;
-                        const int ea = i < kh ? __ldg(row + i) : -1, eb = i < kh && pq.y >= 0 ? __ldg(row + a.kmax + i) : -1;
-                        const int m = min(32, kh - i0);
-#pragma unroll 4
-                        for (int q = 0; q < m; ++q) {
-                            const int ja = __shfl_sync(0xffffffffu, ea, q), jb = __shfl_sync(0xffffffffu, eb, q);
-                            if (ja >= 0 && ja < NB && (ja >> 5) == lane) ba |= 1u << (ja & 31);
-                            if (jb >= 0 && jb < NB && (jb >> 5) == lane) bb |= 1u << (jb & 31);
-                        }
-                    }
-                    uint32_t u = ba | bb;
-                    const int incl = warp_incl_scan(__popc(u));
-                    nU = __shfl_sync(0xffffffffu, incl, 31);
-                    for (int at = 16 + incl - __popc(u); u != 0; u &= u - 1) {
-                        const int bit = __ffs(u) - 1;
-                        hdr[at++] = ((lane * 32 + bit) << 2) | ((ba >> bit) & 1u) | (((bb >> bit) & 1u) << 1);
-                    }
-                    __syncwarp();
-                } else {
-                    pq = a.pairs[((int64_t)b * a.H + h) * NP + pair];   // similarity-driven pairing
-                    pl = a.lists + b * a.list_batch + a.list_off[h] + (int64_t)pair * list_stride(a.k_per_head[h], NB);
-                    nU = __ldg(pl);
-                }
-                if (nU == 0) {
-                    if (DIRECT && lane < 2 && (lane == 0 || pq.y >= 0))
-                        reinterpret_cast<uint16_t*>(a.fallback_list)[(int64_t)bh_ord * NB + pq.x + lane] = 0;
-                    // no valid key block at all: defined output (zeros, log-sum-exp 0), as the exact kernel does
-                    __nv_bfloat16* O = a.o + b * a.so.sb + h * a.so.sh;
-                    for (int idx = lane; idx < 128 * (D / 8); idx += 32) {
-                        const int rr = idx / (D / 8), cc = idx % (D / 8);
-                        const int Ir = rr < 64 ? pq.x : pq.y;
-                        const int grow = Ir * USV_BLOCK + (rr & 63);
-                        if (Ir >= 0 && grow < N) {
-                            *reinterpret_cast<uint4*>(O + (int64_t)grow * a.so.sn + cc * 8) = make_uint4(0, 0, 0, 0);
-                            if (a.y != nullptr) {
-                                const int u1 = a.unmerge_off[(int64_t)b * (N + 1) + grow + 1];
-                                for (int u = a.unmerge_off[(int64_t)b * (N + 1) + grow]; u < u1; ++u)
-                                    *reinterpret_cast<uint4*>(a.y + ((int64_t)b * a.N_full + a.unmerge_idx[(int64_t)b * a.N_full + u]) *
-                                                                        ((int64_t)a.H * D) + h * D + cc * 8) = make_uint4(0, 0, 0, 0);
-                            }
-                            const int64_t grow_bh = ((int64_t)b * a.H + h) * N + grow;
-                            if (a.o_f32 != nullptr) {
-                                float4* o32 = reinterpret_cast<float4*>(a.o_f32 + grow_bh * D + cc * 8);
-                                o32[0] = make_float4(0.f, 0.f, 0.f, 0.f);
-                                o32[1] = make_float4(0.f, 0.f, 0.f, 0.f);
-                            }
-                            if (a.lse != nullptr && cc == 0) a.lse[grow_bh] = 0.f;
-                        }
-                    }
-                    continue;
-                }
-                int srefA = nU, srefB = nU;   // first union slot that block A / block B may see
-                for (int i0 = 0; i0 < nU; i0 += 32) {
-                    const int idx = i0 + lane;
-                    const int e = idx >= nU ? 0 : (DIRECT ? hdr[16 + idx] : __ldg(pl + 1 + idx));
-                    if (!DIRECT && nU <= LCAP && idx < nU) hdr[16 + idx] = e;
-                    const unsigned ba = __ballot_sync(0xffffffffu, e & 1), bb = __ballot_sync(0xffffffffu, e & 2);
-                    if (srefA == nU && ba) srefA = i0 + __ffs(ba) - 1;
-                    if (srefB == nU && bb) srefB = i0 + __ffs(bb) - 1;
-                    if (nU > LCAP && srefA < nU && (srefB < nU || pq.y < 0)) break;   // nothing to copy
-                }
-                if (lane == 0) {
-                    hdr[I_T] = (nU + 1) >> 1;   // 128-key tiles
-                    hdr[I_NU] = nU;
-                    hdr[I_B] = b; hdr[I_H] = h; hdr[I_BH] = bh_ord; hdr[I_IA] = pq.x; hdr[I_IB] = pq.y;
-                    hdr[I_SREFA] = srefA; hdr[I_SREFB] = srefB;
-                    const unsigned long long lp = reinterpret_cast<unsigned long long>(pl + 1);
-                    hdr[I_LIST_LO] = (int)(unsigned)lp; hdr[I_LIST_HI] = (int)(unsigned)(lp >> 32);
-                    s_flag[(n % NSLOT) * 2] = 0;
-                    s_flag[(n % NSLOT) * 2 + 1] = 0;
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar(F::B_IFULL + n % NSLOT));
-                return (nU + 1) >> 1;
-            }
-        };
         // Q rows of published item m -> the Q buffer, once the last S tile of item m - 1 is done.
         auto load_q = [&](int m) -> bool {
             const int* hdr = hdr_of(m);
@@ -345,24 +251,17 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
             return true;
         };
         int g = 0;   // running tile counter
-        int n = 0;   // running item counter
-        int T = publish(0);
-        while (T > 0) {
+        bool ok = true;
+        for (int n = 0; ok; ++n) {
+            if (!mbar_wait(bar(F::B_IFULL + n % NSLOT), (n / NSLOT) & 1, s_abort, a.status, 0x10000)) break;
             const int* hdr = hdr_of(n);
+            const int T = hdr[I_T];
+            if (T < 0) break;
             const int nU = hdr[I_NU];
             const int* list = item_list(hdr);
             const int b = hdr[I_B], h = hdr[I_H];
-            int Tn = 0;
-            bool pub = false, ok = true;
             if (n == 0 && !load_q(0)) break;
             for (int t = 0; t < T; ++t, ++g) {
-                // the next item is drawn and published once this one's first tiles are on their
-                // way: its global round trips then fall into the wait for the K stages to come back
-                if (t == KSTAGES) {
-                    Tn = publish(n + 1);
-                    pub = true;
-                    if (Tn == -2) { ok = false; break; }
-                }
                 const int s = g % KSTAGES;
                 const uint32_t ph = (g / KSTAGES) & 1;
                 const int J0 = list[2 * t] >> 2;
@@ -382,13 +281,6 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
                 // later than that K stage does, and the K tile must not wait for it.
                 if (t == 0 && n > 0 && !load_q(n)) { ok = false; break; }
             }
-            if (!ok) break;
-            if (!pub) {
-                Tn = publish(n + 1);
-                if (Tn == -2) break;
-            }
-            ++n;
-            T = Tn;
         }
     } else if (warp == W_TMA_V) {
         // ===== V producer ========================================================================
@@ -505,12 +397,133 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
             }
         }
     } else if (warp >= W_EPI && warp < W_TMA) {
-        // ===== output warps: thread e <-> TMEM lane e <-> query row e of the item ================
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REG_EPI));
+        // ===== output warps: thread e <-> TMEM lane e <-> query row e of the item; the first is the scout too =======
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REG_EPI));
+        // publish(n): draw work until an item with at least one key block turns up, copy its list
+        // into ring slot n and publish it; a pair without any key block gets its defined output
+        // (zeros) right here and is not published.  Returns the item's tile count, -1 after
+        // publishing the end marker, -2 when a bounded wait gave up.
+        int64_t turn = blockIdx.x;
+        auto publish = [&](int n) -> int {
+            int* hdr = hdr_of(n);
+            if (n >= NSLOT && !mbar_wait(bar(F::B_IFREE + n % NSLOT), ((n / NSLOT) - 1) & 1, s_abort, a.status, 0x8000))
+                return -2;
+            for (;;) {
+                int64_t w;
+                if (DIRECT) {
+                    w = turn;
+                    turn += gridDim.x;
+                } else {
+                    int wi = 0;
+                    if (lane == 0) wi = atomicAdd(a.work_counter, 1);
+                    w = __shfl_sync(0xffffffffu, wi, 0);
+                }
+                if (w >= nitems) {
+                    if (lane == 0) hdr[I_T] = -1;
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(F::B_IFULL + n % NSLOT));
+                    return -1;
+                }
+                const int pair = (int)(w % NP);
+                const int b = (int)(w / NP) / heads;
+                const int bh_ord = b * a.H + a.full_heads + (int)(w / NP) % heads;
+                const int h = a.head_order[bh_ord - b * a.H];
+                int2 pq;
+                const int* pl = nullptr;
+                int nU;
+                if (DIRECT) {
+                    // a word of either row's bitmap per lane, the union as a list in the ring slot
+                    pq = make_int2(2 * pair, 2 * pair + 1 < NB ? 2 * pair + 1 : -1);
+                    const int kh = a.k_per_head[h];
+                    const int32_t* row = a.sel + (((int64_t)b * a.H + h) * NB + pq.x) * a.kmax;
+                    uint32_t ba = 0, bb = 0;
+                    for (int i0 = 0; i0 < kh; i0 += 32) {
+                        const int i = i0 + lane;
+                        const int ea = i < kh ? __ldg(row + i) : -1, eb = i < kh && pq.y >= 0 ? __ldg(row + a.kmax + i) : -1;
+                        const int m = min(32, kh - i0);
+#pragma unroll 4
+                        for (int q = 0; q < m; ++q) {
+                            const int ja = __shfl_sync(0xffffffffu, ea, q), jb = __shfl_sync(0xffffffffu, eb, q);
+                            if (ja >= 0 && ja < NB && (ja >> 5) == lane) ba |= 1u << (ja & 31);
+                            if (jb >= 0 && jb < NB && (jb >> 5) == lane) bb |= 1u << (jb & 31);
+                        }
+                    }
+                    uint32_t u = ba | bb;
+                    const int incl = warp_incl_scan(__popc(u));
+                    nU = __shfl_sync(0xffffffffu, incl, 31);
+                    for (int at = 16 + incl - __popc(u); u != 0; u &= u - 1) {
+                        const int bit = __ffs(u) - 1;
+                        hdr[at++] = ((lane * 32 + bit) << 2) | ((ba >> bit) & 1u) | (((bb >> bit) & 1u) << 1);
+                    }
+                    __syncwarp();
+                } else {
+                    pq = a.pairs[((int64_t)b * a.H + h) * NP + pair];   // similarity-driven pairing
+                    pl = a.lists + b * a.list_batch + a.list_off[h] + (int64_t)pair * list_stride(a.k_per_head[h], NB);
+                    nU = __ldg(pl);
+                }
+                if (nU == 0) {
+                    if (DIRECT && lane < 2 && (lane == 0 || pq.y >= 0))
+                        reinterpret_cast<uint16_t*>(a.fallback_list)[(int64_t)bh_ord * NB + pq.x + lane] = 0;
+                    // no valid key block at all: defined output (zeros, log-sum-exp 0), as the exact kernel does
+                    __nv_bfloat16* O = a.o + b * a.so.sb + h * a.so.sh;
+                    for (int idx = lane; idx < 128 * (D / 8); idx += 32) {
+                        const int rr = idx / (D / 8), cc = idx % (D / 8);
+                        const int Ir = rr < 64 ? pq.x : pq.y;
+                        const int grow = Ir * USV_BLOCK + (rr & 63);
+                        if (Ir >= 0 && grow < N) {
+                            *reinterpret_cast<uint4*>(O + (int64_t)grow * a.so.sn + cc * 8) = make_uint4(0, 0, 0, 0);
+                            if (a.y != nullptr) {
+                                const int u1 = a.unmerge_off[(int64_t)b * (N + 1) + grow + 1];
+                                for (int u = a.unmerge_off[(int64_t)b * (N + 1) + grow]; u < u1; ++u)
+                                    *reinterpret_cast<uint4*>(a.y + ((int64_t)b * a.N_full + a.unmerge_idx[(int64_t)b * a.N_full + u]) *
+                                                                        ((int64_t)a.H * D) + h * D + cc * 8) = make_uint4(0, 0, 0, 0);
+                            }
+                            const int64_t grow_bh = ((int64_t)b * a.H + h) * N + grow;
+                            if (a.o_f32 != nullptr) {
+                                float4* o32 = reinterpret_cast<float4*>(a.o_f32 + grow_bh * D + cc * 8);
+                                o32[0] = make_float4(0.f, 0.f, 0.f, 0.f);
+                                o32[1] = make_float4(0.f, 0.f, 0.f, 0.f);
+                            }
+                            if (a.lse != nullptr && cc == 0) a.lse[grow_bh] = 0.f;
+                        }
+                    }
+                    continue;
+                }
+                int srefA = nU, srefB = nU;   // first union slot that block A / block B may see
+                for (int i0 = 0; i0 < nU; i0 += 32) {
+                    const int idx = i0 + lane;
+                    const int e = idx >= nU ? 0 : (DIRECT ? hdr[16 + idx] : __ldg(pl + 1 + idx));
+                    if (!DIRECT && nU <= LCAP && idx < nU) hdr[16 + idx] = e;
+                    const unsigned ba = __ballot_sync(0xffffffffu, e & 1), bb = __ballot_sync(0xffffffffu, e & 2);
+                    if (srefA == nU && ba) srefA = i0 + __ffs(ba) - 1;
+                    if (srefB == nU && bb) srefB = i0 + __ffs(bb) - 1;
+                    if (nU > LCAP && srefA < nU && (srefB < nU || pq.y < 0)) break;   // nothing to copy
+                }
+                if (lane == 0) {
+                    hdr[I_T] = (nU + 1) >> 1;   // 128-key tiles
+                    hdr[I_NU] = nU;
+                    hdr[I_B] = b; hdr[I_H] = h; hdr[I_BH] = bh_ord; hdr[I_IA] = pq.x; hdr[I_IB] = pq.y;
+                    hdr[I_SREFA] = srefA; hdr[I_SREFB] = srefB;
+                    const unsigned long long lp = reinterpret_cast<unsigned long long>(pl + 1);
+                    hdr[I_LIST_LO] = (int)(unsigned)lp; hdr[I_LIST_HI] = (int)(unsigned)(lp >> 32);
+                    s_flag[(n % NSLOT) * 2] = 0;
+                    s_flag[(n % NSLOT) * 2 + 1] = 0;
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(F::B_IFULL + n % NSLOT));
+                return (nU + 1) >> 1;
+            }
+        };
         const int e = threadIdx.x - NSOFT;
         const int side = e >> 6;                         // 0: block A, 1: block B (uniform per warp)
         const uint32_t lane_base = tmem + ((uint32_t)((warp - W_EPI) * 32) << 16);
+        int next = warp == W_EPI ? 0 : -1;               // item to publish; -1: none (any more)
         for (int m = 0;; ++m) {
+            while (next >= 0 && next <= m + LOOK) {
+                const int T = publish(next);
+                if (T == -2) break;
+                next = T < 0 ? -1 : next + 1;
+            }
             const int slot = m % NSLOT;
             if (!mbar_wait(bar(F::B_IFULL + slot), (m / NSLOT) & 1, s_abort, a.status, 0x10000)) break;
             const int* hdr = hdr_of(m);
@@ -526,9 +539,10 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
 #pragma unroll
                 for (int q = 0; q < NWG; ++q) lx += sums[q * 128 + e];
             }
+            const float nref = has_ref ? s_refv[slot * 128 + e] : 0.f;
+            if (!mbar_wait(bar(F::B_OFULL), m & 1, s_abort, a.status, 0x200)) break;
+            fence_after();
             if (F::SUM_COL) {
-                if (!mbar_wait(bar(F::B_OFULL), m & 1, s_abort, a.status, 0x200)) break;
-                fence_after();
                 uint32_t sum;
                 tmem_ld1(lane_base + TO + D, sum);
                 tmem_wait_ld();
@@ -536,61 +550,27 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
             } else {
                 l = lx;
             }
-            const float nref = has_ref ? s_refv[slot * 128 + e] : 0.f;
             const bool in_range = l > 7.9e-31f && l < 1.2e30f;   // ~[2^-100, 2^100]
             uint64_t z0 = 0, z1 = 0;   // four fp32 sums that stay 0 unless a value of the row is not finite
             const float inv = l > 0.f ? 1.0f / l : 0.f;
-            if (SUM != SUM_NONE && a.lse != nullptr && live)
-                a.lse[((int64_t)ib * a.H + ih) * N + row] = (log2f(lx) - nref) * 0.69314718055994531f;
-            if (!F::SUM_COL) {
-                if (!mbar_wait(bar(F::B_OFULL), m & 1, s_abort, a.status, 0x200)) break;
-                fence_after();
-            }
-            // The row leaves TMEM a quarter (32 columns) at a time and is stored from registers; the
-            // accumulator and the ring slot go back as soon as the last quarter has been read.
+            // The row leaves TMEM a quarter (32 columns) at a time and is kept as bf16 pairs, so that the accumulator and the
+            // ring slot go back before anything is stored: the next item's first P.V waits for them (stored a quarter at a
+            // time in between, they came back 4000 to 7000 cycles later).
             float* o32 = (a.o_f32 != nullptr && live) ? a.o_f32 + (((int64_t)ib * a.H + ih) * N + row) * D : nullptr;
-            __nv_bfloat16* O = a.o + ib * a.so.sb + ih * a.so.sh + (int64_t)row * a.so.sn;
-            // fused unmerge: the row goes to every original token that reads it back
-            int u0 = 0, u1 = 0;
-            if (a.y != nullptr && live) {
-                u0 = a.unmerge_off[(int64_t)ib * (N + 1) + row];
-                u1 = a.unmerge_off[(int64_t)ib * (N + 1) + row + 1];
-            }
-#pragma unroll 1
+            uint32_t pk[D / 2];
+#pragma unroll
             for (int qd = 0; qd < D / 32; ++qd) {
                 uint32_t r0[32];
                 tmem_ld32(lane_base + TO + qd * 32, r0);
-                tmem_wait_ld();
+                tmem_wait_ld32(r0);
 #pragma unroll
                 for (int j = 0; F::CHECK_FINITE && j < 8; ++j) {
                     z0 = fma_f32x2(pack_f32x2(__uint_as_float(r0[4 * j]), __uint_as_float(r0[4 * j + 1])), 0ull, z0);
                     z1 = fma_f32x2(pack_f32x2(__uint_as_float(r0[4 * j + 2]), __uint_as_float(r0[4 * j + 3])), 0ull, z1);
                 }
-                if (qd == D / 32 - 1) {
-                    // A row whose sum left the safe range, or that is not finite (see CHECK_FINITE): the
-                    // first row of a query block to notice hands the block to the exact kernel, which
-                    // keeps query blocks apart.
-                    bool finite = true;
-                    if (F::CHECK_FINITE) {
-                        float za, zb;
-                        unpack_f32x2(add_f32x2(z0, z1), za, zb);
-                        finite = za + zb == 0.f;
-                    }
-                    if (DIRECT) {
-                        const bool any = __any_sync(0xffffffffu, live && !(in_range && finite));
-                        if (lane == 0 && iq >= 0)
-                            reinterpret_cast<uint8_t*>(a.fallback_list)[2 * ((int64_t)ibh * NB + iq) + (warp & 1)] = any;
-                    } else if (live && !(in_range && finite) && a.fallback_list != nullptr &&
-                               atomicExch(&s_flag[slot * 2 + side], 1) == 0) {
-                        a.fallback_list[atomicAdd(a.fallback_count, 1)] = ibh * NB + iq;
-                    }
-                    fence_before();
-                    __syncwarp();
-                    if (lane == 0) {
-                        mbar_arrive(bar(F::B_OFREE));
-                        mbar_arrive(bar(F::B_IFREE + slot));
-                    }
-                }
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                    pk[qd * 16 + j] = pack_bf16x2(__uint_as_float(r0[2 * j]) * inv, __uint_as_float(r0[2 * j + 1]) * inv);
                 if (o32 != nullptr) {
 #pragma unroll
                     for (int j = 0; j < 8; ++j)
@@ -598,25 +578,56 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
                             make_float4(__uint_as_float(r0[4 * j]) * inv, __uint_as_float(r0[4 * j + 1]) * inv,
                                         __uint_as_float(r0[4 * j + 2]) * inv, __uint_as_float(r0[4 * j + 3]) * inv);
                 }
-                if (live) {
-                    uint4 pk[4];
+            }
+            // A row whose sum left the safe range, or that is not finite (see CHECK_FINITE): the
+            // first row of a query block to notice hands the block to the exact kernel, which
+            // keeps query blocks apart.
+            bool finite = true;
+            if (F::CHECK_FINITE) {
+                float za, zb;
+                unpack_f32x2(add_f32x2(z0, z1), za, zb);
+                finite = za + zb == 0.f;
+            }
+            if (DIRECT) {
+                const bool any = __any_sync(0xffffffffu, live && !(in_range && finite));
+                if (lane == 0 && iq >= 0)
+                    reinterpret_cast<uint8_t*>(a.fallback_list)[2 * ((int64_t)ibh * NB + iq) + (warp & 1)] = any;
+            } else if (live && !(in_range && finite) && a.fallback_list != nullptr &&
+                       atomicExch(&s_flag[slot * 2 + side], 1) == 0) {
+                a.fallback_list[atomicAdd(a.fallback_count, 1)] = ibh * NB + iq;
+            }
+            fence_before();
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(bar(F::B_OFREE));
+                mbar_arrive(bar(F::B_IFREE + slot));
+            }
+            if (SUM != SUM_NONE && a.lse != nullptr && live)
+                a.lse[((int64_t)ib * a.H + ih) * N + row] = (log2f(lx) - nref) * 0.69314718055994531f;
+            if (a.y == nullptr) {
+                // Four lanes turn their four rows of 64 bytes into pieces of 16 bytes of all four: a store of the warp then
+                // covers eight rows of 64 consecutive bytes, not 16 bytes of 32.
+                const int rw = iq * USV_BLOCK + ((warp & 1) * 32 + (lane & ~3));
+                __nv_bfloat16* O = a.o + ib * a.so.sb + ih * a.so.sh + (lane & 3) * 8;
+#pragma unroll
+                for (int qd = 0; qd < D / 32; ++qd) {
+                    uint32_t* x = pk + qd * 16;
+                    quad_transpose(x, lane);
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
-                        pk[i] = make_uint4(pack_bf16x2(__uint_as_float(r0[8 * i]) * inv, __uint_as_float(r0[8 * i + 1]) * inv),
-                                           pack_bf16x2(__uint_as_float(r0[8 * i + 2]) * inv, __uint_as_float(r0[8 * i + 3]) * inv),
-                                           pack_bf16x2(__uint_as_float(r0[8 * i + 4]) * inv, __uint_as_float(r0[8 * i + 5]) * inv),
-                                           pack_bf16x2(__uint_as_float(r0[8 * i + 6]) * inv, __uint_as_float(r0[8 * i + 7]) * inv));
-                    if (a.y == nullptr) {
+                        if (iq >= 0 && rw + i < N)
+                            *reinterpret_cast<uint4*>(O + (int64_t)(rw + i) * a.so.sn + qd * 32) =
+                                make_uint4(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]);
+                }
+            } else if (live) {
+                // fused unmerge: the row goes to every original token that reads it back
+                const int u0 = a.unmerge_off[(int64_t)ib * (N + 1) + row], u1 = a.unmerge_off[(int64_t)ib * (N + 1) + row + 1];
+                for (int u = u0; u < u1; ++u) {
+                    const int tok = a.unmerge_idx[(int64_t)ib * a.N_full + u];
+                    __nv_bfloat16* Y = a.y + ((int64_t)ib * a.N_full + tok) * ((int64_t)a.H * D) + ih * D;
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) *reinterpret_cast<uint4*>(O + qd * 32 + 8 * i) = pk[i];
-                    } else {
-                        for (int u = u0; u < u1; ++u) {
-                            const int tok = a.unmerge_idx[(int64_t)ib * a.N_full + u];
-                            __nv_bfloat16* Y = a.y + ((int64_t)ib * a.N_full + tok) * ((int64_t)a.H * D) + ih * D + qd * 32;
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) *reinterpret_cast<uint4*>(Y + 8 * i) = pk[i];
-                        }
-                    }
+                    for (int i = 0; i < D / 8; ++i)
+                        *reinterpret_cast<uint4*>(Y + 8 * i) = make_uint4(pk[4 * i], pk[4 * i + 1], pk[4 * i + 2], pk[4 * i + 3]);
                 }
             }
         }
