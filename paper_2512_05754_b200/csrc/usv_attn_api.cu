@@ -100,6 +100,12 @@ static int sparse_attn_impl(int B, int H, int N, int d, const void* q, const usv
     // 104 / 91; 15 216, keep 1 137 / 157); between the two lines only keep 1 and 2 would gain (768, 8.9 / 15.1 and 13.3 / 17.1).
     const int64_t blocks = (int64_t)B * H * NB;
     const bool small = d == 64 && ((kmx <= 4 && blocks <= 384) || (kmx == 1 && blocks > 1800));
+    // Where every query block has an SM to itself, four groups of warps walk its list side by side: 32 blocks, keep 4 8.3 / 7.0,
+    // 8 11.4 / 9.4, 16 13.7 / 15.2; 128, keep 2 8.3 / 7.0, 4 11.6 / 7.2, 8 12.1 / 9.7; 100, keep 10 13.7 / 11.5; 256, keep 4 11.9 / 12.9
+    // (other kernels / this one).  At d = 128 it never pays (32, keep 4 10.8 / 13.1).
+    int sms;
+    if ((rc = sm_count(&sms)) != USV_OK) return rc;
+    if (impl == 0 && d == 64 && y == nullptr && blocks <= sms && kmx <= 10) return launch_attn_split(a, kmx, st);
     if (impl == 0 && !small && attn_pair_supported(a, d)) {
         int rc2;
         if (attn_pair_direct(a, d)) {

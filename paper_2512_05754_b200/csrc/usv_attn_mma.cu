@@ -9,15 +9,22 @@
 
 namespace usv {
 
-template <int D>
+// G groups of 4 warps share a query block: group i takes the entries i, i + G, ... of its list, and the groups' results, each
+// relative to its own row maxima, are put together at the end.  NBUF: K/V tiles a group has room for.
+template <int D, int G, int NBUF>
 __device__ __forceinline__ void attn_mma_block(const AttnArgs& a, const int work, unsigned char* smem_raw) {
     constexpr int LD = MmaSmem<D>::LD;
     constexpr int TILE = MmaSmem<D>::TILE;
     constexpr int KT = D / 16;  // k-steps of QK^T
     constexpr int NT = D / 8;   // n-tiles of the output
+    const int grp = G == 1 ? 0 : threadIdx.x >> 7;
     __nv_bfloat16* Qs = reinterpret_cast<__nv_bfloat16*>(smem_raw);
-    __nv_bfloat16* Ks = Qs + TILE;
-    __nv_bfloat16* Vs = Ks + 2 * TILE;
+    __nv_bfloat16* Ks = Qs + TILE + grp * (2 * NBUF * TILE);
+    __nv_bfloat16* Vs = Ks + NBUF * TILE;
+    auto group_sync = [&] {
+        if (G == 1) __syncthreads();
+        else asm volatile("barrier.sync %0, 128;" ::"r"(grp + 1) : "memory");
+    };
 
     const int I = work % a.NB;
     const int bh_ord = work / a.NB;
@@ -31,14 +38,14 @@ __device__ __forceinline__ void attn_mma_block(const AttnArgs& a, const int work
     const __nv_bfloat16* K = a.k + b * a.sk.sb + h * a.sk.sh;
     const __nv_bfloat16* V = a.v + b * a.sv.sb + h * a.sv.sh;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;
     const int g = lane >> 2, tig = lane & 3;
 
     // first valid entry of the selection
-    int t = 0;
-    while (t < kh && sel[t] < 0) ++t;
+    int t = grp;
+    while (t < kh && sel[t] < 0) t += G;
 
-    load_tile<D>(Qs, Q, a.sq.sn, I * USV_BLOCK, N);
+    load_tile<D, G>(Qs, Q, a.sq.sn, I * USV_BLOCK, N);
     if (t < kh) {
         load_tile<D>(Ks, K, a.sk.sn, sel[t] * USV_BLOCK, N);
         load_tile<D>(Vs, V, a.sv.sn, sel[t] * USV_BLOCK, N);
@@ -59,14 +66,18 @@ __device__ __forceinline__ void attn_mma_block(const AttnArgs& a, const int work
 
     int buf = 0;
     bool first = true;
+    if (G > 1) {   // the Q tile came through all groups
+        cp_async_wait_all();
+        __syncthreads();
+    }
     while (t < kh) {
         const int J = sel[t];
-        int tn = t + 1;
-        while (tn < kh && sel[tn] < 0) ++tn;
+        int tn = t + G;
+        while (tn < kh && sel[tn] < 0) tn += G;
 
         cp_async_wait_all();
-        __syncthreads();  // tile t is visible; every warp has left the tile of the step before
-        if (tn < kh) {
+        group_sync();  // tile t is visible; every warp has left the tile of the step before
+        if (NBUF == 2 && tn < kh) {
             load_tile<D>(Ks + (buf ^ 1) * TILE, K, a.sk.sn, sel[tn] * USV_BLOCK, N);
             load_tile<D>(Vs + (buf ^ 1) * TILE, V, a.sv.sn, sel[tn] * USV_BLOCK, N);
         }
@@ -166,7 +177,7 @@ __device__ __forceinline__ void attn_mma_block(const AttnArgs& a, const int work
                 mma_bf16_16816(o[2 * n2 + 1], pf[kt], bfr[2], bfr[3]);
             }
         }
-        buf ^= 1;
+        if (NBUF == 2) buf ^= 1;   // (with one tile there is no next one: lists of at most G entries)
         t = tn;
     }
     cp_async_wait_all();
@@ -178,6 +189,62 @@ __device__ __forceinline__ void attn_mma_block(const AttnArgs& a, const int work
         l[r] += __shfl_xor_sync(0xffffffffu, l[r], 2);
         lr[r] += __shfl_xor_sync(0xffffffffu, lr[r], 1);
         lr[r] += __shfl_xor_sync(0xffffffffu, lr[r], 2);
+    }
+    if constexpr (G > 1) {
+        // each group's rows of O where its tiles were, its maxima and sums behind all tiles; then a thread puts 8 columns
+        // of a row together
+        static_assert(64 * (D + 8) * 4 <= 2 * TILE * 2, "a group's rows of O fit where a K and a V tile were");
+        constexpr int OLD = D + 8;
+        float* stat = reinterpret_cast<float*>(Qs + TILE + G * (2 * NBUF * TILE));   // [G][3][64]
+        auto rows_of = [&](int i) { return reinterpret_cast<float*>(Qs + TILE + i * (2 * NBUF * TILE)); };
+        group_sync();   // every warp of the group has left its tiles
+        float* mine = rows_of(grp) + (warp * 16 + g) * OLD + 2 * tig;
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+            *reinterpret_cast<float2*>(mine + n * 8) = make_float2(o[n][0], o[n][1]);
+            *reinterpret_cast<float2*>(mine + 8 * OLD + n * 8) = make_float2(o[n][2], o[n][3]);
+        }
+        if (tig == 0) {
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                float* st = stat + grp * 192 + warp * 16 + g + 8 * r;
+                st[0] = m[r];
+                st[64] = l[r];
+                st[128] = lr[r];
+            }
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < USV_BLOCK * (D / 8); i += 128 * G) {
+            const int rr = i / (D / 8), cc = i % (D / 8) * 8, row = I * USV_BLOCK + rr;
+            if (row >= N) continue;
+            float mx = -INFINITY;
+#pragma unroll
+            for (int q = 0; q < G; ++q) mx = fmaxf(mx, stat[q * 192 + rr]);
+            const float ms = mx == -INFINITY ? 0.f : mx;
+            float ls = 0.f, ln = 0.f, y[8] = {};
+#pragma unroll
+            for (int q = 0; q < G; ++q) {
+                const float w = exp2f(stat[q * 192 + rr] - ms);
+                ls += w * stat[q * 192 + 64 + rr];
+                ln += w * stat[q * 192 + 128 + rr];
+                const float4* x = reinterpret_cast<const float4*>(rows_of(q) + rr * OLD + cc);
+                const float4 u = x[0], v = x[1];
+                y[0] += w * u.x; y[1] += w * u.y; y[2] += w * u.z; y[3] += w * u.w;
+                y[4] += w * v.x; y[5] += w * v.y; y[6] += w * v.z; y[7] += w * v.w;
+            }
+            const float inv = ln > 0.f ? 1.f / ln : 0.f;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) y[e] *= inv;
+            const int64_t at = ((int64_t)b * a.H + h) * N + row;
+            if (a.lse != nullptr && cc == 0) a.lse[at] = ls > 0.f ? (mx + log2f(ls)) * 0.69314718055994531f : 0.f;
+            if (a.o_f32 != nullptr) {
+                float4* dst = reinterpret_cast<float4*>(a.o_f32 + at * D + cc);
+                dst[0] = make_float4(y[0], y[1], y[2], y[3]);
+                dst[1] = make_float4(y[4], y[5], y[6], y[7]);
+            }
+            *reinterpret_cast<uint4*>(a.o + b * a.so.sb + h * a.so.sh + (int64_t)row * a.so.sn + cc) = float8_to_bf16x8(y);
+        }
+        return;
     }
     const float inv[2] = {lr[0] > 0.f ? 1.f / lr[0] : 0.f, lr[1] > 0.f ? 1.f / lr[1] : 0.f};
     const int row_g[2] = {I * USV_BLOCK + warp * 16 + g, I * USV_BLOCK + warp * 16 + g + 8};
@@ -253,7 +320,7 @@ __global__ void __launch_bounds__(128) attn_mma_kernel(const AttnArgs a) {
             if (!__syncthreads_or(mine < blocks && a.work_flags[mine] != 0)) continue;
             for (int64_t i = i0; i < blocks && i < i0 + 128 * (int64_t)stride; i += stride)
                 if (a.work_flags[i] != 0) {
-                    attn_mma_block<D>(a, (int)i, smem_raw);
+                    attn_mma_block<D, 1, 2>(a, (int)i, smem_raw);
                     __syncthreads();
                 }
         }
@@ -262,14 +329,38 @@ __global__ void __launch_bounds__(128) attn_mma_kernel(const AttnArgs a) {
     if (a.work_list == nullptr) {
         // the words behind the sticky status word (fallback count, work counter, ...) start at zero
         if (blockIdx.x == 0 && threadIdx.x < (WS_HEADER - 4) / 4) a.status[1 + threadIdx.x] = 0u;
-        attn_mma_block<D>(a, blockIdx.x, smem_raw);
+        attn_mma_block<D, 1, 2>(a, blockIdx.x, smem_raw);
         return;
     }
     const int n = *a.work_count;
     for (int i = blockIdx.x; i < n; i += gridDim.x) {
-        attn_mma_block<D>(a, a.work_list[i], smem_raw);
+        attn_mma_block<D, 1, 2>(a, a.work_list[i], smem_raw);
         __syncthreads();
     }
+}
+
+// One CTA per query block, G groups.  A call of few blocks takes as long as one walk over a list: loads, two short chains of
+// MMAs and the softmax between them, 1.3 us a key block at D = 64; G of them run side by side.
+template <int D, int G, int NBUF>
+__global__ void __launch_bounds__(128 * G) attn_split_kernel(const AttnArgs a) {
+    dep_sync();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (blockIdx.x == 0 && threadIdx.x < (WS_HEADER - 4) / 4) a.status[1 + threadIdx.x] = 0u;   // (as attn_mma_kernel does)
+    attn_mma_block<D, G, NBUF>(a, blockIdx.x, smem_raw);
+}
+
+template <int D, int G, int NBUF>
+static int launch_split(const AttnArgs& a, cudaStream_t st) {
+    constexpr size_t smem = (size_t)MmaSmem<D>::TILE * (1 + 2 * G * NBUF) * sizeof(__nv_bfloat16) + G * 192 * sizeof(float);
+    static_assert(smem <= 232448, "shared memory budget");
+    cudaFuncSetAttribute(attn_split_kernel<D, G, NBUF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    launch_dep_smem(attn_split_kernel<D, G, NBUF>, dim3((unsigned)(a.B * a.H * a.NB)), dim3(128 * G), smem, st, a);
+    USV_CHECK_LAUNCH("attn_split_kernel");
+    return USV_OK;
+}
+
+int launch_attn_split(const AttnArgs& a, int most, cudaStream_t st) {
+    return most <= 4 ? launch_split<64, 4, 1>(a, st) : launch_split<64, 4, 2>(a, st);
 }
 
 int launch_attn_mma(const AttnArgs& a, int d, cudaStream_t st) {

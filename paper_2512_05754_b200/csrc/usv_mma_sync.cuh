@@ -35,13 +35,13 @@ __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t* r, const void* smem_
 }
 
 // Copies rows [row0, row0+64) of one [N, D] matrix (token stride sn) into a padded smem tile;
-// rows at or beyond N are zero-filled without touching memory.
-template <int D>
+// rows at or beyond N are zero-filled without touching memory.  128 threads take part (a group of them), or 128 G.
+template <int D, int G = 1>
 __device__ __forceinline__ void load_tile(__nv_bfloat16* dst, const __nv_bfloat16* src, int64_t sn,
                                           int row0, int N) {
     constexpr int LD = MmaSmem<D>::LD;
     constexpr int VPR = D / 8;  // 16-byte vectors per row
-    for (int idx = threadIdx.x; idx < USV_BLOCK * VPR; idx += 128) {
+    for (int idx = G == 1 ? threadIdx.x & 127 : threadIdx.x; idx < USV_BLOCK * VPR; idx += 128 * G) {
         const int r = idx / VPR, c = idx % VPR;
         const int row = row0 + r;
         const int ok = row < N;
