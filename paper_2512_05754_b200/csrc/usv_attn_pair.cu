@@ -29,8 +29,8 @@
 //   warps 0-15   four softmax warpgroups sharing the 128 rows (thread r of every group <-> TMEM
 //                lane r <-> query row r).  Group g works on the tiles of running parity g >> 1
 //                and there on key block g & 1 of the tile (64 logit columns).
-//   warps 16-19  output: thread e <-> query row e reads the finished O row out of TMEM, hands the
-//                accumulator back and stores from registers (to o, or, with the
+//   warps 16-19  output: thread e <-> query row e reads the finished O row out of TMEM a quarter at
+//                a time, hands the accumulator back and stores from registers (to o, or, with the
 //                unmerge folded in, to every original token that reads the row back), while the
 //                softmax groups are already in the next item.  Warp 16 is the scout too: it draws items two
 //                ahead, copies their key-block lists into ring slots in shared memory and publishes them.  (That takes
@@ -41,7 +41,7 @@
 //   warp 22      V producer (TMA).
 //   warp 23      S issuer.
 // The CTA is launched with 80 registers per thread and the roles re-divide them at their start
-// (setmaxnreg): softmax and output (a whole row as bf16 pairs) need more than the launch allows for 768 threads, the others less.
+// (setmaxnreg): the softmax loop and the scout need more than the launch allows for 768 threads, the others less.
 //
 // TMEM holds O and THREE S buffers; running tile g uses buffer g mod 3.  The weights P are
 // written back, as bf16 pairs, into the columns their logits came from, so a buffer goes
@@ -141,24 +141,6 @@ __device__ __forceinline__ const int* item_list(const int* hdr) {
     return hdr[I_NU] <= LCAP ? hdr + 16
                              : reinterpret_cast<const int*>(((unsigned long long)(unsigned)hdr[I_LIST_HI] << 32) |
                                                             (unsigned)hdr[I_LIST_LO]);
-}
-
-// Four lanes of a warp, four pieces of 16 bytes each: lane i of the four gets piece i of all four.
-__device__ __forceinline__ void quad_transpose(uint32_t* x, int lane) {
-#pragma unroll
-    for (int o = 1; o < 4; o <<= 1) {
-        const bool up = lane & o;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            if (i & o) continue;
-#pragma unroll
-            for (int w = 0; w < 4; ++w) {
-                const uint32_t got = __shfl_xor_sync(0xffffffffu, up ? x[4 * i + w] : x[4 * (i + o) + w], o);
-                if (up) x[4 * i + w] = got;
-                else x[4 * (i + o) + w] = got;
-            }
-        }
-    }
 }
 
 // DIRECT: no pairing plan (see attn_pair_direct).  Neighbouring query blocks share an item, the CTAs take the
@@ -436,24 +418,34 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
                     pq = make_int2(2 * pair, 2 * pair + 1 < NB ? 2 * pair + 1 : -1);
                     const int kh = a.k_per_head[h];
                     const int32_t* row = a.sel + (((int64_t)b * a.H + h) * NB + pq.x) * a.kmax;
-                    uint32_t ba = 0, bb = 0;
-                    for (int i0 = 0; i0 < kh; i0 += 32) {
-                        const int i = i0 + lane;
-                        const int ea = i < kh ? __ldg(row + i) : -1, eb = i < kh && pq.y >= 0 ? __ldg(row + a.kmax + i) : -1;
-                        const int m = min(32, kh - i0);
+                    if (kh == 1) {
+                        // one or two entries
+                        const int ja = __ldg(row), jb = pq.y >= 0 ? __ldg(row + a.kmax) : -1;
+                        const bool va = ja >= 0 && ja < NB, vb = jb >= 0 && jb < NB, same = va && vb && ja == jb;
+                        const int first = va && !(vb && jb < ja) ? (ja << 2) | 1 | (same ? 2 : 0) : (jb << 2) | 2;
+                        const int second = (first & 1) ? (jb << 2) | 2 : (ja << 2) | 1;
+                        nU = same ? 1 : (int)va + (int)vb;
+                        if (lane < 2) hdr[16 + lane] = lane == 0 ? first : second;
+                    } else {
+                        uint32_t ba = 0, bb = 0;
+                        for (int i0 = 0; i0 < kh; i0 += 32) {
+                            const int i = i0 + lane;
+                            const int ea = i < kh ? __ldg(row + i) : -1, eb = i < kh && pq.y >= 0 ? __ldg(row + a.kmax + i) : -1;
+                            const int m = min(32, kh - i0);
 #pragma unroll 4
-                        for (int q = 0; q < m; ++q) {
-                            const int ja = __shfl_sync(0xffffffffu, ea, q), jb = __shfl_sync(0xffffffffu, eb, q);
-                            if (ja >= 0 && ja < NB && (ja >> 5) == lane) ba |= 1u << (ja & 31);
-                            if (jb >= 0 && jb < NB && (jb >> 5) == lane) bb |= 1u << (jb & 31);
+                            for (int q = 0; q < m; ++q) {
+                                const int ja = __shfl_sync(0xffffffffu, ea, q), jb = __shfl_sync(0xffffffffu, eb, q);
+                                if (ja >= 0 && ja < NB && (ja >> 5) == lane) ba |= 1u << (ja & 31);
+                                if (jb >= 0 && jb < NB && (jb >> 5) == lane) bb |= 1u << (jb & 31);
+                            }
                         }
-                    }
-                    uint32_t u = ba | bb;
-                    const int incl = warp_incl_scan(__popc(u));
-                    nU = __shfl_sync(0xffffffffu, incl, 31);
-                    for (int at = 16 + incl - __popc(u); u != 0; u &= u - 1) {
-                        const int bit = __ffs(u) - 1;
-                        hdr[at++] = ((lane * 32 + bit) << 2) | ((ba >> bit) & 1u) | (((bb >> bit) & 1u) << 1);
+                        uint32_t u = ba | bb;
+                        const int incl = warp_incl_scan(__popc(u));
+                        nU = __shfl_sync(0xffffffffu, incl, 31);
+                        for (int at = 16 + incl - __popc(u); u != 0; u &= u - 1) {
+                            const int bit = __ffs(u) - 1;
+                            hdr[at++] = ((lane * 32 + bit) << 2) | ((ba >> bit) & 1u) | (((bb >> bit) & 1u) << 1);
+                        }
                     }
                     __syncwarp();
                 } else {
@@ -539,10 +531,9 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
 #pragma unroll
                 for (int q = 0; q < NWG; ++q) lx += sums[q * 128 + e];
             }
-            const float nref = has_ref ? s_refv[slot * 128 + e] : 0.f;
-            if (!mbar_wait(bar(F::B_OFULL), m & 1, s_abort, a.status, 0x200)) break;
-            fence_after();
             if (F::SUM_COL) {
+                if (!mbar_wait(bar(F::B_OFULL), m & 1, s_abort, a.status, 0x200)) break;
+                fence_after();
                 uint32_t sum;
                 tmem_ld1(lane_base + TO + D, sum);
                 tmem_wait_ld();
@@ -550,27 +541,61 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
             } else {
                 l = lx;
             }
+            const float nref = has_ref ? s_refv[slot * 128 + e] : 0.f;
             const bool in_range = l > 7.9e-31f && l < 1.2e30f;   // ~[2^-100, 2^100]
             uint64_t z0 = 0, z1 = 0;   // four fp32 sums that stay 0 unless a value of the row is not finite
             const float inv = l > 0.f ? 1.0f / l : 0.f;
-            // The row leaves TMEM a quarter (32 columns) at a time and is kept as bf16 pairs, so that the accumulator and the
-            // ring slot go back before anything is stored: the next item's first P.V waits for them (stored a quarter at a
-            // time in between, they came back 4000 to 7000 cycles later).
+            if (SUM != SUM_NONE && a.lse != nullptr && live)
+                a.lse[((int64_t)ib * a.H + ih) * N + row] = (log2f(lx) - nref) * 0.69314718055994531f;
+            if (!F::SUM_COL) {
+                if (!mbar_wait(bar(F::B_OFULL), m & 1, s_abort, a.status, 0x200)) break;
+                fence_after();
+            }
+            // The row leaves TMEM a quarter (32 columns) at a time and is stored from registers; the
+            // accumulator and the ring slot go back as soon as the last quarter has been read.
             float* o32 = (a.o_f32 != nullptr && live) ? a.o_f32 + (((int64_t)ib * a.H + ih) * N + row) * D : nullptr;
-            uint32_t pk[D / 2];
-#pragma unroll
+            __nv_bfloat16* O = a.o + ib * a.so.sb + ih * a.so.sh + (int64_t)row * a.so.sn;
+            // fused unmerge: the row goes to every original token that reads it back
+            int u0 = 0, u1 = 0;
+            if (a.y != nullptr && live) {
+                u0 = a.unmerge_off[(int64_t)ib * (N + 1) + row];
+                u1 = a.unmerge_off[(int64_t)ib * (N + 1) + row + 1];
+            }
+#pragma unroll 1
             for (int qd = 0; qd < D / 32; ++qd) {
                 uint32_t r0[32];
                 tmem_ld32(lane_base + TO + qd * 32, r0);
-                tmem_wait_ld32(r0);
+                tmem_wait_ld();
 #pragma unroll
                 for (int j = 0; F::CHECK_FINITE && j < 8; ++j) {
                     z0 = fma_f32x2(pack_f32x2(__uint_as_float(r0[4 * j]), __uint_as_float(r0[4 * j + 1])), 0ull, z0);
                     z1 = fma_f32x2(pack_f32x2(__uint_as_float(r0[4 * j + 2]), __uint_as_float(r0[4 * j + 3])), 0ull, z1);
                 }
-#pragma unroll
-                for (int j = 0; j < 16; ++j)
-                    pk[qd * 16 + j] = pack_bf16x2(__uint_as_float(r0[2 * j]) * inv, __uint_as_float(r0[2 * j + 1]) * inv);
+                if (qd == D / 32 - 1) {
+                    // A row whose sum left the safe range, or that is not finite (see CHECK_FINITE): the
+                    // first row of a query block to notice hands the block to the exact kernel, which
+                    // keeps query blocks apart.
+                    bool finite = true;
+                    if (F::CHECK_FINITE) {
+                        float za, zb;
+                        unpack_f32x2(add_f32x2(z0, z1), za, zb);
+                        finite = za + zb == 0.f;
+                    }
+                    if (DIRECT) {
+                        const bool any = __any_sync(0xffffffffu, live && !(in_range && finite));
+                        if (lane == 0 && iq >= 0)
+                            reinterpret_cast<uint8_t*>(a.fallback_list)[2 * ((int64_t)ibh * NB + iq) + (warp & 1)] = any;
+                    } else if (live && !(in_range && finite) && a.fallback_list != nullptr &&
+                               atomicExch(&s_flag[slot * 2 + side], 1) == 0) {
+                        a.fallback_list[atomicAdd(a.fallback_count, 1)] = ibh * NB + iq;
+                    }
+                    fence_before();
+                    __syncwarp();
+                    if (lane == 0) {
+                        mbar_arrive(bar(F::B_OFREE));
+                        mbar_arrive(bar(F::B_IFREE + slot));
+                    }
+                }
                 if (o32 != nullptr) {
 #pragma unroll
                     for (int j = 0; j < 8; ++j)
@@ -578,56 +603,25 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
                             make_float4(__uint_as_float(r0[4 * j]) * inv, __uint_as_float(r0[4 * j + 1]) * inv,
                                         __uint_as_float(r0[4 * j + 2]) * inv, __uint_as_float(r0[4 * j + 3]) * inv);
                 }
-            }
-            // A row whose sum left the safe range, or that is not finite (see CHECK_FINITE): the
-            // first row of a query block to notice hands the block to the exact kernel, which
-            // keeps query blocks apart.
-            bool finite = true;
-            if (F::CHECK_FINITE) {
-                float za, zb;
-                unpack_f32x2(add_f32x2(z0, z1), za, zb);
-                finite = za + zb == 0.f;
-            }
-            if (DIRECT) {
-                const bool any = __any_sync(0xffffffffu, live && !(in_range && finite));
-                if (lane == 0 && iq >= 0)
-                    reinterpret_cast<uint8_t*>(a.fallback_list)[2 * ((int64_t)ibh * NB + iq) + (warp & 1)] = any;
-            } else if (live && !(in_range && finite) && a.fallback_list != nullptr &&
-                       atomicExch(&s_flag[slot * 2 + side], 1) == 0) {
-                a.fallback_list[atomicAdd(a.fallback_count, 1)] = ibh * NB + iq;
-            }
-            fence_before();
-            __syncwarp();
-            if (lane == 0) {
-                mbar_arrive(bar(F::B_OFREE));
-                mbar_arrive(bar(F::B_IFREE + slot));
-            }
-            if (SUM != SUM_NONE && a.lse != nullptr && live)
-                a.lse[((int64_t)ib * a.H + ih) * N + row] = (log2f(lx) - nref) * 0.69314718055994531f;
-            if (a.y == nullptr) {
-                // Four lanes turn their four rows of 64 bytes into pieces of 16 bytes of all four: a store of the warp then
-                // covers eight rows of 64 consecutive bytes, not 16 bytes of 32.
-                const int rw = iq * USV_BLOCK + ((warp & 1) * 32 + (lane & ~3));
-                __nv_bfloat16* O = a.o + ib * a.so.sb + ih * a.so.sh + (lane & 3) * 8;
-#pragma unroll
-                for (int qd = 0; qd < D / 32; ++qd) {
-                    uint32_t* x = pk + qd * 16;
-                    quad_transpose(x, lane);
+                if (live) {
+                    uint4 pk[4];
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
-                        if (iq >= 0 && rw + i < N)
-                            *reinterpret_cast<uint4*>(O + (int64_t)(rw + i) * a.so.sn + qd * 32) =
-                                make_uint4(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]);
-                }
-            } else if (live) {
-                // fused unmerge: the row goes to every original token that reads it back
-                const int u0 = a.unmerge_off[(int64_t)ib * (N + 1) + row], u1 = a.unmerge_off[(int64_t)ib * (N + 1) + row + 1];
-                for (int u = u0; u < u1; ++u) {
-                    const int tok = a.unmerge_idx[(int64_t)ib * a.N_full + u];
-                    __nv_bfloat16* Y = a.y + ((int64_t)ib * a.N_full + tok) * ((int64_t)a.H * D) + ih * D;
+                        pk[i] = make_uint4(pack_bf16x2(__uint_as_float(r0[8 * i]) * inv, __uint_as_float(r0[8 * i + 1]) * inv),
+                                           pack_bf16x2(__uint_as_float(r0[8 * i + 2]) * inv, __uint_as_float(r0[8 * i + 3]) * inv),
+                                           pack_bf16x2(__uint_as_float(r0[8 * i + 4]) * inv, __uint_as_float(r0[8 * i + 5]) * inv),
+                                           pack_bf16x2(__uint_as_float(r0[8 * i + 6]) * inv, __uint_as_float(r0[8 * i + 7]) * inv));
+                    if (a.y == nullptr) {
 #pragma unroll
-                    for (int i = 0; i < D / 8; ++i)
-                        *reinterpret_cast<uint4*>(Y + 8 * i) = make_uint4(pk[4 * i], pk[4 * i + 1], pk[4 * i + 2], pk[4 * i + 3]);
+                        for (int i = 0; i < 4; ++i) *reinterpret_cast<uint4*>(O + qd * 32 + 8 * i) = pk[i];
+                    } else {
+                        for (int u = u0; u < u1; ++u) {
+                            const int tok = a.unmerge_idx[(int64_t)ib * a.N_full + u];
+                            __nv_bfloat16* Y = a.y + ((int64_t)ib * a.N_full + tok) * ((int64_t)a.H * D) + ih * D + qd * 32;
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) *reinterpret_cast<uint4*>(Y + 8 * i) = pk[i];
+                        }
+                    }
                 }
             }
         }
@@ -806,7 +800,7 @@ bool attn_pair_supported(const AttnArgs& a, int d) {
 // 38 k 81 / 93.  (Beyond 1024 blocks or lists of 256 the scout's registers and ring slots do not hold a union.)
 // With short lists the scout's work per item counts, which bounds the number of blocks too, lower where a
 // tile takes longer: D = 128, 3 heads x 220 blocks, keep 11 45.1 / 40.7, 24 x 72, keep 4 47.2 / 48.3, 12 x 120,
-// keep 6 48.3 / 47.2, 16 x 120, keep 3 48.0 / 51.4, 24 x 317, keep 1 114 / 140; D = 64, 24 x 72, keep 4 38.8 / 35.4.
+// keep 6 48.3 / 47.2, 16 x 120, keep 3 48.0 / 51.4, D = 64, 24 x 72, keep 4 38.8 / 35.4.
 bool attn_pair_direct(const AttnArgs& a, int d) {
     constexpr int64_t DIRECT_WORK = 10000;
     const int64_t most_blocks = d == 64 ? 1800 : 1000;
@@ -816,6 +810,9 @@ bool attn_pair_direct(const AttnArgs& a, int d) {
         kept += a.k_per_head[h];
         most = a.k_per_head[h] > most ? a.k_per_head[h] : most;
     }
+    // Single kept blocks need neither bitmaps nor pairs, whatever their number: 24 heads x 100 blocks, D = 128, 47.2 / 42.0,
+    // 24 x 317 107 / 88, 40 x 300 154 / 137.
+    if (a.y == nullptr && most == 1) return true;
     return a.y == nullptr && a.NB <= 1024 && 2 * most <= pr::LCAP && (int64_t)a.B * a.H * a.NB <= most_blocks &&
            (int64_t)a.B * a.NB * kept <= DIRECT_WORK;
 }
