@@ -792,29 +792,30 @@ bool attn_pair_supported(const AttnArgs& a, int d) {
     return (d == 64 || d == 128) && a.NB <= pr::MAX_NB && a.work_counter != nullptr;
 }
 
-// The pairing plan takes 8 to 10 us, partly hidden, before the first query block is computed, and saves a
-// tenth to a sixth of the attention kernel's work: it does not pay in small calls, here those that keep at
-// most DIRECT_WORK key blocks over all query blocks.  Whole calls, us, with the plan / without it, at key
-// blocks kept: D = 128, 2.7 k 29.1 / 26.4, 3.5 k 32.3 / 26.7, 5 k (two heads of 160 blocks) 42.2 / 35.2, 7 k
-// 40.8 / 39.5, 12 k 51.4 / 50.8, 14 k 55.5 / 61.0, 24 k 76 / 80; D = 64, 4.6 k 30.3 / 25.4, 14 k 45.8 / 47.4,
-// 38 k 81 / 93.  (Beyond 1024 blocks or lists of 256 the scout's registers and ring slots do not hold a union.)
-// With short lists the scout's work per item counts, which bounds the number of blocks too, lower where a
-// tile takes longer: D = 128, 3 heads x 220 blocks, keep 11 45.1 / 40.7, 24 x 72, keep 4 47.2 / 48.3, 12 x 120,
-// keep 6 48.3 / 47.2, 16 x 120, keep 3 48.0 / 51.4, D = 64, 24 x 72, keep 4 38.8 / 35.4.
+// The pairing plan takes 10 to 15 us before the first query block is computed, and saves a tenth to a quarter of the attention
+// kernel's work: it does not pay in small calls.  With short lists the scout's work per item counts, which bounds the number of
+// blocks too.  Whole calls on video inputs, us, with the plan / without it, at key blocks kept over all query blocks:
+//   D = 128: 2.7 k 28.3 / 21.0, 6.8 k (2280 blocks) 49.3 / 43.3, 10 k (684) 46.8 / 40.6, 11 k (2256) 60.4 / 58.6, 14 k (1952)
+//     66.9 / 64.4, 14 k (2280) 65.3 / 67.1, 15 k (1824) 62.1 / 64.1, 19 k (1464) 73.4 / 70.8, 19 k (1760) 79.3 / 76.6, 21 k (1128) 71.4 / 65.5,
+//     22 k (2256) 86.4 / 89.9, 27 k (1024) 92.4 / 96.9, 30 k (976) 94.6 / 101.5, 37 k (1464) 112.9 / 119.4
+//   D = 64: 2.7 k 24.1 / 17.3, 8.2 k 35.6 / 30.5, 14 k (4560 blocks) 62.8 / 66.3, 19 k 51.4 / 44.6, 22 k (2256) 56.0 / 54.5,
+//     37 k (1464) 74.9 / 71.2, 38 k (2928) 86.7 / 89.6, 39 k (1760) 79.0 / 77.6, 43 k (2256) 82.5 / 86.3, 58 k (2640) 115.8 / 127.6
+// (Beyond 1024 blocks or lists of 256 the scout's registers and ring slots do not hold a union.)
 bool attn_pair_direct(const AttnArgs& a, int d) {
-    constexpr int64_t DIRECT_WORK = 10000;
-    const int64_t most_blocks = d == 64 ? 1800 : 1000;
     int64_t kept = 0;
     int most = 0;
     for (int h = 0; h < a.H; ++h) {
         kept += a.k_per_head[h];
         most = a.k_per_head[h] > most ? a.k_per_head[h] : most;
     }
+    const int64_t blocks = (int64_t)a.B * a.H * a.NB;
+    kept *= (int64_t)a.B * a.NB;
     // Single kept blocks need neither bitmaps nor pairs, whatever their number: 24 heads x 100 blocks, D = 128, 47.2 / 42.0,
     // 24 x 317 107 / 88, 40 x 300 154 / 137.
     if (a.y == nullptr && most == 1) return true;
-    return a.y == nullptr && a.NB <= 1024 && 2 * most <= pr::LCAP && (int64_t)a.B * a.H * a.NB <= most_blocks &&
-           (int64_t)a.B * a.NB * kept <= DIRECT_WORK;
+    const bool few = d == 64 ? (kept <= 36000 && blocks <= 1800) || (kept <= 24000 && blocks <= 2400)
+                             : (kept <= 20000 && blocks <= 1700) || (kept <= 13000 && blocks <= 2300);
+    return a.y == nullptr && a.NB <= 1024 && 2 * most <= pr::LCAP && few;
 }
 
 template <int D, bool DIRECT, bool LSE>
