@@ -5,6 +5,7 @@
 //                   rows of a block.  It also writes the three bf16 planes
 //                   (mean = hi + mid + lo) that the tensor-core score kernel multiplies, so the
 //                   fp32 means are not read back for a separate split pass.
+//   scores_cluster_kernel : pooling and scores of short sequences in one launch.
 //   scores_small_kernel : the scores of small calls, fp32 CUDA cores (both head widths).
 //   scores_kernel : fp32 CUDA-core NT GEMM per (b,h), 64x64 output tile, 4x4 per thread, for the entry
 //                   point without caller scratch, which has no room for the planes.
@@ -236,6 +237,126 @@ __global__ void __launch_bounds__(256) scores_small_kernel(const float* __restri
         }
 }
 
+// Pooling and scores of short sequences in one kernel: a cluster of CLC CTAs per (b, h).  Each pools its share of the query and of
+// the key blocks (sums in the order of pool_kernel), writes its key means into the shared memory of
+// all of them, and after one cluster barrier computes its query rows of scores (features in ascending order, as above).  Two
+// launches, a round trip of the means through the L2 and the wait between them are saved.
+constexpr int CLC = 8, CL_MAX = 48;   // CTAs of a cluster; blocks of the longest sequence
+
+template <int D, int G>
+constexpr size_t cluster_smem() {     // key means, the CTA's query means, partial sums of two rounds of blocks
+    return (size_t)(CL_MAX + CL_MAX / CLC) * (D + 4) * 4 + 2 * (size_t)G * (128 / (D / 8)) * (D + 4) * 4;
+}
+
+// G groups of 128 threads, each with a block at a time; PER CTAs an SM
+template <int D, int G, int PER>
+__global__ void __launch_bounds__(128 * G, PER) __cluster_dims__(CLC, 1, 1) scores_cluster_kernel(const PoolArgs a, float* __restrict__ scores, float scale) {
+    extern __shared__ __align__(16) float s_mem[];
+    constexpr int LD = D + 4, TPR = D / 8, RPI = 128 / TPR, ITERS = USV_BLOCK / RPI;
+    float* s_k = s_mem;                          // [CL_MAX][LD]
+    float* s_q = s_k + CL_MAX * LD;              // [CL_MAX / CLC][LD]
+    float* s_red = s_q + CL_MAX / CLC * LD;      // [2 buffers][2 blocks][RPI][LD]
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // (waited for before anything is written to a neighbour)
+    dep_sync();
+    const int rank = blockIdx.x, bh = blockIdx.y;
+    const int b = bh / a.H, h = bh % a.H;
+    const int half = threadIdx.x >> 7, tid = threadIdx.x & 127;
+    const int col = tid % TPR, rg = tid / TPR;
+    const int per_q = (a.NB[0] + CLC - 1) / CLC, per_k = (a.NB[1] + CLC - 1) / CLC;
+    const int nq = max(0, min(per_q, a.NB[0] - rank * per_q)), nk = max(0, min(per_k, a.NB[1] - rank * per_k));
+    const int n = nk + nq;                       // the CTA's blocks, keys first
+    auto load = [&](int i, uint4* v) {
+        const int which = i < nk ? 1 : 0, I = i < nk ? rank * per_k + i : rank * per_q + i - nk;
+        const __nv_bfloat16* base = a.x[which] + b * a.sb[which] + h * a.sh[which] + (int64_t)col * 8;
+        const int nvalid = i < n ? min(USV_BLOCK, a.N[which] - I * USV_BLOCK) : 0;
+#pragma unroll
+        for (int it = 0; it < ITERS; ++it) {
+            const int r = it * RPI + rg;
+            v[it] = r < nvalid ? __ldg(reinterpret_cast<const uint4*>(base + (int64_t)(I * USV_BLOCK + r) * a.sn[which])) : make_uint4(0, 0, 0, 0);
+        }
+    };
+    uint4 v[ITERS], vn[ITERS];
+    load(half, v);
+    bool first = true;
+    int buf = 0;
+    for (int i0 = 0; i0 < n; i0 += G, buf ^= 1) {
+        const int i = i0 + half;
+        if (i0 + G < n) load(i + G, vn);
+        float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+#pragma unroll
+        for (int it = 0; it < ITERS; ++it) {
+            float f[8];
+            bf16x8_to_float(v[it], f);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[e] += f[e];
+        }
+        float* rd = s_red + (buf * G + half) * RPI * LD;   // two buffers: one barrier a round is enough
+#pragma unroll
+        for (int e = 0; e < 8; ++e) rd[rg * LD + col * 8 + e] = acc[e];
+        __syncthreads();
+        if (first) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        first = false;
+        if (tid < D && i < n) {
+            const int which = i < nk ? 1 : 0, I = i < nk ? rank * per_k + i : rank * per_q + i - nk;
+            const int nvalid = min(USV_BLOCK, a.N[which] - I * USV_BLOCK);
+            float s = 0.f;
+#pragma unroll
+            for (int g = 0; g < RPI; ++g) s += rd[g * LD + tid];
+            const float mean = s / (float)nvalid;
+            if (which == 0) {
+                s_q[(i - nk) * LD + tid] = mean;
+            } else {
+                const uint32_t at = (uint32_t)__cvta_generic_to_shared(s_k + I * LD + tid);
+#pragma unroll
+                for (int c = 0; c < CLC; ++c) {
+                    uint32_t to;
+                    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(to) : "r"(at), "r"(c));
+                    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(to), "f"(mean) : "memory");
+                }
+            }
+        }
+#pragma unroll
+        for (int it = 0; it < ITERS; ++it) v[it] = vn[it];
+    }
+    if (first) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    const int NBk = a.NB[1];
+    float* out = scores + ((int64_t)bh * a.NB[0] + rank * per_q) * NBk;
+    for (int i = threadIdx.x; i < nq * NBk; i += 128 * G) {
+        const int I = i / NBk, J = i - I * NBk;
+        const float4* x = reinterpret_cast<const float4*>(s_q + I * LD);
+        const float4* y = reinterpret_cast<const float4*>(s_k + J * LD);
+        float acc = 0.f;
+#pragma unroll 8
+        for (int e = 0; e < D / 4; ++e) {
+            const float4 av = x[e], bv = y[e];
+            acc = fmaf(av.w, bv.w, fmaf(av.z, bv.z, fmaf(av.y, bv.y, fmaf(av.x, bv.x, acc))));
+        }
+        out[i] = acc * scale;
+    }
+}
+
+template <int D, int G, int PER>
+static int launch_scores_cluster(const PoolArgs& a, int BH, float* scores, float scale, cudaStream_t st) {
+    constexpr size_t smem = cluster_smem<D, G>();
+    cudaError_t e = cudaFuncSetAttribute(scores_cluster_kernel<D, G, PER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return fail(USV_ERR_CUDA, "block_scores: smem attribute: %s", cudaGetErrorString(e));
+    launch_dep_smem(scores_cluster_kernel<D, G, PER>, dim3(CLC, BH), dim3(128 * G), smem, st, a, scores, scale);
+    USV_CHECK_LAUNCH("scores_cluster_kernel");
+    return USV_OK;
+}
+
+// Calls that are better off with it, as groups of 128 threads a CTA (0: none): a cluster has an eighth of a (b, h)'s blocks a CTA,
+// so sequences are short, and its CTAs are resident together.  Whole calls, us, two kernels / this one: d = 64, 2 heads x 16 blocks
+// 5.4 / 3.0, 12 x 32 5.3 / 5.0, 12 x 48 6.1 / 7.1, 24 x 16 5.3 / 3.8, 40 x 16 5.8 / 5.2; d = 128, 2 x 16 5.4 / 3.7, 12 x 32 6.6 / 5.3,
+// 12 x 48 8.2 / 7.0, 12 x 64 8.0 / 9.0, 24 x 16 7.0 / 5.0, 24 x 32 7.6 / 7.5, 40 x 16 8.0 / 5.7, 40 x 32 9.1 / 9.9, 80 x 16 9.0 / 10.4.
+static int cluster_groups(int BH, int NBq, int NBk, int d, int sms) {
+    const int ctas = BH * CLC, nb = NBq > NBk ? NBq : NBk;
+    if (ctas <= sms && nb <= (d == 128 ? CL_MAX : 32)) return 4;
+    if (ctas <= 2 * sms && nb <= (d == 128 ? 16 : 32)) return 4;
+    return ctas <= (d == 128 ? 3 : 4) * sms && nb <= 16 ? 2 : 0;
+}
+
 // The small form takes calls of at most this many 32 x 32 tiles.  Whole calls, us, with the tensor-core kernel / with
 // this one: d = 64, 12 heads x 32 blocks (12 tiles) 9.9 / 4.9, 24 x 64 (96) 11.7 / 7.2, 4 x 256 (256) 10.1 / 6.8, 2 x 512 (512)
 // 10.2 / 8.8, 12 x 220 (588) 13.6 / 12.4, 3 x 512 (768) 11.1 / 11.2; d = 128, in that order, 15.1 / 6.4, 18.6 / 10.8, 16.2 / 9.9,
@@ -296,12 +417,18 @@ extern "C" int usv_block_scores(int B, int H, int Nq, int Nk, int d, const void*
     int sms;
     if ((rc = sm_count(&sms)) != USV_OK) return rc;
     a.span = pool_span((int64_t)B * H * (NBq + NBk), sms);
+    const float sc = 1.0f / sqrtf((float)d);
+    const int groups = small ? cluster_groups(B * H, NBq, NBk, d, sms) : 0;
+    if (groups == 2)
+        return d == 128 ? launch_scores_cluster<128, 2, 2>(a, B * H, scores, sc, st) : launch_scores_cluster<64, 2, 2>(a, B * H, scores, sc, st);
+    if (groups == 4 && d == 64) return launch_scores_cluster<64, 4, 2>(a, B * H, scores, sc, st);
+    if (groups == 4)
+        return B * H * CLC <= sms ? launch_scores_cluster<128, 4, 1>(a, B * H, scores, sc, st) : launch_scores_cluster<128, 4, 2>(a, B * H, scores, sc, st);
     dim3 pg(ceil_div(NBq > NBk ? NBq : NBk, a.span), B * H, 2);
     if (d == 128) launch_dep(pool_kernel<128>, dim3(pg), dim3(128), 0, st, a);
     else launch_dep(pool_kernel<64>, dim3(pg), dim3(128), 0, st, a);
     USV_CHECK_LAUNCH("pool_kernel");
 
-    const float sc = 1.0f / sqrtf((float)d);
     if (small) {
         dim3 tg(ceil_div(NBk, SCT), ceil_div(NBq, SCT), B * H);
         if (d == 128) launch_dep(scores_small_kernel<128>, tg, dim3(256), 0, st, qbar, kbar, scores, NBq, NBk, sc);
