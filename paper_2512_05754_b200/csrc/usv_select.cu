@@ -360,6 +360,61 @@ __global__ void __launch_bounds__(W == 1 ? 256 : W * 32) select_kernel(const flo
         for (uint32_t m = take[q]; m; m &= m - 1) out[at++] = first + q * 32 + __ffs(m) - 1;
 }
 
+// Rows of at most 32 KPL scores (KPL = 1, 2), one warp each: every score is ranked against all the others, in a quarter of the
+// instructions of the search above and without its chain of dependent steps, which a call of few rows waits for.
+// Calls back to back, us, search / ranking: 384 rows of 32 3.2 / 1.7, 60 000 44.8 / 23.4, 684 of 57 3.5 / 2.8, 4560 of 57 4.9 / 5.2.
+template <int KPL>
+__global__ void __launch_bounds__(256) select_rank_kernel(const float* __restrict__ scores, int32_t* __restrict__ sel, int H,
+                                                          int NBq, int NBk, int kmax, const SelHeads heads, int64_t rows) {
+    dep_sync();
+    const int lane = threadIdx.x & 31;
+    const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (row >= rows) return;
+    const int k = min(heads.k[(row / NBq) % H], NBk);
+    int32_t* out = sel + row * kmax;
+    for (int t = k + lane; t < kmax; t += 32) out[t] = -1;
+    if (k == NBk) {   // keep everything (uniform over the row)
+#pragma unroll
+        for (int i = 0; i < KPL; ++i)
+            if (i * 32 + lane < NBk) out[i * 32 + lane] = i * 32 + lane;
+        return;
+    }
+    uint32_t key[KPL];
+    int rank[KPL];
+#pragma unroll
+    for (int i = 0; i < KPL; ++i) {
+        const int j = i * 32 + lane;
+        key[i] = j < NBk ? float_key_any(scores[row * NBk + j]) : 0u;   // 0: below every key
+        rank[i] = 0;
+    }
+#pragma unroll 8
+    for (int q = 0; q < 32; ++q) {
+        const uint32_t before = q < lane ? 1u : 0u;   // of equal scores the one of the lower index comes first
+#pragma unroll
+        for (int p = 0; p < KPL; ++p) {
+            const uint32_t other = __shfl_sync(0xffffffffu, key[p], q);
+#pragma unroll
+            for (int i = 0; i < KPL; ++i)
+                if (p == i ? other + before > key[i] : (p < i ? other >= key[i] : other > key[i])) ++rank[i];
+        }
+    }
+    int at = 0;
+#pragma unroll
+    for (int i = 0; i < KPL; ++i) {
+        const bool kept = i * 32 + lane < NBk && rank[i] < k;
+        const uint32_t m = __ballot_sync(0xffffffffu, kept);
+        if (kept) out[at + __popc(m & ((1u << lane) - 1u))] = i * 32 + lane;
+        at += __popc(m);
+    }
+}
+
+template <int KPL>
+static cudaError_t launch_rank(const float* scores, int32_t* sel, int H, int NBq, int NBk, int kmax, const SelHeads& heads,
+                               int64_t rows, cudaStream_t st) {
+    return launch_dep_smem(select_rank_kernel<KPL>, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, scores, sel, H, NBq, NBk, kmax,
+                           heads, rows);
+}
+
 template <int W, int KPL>
 static cudaError_t launch_select(const float* scores, int32_t* sel, int H, int NBq, int NBk, int kmax, const SelHeads& heads,
                                  int64_t rows, cudaStream_t st) {
@@ -414,10 +469,13 @@ extern "C" int usv_select_blocks(int B, int H, int NBq, int NBk, const float* sc
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     for (int h = 0; h < H; ++h) first_probes(heads, h, NBk);
 #define USV_SEL(W, KPL) launch_select<W, KPL>(scores, sel, H, NBq, NBk, kmax, heads, rows, st)
-    // The smallest form that holds the row.  One warp a row up to 544 scores (512 scores, 12 288 rows: 16.7 us,
+    // The smallest form that holds the row; up to 64 scores they are ranked, where a call of 33 to 64 has few rows (see
+    // select_rank_kernel).  One warp a row up to 544 scores (512 scores, 12 288 rows: 16.7 us,
     // 22.4 with two warps), then two: at 1182 scores and 47 280 rows two warps of 19 scores a lane take
     // 113 us and one warp of 37 119 us; at 3023 and 36 276 rows two warps take 186 us, four 239 us.
-    if (NBk <= 288) USV_SEL(1, 9);
+    if (NBk <= 32) launch_rank<1>(scores, sel, H, NBq, NBk, kmax, heads, rows, st);
+    else if (NBk <= 64 && rows <= 1500) launch_rank<2>(scores, sel, H, NBq, NBk, kmax, heads, rows, st);
+    else if (NBk <= 288) USV_SEL(1, 9);
     else if (NBk <= 352) USV_SEL(1, 11);
     else if (NBk <= 544) USV_SEL(1, 17);
     else if (NBk <= 832) USV_SEL(2, 13);
