@@ -43,6 +43,8 @@ struct AttnArgs {
 int launch_attn_mma(const AttnArgs& a, int d, cudaStream_t st);
 // the same for small calls at d = 64, four groups of warps a query block; most: longest list
 int launch_attn_split(const AttnArgs& a, int most, cudaStream_t st);
+// the same for lists of one block at d = 64
+int launch_attn_one(const AttnArgs& a, cudaStream_t st);
 bool attn_pair_supported(const AttnArgs& a, int d);
 // whether the call is too small for a pairing plan: a.pairs stays NULL, and fallback_list takes flags
 bool attn_pair_direct(const AttnArgs& a, int d);

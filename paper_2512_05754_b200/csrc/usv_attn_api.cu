@@ -92,20 +92,21 @@ static int sparse_attn_impl(int B, int H, int N, int d, const void* q, const usv
     // The status word (word 0) is sticky; everything behind it starts at zero (the first kernel of
     // either path does that itself: a memset between two kernels costs them their overlapped launch).
     //
-    // Short lists at d = 64 go to the mma.sync kernel alone: one launch, no pairing, ~3 us + 1.3 us per kept key block with
+    // Short lists at d = 64 go to the mma.sync kernels alone: one launch, no pairing, ~3 us + 1.3 us per kept key block with
     // all its CTAs resident at once, where the tcgen05 kernel takes 8 us before the lists matter (without a plan; 15 to 20
     // with one).  Calls, us, mma.sync / tcgen05: 128 query blocks, keep 1 4.8 / 8.4, 3 8.6 / 9.4, 4 10.4 / 9.9, 8 17.9 / 11.7; 384,
-    // keep 4 11.6 / 14.2, 6 15.9 / 16.1, 8 20.0 / 17.6; 512, keep 2 11.5 / 13.1, 3 15.0 / 13.9.  Single blocks go there again
-    // beyond the calls without a plan, whatever their number (2880, keep 1 27 / 44, 2 40 / 45, 3 54 / 47; 7608, keep 1 71 / 88, 2
-    // 104 / 91; 15 216, keep 1 137 / 157); between the two lines only keep 1 and 2 would gain (768, 8.9 / 15.1 and 13.3 / 17.1).
+    // keep 4 11.6 / 14.2, 6 15.9 / 16.1, 8 20.0 / 17.6; 512, keep 2 11.5 / 13.1, 3 15.0 / 13.9.
     const int64_t blocks = (int64_t)B * H * NB;
-    const bool small = d == 64 && ((kmx <= 4 && blocks <= 384) || (kmx == 1 && blocks > 1800));
+    const bool small = d == 64 && kmx <= 4 && blocks <= 384;
     // Where every query block has an SM to itself, four groups of warps walk its list side by side: 32 blocks, keep 4 8.3 / 7.0,
     // 8 11.4 / 9.4, 16 13.7 / 15.2; 128, keep 2 8.3 / 7.0, 4 11.6 / 7.2, 8 12.1 / 9.7; 100, keep 10 13.7 / 11.5; 256, keep 4 11.9 / 12.9
     // (other kernels / this one).  At d = 128 it never pays (32, keep 4 10.8 / 13.1).
     int sms;
     if ((rc = sm_count(&sms)) != USV_OK) return rc;
-    if (impl == 0 && d == 64 && y == nullptr && blocks <= sms && kmx <= 10) return launch_attn_split(a, kmx, st);
+    if (impl == 0 && d == 64 && blocks <= sms && kmx >= 2 && kmx <= 10) return launch_attn_split(a, kmx, st);
+    // Many single blocks at d = 64, mma.sync with two buffers / with one: 2400 23.2 / 21.5, 7608 73.3 / 69.7, 12 000 113 / 107 (the
+    // tcgen05 kernel: 26.3, 72.8, 110).
+    if (impl == 0 && d == 64 && blocks > 1800 && kmx == 1) return launch_attn_one(a, st);
     if (impl == 0 && !small && attn_pair_supported(a, d)) {
         int rc2;
         if (attn_pair_direct(a, d)) {

@@ -359,6 +359,25 @@ static int launch_split(const AttnArgs& a, cudaStream_t st) {
     return USV_OK;
 }
 
+// Lists of one block: nothing follows the first K and V tile, and without a second buffer twice as many CTAs share an SM.
+template <int D>
+__global__ void __launch_bounds__(128, 4) attn_one_kernel(const AttnArgs a) {
+    dep_sync();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (blockIdx.x == 0 && threadIdx.x < (WS_HEADER - 4) / 4) a.status[1 + threadIdx.x] = 0u;   // (as attn_mma_kernel does)
+    attn_mma_block<D, 1, 1>(a, blockIdx.x, smem_raw);
+}
+
+int launch_attn_one(const AttnArgs& a, cudaStream_t st) {
+    constexpr size_t smem = (size_t)MmaSmem<64>::TILE * 3 * sizeof(__nv_bfloat16);
+    static_assert(smem <= 48 * 1024, "no attribute needed");
+    const int64_t blocks = (int64_t)a.B * a.H * a.NB;
+    if (blocks > 2147483647LL) return fail(USV_ERR_UNSUPPORTED, "sparse_attn: too many query blocks");
+    launch_dep_smem(attn_one_kernel<64>, dim3((unsigned)blocks), dim3(128), smem, st, a);
+    USV_CHECK_LAUNCH("attn_one_kernel");
+    return USV_OK;
+}
+
 int launch_attn_split(const AttnArgs& a, int most, cudaStream_t st) {
     return most <= 4 ? launch_split<64, 4, 1>(a, st) : launch_split<64, 4, 2>(a, st);
 }
