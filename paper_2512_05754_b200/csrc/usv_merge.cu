@@ -329,83 +329,113 @@ __global__ void __launch_bounds__(1024) row_scan_kernel(int nB, const int32_t* _
 // candidates in ascending order at a time: the lanes split the descriptors, all candidates' rows are
 // requested before any is used, and the 32 sums over lanes are taken together (at every step a lane
 // hands half of its candidates over: 31 shuffles, where one candidate after the other takes 160), which
-// leaves candidate l in lane l.  Bound: issue slots and the reads of the candidates from L1.  2 x 16 380
-// sources, 27 candidates of 128: 73 -> 41 us (46 us without the bound on registers).  A window of the own block alone
-// has one candidate: whole merges of 118 800 tokens 410 us with one candidate after the other, 444 in groups of 32,
-// 416 so.
-template <int DM>
-__global__ void __launch_bounds__(256, 3) match_local_kernel(const float* __restrict__ mhat, Part p, int N, int nA,
+// leaves candidate l in lane l.  Rows of three destinations (the window reaches one block along x) are asked for from one address a
+// row, 30 candidates at a time.  Bound: the reads of the candidates from L1 (a third of the adds and shuffles less changed
+// nothing).  2 x 16 380 sources, 27 candidates of 128: 73 -> 41 us (46 us without the bound on registers).
+// A CTA goes through neighbouring sources, whose windows share most of their rows in L1, where there are several waves of
+// them.  Whole merges, us, one source a warp / rows of three and several sources: 2 x 16 380 122 / 120, 4 x 24 570 196 / 181, 65 480
+// 144 / 136, 8 x 17 550 239 / 224.  OWN: a window of the own block alone has one candidate and needs no registers for 32: 2 x 16 380
+// 63.6 / 57.0, 37 800 78.5 / 71.6, 2 x 59 400 222 / 189, 138 000 206 / 165.
+template <int DM, bool OWN>
+__global__ void __launch_bounds__(256, OWN ? 6 : 3) match_local_kernel(const float* __restrict__ mhat, Part p, int N, int nA,
                                                           int wt, int wh, int ww,
                                                           const int32_t* __restrict__ src_idx,
                                                           int32_t* __restrict__ jstar_s, float* __restrict__ u_s) {
     dep_sync();
     constexpr int V = DM / 32;   // floats per lane
     struct alignas(4 * V) Vec { float f[V]; };
-    const int a = blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (a >= nA) return;
+    const int per = (nA + (int)gridDim.x - 1) / (int)gridDim.x;   // consecutive sources of the CTA
+    const int end = min(nA, ((int)blockIdx.x + 1) * per);
+    int a = blockIdx.x * per + (threadIdx.x >> 5);
+    if (a >= end) return;
     const int b = blockIdx.y;
     const int lane = threadIdx.x & 31;
     const float* mb = mhat + (int64_t)b * N * DM + lane * V;
-    const int i = src_idx[a];
-    int t, y, x;
-    p.coords(i, t, y, x);
-    const int bt = p.dst.quot(t), by = p.dsh.quot(y), bx = p.dsw.quot(x);
     const int nBt = p.nB / (p.nHy * p.nWx);
-    const int t0 = max(bt - wt, 0), y0 = max(by - wh, 0), x0 = max(bx - ww, 0);
-    const int ny = min(by + wh, p.nHy - 1) - y0 + 1, nx = min(bx + ww, p.nWx - 1) - x0 + 1;
-    const int64_t count = (int64_t)(min(bt + wt, nBt - 1) - t0 + 1) * ny * nx;   // (the block's own destination is among them)
-    const Vec mi = *reinterpret_cast<const Vec*>(mb + (int64_t)i * DM);
-    float best = -INFINITY;
-    int jbest = ((bt * p.st) * p.Hh + by * p.sh) * p.W + bx * p.sw;   // no comparable cosine (NaN in the metric): its own block
-    if (count == 1) {   // the window is its own block: one cosine, its products added in the same order
-        const Vec mj = *reinterpret_cast<const Vec*>(mb + (int64_t)jbest * DM);
-        float c = 0.f;
+    int i = src_idx[a];
+    Vec mi = *reinterpret_cast<const Vec*>(mb + (int64_t)i * DM);
+    for (; a < end; a += 8) {
+        int t, y, x;
+        p.coords(i, t, y, x);
+        const int bt = p.dst.quot(t), by = p.dsh.quot(y), bx = p.dsw.quot(x);
+        const int t0 = max(bt - wt, 0), y0 = max(by - wh, 0), x0 = max(bx - ww, 0);
+        const int ny = min(by + wh, p.nHy - 1) - y0 + 1, nx = min(bx + ww, p.nWx - 1) - x0 + 1;
+        const int64_t count = (int64_t)(min(bt + wt, nBt - 1) - t0 + 1) * ny * nx;   // (the block's own destination is among them)
+        float best = -INFINITY;
+        int jbest = ((bt * p.st) * p.Hh + by * p.sh) * p.W + bx * p.sw;   // no comparable cosine (NaN in the metric): its own block
+        if (OWN || count == 1) {   // the window is its own block: one cosine, its products added in the same order
+            const Vec mj = *reinterpret_cast<const Vec*>(mb + (int64_t)jbest * DM);
+            float c = 0.f;
 #pragma unroll
-        for (int e = 0; e < V; ++e) c = fmaf(mi.f[e], mj.f[e], c);
+            for (int e = 0; e < V; ++e) c = fmaf(mi.f[e], mj.f[e], c);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-        if (c > best) best = c;
-    }
-    for (int64_t k0 = 0; k0 < count && count > 1; k0 += 32) {
-        const int n = (int)min((int64_t)32, count - k0);
-        const int k = (int)k0 + min(lane, n - 1);
-        const int row = k / nx, ct = row / ny;
-        const int jk = (((t0 + ct) * p.st) * p.Hh + (y0 + row - ct * ny) * p.sh) * p.W + (x0 + k - row * nx) * p.sw;
-        float c[32];
-#pragma unroll
-        for (int q0 = 0; q0 < 32; q0 += 8) {
-#pragma unroll
-            for (int q = q0; q < q0 + 8; ++q) c[q] = 0.f;
-            if (q0 < n) {
-                Vec mj[8];
-#pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    mj[q] = *reinterpret_cast<const Vec*>(mb + (int64_t)__shfl_sync(0xffffffffu, jk, q0 + q) * DM);
-#pragma unroll
-                for (int q = 0; q < 8; ++q)
-#pragma unroll
-                    for (int e = 0; e < V; ++e) c[q0 + q] = fmaf(mi.f[e], mj[q].f[e], c[q0 + q]);
-            }
+            for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+            if (c > best) best = c;
         }
+        const bool rows3 = nx == 3;   // rows of three: their candidates follow from one address a row
+        const int step = rows3 ? 30 : 32, dx = p.sw * 32;
+        for (int64_t k0 = 0; !OWN && k0 < count && count > 1; k0 += step) {
+            const int n = (int)min((int64_t)step, count - k0);
+            const int k = (int)k0 + min(lane, n - 1);
+            const int row = k / nx, ct = row / ny;
+            const int jk = (((t0 + ct) * p.st) * p.Hh + (y0 + row - ct * ny) * p.sh) * p.W + (x0 + k - row * nx) * p.sw;
+            float c[32];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const bool up = lane & o;
+            for (int q = 0; q < 32; ++q) c[q] = 0.f;
+            if (rows3) {
 #pragma unroll
-            for (int q = 0; q < o; ++q) {
-                const float give = up ? c[q] : c[q + o], keep = up ? c[q + o] : c[q];
-                c[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                for (int q0 = 0; q0 < 30; q0 += 9) {
+                    if (q0 >= n) continue;
+                    Vec mj[9];
+#pragma unroll
+                    for (int q = 0; q < 9 && q0 + q < 30; q += 3) {
+                        const Vec* at = reinterpret_cast<const Vec*>(mb + (int64_t)__shfl_sync(0xffffffffu, jk, min(q0 + q, n - 3)) * DM);   // (past n: the last row again)
+                        mj[q] = at[0];
+                        mj[q + 1] = at[dx];
+                        mj[q + 2] = at[2 * dx];
+                    }
+#pragma unroll
+                    for (int q = 0; q < 9 && q0 + q < 30; ++q)
+#pragma unroll
+                        for (int e = 0; e < V; ++e) c[q0 + q] = fmaf(mi.f[e], mj[q].f[e], c[q0 + q]);
+                }
+            } else {
+#pragma unroll
+                for (int q0 = 0; q0 < 32; q0 += 8) {
+                    if (q0 >= n) continue;
+                    Vec mj[8];
+#pragma unroll
+                    for (int q = 0; q < 8; ++q)
+                        mj[q] = *reinterpret_cast<const Vec*>(mb + (int64_t)__shfl_sync(0xffffffffu, jk, q0 + q) * DM);
+#pragma unroll
+                    for (int q = 0; q < 8; ++q)
+#pragma unroll
+                        for (int e = 0; e < V; ++e) c[q0 + q] = fmaf(mi.f[e], mj[q].f[e], c[q0 + q]);
+                }
             }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const bool up = lane & o;
+#pragma unroll
+                for (int q = 0; q < o; ++q) {
+                    const float give = up ? c[q] : c[q + o], keep = up ? c[q + o] : c[q];
+                    c[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                }
+            }
+            const uint32_t key = lane < n && c[0] > -INFINITY ? float_key(c[0]) : 0u;   // NaN never wins
+            const uint32_t top = __reduce_max_sync(0xffffffffu, key);
+            const int w = __ffs(__ballot_sync(0xffffffffu, key == top)) - 1;
+            const float cw = __shfl_sync(0xffffffffu, c[0], w);
+            const int jw = __shfl_sync(0xffffffffu, jk, w);
+            if (top != 0 && cw > best) { best = cw; jbest = jw; }
         }
-        const uint32_t key = lane < n && c[0] > -INFINITY ? float_key(c[0]) : 0u;   // NaN never wins
-        const uint32_t top = __reduce_max_sync(0xffffffffu, key);
-        const int w = __ffs(__ballot_sync(0xffffffffu, key == top)) - 1;
-        const float cw = __shfl_sync(0xffffffffu, c[0], w);
-        const int jw = __shfl_sync(0xffffffffu, jk, w);
-        if (top != 0 && cw > best) { best = cw; jbest = jw; }
-    }
-    if (lane == 0) {
-        jstar_s[(int64_t)b * nA + a] = jbest;
-        u_s[(int64_t)b * nA + a] = best;
+        if (lane == 0) {
+            jstar_s[(int64_t)b * nA + a] = jbest;
+            u_s[(int64_t)b * nA + a] = best;
+        }
+        if (a + 8 >= end) return;
+        i = src_idx[a + 8];
+        mi = *reinterpret_cast<const Vec*>(mb + (int64_t)i * DM);
     }
 }
 
@@ -782,9 +812,16 @@ static int token_merge_impl(int B, int N, int C, const void* x, int Hm, int dm,
         USV_CHECK_LAUNCH("desc_kernel");
         if (nA > 0) {
             if (win != nullptr) {
-                dim3 lg(ceil_div(nA, 8), B);
-                if (dm == 128) launch_dep(match_local_kernel<128>, dim3(lg), dim3(256), 0, s, mhat, p, N, nA, win[0], win[1], win[2], src_idx, jstar_s, u_s);
-                else launch_dep(match_local_kernel<64>, dim3(lg), dim3(256), 0, s, mhat, p, N, nA, win[0], win[1], win[2], src_idx, jstar_s, u_s);
+                int sms;   // one wave of CTAs (their launch bounds) from two waves of single sources on
+                if (int e = sm_count(&sms); e != USV_OK) return e;
+                const bool own = win[0] == 0 && win[1] == 0 && win[2] == 0;
+                const int groups = ceil_div(nA, 8), wave = std::max(1, (own ? 6 : 3) * sms / B);
+                dim3 lg(groups > 2 * wave ? wave : groups, B);
+                auto match = [&](auto kernel) {
+                    launch_dep(kernel, lg, dim3(256), 0, s, mhat, p, N, nA, win[0], win[1], win[2], src_idx, jstar_s, u_s);
+                };
+                if (dm == 128) own ? match(match_local_kernel<128, true>) : match(match_local_kernel<128, false>);
+                else own ? match(match_local_kernel<64, true>) : match(match_local_kernel<64, false>);
                 USV_CHECK_LAUNCH("match_local_kernel");
             } else {
                 // tensor cores: fp16 cosines propose, fp32 decides (usv_match_tc.cu)
