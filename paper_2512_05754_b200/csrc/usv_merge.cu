@@ -283,6 +283,118 @@ __global__ void __launch_bounds__(1024) plan_assign_kernel(Part p, int N, int nA
     }
 }
 
+// Both steps in one launch for few sources: one CTA per batch element holds every key in registers, a warp 32 * PER consecutive
+// ones, so that the ranks among the unmerged sources follow from ballots and one sum over the warps.  Bound: the chain of a launch,
+// reads and barriers.  Whole merges with two kernels / with this one, us: 96 sources 17.3 / 15.8, 2 x 1024 20.7 / 17.1, 840 with a matching of
+// all destinations 46.5 / 42.5, 2880 20.6 / 19.2; 4500 25.3 / 26.9, 7500 29.0 / 32.2 (one SM's atomics and scattered stores).
+template <int PER>
+__global__ void __launch_bounds__(1024) plan_small_kernel(Part p, int N, int nA, int r, const int32_t* __restrict__ src_idx,
+                                                          const int32_t* __restrict__ jstar_s, const float* __restrict__ u_s,
+                                                          int32_t* __restrict__ dst_of, int32_t* __restrict__ pos,
+                                                          float* __restrict__ u_out, int32_t* __restrict__ jstar_out,
+                                                          const MergeLists lists) {
+    __shared__ int s_hist[4][256];
+    __shared__ uint32_t s_prefix, s_warp[32];   // s_warp: (keys above T) << 16 | keys equal to T
+    __shared__ int s_remaining;
+    (&s_hist[0][0])[threadIdx.x] = 0;
+    if (threadIdx.x == 0) {
+        s_prefix = 0;
+        s_remaining = r;
+    }
+    dep_sync();
+    const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const float* u = u_s + (int64_t)b * nA;
+    const int32_t* js = jstar_s + (int64_t)b * nA;
+    int32_t* d_of = dst_of + (int64_t)b * N;
+    int32_t* ps = pos + (int64_t)b * N;
+    const int nU = nA - r;
+    const int first = warp * 32 * PER + lane;   // element i of the thread: first + 32 i
+    uint32_t key[PER];
+    int src[PER], to[PER];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int a = first + 32 * i;
+        const bool in = a < nA;
+        key[i] = in ? float_key(u[a]) : 0u;
+        src[i] = in ? src_idx[a] : 0;
+        to[i] = in ? js[a] : 0;
+    }
+    for (int o = threadIdx.x; o < p.nB; o += 1024) {
+        const int n = p.dst_token(o);
+        d_of[n] = -1;
+        ps[n] = nU + o;
+        if (u_out) u_out[(int64_t)b * N + n] = __int_as_float(0x7fc00000);
+        if (jstar_out) jstar_out[(int64_t)b * N + n] = -1;
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int pass = 0; pass < 4; ++pass) {
+        const int shift = 24 - 8 * pass;
+        const uint32_t prefix = s_prefix, mask = pass == 0 ? 0u : (0xffffffffu << (shift + 8));
+#pragma unroll
+        for (int i = 0; i < PER; ++i)
+            if (first + 32 * i < nA && (key[i] & mask) == prefix) atomicAdd(&s_hist[pass][(key[i] >> shift) & 255], 1);
+        __syncthreads();
+        if (warp == 0) {
+            const int remaining = s_remaining;
+            int local[8], sum = 0;
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                local[t] = s_hist[pass][255 - (lane * 8 + t)];
+                sum += local[t];
+            }
+            int before = warp_incl_scan(sum) - sum;
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                if (before < remaining && remaining <= before + local[t]) {
+                    s_prefix = prefix | ((uint32_t)(255 - (lane * 8 + t)) << shift);
+                    s_remaining = remaining - before;
+                }
+                before += local[t];
+            }
+        }
+        __syncthreads();
+    }
+    const uint32_t T = s_prefix;
+    const int need_eq = s_remaining;
+    uint32_t gt[PER], eq[PER];
+    int n_gt = 0, n_eq = 0;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const bool in = first + 32 * i < nA;
+        gt[i] = __ballot_sync(0xffffffffu, in && key[i] > T);
+        eq[i] = __ballot_sync(0xffffffffu, in && key[i] == T);
+        n_gt += __popc(gt[i]);
+        n_eq += __popc(eq[i]);
+    }
+    if (lane == 0) s_warp[warp] = (uint32_t)n_gt << 16 | (uint32_t)n_eq;
+    __syncthreads();
+    const uint32_t ahead = __reduce_add_sync(0xffffffffu, lane < warp ? s_warp[lane] : 0u);
+    int gt_b = (int)(ahead >> 16), eq_b = (int)(ahead & 0xffffu);
+    const uint32_t below = (1u << lane) - 1u;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int a = first + 32 * i, n = src[i], j = to[i];
+        const int g = gt_b + __popc(gt[i] & below), e = eq_b + __popc(eq[i] & below);
+        gt_b += __popc(gt[i]);
+        eq_b += __popc(eq[i]);
+        if (a >= nA) continue;
+        if (key[i] > T || (key[i] == T && e < need_eq)) {
+            const int o = p.ord(j);
+            d_of[n] = j;
+            ps[n] = nU + o;
+            lists.push(b, o, (int64_t)b * N, n);
+        } else {
+            const int un_rank = a - g - min(e, need_eq);
+            d_of[n] = -1;
+            ps[n] = un_rank;
+            lists.row_src[(int64_t)b * nU + un_rank] = n;
+        }
+        if (u_out) u_out[(int64_t)b * N + n] = u[a];
+        if (jstar_out) jstar_out[(int64_t)b * N + n] = j;
+    }
+}
+
 // The same lists from a stored plan.  cnt and head start at zero.
 __global__ void __launch_bounds__(256) plan_lists_kernel(Part p, int N, int nU,
                                                          const int32_t* __restrict__ dst_of,
@@ -828,6 +940,16 @@ static int token_merge_impl(int B, int N, int C, const void* x, int Hm, int dm,
                 rc = launch_match_tc(mhat, m, dm, s);
                 if (rc != USV_OK) return rc;
             }
+        }
+        auto small = [&](auto kernel) {   // (see plan_small_kernel for where it ends)
+            launch_dep(kernel, dim3(B), dim3(1024), 0, s, p, N, nA, r, src_idx, jstar_s, u_s, dst_of, pos, u_out, jstar_out, lists);
+        };
+        if (r > 0 && r < nA && nA <= 3 * 1024) {
+            if (nA <= 1024) small(plan_small_kernel<1>);
+            else if (nA <= 2048) small(plan_small_kernel<2>);
+            else small(plan_small_kernel<3>);
+            USV_CHECK_LAUNCH("plan_small_kernel");
+            return launch_merge(p, B, N, C, nU, Nm, x, lists, dst_of, x_merged, s);
         }
         const int2* tsel = nullptr;
         if (r > 0 && r < nA) {
