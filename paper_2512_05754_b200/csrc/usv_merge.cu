@@ -8,6 +8,7 @@
 //   plan_select_kernel Eq. 10         radix-select of the r-th most confident source
 //   plan_assign_kernel Eq. 11, 14     ordered compaction, dst_of / pos
 //                                and the lists of merged sources per destination (Eq. 12)
+//   plan_held_kernel             both in one launch, by source counts
 //   merge_kernel       Eq. 13-14 warp-per-row gather + mean, 16-byte accesses
 //   unmerge_kernel     Eq. 15    warp-per-row gather copy, 16-byte accesses
 #include <cuda_fp16.h>
@@ -283,18 +284,20 @@ __global__ void __launch_bounds__(1024) plan_assign_kernel(Part p, int N, int nA
     }
 }
 
-// Both steps in one launch for few sources: one CTA per batch element holds every key in registers, a warp 32 * PER consecutive
-// ones, so that the ranks among the unmerged sources follow from ballots and one sum over the warps.  Bound: the chain of a launch,
-// reads and barriers.  Whole merges with two kernels / with this one, us: 96 sources 17.3 / 15.8, 2 x 1024 20.7 / 17.1, 840 with a matching of
-// all destinations 46.5 / 42.5, 2880 20.6 / 19.2; 4500 25.3 / 26.9, 7500 29.0 / 32.2 (one SM's atomics and scattered stores).
-template <int PER>
-__global__ void __launch_bounds__(1024) plan_small_kernel(Part p, int N, int nA, int r, const int32_t* __restrict__ src_idx,
-                                                          const int32_t* __restrict__ jstar_s, const float* __restrict__ u_s,
-                                                          int32_t* __restrict__ dst_of, int32_t* __restrict__ pos,
-                                                          float* __restrict__ u_out, int32_t* __restrict__ jstar_out,
-                                                          const MergeLists lists) {
-    __shared__ int s_hist[4][256];
-    __shared__ uint32_t s_prefix, s_warp[32];   // s_warp: (keys above T) << 16 | keys equal to T
+// Both steps in one launch: the CTA, or the cluster of eight, of a batch element holds every key in registers, a warp 32 * PER
+// consecutive ones, so that the ranks among the unmerged sources follow from ballots and sums over warps and CTAs.  Every CTA counts
+// digits in its own shared memory, and one cluster barrier a pass later adds up all counts.  Bound: the chain of a launch, reads
+// and barriers, and beyond about 50 000 sources the scattered stores and atomics of eight SMs.  Whole merges with two kernels /
+// with this one, us.  One CTA: 96 sources 17.2 / 15.6, 2 x 1024 20.7 / 17.1, 840 with a matching of all destinations 46.5 / 42.5, 2880 20.6 /
+// 18.8, but 4500 25.3 / 26.9, 7500 29.0 / 32.2.  Eight: 1024 20.4 / 24.0, 10 140 38.0 / 38.5, 15 210 44.9 / 41.8, 2 x 16 380 119.9 / 116.9,
+// 4 x 24 570 181 / 176, 37 800 71.4 / 68.1, 65 480 136 / 123, 2 x 59 400 189 / 182, 2 x 88 440 216 / 191.
+template <int CL, int PER>
+__global__ void __launch_bounds__(1024) __cluster_dims__(CL, 1, 1)
+plan_held_kernel(Part p, int N, int nA, int r, const int32_t* __restrict__ src_idx, const int32_t* __restrict__ jstar_s,
+                 const float* __restrict__ u_s, int32_t* __restrict__ dst_of, int32_t* __restrict__ pos,
+                 float* __restrict__ u_out, int32_t* __restrict__ jstar_out, const MergeLists lists) {
+    __shared__ __align__(16) int s_hist[4][256];          // one a pass: peers may still read the one before
+    __shared__ uint32_t s_prefix, s_total, s_warp[32];   // s_warp, s_total: (keys above T) << 16 | keys equal to T
     __shared__ int s_remaining;
     (&s_hist[0][0])[threadIdx.x] = 0;
     if (threadIdx.x == 0) {
@@ -302,30 +305,38 @@ __global__ void __launch_bounds__(1024) plan_small_kernel(Part p, int N, int nA,
         s_remaining = r;
     }
     dep_sync();
-    const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int rank = blockIdx.x, b = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float* u = u_s + (int64_t)b * nA;
     const int32_t* js = jstar_s + (int64_t)b * nA;
     int32_t* d_of = dst_of + (int64_t)b * N;
     int32_t* ps = pos + (int64_t)b * N;
     const int nU = nA - r;
-    const int first = warp * 32 * PER + lane;   // element i of the thread: first + 32 i
+    const int first = (rank * 32 + warp) * 32 * PER + lane;   // element i of the thread: first + 32 i
+    constexpr int AHEAD = CL == 1 ? PER : 1;   // sources and destinations read before they are needed
     uint32_t key[PER];
-    int src[PER], to[PER];
+    int src[AHEAD], to[AHEAD];
 #pragma unroll
     for (int i = 0; i < PER; ++i) {
         const int a = first + 32 * i;
         const bool in = a < nA;
         key[i] = in ? float_key(u[a]) : 0u;
-        src[i] = in ? src_idx[a] : 0;
-        to[i] = in ? js[a] : 0;
+        if (CL == 1) {
+            src[i] = in ? src_idx[a] : 0;
+            to[i] = in ? js[a] : 0;
+        }
     }
-    for (int o = threadIdx.x; o < p.nB; o += 1024) {
+    for (int o = rank * 1024 + threadIdx.x; o < p.nB; o += CL * 1024) {
         const int n = p.dst_token(o);
         d_of[n] = -1;
         ps[n] = nU + o;
         if (u_out) u_out[(int64_t)b * N + n] = __int_as_float(0x7fc00000);
         if (jstar_out) jstar_out[(int64_t)b * N + n] = -1;
     }
+    auto peer = [](const void* at, int cta) {
+        uint32_t to;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(to) : "r"((uint32_t)__cvta_generic_to_shared(at)), "r"(cta));
+        return to;
+    };
     __syncthreads();
 #pragma unroll 1
     for (int pass = 0; pass < 4; ++pass) {
@@ -334,20 +345,34 @@ __global__ void __launch_bounds__(1024) plan_small_kernel(Part p, int N, int nA,
 #pragma unroll
         for (int i = 0; i < PER; ++i)
             if (first + 32 * i < nA && (key[i] & mask) == prefix) atomicAdd(&s_hist[pass][(key[i] >> shift) & 255], 1);
-        __syncthreads();
+        if (CL > 1) {
+            __syncwarp();
+            asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        } else {
+            __syncthreads();
+        }
         if (warp == 0) {
             const int remaining = s_remaining;
-            int local[8], sum = 0;
+            int local[8] = {0, 0, 0, 0, 0, 0, 0, 0}, sum = 0;   // bins 248 - 8 lane and up, of all CTAs
 #pragma unroll
-            for (int t = 0; t < 8; ++t) {
-                local[t] = s_hist[pass][255 - (lane * 8 + t)];
-                sum += local[t];
+            for (int c = 0; c < CL; ++c) {
+                int v[8];
+                const int* at = &s_hist[pass][248 - 8 * lane];
+                if (CL > 1) {
+                    const uint32_t far = peer(at, c);
+                    asm volatile("ld.shared::cluster.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(far) : "memory");
+                    asm volatile("ld.shared::cluster.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "r"(far + 16) : "memory");
+                }
+#pragma unroll
+                for (int t = 0; t < 8; ++t) local[t] += CL > 1 ? v[t] : at[t];
             }
+#pragma unroll
+            for (int t = 0; t < 8; ++t) sum += local[t];
             int before = warp_incl_scan(sum) - sum;
 #pragma unroll
-            for (int t = 0; t < 8; ++t) {
+            for (int t = 7; t >= 0; --t) {
                 if (before < remaining && remaining <= before + local[t]) {
-                    s_prefix = prefix | ((uint32_t)(255 - (lane * 8 + t)) << shift);
+                    s_prefix = prefix | ((uint32_t)(248 - 8 * lane + t) << shift);
                     s_remaining = remaining - before;
                 }
                 before += local[t];
@@ -369,16 +394,30 @@ __global__ void __launch_bounds__(1024) plan_small_kernel(Part p, int N, int nA,
     }
     if (lane == 0) s_warp[warp] = (uint32_t)n_gt << 16 | (uint32_t)n_eq;
     __syncthreads();
-    const uint32_t ahead = __reduce_add_sync(0xffffffffu, lane < warp ? s_warp[lane] : 0u);
+    const uint32_t mine = s_warp[lane];
+    const uint32_t ahead = __reduce_add_sync(0xffffffffu, lane < warp ? mine : 0u);
     int gt_b = (int)(ahead >> 16), eq_b = (int)(ahead & 0xffffu);
+    if (CL > 1) {   // what the CTAs before hold
+        const uint32_t total = __reduce_add_sync(0xffffffffu, mine);
+        if (threadIdx.x == 0) s_total = total;
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        uint32_t other = 0;
+        if (lane < rank) asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(other) : "r"(peer(&s_total, lane)) : "memory");
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // (nobody leaves while a peer may read)
+        gt_b += (int)__reduce_add_sync(0xffffffffu, other >> 16);
+        eq_b += (int)__reduce_add_sync(0xffffffffu, other & 0xffffu);
+    }
     const uint32_t below = (1u << lane) - 1u;
 #pragma unroll
     for (int i = 0; i < PER; ++i) {
-        const int a = first + 32 * i, n = src[i], j = to[i];
+        const int a = first + 32 * i;
         const int g = gt_b + __popc(gt[i] & below), e = eq_b + __popc(eq[i] & below);
         gt_b += __popc(gt[i]);
         eq_b += __popc(eq[i]);
         if (a >= nA) continue;
+        const int n = CL == 1 ? src[CL == 1 ? i : 0] : src_idx[a], j = CL == 1 ? to[CL == 1 ? i : 0] : js[a];
         if (key[i] > T || (key[i] == T && e < need_eq)) {
             const int o = p.ord(j);
             d_of[n] = j;
@@ -392,6 +431,10 @@ __global__ void __launch_bounds__(1024) plan_small_kernel(Part p, int N, int nA,
         }
         if (u_out) u_out[(int64_t)b * N + n] = u[a];
         if (jstar_out) jstar_out[(int64_t)b * N + n] = j;
+    }
+    if (CL > 1) {
+        __syncwarp();
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     }
 }
 
@@ -941,14 +984,21 @@ static int token_merge_impl(int B, int N, int C, const void* x, int Hm, int dm,
                 if (rc != USV_OK) return rc;
             }
         }
-        auto small = [&](auto kernel) {   // (see plan_small_kernel for where it ends)
-            launch_dep(kernel, dim3(B), dim3(1024), 0, s, p, N, nA, r, src_idx, jstar_s, u_s, dst_of, pos, u_out, jstar_out, lists);
+        auto held = [&](auto kernel, int ctas) {   // (see plan_held_kernel for where the lines are)
+            launch_dep(kernel, dim3(ctas, B), dim3(1024), 0, s, p, N, nA, r, src_idx, jstar_s, u_s, dst_of, pos, u_out, jstar_out, lists);
         };
-        if (r > 0 && r < nA && nA <= 3 * 1024) {
-            if (nA <= 1024) small(plan_small_kernel<1>);
-            else if (nA <= 2048) small(plan_small_kernel<2>);
-            else small(plan_small_kernel<3>);
-            USV_CHECK_LAUNCH("plan_small_kernel");
+        if (r > 0 && r < nA && (nA <= 3 * 1024 || (nA > 12 * 1024 && nA <= 16 * 8 * 1024))) {
+            const int per = ceil_div(nA, nA <= 3 * 1024 ? 1024 : 8 * 1024);
+            if (nA <= 3 * 1024) per == 1 ? held(plan_held_kernel<1, 1>, 1) : per == 2 ? held(plan_held_kernel<1, 2>, 1) : held(plan_held_kernel<1, 3>, 1);
+            else if (per <= 2) held(plan_held_kernel<8, 2>, 8);
+            else if (per <= 3) held(plan_held_kernel<8, 3>, 8);
+            else if (per <= 4) held(plan_held_kernel<8, 4>, 8);
+            else if (per <= 5) held(plan_held_kernel<8, 5>, 8);
+            else if (per <= 6) held(plan_held_kernel<8, 6>, 8);
+            else if (per <= 8) held(plan_held_kernel<8, 8>, 8);
+            else if (per <= 11) held(plan_held_kernel<8, 11>, 8);
+            else held(plan_held_kernel<8, 16>, 8);
+            USV_CHECK_LAUNCH("plan_held_kernel");
             return launch_merge(p, B, N, C, nU, Nm, x, lists, dst_of, x_merged, s);
         }
         const int2* tsel = nullptr;
