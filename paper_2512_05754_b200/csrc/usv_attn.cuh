@@ -41,8 +41,10 @@ struct AttnArgs {
 };
 
 int launch_attn_mma(const AttnArgs& a, int d, cudaStream_t st);
-// the same for small calls at d = 64, four groups of warps a query block; most: longest list
-int launch_attn_split(const AttnArgs& a, int most, cudaStream_t st);
+// the same, bit for bit, for small calls at d = 64 with lists of at most four blocks, four groups of warps a query block
+int launch_attn_four(const AttnArgs& a, cudaStream_t st);
+// small calls at d = 64 with longer lists, four groups of warps a query block
+int launch_attn_split(const AttnArgs& a, cudaStream_t st);
 // the same for lists of one block at d = 64
 int launch_attn_one(const AttnArgs& a, cudaStream_t st);
 bool attn_pair_supported(const AttnArgs& a, int d);

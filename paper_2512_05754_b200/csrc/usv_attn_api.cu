@@ -98,12 +98,12 @@ static int sparse_attn_impl(int B, int H, int N, int d, const void* q, const usv
     // keep 4 11.6 / 14.2, 6 15.9 / 16.1, 8 20.0 / 17.6; 512, keep 2 11.5 / 13.1, 3 15.0 / 13.9.
     const int64_t blocks = (int64_t)B * H * NB;
     const bool small = d == 64 && kmx <= 4 && blocks <= 384;
-    // Where every query block has an SM to itself, four groups of warps walk its list side by side: 32 blocks, keep 4 8.3 / 7.0,
-    // 8 11.4 / 9.4, 16 13.7 / 15.2; 128, keep 2 8.3 / 7.0, 4 11.6 / 7.2, 8 12.1 / 9.7; 100, keep 10 13.7 / 11.5; 256, keep 4 11.9 / 12.9
-    // (other kernels / this one).  At d = 128 it never pays (32, keep 4 10.8 / 13.1).
+    // Where every query block has an SM to itself, four groups of warps take its list side by side: 32 blocks, keep 4 8.3 / 7.35,
+    // 8 11.4 / 9.4, 16 13.7 / 15.2; 128, keep 2 7.0 / 5.4, 4 10.7 / 7.4, 8 12.1 / 9.7; 100, keep 10 13.7 / 11.5; 256, keep 4 11.9 / 12.9
+    // (other kernels / these).  At d = 128 it never pays (32, keep 4 10.8 / 13.1).
     int sms;
     if ((rc = sm_count(&sms)) != USV_OK) return rc;
-    if (impl == 0 && d == 64 && blocks <= sms && kmx >= 2 && kmx <= 10) return launch_attn_split(a, kmx, st);
+    if (impl == 0 && d == 64 && blocks <= sms && kmx >= 2 && kmx <= 10) return kmx <= 4 ? launch_attn_four(a, st) : launch_attn_split(a, st);
     // Many single blocks at d = 64, mma.sync with two buffers / with one: 2400 23.2 / 21.5, 7608 73.3 / 69.7, 12 000 113 / 107 (the
     // tcgen05 kernel: 26.3, 72.8, 110).
     if (impl == 0 && d == 64 && blocks > 1800 && kmx == 1) return launch_attn_one(a, st);

@@ -9,13 +9,92 @@
 
 namespace usv {
 
+// Weights of a 64-key tile from its logits, relative to ms (rows g and g + 8 of the warp): pf gets them as bf16, in the layout
+// of an A operand, and add(nt, r, e, w) sees the sum of the unrounded pair of 8-key piece nt and row r, and the rounded pair.
+template <typename Add>
+__device__ __forceinline__ void tile_weights(const float (&s)[8][4], float c, const float (&ms)[2], uint32_t (&pf)[4][4], Add add) {
+#pragma unroll
+    for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const float e0 = exp2f(fmaf(s[nt][2 * r], c, -ms[r]));
+            const float e1 = exp2f(fmaf(s[nt][2 * r + 1], c, -ms[r]));
+            const uint32_t w = pack_bf16x2(e0, e1);
+            pf[nt >> 1][(nt & 1) * 2 + r] = w;
+            add(nt, r, e0 + e1, w);
+        }
+}
+__device__ __forceinline__ float sum_bf16x2(uint32_t w) { return __uint_as_float(w << 16) + __uint_as_float(w & 0xffff0000u); }
+
+// Q fragments of the warp's 16 rows, and the logits of one K tile
+template <int D>
+__device__ __forceinline__ void load_q_frags(uint32_t (&qf)[D / 16][4], const __nv_bfloat16* Qs, int warp, int lane) {
+    constexpr int LD = MmaSmem<D>::LD;
+    const __nv_bfloat16* qrow = Qs + (warp * 16 + (lane >> 2)) * LD + 2 * (lane & 3);
+#pragma unroll
+    for (int kt = 0; kt < D / 16; ++kt) {
+        qf[kt][0] = *reinterpret_cast<const uint32_t*>(qrow + kt * 16);
+        qf[kt][1] = *reinterpret_cast<const uint32_t*>(qrow + 8 * LD + kt * 16);
+        qf[kt][2] = *reinterpret_cast<const uint32_t*>(qrow + kt * 16 + 8);
+        qf[kt][3] = *reinterpret_cast<const uint32_t*>(qrow + 8 * LD + kt * 16 + 8);
+    }
+}
+// s: 16 x 64 logits, keys from nvalid on -inf; mx: the maxima of rows g and g + 8
+template <int D>
+__device__ __forceinline__ void tile_logits(float (&s)[8][4], float (&mx)[2], const uint32_t (&qf)[D / 16][4], const __nv_bfloat16* Kt,
+                                            int nvalid, int lane) {
+    constexpr int LD = MmaSmem<D>::LD;
+    const int g = lane >> 2, tig = lane & 3;
+#pragma unroll
+    for (int nt = 0; nt < 8; ++nt) {
+        s[nt][0] = s[nt][1] = s[nt][2] = s[nt][3] = 0.f;
+        const __nv_bfloat16* krow = Kt + (nt * 8 + g) * LD + 2 * tig;
+#pragma unroll
+        for (int kt = 0; kt < D / 16; ++kt) {
+            const uint32_t b0 = *reinterpret_cast<const uint32_t*>(krow + kt * 16);
+            const uint32_t b1 = *reinterpret_cast<const uint32_t*>(krow + kt * 16 + 8);
+            mma_bf16_16816(s[nt], qf[kt], b0, b1);
+        }
+    }
+    if (nvalid < USV_BLOCK) {
+#pragma unroll
+        for (int nt = 0; nt < 8; ++nt) {
+            const int col = nt * 8 + 2 * tig;
+            if (col >= nvalid) s[nt][0] = s[nt][2] = -INFINITY;
+            if (col + 1 >= nvalid) s[nt][1] = s[nt][3] = -INFINITY;
+        }
+    }
+    mx[0] = mx[1] = -INFINITY;
+#pragma unroll
+    for (int nt = 0; nt < 8; ++nt) {
+        mx[0] = fmaxf(mx[0], fmaxf(s[nt][0], s[nt][1]));
+        mx[1] = fmaxf(mx[1], fmaxf(s[nt][2], s[nt][3]));
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 1));
+        mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 2));
+    }
+}
+// The running maximum m of a row of scaled (base-2) logits past a tile whose maximum is mx * c: returns the factor for what was
+// summed so far; ms is what the tile's weights are relative to.
+__device__ __forceinline__ float next_max(float& m, float mx, float c, float& ms) {
+    const float mnew = fmaxf(m, mx * c);
+    ms = mnew == -INFINITY ? 0.f : mnew;
+    const float alpha = exp2f(m - ms);
+    m = mnew;
+    return alpha;
+}
+
 // G groups of 4 warps share a query block: group i takes the entries i, i + G, ... of its list, and the groups' results, each
-// relative to its own row maxima, are put together at the end.  NBUF: K/V tiles a group has room for.
+// relative to its own row maxima, are put together at the end.  (Each group's weights are rounded to bf16 relative to maxima of its
+// own: results differ from those of one group by that rounding, and are no further from fp64.  Lists of 5 to 10 entries of white
+// noise: 2.1e-4 to 3.5e-4 relative, 2.2e-4 to 3.7e-4 with one group, 3.0e-4 to 4.3e-4 on the tcgen05 kernel.)
+// NBUF: K/V tiles a group has room for.
 template <int D, int G, int NBUF>
 __device__ __forceinline__ void attn_mma_block(const AttnArgs& a, const int work, unsigned char* smem_raw) {
     constexpr int LD = MmaSmem<D>::LD;
     constexpr int TILE = MmaSmem<D>::TILE;
-    constexpr int KT = D / 16;  // k-steps of QK^T
     constexpr int NT = D / 8;   // n-tiles of the output
     const int grp = G == 1 ? 0 : threadIdx.x >> 7;
     __nv_bfloat16* Qs = reinterpret_cast<__nv_bfloat16*>(smem_raw);
@@ -52,7 +131,7 @@ __device__ __forceinline__ void attn_mma_block(const AttnArgs& a, const int work
     }
     cp_async_commit();
 
-    uint32_t qf[KT][4];
+    uint32_t qf[D / 16][4];
     float o[NT][4];
 #pragma unroll
     for (int n = 0; n < NT; ++n) o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f;
@@ -83,80 +162,20 @@ __device__ __forceinline__ void attn_mma_block(const AttnArgs& a, const int work
         }
         cp_async_commit();
 
-        if (first) {
-            const __nv_bfloat16* qrow = Qs + (warp * 16 + g) * LD + 2 * tig;
-#pragma unroll
-            for (int kt = 0; kt < KT; ++kt) {
-                qf[kt][0] = *reinterpret_cast<const uint32_t*>(qrow + kt * 16);
-                qf[kt][1] = *reinterpret_cast<const uint32_t*>(qrow + 8 * LD + kt * 16);
-                qf[kt][2] = *reinterpret_cast<const uint32_t*>(qrow + kt * 16 + 8);
-                qf[kt][3] = *reinterpret_cast<const uint32_t*>(qrow + 8 * LD + kt * 16 + 8);
-            }
-            first = false;
-        }
+        if (first) load_q_frags<D>(qf, Qs, warp, lane);
+        first = false;
 
-        const __nv_bfloat16* Kt = Ks + buf * TILE;
         const __nv_bfloat16* Vt = Vs + buf * TILE;
-
-        float s[8][4];
-#pragma unroll
-        for (int nt = 0; nt < 8; ++nt) {
-            s[nt][0] = s[nt][1] = s[nt][2] = s[nt][3] = 0.f;
-            const __nv_bfloat16* krow = Kt + (nt * 8 + g) * LD + 2 * tig;
-#pragma unroll
-            for (int kt = 0; kt < KT; ++kt) {
-                const uint32_t b0 = *reinterpret_cast<const uint32_t*>(krow + kt * 16);
-                const uint32_t b1 = *reinterpret_cast<const uint32_t*>(krow + kt * 16 + 8);
-                mma_bf16_16816(s[nt], qf[kt], b0, b1);
-            }
-        }
-        const int nvalid = N - J * USV_BLOCK;  // keys of this block with index < N
-        if (nvalid < USV_BLOCK) {
-#pragma unroll
-            for (int nt = 0; nt < 8; ++nt) {
-                const int col = nt * 8 + 2 * tig;
-                if (col >= nvalid) s[nt][0] = s[nt][2] = -INFINITY;
-                if (col + 1 >= nvalid) s[nt][1] = s[nt][3] = -INFINITY;
-            }
-        }
+        float s[8][4], mx[2], alpha[2], ms[2];
+        tile_logits<D>(s, mx, qf, Ks + buf * TILE, N - J * USV_BLOCK, lane);
         // online softmax (rows g -> elements 0,1; row g+8 -> elements 2,3)
-        float mx[2] = {-INFINITY, -INFINITY};
 #pragma unroll
-        for (int nt = 0; nt < 8; ++nt) {
-            mx[0] = fmaxf(mx[0], fmaxf(s[nt][0], s[nt][1]));
-            mx[1] = fmaxf(mx[1], fmaxf(s[nt][2], s[nt][3]));
-        }
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 1));
-            mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 2));
-        }
-        float alpha[2], mnew[2];
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            mnew[r] = fmaxf(m[r], mx[r] * c);
-            const float ms = mnew[r] == -INFINITY ? 0.f : mnew[r];
-            alpha[r] = exp2f(m[r] - ms);
-            m[r] = mnew[r];
-            mnew[r] = ms;
-            l[r] *= alpha[r];
-            lr[r] *= alpha[r];
-        }
+        for (int r = 0; r < 2; ++r) alpha[r] = next_max(m[r], mx[r], c, ms[r]);
         uint32_t pf[4][4];
-#pragma unroll
-        for (int nt = 0; nt < 8; ++nt) {
-            const float p0 = exp2f(fmaf(s[nt][0], c, -mnew[0]));
-            const float p1 = exp2f(fmaf(s[nt][1], c, -mnew[0]));
-            const float p2 = exp2f(fmaf(s[nt][2], c, -mnew[1]));
-            const float p3 = exp2f(fmaf(s[nt][3], c, -mnew[1]));
-            l[0] += p0 + p1;
-            l[1] += p2 + p3;
-            const uint32_t w01 = pack_bf16x2(p0, p1), w23 = pack_bf16x2(p2, p3);
-            lr[0] += __uint_as_float(w01 << 16) + __uint_as_float(w01 & 0xffff0000u);
-            lr[1] += __uint_as_float(w23 << 16) + __uint_as_float(w23 & 0xffff0000u);
-            pf[nt >> 1][(nt & 1) * 2 + 0] = w01;
-            pf[nt >> 1][(nt & 1) * 2 + 1] = w23;
-        }
+        tile_weights(s, c, ms, pf, [&](int nt, int r, float e, uint32_t w) {
+            l[r] = nt == 0 ? fmaf(l[r], alpha[r], e) : l[r] + e;
+            lr[r] = nt == 0 ? fmaf(lr[r], alpha[r], sum_bf16x2(w)) : lr[r] + sum_bf16x2(w);
+        });
 #pragma unroll
         for (int n = 0; n < NT; ++n) {
             o[n][0] *= alpha[0];
@@ -177,7 +196,7 @@ __device__ __forceinline__ void attn_mma_block(const AttnArgs& a, const int work
                 mma_bf16_16816(o[2 * n2 + 1], pf[kt], bfr[2], bfr[3]);
             }
         }
-        if (NBUF == 2) buf ^= 1;   // (with one tile there is no next one: lists of at most G entries)
+        if (NBUF == 2) buf ^= 1;   // (with one tile there is no next one)
         t = tn;
     }
     cp_async_wait_all();
@@ -339,8 +358,8 @@ __global__ void __launch_bounds__(128) attn_mma_kernel(const AttnArgs a) {
     }
 }
 
-// One CTA per query block, G groups.  A call of few blocks takes as long as one walk over a list: loads, two short chains of
-// MMAs and the softmax between them, 1.3 us a key block at D = 64; G of them run side by side.
+// One CTA per query block, G groups, lists of five to ten blocks.  A call of few blocks takes as long as one walk over a list:
+// loads, two short chains of MMAs and the softmax between them, 1.3 us a key block at D = 64; G of them run side by side.
 template <int D, int G, int NBUF>
 __global__ void __launch_bounds__(128 * G) attn_split_kernel(const AttnArgs a) {
     dep_sync();
@@ -349,13 +368,181 @@ __global__ void __launch_bounds__(128 * G) attn_split_kernel(const AttnArgs a) {
     attn_mma_block<D, G, NBUF>(a, blockIdx.x, smem_raw);
 }
 
-template <int D, int G, int NBUF>
-static int launch_split(const AttnArgs& a, cudaStream_t st) {
+int launch_attn_split(const AttnArgs& a, cudaStream_t st) {
+    constexpr int D = 64, G = 4, NBUF = 2;
     constexpr size_t smem = (size_t)MmaSmem<D>::TILE * (1 + 2 * G * NBUF) * sizeof(__nv_bfloat16) + G * 192 * sizeof(float);
     static_assert(smem <= 232448, "shared memory budget");
-    cudaFuncSetAttribute(attn_split_kernel<D, G, NBUF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(attn_split_kernel<D, G, NBUF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return fail(USV_ERR_CUDA, "sparse_attn: smem attribute: %s", cudaGetErrorString(e));
     launch_dep_smem(attn_split_kernel<D, G, NBUF>, dim3((unsigned)(a.B * a.H * a.NB)), dim3(128 * G), smem, st, a);
     USV_CHECK_LAUNCH("attn_split_kernel");
+    return USV_OK;
+}
+
+// Lists of up to four blocks where every query block has an SM to itself, one CTA per query block, four groups of 4 warps: group
+// i loads entry i and takes its logits and, when the four maxima of a row are known, its weights, which every group
+// then multiplies with a quarter of V's columns.  Maxima, sums and products come in the order of the list, so the result is that
+// of attn_mma_block bit for bit.  Bound: the chain launch, loads, MMAs and the softmax between them, and 0.85 us an entry for its
+// MMAs.  Calls at D = 64, us, one group / groups with maxima of their own / this kernel: 32 blocks, keep 4 8.3 / 7.3 / 7.35; 128, keep
+// 2 7.0 / 5.8 / 5.4, keep 4 10.7 / 7.4 / 7.4; 40, keep 3 7.3 / 6.45 / 6.35.  (Several rounds of four entries, with all groups waiting for
+// one another in each, take longer than groups of their own: 128 blocks, keep 8 11.9 / 9.9.)
+template <int D>
+struct FourSmem {
+    static constexpr int TILE = MmaSmem<D>::TILE, G = 4;
+    static constexpr size_t TILES = (size_t)TILE * (1 + 2 * G) * sizeof(__nv_bfloat16);   // Q, K and V; P takes the place of K
+    static constexpr size_t MAXIMA = G * USV_BLOCK * sizeof(float);
+    static constexpr size_t SUMS = (size_t)G * 8 * USV_BLOCK * 4 * sizeof(float);   // unrounded pairs, for the log-sum-exp
+    static constexpr size_t BYTES = TILES + MAXIMA + SUMS;
+};
+
+template <int D>
+__global__ void __launch_bounds__(512) attn_four_kernel(const AttnArgs a) {
+    dep_sync();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    using F = FourSmem<D>;
+    constexpr int LD = MmaSmem<D>::LD, TILE = F::TILE, G = F::G;
+    constexpr int NC = D / G / 8;   // n-tiles of the output a group has
+    static_assert(NC == 2, "one ldmatrix of V per k-step");
+    if (blockIdx.x == 0 && threadIdx.x < (WS_HEADER - 4) / 4) a.status[1 + threadIdx.x] = 0u;   // (as attn_mma_kernel does)
+    __nv_bfloat16* Qs = reinterpret_cast<__nv_bfloat16*>(smem_raw);
+    auto k_tile = [&](int grp) { return Qs + TILE * (1 + 2 * grp); };   // V behind it
+    float* s_max = reinterpret_cast<float*>(smem_raw + F::TILES);                 // [G][64]
+    float* s_sum = reinterpret_cast<float*>(smem_raw + F::TILES + F::MAXIMA);     // [G][8][64][4]
+
+    const int I = blockIdx.x % a.NB, bh_ord = blockIdx.x / a.NB;
+    const int b = bh_ord / a.H, h = a.head_order[bh_ord % a.H];
+    const int kh = a.k_per_head[h], N = a.N;
+    const int32_t* sel = a.sel + (((int64_t)b * a.H + h) * a.NB + I) * a.kmax;
+    const __nv_bfloat16* K = a.k + b * a.sk.sb + h * a.sk.sh;
+    const __nv_bfloat16* V = a.v + b * a.sv.sb + h * a.sv.sh;
+    const int grp = threadIdx.x >> 7, warp = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;
+    const int g = lane >> 2, tig = lane & 3;
+
+    // the group's entry: the grp-th of the valid ones
+    const int e_lane = lane < kh ? sel[lane] : -1;
+    const unsigned valid = __ballot_sync(0xffffffffu, e_lane >= 0);
+    const int entries = __popc(valid);   // at most G
+    const unsigned here = __ballot_sync(0xffffffffu, e_lane >= 0 && __popc(valid & ((1u << lane) - 1u)) == grp);
+    const int J = __shfl_sync(0xffffffffu, e_lane, here ? __ffs(here) - 1 : 0);
+    load_tile<D, G>(Qs, a.q + b * a.sq.sb + h * a.sq.sh, a.sq.sn, I * USV_BLOCK, N);
+    if (grp < entries) load_tile<D>(k_tile(grp), K, a.sk.sn, J * USV_BLOCK, N);
+    cp_async_commit();
+    if (grp < entries) load_tile<D>(k_tile(grp) + TILE, V, a.sv.sn, J * USV_BLOCK, N);
+    cp_async_commit();
+    asm volatile("cp.async.wait_group 1;\n" ::: "memory");   // Q and K
+    __syncthreads();
+
+    uint32_t qf[D / 16][4];
+    float o[NC][4] = {};
+    float m[2] = {-INFINITY, -INFINITY};   // (as in attn_mma_block)
+    // Of the sums over a row's weights each group takes one: of the rounded ones of rows g (0) and g + 8 (1), of the others (2, 3).
+    const int own = grp & 1;
+    float sum = 0.f;
+    const float c = a.scale_log2;
+    const int row = warp * 16 + g;
+    load_q_frags<D>(qf, Qs, warp, lane);
+    float s[8][4];
+    if (grp < entries) {
+        float mx[2];
+        tile_logits<D>(s, mx, qf, k_tile(grp), N - J * USV_BLOCK, lane);
+        if (tig < 2) s_max[grp * USV_BLOCK + row + 8 * tig] = tig ? mx[1] : mx[0];
+    }
+    __syncthreads();
+    float alpha[G][2], ms[2] = {0.f, 0.f};
+#pragma unroll
+    for (int t = 0; t < G; ++t)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            float at;
+            alpha[t][r] = t < entries ? next_max(m[r], s_max[t * USV_BLOCK + row + 8 * r], c, at) : 1.f;
+            if (t == grp && t < entries) ms[r] = at;
+        }
+    if (grp < entries) {
+        uint32_t pf[4][4];
+        float* sums = s_sum + grp * (8 * USV_BLOCK * 4) + row * 4 + tig;
+        tile_weights(s, c, ms, pf, [&](int nt, int r, float e, uint32_t) {
+            if (a.lse != nullptr) sums[nt * (USV_BLOCK * 4) + r * 32] = e;
+        });
+        __nv_bfloat16* P = k_tile(grp) + row * LD + 2 * tig;   // (nobody reads the K tile any more)
+#pragma unroll
+        for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+                *reinterpret_cast<uint32_t*>(P + 8 * r * LD + nt * 8) = pf[nt >> 1][(nt & 1) * 2 + r];
+    }
+    cp_async_wait_all();   // V
+    __syncthreads();
+#pragma unroll
+    for (int t = 0; t < G; ++t) {
+        if (t >= entries) break;
+        const __nv_bfloat16* prow = k_tile(t) + (warp * 16 + (lane & 15)) * LD + (lane >> 4) * 8;
+        const __nv_bfloat16* vrow = k_tile(t) + TILE + (lane & 15) * LD + grp * (8 * NC) + (lane >> 4) * 8;
+#pragma unroll
+        for (int i = 0; i < NC; ++i)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) o[i][e] *= alpha[t][e >> 1];
+#pragma unroll
+        for (int kt = 0; kt < 4; ++kt) {
+            uint32_t pf[4], bfr[4];
+            ldmatrix_x4(pf, prow + kt * 16);
+            ldmatrix_x4_trans(bfr, vrow + kt * 16 * LD);
+            mma_bf16_16816(o[0], pf, bfr[0], bfr[1]);
+            mma_bf16_16816(o[1], pf, bfr[2], bfr[3]);
+            if (grp < 2) {
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {   // 8-key piece 2 kt + e
+                    const float w = sum_bf16x2(own ? pf[2 * e + 1] : pf[2 * e]);
+                    sum = kt == 0 && e == 0 ? fmaf(sum, own ? alpha[t][1] : alpha[t][0], w) : sum + w;
+                }
+            }
+        }
+        if (grp >= 2 && a.lse != nullptr) {
+            const float* sums = s_sum + t * (8 * USV_BLOCK * 4) + (row + 8 * own) * 4 + tig;
+#pragma unroll
+            for (int nt = 0; nt < 8; ++nt) {
+                const float e = sums[nt * (USV_BLOCK * 4)];
+                sum = nt == 0 ? fmaf(sum, own ? alpha[t][1] : alpha[t][0], e) : sum + e;
+            }
+        }
+    }
+
+    sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+    sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+    if (tig == 0 && grp < 2) s_max[grp * USV_BLOCK + row] = sum;   // (nobody reads the maxima any more)
+    if (tig == 0 && grp >= 2 && a.lse != nullptr) {
+        const int at = I * USV_BLOCK + row + 8 * own;
+        if (at < N) a.lse[((int64_t)b * a.H + h) * N + at] = sum > 0.f ? ((own ? m[1] : m[0]) + log2f(sum)) * 0.69314718055994531f : 0.f;
+    }
+    __syncthreads();
+    // the group's columns, the bf16 ones through the (now idle) Q tile for 16-byte stores
+    __nv_bfloat16* stage = Qs + warp * 16 * LD + grp * (8 * NC);
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const float lr = s_max[r * USV_BLOCK + row], inv = lr > 0.f ? 1.f / lr : 0.f;
+        const int at = I * USV_BLOCK + row + 8 * r;
+        const int64_t at_bh = ((int64_t)b * a.H + h) * N + at;
+#pragma unroll
+        for (int i = 0; i < NC; ++i) {
+            const float y0 = o[i][2 * r] * inv, y1 = o[i][2 * r + 1] * inv;
+            if (a.o_f32 != nullptr && at < N)
+                *reinterpret_cast<float2*>(a.o_f32 + at_bh * D + grp * (8 * NC) + i * 8 + 2 * tig) = make_float2(y0, y1);
+            *reinterpret_cast<uint32_t*>(stage + (g + 8 * r) * LD + i * 8 + 2 * tig) = pack_bf16x2(y0, y1);
+        }
+    }
+    __syncwarp();
+    const int out_row = I * USV_BLOCK + warp * 16 + (lane >> 1);
+    if (out_row < N)
+        *reinterpret_cast<uint4*>(a.o + b * a.so.sb + h * a.so.sh + (int64_t)out_row * a.so.sn + grp * (8 * NC) + (lane & 1) * 8) =
+            *reinterpret_cast<const uint4*>(stage + (lane >> 1) * LD + (lane & 1) * 8);
+}
+
+int launch_attn_four(const AttnArgs& a, cudaStream_t st) {
+    constexpr size_t smem = FourSmem<64>::BYTES;
+    static_assert(smem <= 232448, "shared memory budget");
+    cudaError_t e = cudaFuncSetAttribute(attn_four_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return fail(USV_ERR_CUDA, "sparse_attn: smem attribute: %s", cudaGetErrorString(e));
+    launch_dep_smem(attn_four_kernel<64>, dim3((unsigned)(a.B * a.H * a.NB)), dim3(512), smem, st, a);
+    USV_CHECK_LAUNCH("attn_four_kernel");
     return USV_OK;
 }
 
@@ -376,10 +563,6 @@ int launch_attn_one(const AttnArgs& a, cudaStream_t st) {
     launch_dep_smem(attn_one_kernel<64>, dim3((unsigned)blocks), dim3(128), smem, st, a);
     USV_CHECK_LAUNCH("attn_one_kernel");
     return USV_OK;
-}
-
-int launch_attn_split(const AttnArgs& a, int most, cudaStream_t st) {
-    return most <= 4 ? launch_split<64, 4, 1>(a, st) : launch_split<64, 4, 2>(a, st);
 }
 
 int launch_attn_mma(const AttnArgs& a, int d, cudaStream_t st) {
