@@ -348,8 +348,11 @@ attn_dense_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
         }
     } else if (warp < W_EPI) {
         // ===== softmax warpgroups ================================================================
-        // Slot n % NSLOT of the sums and references is used again by item n + NSLOT, whose first S tile waits for a P.V
-        // of item n + 1 at the earliest, and that for the output warps to have read item n (OFREE).
+        // Slot n % NSLOT of the sums and references is used again by item n + NSLOT.  With two tiles an item and more (attn_dense_heads
+        // sees to that) every group has a tile in every item, and the first S tile of item n + 4 waits for the P.V of a tile three
+        // before it, of item n + 2 at the earliest.  That was issued behind the first P.V of its item, which waits for
+        // the output warps to have read item n + 1 (OFREE), and so item n.  (With one tile a group without it would
+        // wait for nothing, and its arrival for item n + 4 could be counted for item n.)
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REG_SOFT));
         const int grp = warp >> 2;                       // tiles of running parity grp >> 1, key block grp & 1
         const int tp = grp >> 1, hb = grp & 1;
@@ -476,15 +479,19 @@ static int dense_clusters() {
     return n;
 }
 
-// Calls whose heads are all full, beyond those without a plan (which look at the lists for holes), always go here (us, pair
-// kernel / this one: 12 heads x 30 blocks 37.0 / 34.8; 24 x 30 50.6 / 47.1; 1 x 317 250 / 224; 4 x 317 672 / 607; 12 x 317 1899 / 1687; 1 x 1857 5671 /
-// 5102).  Where other heads are sparse the two kernels run one after the other, and what the last, partly empty wave of
+// Calls whose heads are all full, beyond those without a plan, go here (us, pair kernel with a plan / this one: 12 heads x 30 blocks
+// 42.5 / 40.9; 24 x 28 48.2 / 45.4; 1 x 140 62.6 / 58.2; 1 x 317 250 / 224; 4 x 317 672 / 607; 12 x 317 1899 / 1687; 1 x 1857 5671 / 5102; 1000 x 3
+// 88.5 / 64.6; 2400 x 5 267 / 252; 1600 x 7 288 / 249; 800 x 8 190 / 167).  An item has four query blocks however many of them there are: with one
+// or two left for the last item, sequences of 9 to 18 blocks are faster there (900 x 9 258 / 267, 800 x 10 215 / 221, 600 x 13 267 / 277, 600 x 14
+// 276 / 289, 400 x 17 289 / 291; but 400 x 21 401 / 397, 200 x 25 278 / 268).  Two tiles an item are the least (see the softmax warps).
+// Where other heads are sparse the two kernels run one after the other, and what the last, partly empty wave of
 // this one leaves idle has to be won back: 16 heads x 317 blocks, four of them full (4.3 waves), 978 / 1007; 24 heads, six full
 // (6.5 waves), 1435 / 1403; 48 x 122, twelve full (5.0 waves), 491 / 502.
 int attn_dense_heads(const AttnArgs& a, int d) {
     int full = 0;
     while (full < a.H && a.k_per_head[a.head_order[full]] >= a.NB) ++full;
-    if (full == 0 || d != dn::D || a.y != nullptr) return 0;
+    if (full == 0 || d != dn::D || a.y != nullptr || a.NB < 3) return 0;
+    if ((a.NB & 3) != 0 && (a.NB & 3) != 3 && a.NB >= 9 && a.NB <= 18) return 0;
     const int64_t items = (int64_t)a.B * full * ((a.NB + 3) / 4);
     if (items > 1000000000LL) return 0;
     const int clusters = dense_clusters();

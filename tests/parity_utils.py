@@ -46,6 +46,22 @@ def check_selection(sel_gpu, scores64, k_per_head):
     return B * H * NBq, ambiguous, differing
 
 
+def attention_path(call, query_blocks):
+    """Which kernels call(), one sparse_attn_fwd on the current stream that recomputes fewer than half of its query blocks, ran: "one
+    kernel", "no plan", "dense", "plan" or "plan, dense".  Told by the launches (plan and dense kernel one each, an ordered plan three
+    more) and by the scratch buffer: calls without a plan write a flag for every query block, the others list the few recomputed ones."""
+    from paper_2512_05754_b200 import binding
+    call()                                                   # (the buffer has its size)
+    flags = binding._workspace(torch.device("cuda", torch.cuda.current_device()), 0)[256:256 + 2 * query_blocks]
+    flags.fill_(0xab)
+    before = binding.kernel_launches()
+    call()
+    n = binding.kernel_launches() - before
+    if n == 2:
+        return "dense" if bool((flags == 0xab).any()) else "no plan"
+    return {1: "one kernel", 3: "plan", 4: "plan, dense", 6: "plan", 7: "plan, dense"}[n]
+
+
 def attn_errors(o_gpu, o_ref):
     """(max abs error, relative L2 error) of two arrays of the same shape (fp64 math)."""
     a = np.asarray(o_gpu, dtype=np.float64)
