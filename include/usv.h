@@ -135,7 +135,8 @@ int usv_select_blocks(int B, int H, int NBq, int NBk, const float* scores,
  * bf16 operands on the tensor cores, fp32 online softmax and accumulation, bf16 output.
  *
  * q,k,v: bf16 views [B,H,N,d] (self-attention: one N); d in {64,128}.
- * sel: int32 [B,H,NB,kmax], entries in [0,NB), -1 entries are skipped.
+ * sel: int32 [B,H,NB,kmax], entries in [0,NB), -1 entries are skipped (also in lists of NB entries; of those, which otherwise
+ * are the full set, the d = 128 kernel of large calls hands the ones with -1 entries to the exact kernel, which is slower).
  * k_per_head: HOST int32[H].  o: bf16 view [B,H,N,d] (written, rows < N only).
  * o_f32: optional fp32 [B,H,N,d] contiguous copy of the un-rounded output (NULL to skip).
  * lse: optional fp32 [B,H,N], natural-log of the softmax denominator (NULL to skip).  At d = 64, and with impl 1, it is
@@ -188,7 +189,8 @@ int usv_sparse_attn_fwd_unmerge(int B, int H, int N, int d, const void* q, const
                                 void* stream);
 
 /* After usv_sparse_attn_fwd with impl 0: how many query blocks the tcgen05 kernel handed to the
- * exact kernel because their softmax sums left the safe exponent range (normally 0).
+ * exact kernel because their softmax sums left the safe exponent range or (large calls at d = 128)
+ * a list of NB entries had a -1 among them (normally 0).
  * Synchronises `stream`.  ws is the workspace that call used. */
 int usv_sparse_attn_fallbacks(const void* ws, void* stream, int* count);
 

@@ -59,10 +59,9 @@ int launch_scatter_fallbacks(const AttnArgs& a, int d, cudaStream_t st);
 // ints one pair's list occupies for a head that keeps k of NB key blocks (header + entries)
 __host__ __device__ inline int64_t list_stride(int k, int NB) { return 1 + (int64_t)(2 * (int64_t)k < NB ? 2 * k : NB); }
 size_t pair_plan_bytes(int B, int H, int NB, const int32_t* k_per_head);
-// Fills a.pairs / a.lists / a.list_* (pointing into mem) and enqueues the plan kernels.  as_listed: a list of as many
-// entries as there are key blocks may have holes (the attention takes it for the full set).  What the attention kernel
+// Fills a.pairs / a.lists / a.list_* (pointing into mem) and enqueues the plan kernels.  What the attention kernel
 // counts in the header starts at zero where a.work_counter is given.
-int launch_pair_plan(AttnArgs& a, void* mem, bool as_listed, cudaStream_t st);
+int launch_pair_plan(AttnArgs& a, void* mem, cudaStream_t st);
 constexpr int PLAN_MAX_NB = 4096;   // key blocks of the longest sequence a plan covers
 
 }  // namespace usv

@@ -116,7 +116,7 @@ static int sparse_attn_impl(int B, int H, int N, int d, const void* q, const usv
         }
         a.full_heads = attn_dense_heads(a, d);
         if (a.full_heads < H) {
-            if ((rc2 = launch_pair_plan(a, plan_mem, false, st)) != USV_OK) return rc2;
+            if ((rc2 = launch_pair_plan(a, plan_mem, st)) != USV_OK) return rc2;
         } else {
             cudaError_t e = cudaMemsetAsync(a.status + 1, 0, WS_HEADER - 4, st);   // (what the plan does otherwise)
             if (e != cudaSuccess) return fail(USV_ERR_CUDA, "sparse_attn: memset: %s", cudaGetErrorString(e));

@@ -42,7 +42,6 @@ struct Order {
     uint8_t* taken;            // [B*H][NB] written by the first pass: 1 = paired
     int* count;                // [B*H] pairs written so far (starts at zero)
     int pass;                  // 0: one pass in index order (the rest unused); 1, 2: first and second of two
-    int as_listed;             // lists of as many entries as there are key blocks are read too (the marginal's may have holes)
 };
 
 __device__ __forceinline__ uint32_t mix12(uint32_t x, uint32_t a, uint32_t b) {   // a bijection of 0 .. 4095
@@ -136,6 +135,28 @@ __global__ void __launch_bounds__(1024) plan_sort_kernel(int NB, const uint32_t*
         if (4 * t + q < NB) by_rank[base + 4 * t + q] = (uint16_t)(x[q] & 4095u);
 }
 
+// The ascending union of two bitmaps over the key blocks, each entry flagged with the row(s) it is from (bitsB NULL: one row);
+// a warp's work.  out[0]: number of entries.
+__device__ __forceinline__ void write_union(const uint32_t* bitsA, const uint32_t* bitsB, int nwords, int* __restrict__ out) {
+    const int lane = threadIdx.x & 31;
+    int running = 0;
+    for (int w0 = 0; w0 < nwords; w0 += 32) {
+        const int w = w0 + lane;
+        const uint32_t ba = w < nwords ? bitsA[w] : 0u;
+        const uint32_t bb = (w < nwords && bitsB != nullptr) ? bitsB[w] : 0u;
+        uint32_t u = ba | bb;
+        const int incl = warp_incl_scan(__popc(u));
+        int off = running + incl - __popc(u);
+        while (u) {
+            const int bit = __ffs(u) - 1;
+            u &= u - 1;
+            out[1 + off++] = ((w * 32 + bit) << 2) | ((ba >> bit) & 1u) | (((bb >> bit) & 1u) << 1);
+        }
+        running += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    if (lane == 0) out[0] = running;
+}
+
 // One CTA per chunk of CH query blocks of one (batch, head).
 //   1. bitmaps of the chunk's selection rows (shared memory)
 //   2. overlap |sel(I) & sel(J)| of every two blocks of the chunk
@@ -180,7 +201,7 @@ pair_plan_kernel(const AttnArgs a, int2* __restrict__ pairs, int* __restrict__ l
     // its CTAs, already resident, would leave room for one CTA of this kernel an SM instead of two (D = 64, 12 heads x 256
     // blocks, keep 26: 134 us a call, 138 with the wait behind the signal).
     dep_wait();
-    const bool full = kh >= NB && !ord.as_listed;   // every list is the full set: no overlaps to compute
+    const bool full = kh >= NB;   // every list is the full set but for holes: no overlaps to compute
     if (warp == 0 && !full) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(t5::smem_u32(&s_tmem)), "r"(128u) : "memory");
@@ -206,14 +227,34 @@ pair_plan_kernel(const AttnArgs a, int2* __restrict__ pairs, int* __restrict__ l
         if (ord.pass == 2 || a.full_heads > 0) return;   // (done by the first pass, or not wanted)
         out_pairs += blockIdx.x * (CH / 2);
         out_lists += (int64_t)blockIdx.x * (CH / 2) * lstride;
-        // every list is the full set: pairing is arbitrary and every key block belongs to both sides
+        // every list is the full set unless it has holes: pairing is arbitrary and every key block belongs to both sides
         for (int p = threadIdx.x; p < npairs; p += THREADS)
             out_pairs[p] = make_int2(I0 + 2 * p, 2 * p + 1 < nI ? I0 + 2 * p + 1 : -1);
+        uint32_t* mine = bm + 2 * warp * pitch;
         for (int p = warp; p < npairs; p += THREADS / 32) {
             int* out = out_lists + (int64_t)p * lstride;
-            const int flags = 2 * p + 1 < nI ? 3 : 1;
-            for (int j = lane; j < NB; j += 32) out[1 + j] = (j << 2) | flags;
+            const bool two = 2 * p + 1 < nI;
+            const int flags = two ? 3 : 1;
+            const int32_t* row = a.sel + ((int64_t)bh * NB + I0 + 2 * p) * a.kmax;
+            const int32_t* other = two ? row + a.kmax : row;
+            bool hole = false;
+#pragma unroll 4
+            for (int j = lane; j < NB; j += 32) {
+                out[1 + j] = (j << 2) | flags;
+                hole |= (unsigned)__ldg(row + j) >= (unsigned)NB || (unsigned)__ldg(other + j) >= (unsigned)NB;
+            }
             if (lane == 0) out[0] = NB;
+            if (!__any_sync(0xffffffffu, hole)) continue;
+            for (int i = lane; i < 2 * pitch; i += 32) mine[i] = 0u;
+            __syncwarp();
+            for (int j = lane; j < NB; j += 32) {
+                const unsigned ja = __ldg(row + j), jb = two ? __ldg(other + j) : -1;
+                if (ja < (unsigned)NB) atomicOr(&mine[ja >> 5], 1u << (ja & 31));
+                if (jb < (unsigned)NB) atomicOr(&mine[pitch + (jb >> 5)], 1u << (jb & 31));
+            }
+            __syncwarp();
+            write_union(mine, mine + pitch, nwords, out);
+            __syncwarp();
         }
         return;
     }
@@ -423,25 +464,7 @@ pair_plan_kernel(const AttnArgs a, int2* __restrict__ pairs, int* __restrict__ l
     // 5. union lists
     for (int p = warp; p < s_count; p += THREADS / 32) {
         const int i = order[p], j = partner[i];
-        const uint32_t* bitsA = bm + i * pitch;
-        const uint32_t* bitsB = bm + (j >= 0 ? j : i) * pitch;
-        int* out = out_lists + (int64_t)p * lstride;
-        int running = 0;
-        for (int w0 = 0; w0 < nwords; w0 += 32) {
-            const int w = w0 + lane;
-            const uint32_t ba = w < nwords ? bitsA[w] : 0u;
-            const uint32_t bb = (w < nwords && j >= 0) ? bitsB[w] : 0u;
-            uint32_t u = ba | bb;
-            const int incl = warp_incl_scan(__popc(u));
-            int off = running + incl - __popc(u);
-            while (u) {
-                const int bit = __ffs(u) - 1;
-                u &= u - 1;
-                out[1 + off++] = ((w * 32 + bit) << 2) | ((ba >> bit) & 1u) | (((bb >> bit) & 1u) << 1);
-            }
-            running += __shfl_sync(0xffffffffu, incl, 31);
-        }
-        if (lane == 0) out[0] = running;
+        write_union(bm + i * pitch, j >= 0 ? bm + j * pitch : nullptr, nwords, out_lists + (int64_t)p * lstride);
     }
 }
 
@@ -498,7 +521,7 @@ struct PlanLayout {
 
 size_t pair_plan_bytes(int B, int H, int NB, const int32_t* k_per_head) { return PlanLayout(B, H, NB, k_per_head).total; }
 
-int launch_pair_plan(AttnArgs& a, void* mem, bool as_listed, cudaStream_t st) {
+int launch_pair_plan(AttnArgs& a, void* mem, cudaStream_t st) {
     const int NP = (a.NB + 1) / 2, BH = a.B * a.H;
     char* base = static_cast<char*>(mem);
     const PlanLayout L(a.B, a.H, a.NB, a.k_per_head);
@@ -518,11 +541,11 @@ int launch_pair_plan(AttnArgs& a, void* mem, bool as_listed, cudaStream_t st) {
     cudaError_t e = cudaFuncSetAttribute(plan::pair_plan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan::MOST_SMEM);
     if (e != cudaSuccess) return fail(USV_ERR_CUDA, "sparse_attn: plan smem attribute: %s", cudaGetErrorString(e));
     const dim3 grid((a.NB + plan::CH - 1) / plan::CH, BH);
-    plan::Order ord = {nullptr, nullptr, nullptr, 0, as_listed};
+    plan::Order ord = {nullptr, nullptr, nullptr, 0};
     if (plan::plan_ordered(a)) {
         uint32_t* keys = reinterpret_cast<uint32_t*>(base + L.keys);
         uint16_t* by_rank = reinterpret_cast<uint16_t*>(base + L.by_rank);
-        ord = {by_rank, reinterpret_cast<uint8_t*>(base + L.taken), reinterpret_cast<int*>(base + L.count), 1, as_listed};
+        ord = {by_rank, reinterpret_cast<uint8_t*>(base + L.taken), reinterpret_cast<int*>(base + L.count), 1};
         const int64_t rows = (int64_t)BH * a.NB;
         launch_dep_smem(plan::plan_keys_kernel, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, a, keys, ord.count);
         USV_CHECK_LAUNCH("plan_keys_kernel");

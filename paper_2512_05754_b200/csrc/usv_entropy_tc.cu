@@ -375,7 +375,7 @@ int launch_marginal_plan(MargArgs& a, void* mem, cudaStream_t st) {
     p.status = a.status;
     p.B = a.B; p.H = a.H; p.N = a.N; p.NB = a.NB; p.kmax = a.kmax;
     for (int h = 0; h < a.H; ++h) p.k_per_head[h] = a.k_per_head[h];
-    const int rc = launch_pair_plan(p, mem, true, st);
+    const int rc = launch_pair_plan(p, mem, st);
     if (rc != USV_OK) return rc;
     a.pairs = p.pairs;
     a.lists = p.lists;
