@@ -49,7 +49,7 @@ int launch_attn_split(const AttnArgs& a, cudaStream_t st);
 int launch_attn_one(const AttnArgs& a, cudaStream_t st);
 bool attn_pair_supported(const AttnArgs& a, int d);
 // whether the call is too small for a pairing plan: a.pairs stays NULL, and fallback_list takes flags
-bool attn_pair_direct(const AttnArgs& a, int d);
+bool attn_pair_direct(const AttnArgs& a, int d, int sms);
 int launch_attn_pair(const AttnArgs& a, int d, cudaStream_t st);
 // Heads that keep every key block and are better computed by the kernel of usv_attn_dense.cu (the first of a.head_order); 0: none.
 int attn_dense_heads(const AttnArgs& a, int d);

@@ -109,7 +109,7 @@ static int sparse_attn_impl(int B, int H, int N, int d, const void* q, const usv
     if (impl == 0 && d == 64 && blocks > 1800 && kmx == 1) return launch_attn_one(a, st);
     if (impl == 0 && !small && attn_pair_supported(a, d)) {
         int rc2;
-        if (attn_pair_direct(a, d)) {
+        if (attn_pair_direct(a, d, sms)) {
             if ((rc2 = launch_attn_pair(a, d, st)) != USV_OK) return rc2;
             a.work_flags = reinterpret_cast<const uint16_t*>(a.fallback_list);
             return launch_attn_mma(a, d, st);

@@ -801,19 +801,29 @@ bool attn_pair_supported(const AttnArgs& a, int d) {
 //   D = 64: 2.7 k 24.1 / 17.3, 8.2 k 35.6 / 30.5, 14 k (4560 blocks) 62.8 / 66.3, 19 k 51.4 / 44.6, 22 k (2256) 56.0 / 54.5,
 //     37 k (1464) 74.9 / 71.2, 38 k (2928) 86.7 / 89.6, 39 k (1760) 79.0 / 77.6, 43 k (2256) 82.5 / 86.3, 58 k (2640) 115.8 / 127.6
 // (Beyond 1024 blocks or lists of 256 the scout's registers and ring slots do not hold a union.)
-bool attn_pair_direct(const AttnArgs& a, int d) {
+// Full lists have nothing to pair for, and their plan is written in 3 us: with it / without it (dense kernel where it takes them),
+// D = 128, 9 k 33.1 / 33.0 (31.7), 10.8 k 42.5 / 43.2 (40.9), 18 k 49.2 / 50.8 (47.0), 20 k 62.6 / 66.3 (58.2); D = 64, 10.8 k 28.7 / 30.4,
+// 20 k 41.6 / 44.6, 31 k 44.5 / 47.4.  (Of sequences up to six blocks the dense kernel's items are half empty: 300 x 6 44.0, 41.5 without.)
+// At D = 64 the largest calls have lists so long that a last wave of few items shows, which the plan's shorter lists make up for:
+// 4 heads x 150 blocks (2.03 waves) 77.2 / 86.3, 5 x 120 78.6 / 84.6, 3 x 200 83.7 / 87.9, 2 x 180 (1.22 waves) 94.6 / 97.5; but 6 x 110
+// (2.23) 68.2 / 69.7 and 71.1 / 65.8, 8 x 80 (2.16) 64.5 / 58.2, 8 x 90 (2.43) 71.3 / 70.3, 4 x 140 (1.89) 68.4 / 63.1, 12 x 70 (2.84) 62.7 / 56.4.
+bool attn_pair_direct(const AttnArgs& a, int d, int sms) {
     int64_t kept = 0;
-    int most = 0;
+    int most = 0, least = a.NB;
     for (int h = 0; h < a.H; ++h) {
         kept += a.k_per_head[h];
         most = a.k_per_head[h] > most ? a.k_per_head[h] : most;
+        least = a.k_per_head[h] < least ? a.k_per_head[h] : least;
     }
     const int64_t blocks = (int64_t)a.B * a.H * a.NB;
     kept *= (int64_t)a.B * a.NB;
     // Single kept blocks need neither bitmaps nor pairs, whatever their number: 24 heads x 100 blocks, D = 128, 47.2 / 42.0,
     // 24 x 317 107 / 88, 40 x 300 154 / 137.
     if (a.y == nullptr && most == 1) return true;
-    const bool few = d == 64 ? (kept <= 36000 && blocks <= 1800) || (kept <= 24000 && blocks <= 2400)
+    if (least >= a.NB && a.NB > 6 && kept > 10000) return false;
+    const int64_t items = (int64_t)a.B * a.H * ((a.NB + 1) / 2), waves = (items + sms - 1) / sms;
+    const bool idle = waves > 1 && 10 * items < 7 * waves * sms;   // of the last wave, most
+    const bool few = d == 64 ? (kept <= 36000 && blocks <= 1800 && !idle) || (kept <= 24000 && blocks <= 2400)
                              : (kept <= 20000 && blocks <= 1700) || (kept <= 13000 && blocks <= 2300);
     return a.y == nullptr && a.NB <= 1024 && 2 * most <= pr::LCAP && few;
 }

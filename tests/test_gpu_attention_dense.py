@@ -69,7 +69,8 @@ def _check(B, H, N, kph, path, token_major=False, edit=None, d=128, holes=None):
     ("dense", 10, 80, 64 * 3, False), ("dense", 10, 80, 64 * 2 + 5, True), ("dense", 10, 60, 64 * 4 - 9, False), ("dense", 10, 48, 64 * 5, True),
     ("dense", 8, 50, 64 * 5 + 3, False), ("dense", 7, 50, 64 * 7 - 1, False), ("dense", 3, 100, 64 * 8, True), ("dense", 1, 60, 64 * 19 - 7, False),
     ("dense", 2, 24, 64 * 30 + 63, True), ("dense", 1, 2, 64 * 101 + 64, False), ("dense", 1, 1, 64 * 145 + 3, False),
-    ("dense", 1, 2, 64 * 150 + 9, False), ("dense", 2, 2, 64 * 104, True),
+    ("dense", 1, 2, 64 * 150 + 9, False), ("dense", 2, 2, 64 * 104, True), ("dense", 1, 12, 64 * 29 + 1, False), ("no plan", 1, 12, 64 * 28, False),
+    ("dense", 3, 70, 64 * 7 - 3, True),
     ("plan", 20, 60, 65, False), ("plan", 20, 60, 64 * 2, True), ("plan", 3, 80, 64 * 10, False), ("plan", 2, 100, 64 * 12 + 1, False),
     ("no plan", 11, 100, 37, False), ("no plan", 10, 120, 64, True), ("no plan", 9, 60, 65, True), ("no plan", 4, 90, 64 * 3, False),
     ("no plan", 3, 80, 64 * 4 + 1, False), ("no plan", 3, 100, 64 * 5 + 3, True), ("no plan", 4, 75, 64 * 6, False)])
@@ -86,7 +87,7 @@ def test_full_heads_beside_sparse_ones(N):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("path,N", [("dense", 64 * 100), ("dense", 64 * 101 + 5), ("no plan", 64 * 40), ("no plan", 64 * 41 + 5)])
+@pytest.mark.parametrize("path,N", [("dense", 64 * 100), ("dense", 64 * 101 + 5), ("no plan", 64 * 40), ("no plan", 64 * 41 + 5), ("dense", 64 * 60)])
 def test_rows_out_of_range_go_to_the_exact_kernel(path, N):
     """A row's reference is its maximum over the first key block; here later keys of some rows exceed it by more than 100
     powers of two.  Every query block with such a row is counted once."""
