@@ -295,8 +295,11 @@ int usv_attn_entropy(int B, int H, int N, int d, const void* q, const usv_stride
                      float* key_marginal, float* entropy, void* ws, void* stream);
 
 /* The same with scratch memory, with which large calls are faster: query blocks whose lists overlap are paired first.
- * ws: as above, ws_bytes of it; with fewer than usv_attn_entropy_workspace() bytes (or NULL) the call is usv_attn_entropy. */
+ * ws: as above, ws_bytes of it; with fewer than the call's lists need (or NULL) the call is usv_attn_entropy.
+ * usv_attn_entropy_lists_workspace: the bytes that are of use to a call with these lists on the current device, USV_WS_HEADER
+ * where nothing is paired; usv_attn_entropy_workspace: enough for any lists of at most kmax blocks. */
 size_t usv_attn_entropy_workspace(int B, int H, int N, int kmax);
+size_t usv_attn_entropy_lists_workspace(int B, int H, int N, const int32_t* k_per_head);
 int usv_attn_entropy_ws(int B, int H, int N, int d, const void* q, const usv_strides* sq,
                         const void* k, const usv_strides* sk, const int32_t* sel,
                         const int32_t* k_per_head, int kmax, const float* lse, float scale,

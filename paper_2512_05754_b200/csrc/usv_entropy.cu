@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(1024) entropy_kernel(const float* __restrict__
 static int attn_entropy_impl(int B, int H, int N, int d, const void* q, const usv_strides* sq,
                              const void* k, const usv_strides* sk, const int32_t* sel,
                              const int32_t* k_per_head, int kmax, const float* lse, float scale,
-                             float* key_marginal, float* entropy, void* ws, bool room, void* stream) {
+                             float* key_marginal, float* entropy, void* ws, size_t ws_bytes, void* stream) {
     using namespace usv;
     if (B <= 0 || H <= 0 || N <= 0) return fail(USV_ERR_INVALID_ARG, "attn_entropy: B,H,N must be positive");
     if (d != 64 && d != 128) return fail(USV_ERR_UNSUPPORTED, "attn_entropy: d=%d (need 64 or 128)", d);
@@ -83,7 +83,8 @@ static int attn_entropy_impl(int B, int H, int N, int d, const void* q, const us
     if (e != cudaSuccess) return fail(USV_ERR_CUDA, "attn_entropy: memset: %s", cudaGetErrorString(e));
     int sms;
     if ((rc = sm_count(&sms)) != USV_OK) return rc;
-    if (room && marginal_planned(a, sms) && (rc = launch_marginal_plan(a, static_cast<char*>(ws) + WS_HEADER, st)) != USV_OK)
+    if (ws != nullptr && ws_bytes > WS_HEADER && marginal_planned(a, sms) && ws_bytes >= WS_HEADER + pair_plan_bytes(B, H, NB, k_per_head) &&
+        (rc = launch_marginal_plan(a, static_cast<char*>(ws) + WS_HEADER, st)) != USV_OK)
         return rc;
     if ((rc = launch_marginal_tc(a, d, st)) != USV_OK) return rc;
     launch_dep_smem(entropy_kernel, dim3(B), dim3(1024), 0, st, key_marginal, N, entropy);
@@ -95,20 +96,33 @@ extern "C" int usv_attn_entropy(int B, int H, int N, int d, const void* q, const
                                 const void* k, const usv_strides* sk, const int32_t* sel,
                                 const int32_t* k_per_head, int kmax, const float* lse, float scale,
                                 float* key_marginal, float* entropy, void* ws, void* stream) {
-    return attn_entropy_impl(B, H, N, d, q, sq, k, sk, sel, k_per_head, kmax, lse, scale, key_marginal, entropy, ws, false, stream);
+    return attn_entropy_impl(B, H, N, d, q, sq, k, sk, sel, k_per_head, kmax, lse, scale, key_marginal, entropy, ws, 0, stream);
 }
 
 extern "C" size_t usv_attn_entropy_workspace(int B, int H, int N, int kmax) {
-    if (B <= 0 || H <= 0 || N <= 0 || H > USV_MAX_HEADS) return usv::WS_HEADER;
-    return usv::WS_HEADER + usv::marginal_plan_bytes(B, H, usv::ceil_div(N, USV_BLOCK), kmax);
+    using namespace usv;
+    if (B <= 0 || H <= 0 || N <= 0 || H > USV_MAX_HEADS) return WS_HEADER;
+    return WS_HEADER + marginal_plan_bytes(B, H, ceil_div(N, USV_BLOCK), kmax);
+}
+
+extern "C" size_t usv_attn_entropy_lists_workspace(int B, int H, int N, const int32_t* k_per_head) {
+    using namespace usv;
+    MargArgs a;
+    int sms;
+    if (B <= 0 || H <= 0 || N <= 0 || H > USV_MAX_HEADS || k_per_head == nullptr || sm_count(&sms) != USV_OK) return WS_HEADER;
+    a.B = B; a.H = H; a.N = N; a.NB = ceil_div(N, USV_BLOCK);
+    for (int h = 0; h < H; ++h) {
+        if (k_per_head[h] < 1 || k_per_head[h] > a.NB) return WS_HEADER;   // (refused by the call)
+        a.k_per_head[h] = k_per_head[h];
+    }
+    return WS_HEADER + (marginal_planned(a, sms) ? pair_plan_bytes(B, H, a.NB, k_per_head) : 0);
 }
 
 extern "C" int usv_attn_entropy_ws(int B, int H, int N, int d, const void* q, const usv_strides* sq,
                                    const void* k, const usv_strides* sk, const int32_t* sel,
                                    const int32_t* k_per_head, int kmax, const float* lse, float scale,
                                    float* key_marginal, float* entropy, void* ws, size_t ws_bytes, void* stream) {
-    const bool room = ws != nullptr && ws_bytes >= usv_attn_entropy_workspace(B, H, N, kmax);
-    return attn_entropy_impl(B, H, N, d, q, sq, k, sk, sel, k_per_head, kmax, lse, scale, key_marginal, entropy, ws, room, stream);
+    return attn_entropy_impl(B, H, N, d, q, sq, k, sk, sel, k_per_head, kmax, lse, scale, key_marginal, entropy, ws, ws_bytes, stream);
 }
 
 extern "C" int usv_allocate_sparsity(int L, const float* entropy, float gamma, float rho_bar, float rho_min,

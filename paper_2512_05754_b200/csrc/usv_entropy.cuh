@@ -25,7 +25,9 @@ struct MargArgs {
 int launch_marginal_tc(const MargArgs& a, int d, cudaStream_t st);
 // whether a pairing plan pays for the call
 bool marginal_planned(const MargArgs& a, int sms);
+// room for the plan of any call with lists of at most kmax blocks; 0 where none of them pays
 size_t marginal_plan_bytes(int B, int H, int NB, int kmax);
+size_t pair_plan_bytes(int B, int H, int NB, const int32_t* k_per_head);
 // Enqueues the plan of the call in mem and points a to it.
 int launch_marginal_plan(MargArgs& a, void* mem, cudaStream_t st);
 

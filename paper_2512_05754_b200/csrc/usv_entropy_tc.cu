@@ -364,8 +364,10 @@ bool marginal_planned(const MargArgs& a, int sms) {
 }
 
 size_t marginal_plan_bytes(int B, int H, int NB, int kmax) {
+    const int k = kmax < 1 ? 1 : (kmax > NB ? NB : kmax);
+    if (NB > PLAN_MAX_NB || (int64_t)B * H * NB * k < et::PLAN_MIN_WORK) return 0;   // (see marginal_planned)
     int32_t kk[USV_MAX_HEADS];
-    for (int h = 0; h < H; ++h) kk[h] = kmax < 1 ? 1 : (kmax > NB ? NB : kmax);
+    for (int h = 0; h < H; ++h) kk[h] = k;
     return pair_plan_bytes(B, H, NB, kk);
 }
 

@@ -332,7 +332,7 @@ PyObject* attn_entropy(PyObject* const* a) {
         NoGil off;
         marg = fresh({B, N}, at::kFloat, q);
         ent = fresh({B}, at::kFloat, q);
-        Scratch ws(q.device(), usv_attn_entropy_workspace((int)B, (int)H, (int)N, (int)sel.size(3)));
+        Scratch ws(q.device(), usv_attn_entropy_lists_workspace((int)B, (int)H, (int)N, kept.k.data()));
         check(usv_attn_entropy_ws((int)B, (int)H, (int)N, (int)d, ptr(q), &sq, ptr(k), &sk, (const int32_t*)ptr(sel),
                                   kept.k.data(), (int)sel.size(3), (const float*)ptr(lse), scale, (float*)ptr(marg),
                                   (float*)ptr(ent), ws.ptr(), ws.bytes(), stream_of(q)),

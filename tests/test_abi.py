@@ -102,6 +102,13 @@ def test_workspace_sizes(L):
     assert L.usv_block_scores_workspace(1, 12, 32760, 32760, 128) == header + means + planes
     assert L.usv_block_scores_workspace(1, 2, 1024, 1024, 64) == header + 2 * 2 * 16 * 64 * 4   # d = 64: header + means
     assert L.usv_token_merge_workspace(1, 32760, 1536, 12, 128) >= 32760 * 128 * 4
+    # the key marginal: a header, and a plan's room only where lists of that length can pay for one (500 000 kept blocks, 4096 blocks a row)
+    L.usv_attn_entropy_workspace.restype = L.usv_attn_entropy_lists_workspace.restype = ctypes.c_size_t
+    assert L.usv_attn_entropy_workspace(1, 24, 16384 * 64, 1639) == header
+    assert L.usv_attn_entropy_workspace(1, 12, 512 * 64, 52) == header
+    assert L.usv_attn_entropy_workspace(1, 40, 1182 * 64, 60) >= 40 * 591 * 121 * 4
+    assert L.usv_attn_entropy_lists_workspace(1, 2, 64 * 64, (ctypes.c_int32 * 2)(-5, 3)) == header
+    assert L.usv_attn_entropy_lists_workspace(1, 2, 64 * 64, None) == header
 
 
 def test_module_is_tied_to_the_torch_and_interpreter_it_was_built_for(monkeypatch):

@@ -23,7 +23,7 @@ class S(ctypes.Structure):
 def test_planned_marginal_is_the_plain_one(B, H, N, d, kph, holes):
     from paper_2512_05754_b200 import binding
     L = binding.lib()
-    L.usv_attn_entropy_workspace.restype = ctypes.c_size_t
+    L.usv_attn_entropy_workspace.restype = L.usv_attn_entropy_lists_workspace.restype = ctypes.c_size_t
     kph = (kph * H)[:H]
     NB, kmax = -(-N // 64), max(kph)
     assert B * NB * sum(k for k in kph if k < NB) >= 500000
@@ -41,10 +41,11 @@ def test_planned_marginal_is_the_plain_one(B, H, N, d, kph, holes):
         sel[:, :, 1::5, 0] = -1
     s = S(*q.stride()[:3])
     p = lambda t: ctypes.c_void_p(t.data_ptr())
-    n = L.usv_attn_entropy_workspace(B, H, N, kmax)
+    n = L.usv_attn_entropy_lists_workspace(B, H, N, (ctypes.c_int32 * H)(*kph))
+    assert 256 < n <= L.usv_attn_entropy_workspace(B, H, N, kmax)
     ws = torch.zeros(n, dtype=torch.uint8, device=DEV)
     out = []
-    for room in (256, n):
+    for room in (n - 1, n):
         marg, ent = torch.full((B, N), -1.0, device=DEV), torch.full((B,), -1.0, device=DEV)
         ws[4:256].fill_(7)
         before = L.usv_kernel_launches()
@@ -58,3 +59,19 @@ def test_planned_marginal_is_the_plain_one(B, H, N, d, kph, holes):
     assert torch.equal(out[0][0] == 0, out[1][0] == 0)
     assert (out[0][0] - out[1][0]).abs().max() <= 1e-5 * out[0][0].max()
     assert (out[0][1] - out[1][1]).abs().max() <= 1e-5 * out[0][1].abs().max()
+
+
+@pytest.mark.gpu
+def test_calls_without_a_plan_ask_for_no_room():
+    """Lists that a plan does not pay for, although one head keeps everything, take nothing beyond the header from a stream's buffer."""
+    import paper_2512_05754_b200 as usv
+    from paper_2512_05754_b200 import binding
+    H, NB = 2, 300
+    g = torch.Generator(device=DEV).manual_seed(5)
+    q, k = (torch.randn(1, H, 64 * NB, 64, generator=g, device=DEV).to(torch.bfloat16) for _ in range(2))
+    sel = torch.arange(NB, device=DEV, dtype=torch.int32).expand(1, H, NB, NB).contiguous()
+    with torch.cuda.stream(torch.cuda.Stream()):
+        marg, _ = usv.attn_entropy(q, k, sel, [NB, 10], torch.full((1, H, 64 * NB), 6.0, device=DEV))
+        torch.cuda.synchronize()
+        assert binding._workspace(torch.device(DEV), 0).numel() == 256
+    assert bool((marg > 0).all())
