@@ -6,7 +6,7 @@ import torch
 
 import oracle
 import usv_inputs as ui
-from parity_utils import attn_errors
+from parity_utils import attention_path, attn_errors
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -19,11 +19,13 @@ def usv():
     return m
 
 
-# an odd number of query blocks and a partial last block, k just above the small-call line; more
-# query blocks than that line with short lists; union lists beyond a ring slot (512 entries)
-@pytest.mark.parametrize("B,H,grid,kph", [(1, 1, (3, 9, 25), [9]), (2, 3, (5, 31, 33), [3, 1, 8]),
-                                          (1, 1, (9, 62, 66), [515])])
-def test_head_width_64(usv, B, H, grid, kph):
+# an odd number of query blocks and a partial last block on either side of the longest list of small calls (10 entries); more
+# query blocks than those with short lists; union lists beyond a ring slot (512 entries); more work than runs without a plan
+@pytest.mark.parametrize("path,B,H,grid,kph", [
+    ("one kernel", 1, 1, (3, 9, 25), [9]), ("no plan", 1, 1, (3, 12, 25), [11]), ("no plan", 2, 3, (5, 31, 33), [3, 1, 8]),
+    ("plan", 1, 1, (9, 62, 66), [515]), ("plan", 1, 8, (10, 32, 32), [30, 29, 40])])
+def test_head_width_64(usv, path, B, H, grid, kph):
+    kph = (kph * H)[:H]
     wl = ui.Workload("d64_edges", 170 + len(kph), B, H, 64, grid, (100,))
     N, NB = wl.N, wl.NB
     q, k, v = ui.make_qkv(wl, layout="bnhd")
@@ -33,8 +35,9 @@ def test_head_width_64(usv, B, H, grid, kph):
         for h in range(H):
             for i in range(NB):
                 sel[b, h, i, :kph[h]] = np.sort(rng.choice(NB, size=kph[h], replace=False))
-    o, o32, lse = usv.sparse_attn_fwd(q.to(DEV), k.to(DEV), v.to(DEV), torch.from_numpy(sel).to(DEV), kph, N=N,
-                                      return_f32=True, return_lse=True)
+    args = (q.to(DEV), k.to(DEV), v.to(DEV), torch.from_numpy(sel).to(DEV), kph, N)
+    assert attention_path(lambda: usv.sparse_attn_fwd(*args), B * H * NB) == path
+    o, o32, lse = usv.sparse_attn_fwd(*args, return_f32=True, return_lse=True)
     torch.cuda.synchronize()
     assert usv.workspace_status() == 0 and usv.sparse_attn_fallbacks() == 0
     o_ref, lse_ref = oracle.sparse_attn(q, k, v, N, sel, kph)
@@ -45,27 +48,37 @@ def test_head_width_64(usv, B, H, grid, kph):
     assert np.abs(lse.cpu().numpy() - lse_ref.reshape(B, H, NB * 64)[:, :, :N]).max() <= 2e-3
 
 
-def test_an_infinity_reaches_only_the_query_blocks_that_selected_it(usv):
-    """Two query blocks share an item; the second one alone selects a block with an infinity in V.
+# small calls, which keep query blocks apart, items of neighbours, and items of a plan, which pairs the one block with another list
+# with the one that is left of those with the same
+@pytest.mark.parametrize("path,H,NB,K,with_inf", [("one kernel", 1, 12, 9, slice(1, None, 2)), ("no plan", 1, 14, 11, slice(1, None, 2)),
+                                                  ("no plan", 2, 80, 15, slice(7, 8)), ("plan", 4, 120, 80, slice(1, 2))])
+def test_an_infinity_reaches_only_the_query_blocks_that_selected_it(usv, path, H, NB, K, with_inf):
+    """Two query blocks share an item; one alone selects a block with an infinity in V.
     Its own rows are not finite, its partner's equal the result without that block."""
-    N, NB, K, d = 64 * 12, 12, 9, 64
+    N, d = 64 * NB, 64
     g = torch.Generator().manual_seed(d)
-    q, k, v = (torch.randn(1, 1, N, d, generator=g).to(torch.bfloat16) for _ in range(3))
-    v[:, :, 64 * 11 + 5, 3] = float("inf")
-    sel = torch.arange(K, dtype=torch.int32).expand(1, 1, NB, K).clone()
-    sel[0, 0, 1::2, K - 1] = 11
-    args = (q.to(DEV), k.to(DEV), v.to(DEV), sel.to(DEV), [K])
-    o = usv.sparse_attn_fwd(*args).float().cpu()[0, 0].reshape(NB, 64, d)
-    exact = usv.sparse_attn_fwd(*args, impl=1).float().cpu()[0, 0].reshape(NB, 64, d)
-    assert torch.isfinite(o[0::2]).all()
-    assert not torch.isfinite(o[1::2, :, 3]).any()
-    assert (o[0::2] - exact[0::2]).abs().max() <= MAX_ABS
+    q, k, v = (torch.randn(1, H, N, d, generator=g).to(torch.bfloat16) for _ in range(3))
+    v[:, 0, 64 * (NB - 1) + 5, 3] = float("inf")
+    sel = torch.arange(K, dtype=torch.int32).expand(1, H, NB, K).clone()
+    sel[0, 0, with_inf, K - 1] = NB - 1
+    args = (q.to(DEV), k.to(DEV), v.to(DEV), sel.to(DEV), [K] * H)
+    assert attention_path(lambda: usv.sparse_attn_fwd(*args), H * NB) == path
+    o = usv.sparse_attn_fwd(*args).float().cpu()[0].reshape(H, NB, 64, d)
+    if path != "one kernel":
+        assert usv.sparse_attn_fallbacks() == 2 * len(range(NB)[with_inf])        # they did share items, and were recomputed
+    exact = usv.sparse_attn_fwd(*args, impl=1).float().cpu()[0].reshape(H, NB, 64, d)
+    hit = torch.zeros(H, NB, dtype=torch.bool)
+    hit[0, with_inf] = True
+    assert torch.isfinite(o[~hit]).all()
+    assert not torch.isfinite(o[hit][..., 3]).any()
+    assert (o[~hit] - exact[~hit]).abs().max() <= MAX_ABS
 
 
-# without a plan, with one, and the kernel of small calls; the last with logits nine times the size
-@pytest.mark.parametrize("B,H,grid,k,amp", [(1, 2, (4, 20, 24), 6, 1.0), (2, 3, (5, 31, 33), 20, 1.0), (1, 1, (3, 9, 25), 5, 1.0),
-                                            (1, 4, (6, 32, 32), 30, 3.0)])
-def test_log_sum_exp_is_fp32_exact(usv, B, H, grid, k, amp):
+# the kernel of small calls, without a plan, with one; some with logits nine times the size
+@pytest.mark.parametrize("path,B,H,grid,k,amp", [
+    ("one kernel", 1, 2, (4, 20, 24), 6, 1.0), ("no plan", 2, 3, (5, 31, 33), 20, 1.0), ("one kernel", 1, 1, (3, 9, 25), 5, 1.0),
+    ("no plan", 1, 4, (6, 32, 32), 30, 3.0), ("plan", 1, 8, (10, 32, 32), 30, 3.0)])
+def test_log_sum_exp_is_fp32_exact(usv, path, B, H, grid, k, amp):
     """The log-sum-exp comes from unrounded weights.  Bound: logits in base 2 of up to 100 carry an fp32 rounding of
     100 x 2^-24 = 6e-6 each from the product and from the reference, exp2 2^-22 and the sum of up to 1920 weights in
     four chains 480 x 2^-24 = 2.9e-5 if every rounding went the same way; seen: 1.2e-5."""
@@ -74,7 +87,9 @@ def test_log_sum_exp_is_fp32_exact(usv, B, H, grid, k, amp):
     q, kk, v = ui.make_qkv(wl)
     q, kk = (q.float() * amp).to(torch.bfloat16), (kk.float() * amp).to(torch.bfloat16)
     sel = np.sort(np.argsort(np.random.default_rng(k).random((B, H, NB, NB)), axis=-1)[..., :k].astype(np.int32), axis=-1)
-    _, lse = usv.sparse_attn_fwd(q.to(DEV), kk.to(DEV), v.to(DEV), torch.from_numpy(sel).to(DEV), [k] * H, return_lse=True)
+    args = (q.to(DEV), kk.to(DEV), v.to(DEV), torch.from_numpy(sel).to(DEV), [k] * H)
+    assert attention_path(lambda: usv.sparse_attn_fwd(*args, return_lse=True), B * H * NB) == path
+    _, lse = usv.sparse_attn_fwd(*args, return_lse=True)
     assert usv.workspace_status() == 0
     _, ref = oracle.sparse_attn(q, kk, v, N, sel, [k] * H)
     assert np.abs(lse.cpu().numpy() - ref.reshape(B, H, NB * 64)[:, :, :N]).max() <= 4e-5
