@@ -274,7 +274,7 @@ def merge_path_rooflines(usv, device, peak_gbs):
         hbm_entry("usv_token_merge(metric=NULL)", "plan_lists_kernel + merge_kernel", moved, ms_apply, peak_gbs,
                   "merge_kernel streams the bytes; the clearing and building of the lists before it are latency-bound"),
         hbm_entry("usv_token_unmerge", "unmerge_kernel", moved, ms_unm, peak_gbs),
-        {"call": "usv_token_merge(metric)", "kernels": "desc + match_tc + recheck + match_exact + plan_select + plan_assign + merge",
+        {"call": "usv_token_merge(metric)", "kernels": "desc + match_tc + recheck + match_exact + plan_held + merge",
          "bound": "tensor (matching) + hbm (descriptors, merge)", "ms": ms_plan,
          "bytes_descriptors": int(desc_bytes), "bytes_merge": int(moved),
          "note": "whole call; the plan-building part is %.4f ms" % (ms_plan - ms_apply)},

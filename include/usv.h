@@ -148,10 +148,14 @@ int usv_select_blocks(int B, int H, int NBq, int NBk, const float* scores,
  * and gives a key block that only one of them selected zero weight for the other.  Results equal
  * the per-block definition for finite inputs, and at d = 64 for all inputs.  At d = 128 a NaN or
  * infinity in K or V inside a block that one query block of a pair selected can also reach the
- * output rows of its partner (0 * inf); blocks that neither selected are never read.  impl 1 keeps
- * query blocks fully separate.  Short lists at d = 64 (up to four kept key blocks with at most 384 query blocks over all
- * heads; a single one with more than 1800) and sequences of more than 4096 key blocks (262 144 tokens) run the impl 1
- * kernel whatever impl says.
+ * output rows of its partner (0 * inf); blocks that neither selected are never read.  Heads that keep every key
+ * block may be computed four query blocks at a time (d = 128, large calls), all of which see all blocks.  There, in
+ * an eighth of the weights, and at d = 64, in a fifth, what lies below 2^-126 of a row's first maximum counts as 2^-126 and not as 0,
+ * which shows beside values of 1e36 and more.
+ * impl 1 keeps query blocks fully separate.  So do these, whatever impl says: sequences of more than 4096 key blocks
+ * (262 144 tokens) and views whose heads or batch elements share rows (stride 0), on the impl 1 kernel; and at d = 64 short lists,
+ * of up to four kept key blocks with at most 384 query blocks over all heads and of single ones with more than 1800, with the results
+ * of impl 1 bit for bit, and of five to ten with at most as many query blocks as the GPU has SMs, which are summed up in four parts.
  */
 size_t usv_sparse_attn_workspace(int B, int H, int N, int d, int kmax);
 int usv_sparse_attn_fwd(int B, int H, int N, int d, const void* q, const usv_strides* sq,

@@ -208,8 +208,8 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
     fence_after();
     dep_sync();
     const uint32_t tmem = *s_tmem;
-    // Each role starts by handing registers over (service and output warps) or taking them
-    // (softmax warps): setmaxnreg, whole warpgroups.
+    // Each role starts by handing registers over (service warps) or taking them (softmax and output
+    // warps): setmaxnreg, whole warpgroups.
 
     if (warp == W_TMA) {
         // ===== Q and K producer (whole warp in the loop, one elected lane issues) ================

@@ -140,8 +140,8 @@ struct MergeLists {
 // pass that marks the merged sources (ties to the lowest source index) and writes dst_of / pos.
 // Key T of the r-th most confident source and the number of sources equal to T that still merge
 // (Eq. 10 with ties to the lowest index), for 0 < r < nA.  One CTA per batch element.
-// The first HELD * 1024 keys stay in registers over the four passes: 13.5 -> 8 us at 20 691 sources, where
-// every pass waited for the L2 again.
+// The first HELD * 1024 keys stay in registers over the four passes, each of which would wait for the L2 again (13.5 -> 8 us at
+// 20 691 sources, when this kernel still took them; see plan_held_kernel for the counts that it is left with).
 template <int HELD>
 __global__ void __launch_bounds__(1024) plan_select_kernel(int nA, int r, const float* __restrict__ u_s,
                                                            int2* __restrict__ tsel) {
@@ -485,8 +485,8 @@ __global__ void __launch_bounds__(1024) row_scan_kernel(int nB, const int32_t* _
 // requested before any is used, and the 32 sums over lanes are taken together (at every step a lane
 // hands half of its candidates over: 31 shuffles, where one candidate after the other takes 160), which
 // leaves candidate l in lane l.  Rows of three destinations (the window reaches one block along x) are asked for from one address a
-// row, 30 candidates at a time.  Bound: the reads of the candidates from L1 (a third of the adds and shuffles less changed
-// nothing).  2 x 16 380 sources, 27 candidates of 128: 73 -> 41 us (46 us without the bound on registers).
+// row, 30 candidates at a time.  Bound: the L1's data pipe, which the shuffles go through too (71 % busy), and the latency behind it
+// (half of a warp's wait is for loads, issue slots are 56 % busy; a third of the adds and shuffles less changed nothing).  2 x 16 380 sources, 27 candidates of 128: 73 -> 41 us (46 us without the bound on registers).
 // A CTA goes through neighbouring sources, whose windows share most of their rows in L1, where there are several waves of
 // them.  Whole merges, us, one source a warp / rows of three and several sources: 2 x 16 380 122 / 120, 4 x 24 570 196 / 181, 65 480
 // 144 / 136, 8 x 17 550 239 / 224.  OWN: a window of the own block alone has one candidate and needs no registers for 32: 2 x 16 380

@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(128 * G, PER) __cluster_dims__(CLC, 1, 1) scor
     constexpr int LD = D + 4, TPR = D / 8, RPI = 128 / TPR, ITERS = USV_BLOCK / RPI;
     float* s_k = s_mem;                          // [CL_MAX][LD]
     float* s_q = s_k + CL_MAX * LD;              // [CL_MAX / CLC][LD]
-    float* s_red = s_q + CL_MAX / CLC * LD;      // [2 buffers][2 blocks][RPI][LD]
+    float* s_red = s_q + CL_MAX / CLC * LD;      // [2 buffers][G blocks][RPI][LD]
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // (waited for before anything is written to a neighbour)
     dep_sync();
     const int rank = blockIdx.x, bh = blockIdx.y;
