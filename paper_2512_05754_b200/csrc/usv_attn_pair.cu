@@ -32,7 +32,7 @@
 //   warps 16-19  output: thread e <-> query row e reads the finished O row out of TMEM a quarter at
 //                a time, hands the accumulator back and stores from registers (to o, or, with the
 //                unmerge folded in, to every original token that reads the row back), while the
-//                softmax groups are already in the next item.  Warp 16 is the scout too: it draws items two
+//                softmax groups are already in the next item.  Warp 16 is the scout too: it draws items one or two
 //                ahead, copies their key-block lists into ring slots in shared memory and publishes them.  (That takes
 //                3000 to 6000 cycles of round trips to the L2 and of issue slots it has to wait for.  In the K producer, where
 //                it stood before, the third K tile of an item waited for it.)
@@ -63,7 +63,8 @@ constexpr int NWG = 4;                          // softmax warpgroups
 constexpr int VSTAGES = 3;                      // V tile stages
 constexpr int SBUF = 3;                         // S/P buffers in TMEM
 constexpr int NSLOT = 4;                        // item ring
-constexpr int LOOK = 2;                         // items published ahead of the one whose output is next (at most NSLOT - 1)
+constexpr int LOOK = 2;                         // items published ahead of the one whose output is next (at most NSLOT - 1), but
+constexpr int LONG = 8;                         // one where that one has this many tiles (see the scout)
 constexpr int LCAP = 512;                       // list entries a ring slot holds (longer lists are read from global memory)
 constexpr int MAX_NB = PLAN_MAX_NB;             // key blocks per sequence this kernel covers
 constexpr uint32_t ITEM_BYTES = 64 + LCAP * 4;
@@ -511,7 +512,11 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
         const uint32_t lane_base = tmem + ((uint32_t)((warp - W_EPI) * 32) << 16);
         int next = warp == W_EPI ? 0 : -1;               // item to publish; -1: none (any more)
         for (int m = 0;; ++m) {
+            // An item of LONG tiles gives time enough to publish the one after it later.  (Drawn earlier than needed, few items of unequal
+            // lists end up shared out in turn: 24 heads x 69 blocks at d = 64, a quarter of them full, 92.6 us drawn one ahead, 101 two, 85
+            // so; 12 x 70 at d = 128 65.5, 67.5, 64.3; lists of two or three blocks, 40 x 300, 173, 164, 164.)
             while (next >= 0 && next <= m + LOOK) {
+                if (!DIRECT && next == m + LOOK && hdr_of(next - 1)[I_T] >= LONG) break;
                 const int T = publish(next);
                 if (T == -2) break;
                 next = T < 0 ? -1 : next + 1;
