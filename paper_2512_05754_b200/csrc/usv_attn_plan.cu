@@ -230,25 +230,38 @@ pair_plan_kernel(const AttnArgs a, int2* __restrict__ pairs, int* __restrict__ l
         // every list is the full set unless it has holes: pairing is arbitrary and every key block belongs to both sides
         for (int p = threadIdx.x; p < npairs; p += THREADS)
             out_pairs[p] = make_int2(I0 + 2 * p, 2 * p + 1 < nI ? I0 + 2 * p + 1 : -1);
-        uint32_t* mine = bm + 2 * warp * pitch;
-        for (int p = warp; p < npairs; p += THREADS / 32) {
-            int* out = out_lists + (int64_t)p * lstride;
-            const bool two = 2 * p + 1 < nI;
-            const int flags = two ? 3 : 1;
-            const int32_t* row = a.sel + ((int64_t)bh * NB + I0 + 2 * p) * a.kmax;
-            const int32_t* other = two ? row + a.kmax : row;
-            bool hole = false;
-#pragma unroll 4
-            for (int j = lane; j < NB; j += 32) {
-                out[1 + j] = (j << 2) | flags;
-                hole |= (unsigned)__ldg(row + j) >= (unsigned)NB || (unsigned)__ldg(other + j) >= (unsigned)NB;
+        // pairs warp, warp + 16, ...: their rows are read together (one pair after the other 8 heads x 101 blocks took 7 us longer)
+        constexpr int WARPS = THREADS / 32, P = CH / 2 / WARPS;
+        const int32_t* rows = a.sel + ((int64_t)bh * NB + I0 + 2 * warp) * a.kmax;
+        auto row = [&](int i, int side) { return rows + (int64_t)(2 * WARPS * i + side) * a.kmax; };
+        auto in = [&](int i, int side) { return 2 * (warp + WARPS * i) + side < nI; };
+        bool hole[P] = {};
+#pragma unroll 2
+        for (int j = lane; j < NB; j += 32) {
+            int at[P][2];
+#pragma unroll
+            for (int i = 0; i < P; ++i)
+#pragma unroll
+                for (int side = 0; side < 2; ++side) at[i][side] = in(i, side) ? __ldg(row(i, side) + j) : 0;
+#pragma unroll
+            for (int i = 0; i < P; ++i) {
+                hole[i] |= (unsigned)at[i][0] >= (unsigned)NB || (unsigned)at[i][1] >= (unsigned)NB;
+                if (in(i, 0)) out_lists[(int64_t)(warp + WARPS * i) * lstride + 1 + j] = (j << 2) | (in(i, 1) ? 3 : 1);
             }
+        }
+        uint32_t* mine = bm + 2 * warp * pitch;
+#pragma unroll 1
+        for (int i = 0; i < P && in(i, 0); ++i) {
+            int* out = out_lists + (int64_t)(warp + WARPS * i) * lstride;
             if (lane == 0) out[0] = NB;
-            if (!__any_sync(0xffffffffu, hole)) continue;
-            for (int i = lane; i < 2 * pitch; i += 32) mine[i] = 0u;
+            bool any = false;
+#pragma unroll
+            for (int q = 0; q < P; ++q) any = q == i ? hole[q] : any;
+            if (!__any_sync(0xffffffffu, any)) continue;
+            for (int w = lane; w < 2 * pitch; w += 32) mine[w] = 0u;
             __syncwarp();
             for (int j = lane; j < NB; j += 32) {
-                const unsigned ja = __ldg(row + j), jb = two ? __ldg(other + j) : -1;
+                const unsigned ja = __ldg(row(i, 0) + j), jb = in(i, 1) ? __ldg(row(i, 1) + j) : -1;
                 if (ja < (unsigned)NB) atomicOr(&mine[ja >> 5], 1u << (ja & 31));
                 if (jb < (unsigned)NB) atomicOr(&mine[pitch + (jb >> 5)], 1u << (jb & 31));
             }
