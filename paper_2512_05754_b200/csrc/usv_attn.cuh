@@ -52,7 +52,7 @@ bool attn_pair_supported(const AttnArgs& a, int d);
 bool attn_pair_direct(const AttnArgs& a, int d, int sms);
 int launch_attn_pair(const AttnArgs& a, int d, cudaStream_t st);
 // Heads that keep every key block and are better computed by the kernel of usv_attn_dense.cu (the first of a.head_order); 0: none.
-int attn_dense_heads(const AttnArgs& a, int d);
+int attn_dense_heads(const AttnArgs& a, int d, int sms);
 int launch_attn_dense(const AttnArgs& a, cudaStream_t st);
 // fused unmerge: copies the query blocks the exact kernel recomputed (into o) to their original tokens in y
 int launch_scatter_fallbacks(const AttnArgs& a, int d, cudaStream_t st);

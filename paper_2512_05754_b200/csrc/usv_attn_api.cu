@@ -114,7 +114,7 @@ static int sparse_attn_impl(int B, int H, int N, int d, const void* q, const usv
             a.work_flags = reinterpret_cast<const uint16_t*>(a.fallback_list);
             return launch_attn_mma(a, d, st);
         }
-        a.full_heads = attn_dense_heads(a, d);
+        a.full_heads = attn_dense_heads(a, d, sms);
         if (a.full_heads < H) {
             if ((rc2 = launch_pair_plan(a, plan_mem, st)) != USV_OK) return rc2;
         } else {

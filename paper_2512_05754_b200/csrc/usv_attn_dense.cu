@@ -487,25 +487,28 @@ static int dense_clusters() {
     return n;
 }
 
-// Calls whose heads are all full, beyond those without a plan, go here (us, pair kernel with a plan / this one: 12 heads x 30 blocks
-// 42.5 / 40.9; 24 x 28 48.2 / 45.4; 1 x 140 62.6 / 58.2; 1 x 317 250 / 224; 4 x 317 672 / 607; 12 x 317 1899 / 1687; 1 x 1857 5671 / 5102; 1000 x 3
-// 88.5 / 64.6; 2400 x 5 267 / 252; 1600 x 7 288 / 249; 800 x 8 190 / 167).  An item has four query blocks however many of them there are: with one
-// or two left for the last item, sequences of 9 to 18 blocks are faster there (900 x 9 258 / 267, 800 x 10 215 / 221, 600 x 13 267 / 277, 600 x 14
-// 276 / 289, 400 x 17 289 / 291; but 400 x 21 401 / 397, 200 x 25 278 / 268).  Two tiles an item are the least (see the softmax warps).
+// Calls whose heads are all full, beyond those without a plan, go here where waves of items take less time than on the paired kernel,
+// whose items have two query blocks: a wave is a tenth shorter here, but the last one may be emptier, and an item has room for four
+// query blocks however many are left for it.  us, pair kernel with a plan / this one, with the waves of either: 12 heads x 30 blocks 42.5 / 40.9
+// (2 / 2), 24 x 28 48.2 / 45.4 (3 / 3), 1 x 140 62.6 / 58.2 (1 / 1), 24 x 53 131 / 119 (5 / 5), 12 x 101 254 / 229 (5 / 5), 12 x 317 1899 / 1687 (13 / 13),
+// 1 x 1857 5671 / 5102 (7 / 7), 400 x 21 401 / 397 (30 / 33); but 8 x 73 74 / 91 (2 / 3), 16 x 53 79 / 88 (3 / 4), 40 x 21 46 / 52 (3 / 4), 240 x 10
+// 63.4 / 65.5 (9 / 10), 400 x 17 289 / 291 (25 / 28), 600 x 14 276 / 289 (29 / 33), 900 x 9 258 / 267 (31 / 37).  Up to eight blocks what an item costs
+// beside its tiles counts, and there are half as many here: 1000 x 3 88.5 / 64.6, 800 x 4 140 / 99, 2400 x 5 267 / 252, 600 x 6 123 / 117, 800 x 8 190 / 167.
+// Two tiles an item are the least (see the softmax warps).
 // Where other heads are sparse the two kernels run one after the other, and what the last, partly empty wave of
 // this one leaves idle has to be won back: 16 heads x 317 blocks, four of them full (4.3 waves), 978 / 1007; 24 heads, six full
 // (6.5 waves), 1435 / 1403; 48 x 122, twelve full (5.0 waves), 491 / 502.
-int attn_dense_heads(const AttnArgs& a, int d) {
+int attn_dense_heads(const AttnArgs& a, int d, int sms) {
     int full = 0;
     while (full < a.H && a.k_per_head[a.head_order[full]] >= a.NB) ++full;
     if (full == 0 || d != dn::D || a.y != nullptr || a.NB < 3) return 0;
-    if ((a.NB & 3) != 0 && (a.NB & 3) != 3 && a.NB >= 9 && a.NB <= 18) return 0;
-    const int64_t items = (int64_t)a.B * full * ((a.NB + 3) / 4);
+    const int64_t items = (int64_t)a.B * full * ((a.NB + 3) / 4), pairs = (int64_t)a.B * full * ((a.NB + 1) / 2);
     if (items > 1000000000LL) return 0;
     const int clusters = dense_clusters();
     if (clusters <= 0) return 0;
     const int64_t waves = (items + clusters - 1) / clusters;
-    return full == a.H || (waves > 6 && 10 * items >= 9 * waves * clusters) ? full : 0;
+    if (full == a.H) return a.NB <= 8 || 9 * waves < 10 * ((pairs + sms - 1) / sms) ? full : 0;
+    return waves > 6 && 10 * items >= 9 * waves * clusters && 9 * waves * sms < 10 * pairs ? full : 0;
 }
 
 int launch_attn_dense(const AttnArgs& a, cudaStream_t st) {
