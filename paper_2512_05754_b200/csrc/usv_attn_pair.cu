@@ -63,8 +63,7 @@ constexpr int NWG = 4;                          // softmax warpgroups
 constexpr int VSTAGES = 3;                      // V tile stages
 constexpr int SBUF = 3;                         // S/P buffers in TMEM
 constexpr int NSLOT = 4;                        // item ring
-constexpr int LOOK = 2;                         // items published ahead of the one whose output is next (at most NSLOT - 1), but
-constexpr int LONG = 8;                         // one where that one has this many tiles (see the scout)
+constexpr int LOOK = 2;                         // items published ahead of the one whose output is next (at most NSLOT - 1)
 constexpr int LCAP = 512;                       // list entries a ring slot holds (longer lists are read from global memory)
 constexpr int MAX_NB = PLAN_MAX_NB;             // key blocks per sequence this kernel covers
 constexpr uint32_t ITEM_BYTES = 64 + LCAP * 4;
@@ -79,6 +78,7 @@ constexpr uint32_t ITEM_BYTES = 64 + LCAP * 4;
 template <int D>
 struct Cfg {
     static constexpr int NH = D / 64;               // column halves of a tile
+    static constexpr int LONG = D == 64 ? 8 : 10;   // tiles of an item that lets the scout wait (see there)
     static constexpr int KSTAGES = D == 64 ? 4 : 2; // K tile stages
     static constexpr uint32_t TILE_BYTES = KT * D * 2;
     // A NaN or infinity in V of a key block that only one side selected reaches the other side's rows
@@ -512,11 +512,13 @@ attn_pair_kernel(const AttnArgs a, const __grid_constant__ Maps maps) {
         const uint32_t lane_base = tmem + ((uint32_t)((warp - W_EPI) * 32) << 16);
         int next = warp == W_EPI ? 0 : -1;               // item to publish; -1: none (any more)
         for (int m = 0;; ++m) {
-            // An item of LONG tiles gives time enough to publish the one after it later.  (Drawn earlier than needed, few items of unequal
+            // An item of F::LONG tiles gives time enough to publish the one after it later.  (Drawn earlier than needed, few items of unequal
             // lists end up shared out in turn: 24 heads x 69 blocks at d = 64, a quarter of them full, 92.6 us drawn one ahead, 101 two, 85
-            // so; 12 x 70 at d = 128 65.5, 67.5, 64.3; lists of two or three blocks, 40 x 300, 173, 164, 164.)
+            // so; 12 x 70 at d = 128 65.5, 67.5, 64.3; lists of two or three blocks, 40 x 300, 173, 164, 164.  The lines, 8 / 10 / 12 tiles:
+            // d = 128, 16 x 128, keep 13 87.2 / 86.0 / 85.6, 40 x 90, keep 14 138.6 / 136.7 / 136.3, 12 x 140, keep 21 101.3 / 101.5 / 105;
+            // d = 64, 16 x 160, keep 16 85.3 / 87.2 / 85.6, 24 x 120, keep 18 103.9 / 103.9 / 105.5.)
             while (next >= 0 && next <= m + LOOK) {
-                if (!DIRECT && next == m + LOOK && hdr_of(next - 1)[I_T] >= LONG) break;
+                if (!DIRECT && next == m + LOOK && hdr_of(next - 1)[I_T] >= F::LONG) break;
                 const int T = publish(next);
                 if (T == -2) break;
                 next = T < 0 ? -1 : next + 1;
