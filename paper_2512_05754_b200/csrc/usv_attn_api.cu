@@ -98,8 +98,8 @@ static int sparse_attn_impl(int B, int H, int N, int d, const void* q, const usv
     // keep 4 11.6 / 14.2, 6 15.9 / 16.1, 8 20.0 / 17.6; 512, keep 2 11.5 / 13.1, 3 15.0 / 13.9.
     const int64_t blocks = (int64_t)B * H * NB;
     const bool small = d == 64 && kmx <= 4 && blocks <= 384;
-    // Where every query block has an SM to itself, four groups of warps take its list side by side: 32 blocks, keep 4 8.3 / 7.35,
-    // 8 11.4 / 9.4, 16 13.7 / 15.2; 128, keep 2 7.0 / 5.4, 4 10.7 / 7.4, 8 12.1 / 9.7; 100, keep 10 13.7 / 11.5; 256, keep 4 11.9 / 12.9
+    // Where every query block has an SM to itself, four groups of warps take its list side by side: 32 blocks, keep 4 8.3 / 7.0,
+    // 8 11.4 / 9.4, 16 13.7 / 15.2; 128, keep 2 7.0 / 5.2, 4 10.7 / 7.1, 8 12.1 / 9.7; 100, keep 10 13.7 / 11.5; 256, keep 4 11.9 / 12.9
     // (other kernels / these).  At d = 128 it never pays (32, keep 4 10.8 / 13.1).
     int sms;
     if ((rc = sm_count(&sms)) != USV_OK) return rc;

@@ -383,23 +383,26 @@ int launch_attn_split(const AttnArgs& a, cudaStream_t st) {
 // i loads entry i and takes its logits and, when the four maxima of a row are known, its weights, which every group
 // then multiplies with a quarter of V's columns.  Maxima, sums and products come in the order of the list, so the result is that
 // of attn_mma_block bit for bit.  Bound: the chain launch, loads, MMAs and the softmax between them, and 0.85 us an entry for its
-// MMAs.  Calls at D = 64, us, one group / groups with maxima of their own / this kernel: 32 blocks, keep 4 8.3 / 7.3 / 7.35; 128, keep
-// 2 7.0 / 5.8 / 5.4, keep 4 10.7 / 7.4 / 7.4; 40, keep 3 7.3 / 6.45 / 6.35.  (Several rounds of four entries, with all groups waiting for
+// MMAs.  Calls at D = 64, us, one group / groups with maxima of their own / this kernel: 32 blocks, keep 4 8.3 / 7.3 / 7.0; 128, keep
+// 2 7.0 / 5.8 / 5.2, keep 4 10.7 / 7.4 / 7.1; 40, keep 3 7.3 / 6.45 / 6.15.  (Several rounds of four entries, with all groups waiting for
 // one another in each, take longer than groups of their own: 128 blocks, keep 8 11.9 / 9.9.)
-template <int D>
+template <int D, bool LSE>
 struct FourSmem {
     static constexpr int TILE = MmaSmem<D>::TILE, G = 4;
     static constexpr size_t TILES = (size_t)TILE * (1 + 2 * G) * sizeof(__nv_bfloat16);   // Q, K and V; P takes the place of K
     static constexpr size_t MAXIMA = G * USV_BLOCK * sizeof(float);
-    static constexpr size_t SUMS = (size_t)G * 8 * USV_BLOCK * 4 * sizeof(float);   // unrounded pairs, for the log-sum-exp
-    static constexpr size_t BYTES = TILES + MAXIMA + SUMS;
+    static constexpr size_t SUMS = LSE ? (size_t)G * 8 * USV_BLOCK * 4 * sizeof(float) : 0;   // unrounded pairs, for the log-sum-exp
+    // More than half of an SM's, so that no two CTAs share one while others idle (a layer of 8 heads x 15 blocks 14.5 us with 85 KB, 12.2
+    // so: CTAs may start where the kernel before has already left).
+    static constexpr size_t ALONE = 118 * 1024;
+    static constexpr size_t BYTES = TILES + MAXIMA + SUMS > ALONE ? TILES + MAXIMA + SUMS : ALONE;
 };
 
-template <int D>
+template <int D, bool LSE>
 __global__ void __launch_bounds__(512) attn_four_kernel(const AttnArgs a) {
     dep_sync();
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    using F = FourSmem<D>;
+    using F = FourSmem<D, LSE>;
     constexpr int LD = MmaSmem<D>::LD, TILE = F::TILE, G = F::G;
     constexpr int NC = D / G / 8;   // n-tiles of the output a group has
     static_assert(NC == 2, "one ldmatrix of V per k-step");
@@ -448,20 +451,19 @@ __global__ void __launch_bounds__(512) attn_four_kernel(const AttnArgs a) {
         if (tig < 2) s_max[grp * USV_BLOCK + row + 8 * tig] = tig ? mx[1] : mx[0];
     }
     __syncthreads();
-    float alpha[G][2], ms[2] = {0.f, 0.f};
+    float ms[2] = {-INFINITY, -INFINITY};   // the running maxima at the group's entry
 #pragma unroll
     for (int t = 0; t < G; ++t)
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            float at;
-            alpha[t][r] = t < entries ? next_max(m[r], s_max[t * USV_BLOCK + row + 8 * r], c, at) : 1.f;
-            if (t == grp && t < entries) ms[r] = at;
-        }
+        for (int r = 0; r < 2; ++r)
+            if (t <= grp && t < entries) ms[r] = fmaxf(ms[r], s_max[t * USV_BLOCK + row + 8 * r] * c);
+#pragma unroll
+    for (int r = 0; r < 2; ++r) ms[r] = ms[r] == -INFINITY ? 0.f : ms[r];
     if (grp < entries) {
         uint32_t pf[4][4];
         float* sums = s_sum + grp * (8 * USV_BLOCK * 4) + row * 4 + tig;
         tile_weights(s, c, ms, pf, [&](int nt, int r, float e, uint32_t) {
-            if (a.lse != nullptr) sums[nt * (USV_BLOCK * 4) + r * 32] = e;
+            if (LSE) sums[nt * (USV_BLOCK * 4) + r * 32] = e;
         });
         __nv_bfloat16* P = k_tile(grp) + row * LD + 2 * tig;   // (nobody reads the K tile any more)
 #pragma unroll
@@ -472,15 +474,17 @@ __global__ void __launch_bounds__(512) attn_four_kernel(const AttnArgs a) {
     }
     cp_async_wait_all();   // V
     __syncthreads();
+#pragma unroll 4
+    for (int t = 0; t < entries; ++t) {
+        float alpha[2], at;   // (taken here and not for all entries beforehand: the layer of 2 x 16 blocks 12.05 us, 12.45 so)
 #pragma unroll
-    for (int t = 0; t < G; ++t) {
-        if (t >= entries) break;
+        for (int r = 0; r < 2; ++r) alpha[r] = next_max(m[r], s_max[t * USV_BLOCK + row + 8 * r], c, at);
         const __nv_bfloat16* prow = k_tile(t) + (warp * 16 + (lane & 15)) * LD + (lane >> 4) * 8;
         const __nv_bfloat16* vrow = k_tile(t) + TILE + (lane & 15) * LD + grp * (8 * NC) + (lane >> 4) * 8;
 #pragma unroll
         for (int i = 0; i < NC; ++i)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) o[i][e] *= alpha[t][e >> 1];
+            for (int e = 0; e < 4; ++e) o[i][e] *= alpha[e >> 1];
 #pragma unroll
         for (int kt = 0; kt < 4; ++kt) {
             uint32_t pf[4], bfr[4];
@@ -492,16 +496,16 @@ __global__ void __launch_bounds__(512) attn_four_kernel(const AttnArgs a) {
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {   // 8-key piece 2 kt + e
                     const float w = sum_bf16x2(own ? pf[2 * e + 1] : pf[2 * e]);
-                    sum = kt == 0 && e == 0 ? fmaf(sum, own ? alpha[t][1] : alpha[t][0], w) : sum + w;
+                    sum = kt == 0 && e == 0 ? fmaf(sum, own ? alpha[1] : alpha[0], w) : sum + w;
                 }
             }
         }
-        if (grp >= 2 && a.lse != nullptr) {
+        if (LSE && grp >= 2) {
             const float* sums = s_sum + t * (8 * USV_BLOCK * 4) + (row + 8 * own) * 4 + tig;
 #pragma unroll
             for (int nt = 0; nt < 8; ++nt) {
                 const float e = sums[nt * (USV_BLOCK * 4)];
-                sum = nt == 0 ? fmaf(sum, own ? alpha[t][1] : alpha[t][0], e) : sum + e;
+                sum = nt == 0 ? fmaf(sum, own ? alpha[1] : alpha[0], e) : sum + e;
             }
         }
     }
@@ -509,7 +513,7 @@ __global__ void __launch_bounds__(512) attn_four_kernel(const AttnArgs a) {
     sum += __shfl_xor_sync(0xffffffffu, sum, 1);
     sum += __shfl_xor_sync(0xffffffffu, sum, 2);
     if (tig == 0 && grp < 2) s_max[grp * USV_BLOCK + row] = sum;   // (nobody reads the maxima any more)
-    if (tig == 0 && grp >= 2 && a.lse != nullptr) {
+    if (LSE && tig == 0 && grp >= 2) {
         const int at = I * USV_BLOCK + row + 8 * own;
         if (at < N) a.lse[((int64_t)b * a.H + h) * N + at] = sum > 0.f ? ((own ? m[1] : m[0]) + log2f(sum)) * 0.69314718055994531f : 0.f;
     }
@@ -536,14 +540,19 @@ __global__ void __launch_bounds__(512) attn_four_kernel(const AttnArgs a) {
             *reinterpret_cast<const uint4*>(stage + (lane >> 1) * LD + (lane & 1) * 8);
 }
 
-int launch_attn_four(const AttnArgs& a, cudaStream_t st) {
-    constexpr size_t smem = FourSmem<64>::BYTES;
+template <int D, bool LSE>
+static int launch_four(const AttnArgs& a, cudaStream_t st) {
+    constexpr size_t smem = FourSmem<D, LSE>::BYTES;
     static_assert(smem <= 232448, "shared memory budget");
-    cudaError_t e = cudaFuncSetAttribute(attn_four_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(attn_four_kernel<D, LSE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return fail(USV_ERR_CUDA, "sparse_attn: smem attribute: %s", cudaGetErrorString(e));
-    launch_dep_smem(attn_four_kernel<64>, dim3((unsigned)(a.B * a.H * a.NB)), dim3(512), smem, st, a);
+    launch_dep_smem(attn_four_kernel<D, LSE>, dim3((unsigned)(a.B * a.H * a.NB)), dim3(512), smem, st, a);
     USV_CHECK_LAUNCH("attn_four_kernel");
     return USV_OK;
+}
+
+int launch_attn_four(const AttnArgs& a, cudaStream_t st) {
+    return a.lse != nullptr ? launch_four<64, true>(a, st) : launch_four<64, false>(a, st);
 }
 
 // Lists of one block: nothing follows the first K and V tile, and without a second buffer twice as many CTAs share an SM.
